@@ -127,6 +127,11 @@ struct PrbSubStreams {
 int prb_launch_sample(const PrbView& v, uint32_t B, float beta, uint64_t seed, int32_t* d_idx, float* d_w,
                       const PrbBatch& dst, cudaStream_t s, int uniform = 0, uint32_t n_sub = 1,
                       const PrbSubStreams* subs = nullptr, int buffer_norm = 0);
+// The same for short rows of a buffer without frames, in one launch (prb_sample_short.cu).
+int prb_launch_sample_short(const PrbView& v, uint32_t B, float beta, uint64_t seed, int32_t* d_idx, float* d_w, const PrbBatch& dst,
+                            cudaStream_t s, int uniform, int buffer_norm);
+// The scan of the leaves for their smallest positive one, into PrbState::pmin_bits.
+int prb_launch_leaf_min(const PrbView& v, cudaStream_t s);
 // A sample of long rows as two kernels.  The first walks the tree and leaves, in a hand-off area of the
 // slab (one of PrbView::handoff), what the second needs: a header, the leaf index of every stratum and
 // that leaf's priority.  The second copies the rows (and turns the priorities into weights meanwhile).

@@ -478,159 +478,24 @@ prb_sample_kernel(const __grid_constant__ PrbView v, uint32_t B, float beta, uin
     }
 }
 
-// ---- large batches of short rows: one stratum per thread -------------------------------------------
-// With thousands of strata the K-lane groups above keep too few tree reads in flight (a CTA walks
-// 256 / K strata at a time, round after round).  Here every thread walks a stratum of its own: it
-// loads the K children of its node itself (one 8..128-byte group: whole sectors), forms the same
-// left-to-right binary32 prefix sums one after another and enters the first child whose prefix
-// exceeds the binary64 target -- the count of prefixes the target has passed, as the lanes' ballot
-// gives it.  A CTA takes a contiguous range of strata, 256 at a time: targets, descents, index and raw
-// weight per thread; then all its threads copy the rows, granule by granule (consecutive threads,
-// consecutive granules), up to sixteen loads in flight each.  Every CTA raises the batch's largest raw
-// weight with one atomic maximum (positive binary64 values order like their bit patterns); a second,
-// small launch divides all raw weights by it.
-constexpr uint32_t kWideSampleFrom = 2048;      // batches of at least this many strata (short rows)
-constexpr uint32_t kWideSampleStrata = 32;      // ... spread over CTAs of at least this many strata
-
-// Short rows of strata [k_first, k_first + n_rows) by all `nthreads` threads, field by field, in
-// granules of type T: up to U granules per thread are loaded before the first is stored.
-template <typename T, int U>
-__device__ __forceinline__ void gather_field_deep(const T* __restrict__ store, T* __restrict__ out, uint32_t W, uint32_t Wp, uint32_t total,
-                                                  const uint32_t* s_idx, uint32_t rank, uint32_t nthreads)
-{
-    for (uint32_t e0 = rank; e0 < total; e0 += nthreads * U) {
-        T tmp[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const uint32_t e = e0 + u * nthreads;
-            if (e < total) {
-                const uint32_t r = (W == 1) ? e : e / W;
-                tmp[u] = store[(uint64_t)s_idx[r] * Wp + (e - r * W)];     // (s_idx comes from a descent, checked there; Wp: granules per slot)
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const uint32_t e = e0 + u * nthreads;
-            if (e < total) out[e] = tmp[u];
-        }
-    }
-}
-
-__device__ __forceinline__ void gather_short_fields_deep(const PrbView& v, const PrbBatch& dst, uint32_t k_first, uint32_t n_rows,
-                                                         const uint32_t* s_idx, uint32_t rank, uint32_t nthreads)
-{
-    for (int f = 0; f < PRB_NUM_FIELDS; ++f) {
-        if (dst.ptr[f] == nullptr || v.field_bytes[f] == 0) continue;
-        const uint32_t vec = v.field_vec[f], W = v.field_bytes[f] / vec, Wp = v.field_pitch[f] / vec, total = n_rows * W;
-        const unsigned char* src = v.store[f];
-        unsigned char* out = dst.ptr[f] + (uint64_t)k_first * v.field_bytes[f];
-        switch (vec) {
-        case 16: gather_field_deep<uint4, 4>(reinterpret_cast<const uint4*>(src), reinterpret_cast<uint4*>(out), W, Wp, total, s_idx, rank, nthreads); break;
-        case 8: gather_field_deep<uint2, 8>(reinterpret_cast<const uint2*>(src), reinterpret_cast<uint2*>(out), W, Wp, total, s_idx, rank, nthreads); break;
-        case 4: gather_field_deep<uint32_t, 16>(reinterpret_cast<const uint32_t*>(src), reinterpret_cast<uint32_t*>(out), W, Wp, total, s_idx, rank, nthreads); break;
-        case 2: gather_field_deep<uint16_t, 8>(reinterpret_cast<const uint16_t*>(src), reinterpret_cast<uint16_t*>(out), W, Wp, total, s_idx, rank, nthreads); break;
-        default: gather_field_deep<unsigned char, 8>(src, out, W, Wp, total, s_idx, rank, nthreads); break;
-        }
-    }
-}
-
-template <int K>
-__global__ void __launch_bounds__(kThreads, kCtasPerSm)
-prb_sample_wide_kernel(const __grid_constant__ PrbView v, uint32_t B, float beta, uint64_t seed,
-                       int32_t* __restrict__ out_idx, float* __restrict__ out_w, const __grid_constant__ PrbBatch dst,
-                       const __grid_constant__ SamplePlan plan)
-{
-    __shared__ __align__(16) float s_top[top_floats_of(K)];
-    __shared__ uint32_t s_idx[kThreads];
-    __shared__ unsigned long long s_wmax;
-    __shared__ unsigned s_flags;
-    __shared__ unsigned int s_last;
-    const uint32_t tid = threadIdx.x;
-    const unsigned long long calls = v.state->sample_calls;
-    const unsigned long long fill = v.state->fill;
-    const float total32 = __ldg(v.level[0]);
-    {
-        const float4* src = reinterpret_cast<const float4*>(v.level[1]);
-        for (uint32_t q = tid; q < plan.top_vec4; q += kThreads) reinterpret_cast<float4*>(s_top)[q] = __ldg(src + q);
-    }
-    if (tid == 0) { s_wmax = 0ull; s_flags = 0u; }
-    const bool empty = (fill == 0) || !(total32 > 0.0f);
-    const double total = (double)total32;
-    const uint32_t k_lo = (uint32_t)(((uint64_t)blockIdx.x * B) / gridDim.x);
-    const uint32_t k_hi = (uint32_t)(((uint64_t)(blockIdx.x + 1) * B) / gridDim.x);
-    __syncthreads();
-    unsigned long long my_wmax = 0ull;
-    unsigned my_flags = 0u;
-    for (uint32_t kb = k_lo; kb < k_hi && !empty; kb += kThreads) {
-        const uint32_t k = kb + tid, n_here = min(kThreads, k_hi - kb);
-        if (k < k_hi) {
-            // target of stratum k (Eq. 1's x, one per equal segment of the total), then the walk
-            const double x = prb_stratum_target(k, B, total, calls, seed);
-            uint32_t leaf; float p;
-            prb_descend_alone<K>(v, plan.top_levels, plan.top_off, s_top, x, leaf, p, my_flags);
-            s_idx[tid] = leaf;
-            out_idx[k] = (int32_t)leaf;
-            if (out_w != nullptr) {
-                const double wr = pow(__ddiv_rn(__dmul_rn((double)fill, (double)p), total), -(double)beta);
-                v.wraw[k] = wr;
-                my_wmax = max(my_wmax, (unsigned long long)__double_as_longlong(wr));
-            }
-        }
-        __syncthreads();
-        gather_short_fields_deep(v, dst, kb, n_here, s_idx, tid, kThreads);
-        __syncthreads();            // s_idx is rewritten by the next pass
-    }
-    if (my_wmax) atomicMax(&s_wmax, my_wmax);
-    if (my_flags) atomicOr(&s_flags, my_flags);
-    __syncthreads();
-    if (tid == 0) {
-        if (s_flags) atomicOr(&v.state->status, s_flags);
-        if (s_wmax) atomicMax(&v.state->wide_wmax_bits, s_wmax);
-        s_last = (prb_ticket(&v.state->sample_ticket) == gridDim.x - 1) ? 1u : 0u;
-    }
-    __syncthreads();
-    if (tid == 0 && s_last) {
-        // the last CTA to finish: the call's bookkeeping (the weights are divided by a launch of their own)
-        if (empty) atomicOr(&v.state->status, PEARL_ST_EMPTY);
-        else v.state->sample_calls = calls + 1;
-        v.state->sample_ticket = 0u;
-    }
-}
-
-// Second launch of a large-batch sample: w_k = raw weight / the batch's largest, by as many CTAs as
-// it takes (one CTA would need B / 1024 dependent round trips).  The largest raw weight is zero only
-// if the buffer was empty: then nothing is written.  The last CTA to have read it clears it.
-__global__ void __launch_bounds__(kThreads)
-prb_normalise_weights_kernel(const __grid_constant__ PrbView v, uint32_t B, float* __restrict__ out_w)
-{
-    const unsigned long long bits = __ldcg(&v.state->wide_wmax_bits);
-    if (bits) {
-        const double wmax = __longlong_as_double((long long)bits);
-        const uint32_t k0 = blockIdx.x * kThreads * 4u + threadIdx.x;
-        double held[4];
-#pragma unroll
-        for (uint32_t u = 0; u < 4; ++u) if (k0 + u * kThreads < B) held[u] = __ldcg(v.wraw + k0 + u * kThreads);
-#pragma unroll
-        for (uint32_t u = 0; u < 4; ++u) if (k0 + u * kThreads < B) out_w[k0 + u * kThreads] = (float)__ddiv_rn(held[u], wmax);
-    }
-    __syncthreads();        // every thread of the CTA has read the maximum
-    if (threadIdx.x == 0 && prb_ticket(&v.state->sample_ticket) == gridDim.x - 1) {
-        v.state->wide_wmax_bits = 0ull;
-        v.state->sample_ticket = 0u;
-    }
-}
-
 // The smallest positive leaf among the `fill` stored ones, into state->pmin_bits (all ones at creation and
 // again after every sample that used it): positive binary32 values order like their bit patterns.
-__global__ void prb_leaf_min_kernel(const __grid_constant__ PrbView v)
+// Bound by L2 bandwidth (the leaves of up to 2^24 slots stay there): eight 16-byte loads in flight per thread.
+// (a slot beyond the fill count has leaf 0, and so has the padding behind the last one: neither counts)
+__global__ void __launch_bounds__(256) prb_leaf_min_kernel(const __grid_constant__ PrbView v)
 {
-    const unsigned long long fill = v.state->fill;
-    const float* leaves = v.level[v.depth];
+    const float4* leaves = reinterpret_cast<const float4*>(v.level[v.depth]);
+    const uint64_t units = (v.level_alloc[v.depth] + 3u) / 4u, stride = (uint64_t)gridDim.x * blockDim.x;
     unsigned best = 0xFFFFFFFFu;
-    for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < fill;
-         i += (unsigned long long)gridDim.x * blockDim.x) {
-        const float p = __ldg(leaves + i);
-        if (p > 0.0f) best = min(best, __float_as_uint(p));
+    // (a zero leaf wraps to the largest value and never wins)
+    auto take = [&best](float p) { best = min(best, __float_as_uint(p) - 1u); };
+    constexpr int U = 8;
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < units; i += stride * U) {
+        float4 t[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) t[u] = i + u * stride < units ? __ldg(leaves + i + u * stride) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+        for (int u = 0; u < U; ++u) { take(t[u].x); take(t[u].y); take(t[u].z); take(t[u].w); }
     }
     __shared__ unsigned s_best[8];
     best = __reduce_min_sync(0xFFFFFFFFu, best);
@@ -638,7 +503,7 @@ __global__ void prb_leaf_min_kernel(const __grid_constant__ PrbView v)
     __syncthreads();
     if (threadIdx.x == 0) {
         for (unsigned w = 1; w < blockDim.x / 32u; ++w) best = min(best, s_best[w]);
-        if (best != 0xFFFFFFFFu) atomicMin(&v.state->pmin_bits, (unsigned long long)best);      // one atomic per CTA
+        if (best != 0xFFFFFFFFu) atomicMin(&v.state->pmin_bits, (unsigned long long)best + 1ull);      // one atomic per CTA
     }
 }
 
@@ -910,6 +775,16 @@ bool prb_sample_has_long_rows(const PrbView& v, const PrbBatch& dst)
     return v.stack == 0 && plan_row_mode(v, dst, plan);      // (rebuilt observations: the one-kernel sample only)
 }
 
+int prb_launch_leaf_min(const PrbView& v, cudaStream_t s)
+{
+    const uint64_t per_cta = 256ull * 32ull;
+    uint64_t ctas = (v.capacity + per_cta - 1) / per_cta;
+    const uint64_t most = (uint64_t)prb_sm_count() * 4;
+    if (ctas > most) ctas = most;
+    prb_leaf_min_kernel<<<(unsigned)ctas, 256, 0, s>>>(v);
+    return cudaGetLastError() == cudaSuccess ? 1 : -1;
+}
+
 int prb_launch_sample(const PrbView& v, uint32_t B, float beta, uint64_t seed, int32_t* d_idx, float* d_w,
                       const PrbBatch& dst, cudaStream_t s, int uniform, uint32_t n_sub, const PrbSubStreams* subs, int buffer_norm)
 {
@@ -918,6 +793,9 @@ int prb_launch_sample(const PrbView& v, uint32_t B, float beta, uint64_t seed, i
     const int dev = prb_current_device();
     SamplePlan plan;
     const bool row_mode = plan_row_mode(v, dst, plan);
+    // Short rows in one piece have a kernel of their own (prb_sample_short.cu); here: long rows, rebuilt
+    // observations, and the sub-batches of a streamed call.
+    if (!row_mode && n_sub == 1 && v.stack == 0) return prb_launch_sample_short(v, B, beta, seed, d_idx, d_w, dst, s, uniform, buffer_norm);
     plan.n_tasks = B * plan.tps;
     plan.first_task = 0;
     plan.ticket_total = 0;
@@ -928,23 +806,6 @@ int prb_launch_sample(const PrbView& v, uint32_t B, float beta, uint64_t seed, i
     plan_staged_top(v, uniform != 0, plan);
     const uint32_t R = kThreads / v.fanout;
     const int ki = v.log2_fanout;
-    if (!row_mode && n_sub == 1 && !uniform && !buffer_norm && B >= kWideSampleFrom && v.stack == 0) {
-        // a large batch of short rows: one stratum per thread
-        uint32_t grid = (B + kWideSampleStrata - 1) / kWideSampleStrata;
-        const uint32_t one_wave = (uint32_t)sm_count * kCtasPerSm;
-        if (grid > one_wave) grid = one_wave;
-        plan.ring_stages = 0; plan.ring_stage_bytes = 0; plan.pf_groups = 0; plan.pf_off = 0;
-        plan.ticket_total = grid;
-        switch (v.fanout) {
-        case 2: prb_sample_wide_kernel<2><<<grid, kThreads, 0, s>>>(v, B, beta, seed, d_idx, d_w, dst, plan); break;
-        case 4: prb_sample_wide_kernel<4><<<grid, kThreads, 0, s>>>(v, B, beta, seed, d_idx, d_w, dst, plan); break;
-        case 8: prb_sample_wide_kernel<8><<<grid, kThreads, 0, s>>>(v, B, beta, seed, d_idx, d_w, dst, plan); break;
-        case 16: prb_sample_wide_kernel<16><<<grid, kThreads, 0, s>>>(v, B, beta, seed, d_idx, d_w, dst, plan); break;
-        default: prb_sample_wide_kernel<32><<<grid, kThreads, 0, s>>>(v, B, beta, seed, d_idx, d_w, dst, plan); break;
-        }
-        if (d_w != nullptr) prb_normalise_weights_kernel<<<(B + kThreads * 4u - 1) / (kThreads * 4u), kThreads, 0, s>>>(v, B, d_w);
-        return cudaGetLastError() == cudaSuccess ? (d_w != nullptr ? 2 : 1) : -1;
-    }
     // dynamic shared memory a CTA of this kernel may have: what the device allows less its static part
     static uint32_t dyn_max[kPrbMaxDevices][6];
     if (dyn_max[dev][ki] == 0) {
@@ -1040,10 +901,7 @@ int prb_launch_sample(const PrbView& v, uint32_t B, float beta, uint64_t seed, i
     int extra_launches = 0;
     if (plan.buffer_norm && v.min_off == 0) {
         // the scan of the leaves goes first, on the caller's stream (no min-tree to read the minimum from)
-        const uint64_t per_cta = 256ull * 16ull;
-        uint64_t ctas = (v.capacity + per_cta - 1) / per_cta;
-        if (ctas > (uint64_t)sm_count * 4) ctas = (uint64_t)sm_count * 4;
-        prb_leaf_min_kernel<<<(unsigned)ctas, 256, 0, s>>>(v);
+        if (prb_launch_leaf_min(v, s) < 0) return -1;
         extra_launches = 1;
     }
     static bool big_smem[kPrbMaxDevices][2][6];
@@ -1117,10 +975,7 @@ int prb_launch_descend(const PrbView& v, uint32_t B, uint64_t seed, unsigned cha
     int launches = 1;
     if (plan.buffer_norm && v.min_off == 0) {
         // the scan of the leaves goes first, on the same stream (no min-tree to read the minimum from)
-        const uint64_t per_cta = 256ull * 16ull;
-        uint64_t ctas = (v.capacity + per_cta - 1) / per_cta;
-        if (ctas > (uint64_t)sm_count * 4) ctas = (uint64_t)sm_count * 4;
-        prb_leaf_min_kernel<<<(unsigned)ctas, 256, 0, s>>>(v);
+        if (prb_launch_leaf_min(v, s) < 0) return -1;
         launches = 2;
     }
     // one CTA per SM at most (the kernel has to fit beside a row copy's CTAs), each walking its strata

@@ -1,0 +1,60 @@
+"""The short-row sample at the sizes where its two shapes (one cluster, a cooperative grid) and its copy of rows
+change: batches around a warp, a CTA's share and the line between the shapes; rows of 1-, 2- and 4-byte words, shorter
+than half a warp's words and longer than a CTA's; and its weights against binary64."""
+import numpy as np
+import pytest
+import torch
+
+from prb_harness import Pair
+
+pytestmark = pytest.mark.gpu
+
+
+def _fill(pr, rng, N, obs_bytes, act_bytes, chunk):
+    for at in range(0, N, chunk):
+        n = min(chunk, N - at)
+        prio = np.exp(rng.standard_normal(n)).astype(np.float32)
+        prio[rng.random(n) < 0.1] = 0.0
+        pr.insert(dict(obs=rng.integers(0, 256, size=(n, obs_bytes), dtype=np.uint8),
+                       act=rng.integers(0, 256, size=(n, act_bytes), dtype=np.uint8),
+                       rew=rng.standard_normal(n).astype(np.float32),
+                       next_obs=rng.integers(0, 256, size=(n, obs_bytes), dtype=np.uint8),
+                       done=rng.integers(0, 2, size=n, dtype=np.uint8), prio=prio))
+
+
+@pytest.mark.parametrize("K,N", [(2, 5000), (2, 40_001), (4, 20_000), (8, 4097), (16, 70_000), (32, 33_000)])
+@pytest.mark.parametrize("obs_bytes,act_bytes", [(3, 1), (12, 4), (242, 6), (2052, 24)])
+def test_batch_sizes(oracle_mod, K, N, obs_bytes, act_bytes):
+    rng = np.random.default_rng(N + obs_bytes)
+    pr = Pair(oracle_mod, N, K, obs_bytes, act_bytes, 4096)
+    _fill(pr, rng, N, obs_bytes, act_bytes, 4096)
+    for call, B in enumerate([1, 4, 5, 31, 33, 64, 65, 511, 1025, 1536, 1537, 4000]):
+        pr.sample(B, 0.4 if call % 2 else 1.0, 7 + call)
+        pr.compare_state()
+    assert pr.compare_status() in (0, 8)
+    pr.close()
+
+
+@pytest.mark.parametrize("B", [48, 3000, 200_000])
+def test_weights_against_binary64(oracle_mod, B):
+    # (p / p_min)^-beta is formed in binary64 and rounded once to binary32: half a unit in the last place, 2^-24
+    # relative, and nothing else that shows (1e-9 allowed for the two logarithms and the exponential)
+    rng = np.random.default_rng(B)
+    N, K = 200_000, 16
+    pr = Pair(oracle_mod, N, K, 4, 4, 200_000)
+    prio = np.exp(6 * rng.standard_normal(N)).astype(np.float32)
+    pr.insert(dict(obs=np.zeros((N, 4), np.uint8), act=np.zeros((N, 4), np.uint8), rew=np.zeros(N, np.float32),
+                   next_obs=np.zeros((N, 4), np.uint8), done=np.zeros(N, np.uint8), prio=prio))
+    dev = pr.dev
+    idx, w = torch.zeros(B, dtype=torch.int32, device=dev), torch.zeros(B, device=dev)
+    for beta in (0.4, 1.0, 3.7, 0.0):
+        for norm in ("batch", "buffer"):
+            (pr.gpu.sample if norm == "batch" else pr.gpu.sample_buffer_norm)(B, beta, 3, idx, w)
+            p = prio[idx.cpu().numpy()].astype(np.float64)
+            # (the exponent crosses the C ABI as a binary32)
+            want = (p / (p.min() if norm == "batch" else prio[prio > 0].min().astype(np.float64))) ** -float(np.float32(beta))
+            got = w.cpu().numpy().astype(np.float64)
+            normal = want > 2.0 ** -125                                 # below: binary32's subnormals
+            assert np.all(np.abs(got - want)[normal] <= want[normal] * (2.0 ** -24 + 1e-9))
+            assert np.all(np.abs(got - want)[~normal] <= 2.0 ** -149)
+    pr.close()
