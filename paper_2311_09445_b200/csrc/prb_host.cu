@@ -133,8 +133,8 @@ namespace {
 void destroy_fork(PrbFork& f)
 {
     if (f.fork) cudaEventDestroy(f.fork);
-    if (f.join) cudaEventDestroy(f.join);
     if (f.side) cudaStreamDestroy(f.side);
+    if (f.join) cudaEventDestroy(f.join);
     f = PrbFork{nullptr, nullptr, nullptr};
     cudaGetLastError();
 }
@@ -170,7 +170,7 @@ struct pearl_prb {
     bool main_touched = true;                    // since fork.side last waited for the caller's stream, that stream
                                                  // has been given work that reads or writes the tree or the state
     uint32_t handoff_next = 0;
-    unsigned long long after_forked_tree = 0;    // the capture in which the last call was an update + insertion whose tree kernel ran on fork.side (0: it was not)
+    bool after_rows = false;                     // the last call was an update + insertion of long rows: a tree kernel beside a row copy
     unsigned long long main_last_gather = 0;     // the capture in which the last kernel given to the caller's stream was such a row copy (0: it was not)
     ~pearl_prb()
     {
@@ -230,10 +230,8 @@ unsigned long long capture_of(cudaStream_t s)
 // The descents -- chains of dependent L2 reads that keep HBM idle -- read and write nothing of the
 // caller's: the tree, the state and a hand-off area of the slab (leaf indices and priorities; the
 // weights are formed by the row copy's spare warps).  So they are launched on the handle's
-// second stream, where they are ordered after the tree work that stream already holds (the tree kernel
-// of the update + insertion before them) but not after the rows the caller's stream is still copying:
-// in a captured step they run beside the insertion's row copy, and in back-to-back samples beside the
-// row copy of the sample before.  The caller's stream then waits for them and runs the indexed row
+// second stream, where they are ordered after the tree work before them but not after the rows the caller's stream is
+// still copying: in back-to-back samples they run beside the row copy of the sample before.  The caller's stream then waits for them and runs the indexed row
 // copy, which also hands indices and weights to the caller.  Everything the caller can see is written
 // on the caller's stream, in order.  The second stream waits for the caller's stream first whenever
 // that stream has been given tree or state work since (main_touched), and once at the start of every
@@ -267,7 +265,7 @@ int sample_two_kernels(pearl_prb* h, unsigned long long capture, uint32_t B, flo
     h->gather_capture[j] = capture;
     h->handoff_next = (j + 1u) % kPrbHandoffs;
     h->main_last_gather = capture;
-    h->after_forked_tree = 0;
+    h->after_rows = false;
     return k1 + k2 + 1;
 }
 
@@ -458,7 +456,7 @@ int pearl_prb_insert(pearl_prb_t* h, uint32_t n, const void* d_obs, const void* 
     const int k = prb_launch_insert(h->view, n, b, d_prio, h->stream);
     if (k < 0) return PEARL_ERR_CUDA;
     h->launches += (uint64_t)k;
-    h->main_touched = true; h->main_last_gather = 0; h->after_forked_tree = 0;
+    h->main_touched = true; h->main_last_gather = 0; h->after_rows = false;
     return PEARL_OK;
 }
 
@@ -492,11 +490,11 @@ static int sample_common(pearl_prb_t* h, uint32_t B, float beta, uint64_t seed, 
     // form, whose descents are the prologue of the copy, is shorter by a launch.
     const unsigned long long capture = (n_sub == 1 && prb_sample_has_long_rows(h->view, b)) ? capture_of(h->stream) : 0ull;
     int k;
-    if (capture && h->after_forked_tree != capture) {
+    if (capture && !h->after_rows) {
         k = sample_two_kernels(h, capture, B, beta, seed, d_idx, d_w, b, uniform, buffer_norm);
     } else {
         k = prb_launch_sample(h->view, B, beta, seed, d_idx, d_w, b, h->stream, uniform, n_sub, &h->subs, buffer_norm);
-        h->main_touched = true; h->main_last_gather = 0; h->after_forked_tree = 0;
+        h->main_touched = true; h->main_last_gather = 0; h->after_rows = false;
     }
     if (k < 0) return PEARL_ERR_CUDA;
     h->launches += (uint64_t)k;
@@ -551,7 +549,7 @@ static int update_common(pearl_prb_t* h, uint32_t B, const int32_t* d_idx, const
     const int k = prb_launch_update(h->view, B, d_idx, d_val, raw, alpha, eps, h->stream, stale);
     if (k < 0) return PEARL_ERR_CUDA;
     h->launches += (uint64_t)k;
-    h->main_touched = true; h->main_last_gather = 0; h->after_forked_tree = 0;
+    h->main_touched = true; h->main_last_gather = 0; h->after_rows = false;
     return PEARL_OK;
 }
 
@@ -586,7 +584,7 @@ int pearl_prb_get_priorities(pearl_prb_t* h, uint32_t B, const int32_t* d_idx, f
     const int k = prb_launch_get_priorities(h->view, B, d_idx, d_out, h->stream);
     if (k < 0) return PEARL_ERR_CUDA;
     h->launches += (uint64_t)k;
-    h->main_touched = true; h->main_last_gather = 0; h->after_forked_tree = 0;
+    h->main_touched = true; h->main_last_gather = 0; h->after_rows = false;
     return PEARL_OK;
 }
 
@@ -616,20 +614,11 @@ int pearl_prb_update_insert(pearl_prb_t* h, uint32_t B, const int32_t* d_idx, co
     if (!guard.ok) return PEARL_ERR_CUDA;
     PrbBatch b;
     for (int f = 0; f < PRB_NUM_FIELDS; ++f) b.ptr[f] = (unsigned char*)ptrs[f];
-    bool forked = false;
-    const int k = prb_launch_insert(h->view, n, b, d_prio, h->stream, B, d_idx, d_td, 0, alpha, eps, &h->fork, &forked);
+    bool beside = false;
+    const int k = prb_launch_insert(h->view, n, b, d_prio, h->stream, B, d_idx, d_td, 0, alpha, eps, &h->fork, &beside);
     if (k < 0) return PEARL_ERR_CUDA;
     h->launches += (uint64_t)k;
-    if (forked) {
-        // the tree work went to the second stream, which waited for this one first; what this stream got
-        // is the row copy, which touches neither the tree nor the state the descents read
-        h->side_capture = capture_of(h->stream);
-        h->main_touched = false;
-        h->main_last_gather = 0;
-        h->after_forked_tree = h->side_capture;
-    } else {
-        h->main_touched = true; h->main_last_gather = 0; h->after_forked_tree = 0;
-    }
+    h->main_touched = true; h->main_last_gather = 0; h->after_rows = beside;
     return PEARL_OK;
 }
 
@@ -842,8 +831,11 @@ int step_host_duplex(pearl_prb* h, uint32_t B_upd, const int32_t* h_upd_idx, con
     for (int f = 0; f < PRB_NUM_FIELDS; ++f)
         if (in_b.ptr[f] && !to_dev(in_b.ptr[f], src[f], (uint64_t)n * h->view.field_bytes[f], up)) return PEARL_ERR_CUDA;      // (read by the row kernel only)
     unsigned char* area = h->view.handoff[0];
-    int k = prb_launch_update(h->view, B_upd, d_uidx, d_td, 0, alpha, eps, main, 0, n, d_prio, in_b.ptr[F_DONE]);
-    if (k != 1) return PEARL_ERR_CUDA;
+    PrbTreeArgs tree;
+    tree.B = B_upd; tree.idx = d_uidx; tree.val = d_td; tree.alpha = alpha; tree.eps = eps;
+    tree.n = n; tree.prio = d_prio; tree.done = in_b.ptr[F_DONE];
+    const int k = prb_launch_tree(h->view, tree, main, false);
+    if (k < 1) return PEARL_ERR_CUDA;
     if (prb_launch_descend(h->view, B, seed, area, main, 0, 0) != 1) return PEARL_ERR_CUDA;
     if (prb_launch_gather(h->view, B, beta, area, d_idx, d_w, out_b, main, false, 1, n) != 1) return PEARL_ERR_CUDA;
     for (int f = 0; f < PRB_NUM_FIELDS; ++f)
@@ -851,8 +843,8 @@ int step_host_duplex(pearl_prb* h, uint32_t B_upd, const int32_t* h_upd_idx, con
     if (prb_launch_insert(h->view, n, in_b, d_prio, up, 0, nullptr, nullptr, 0, 0.0f, 0.0f, nullptr, nullptr, true) != 1) return PEARL_ERR_CUDA;
     if (cudaEventRecord(h->subs.done[1], up) != cudaSuccess || cudaStreamWaitEvent(main, h->subs.done[1], 0) != cudaSuccess) return PEARL_ERR_CUDA;
     if (prb_launch_gather(h->view, B, beta, area, d_idx, d_w, out_b, main, false, 2, n) != 1) return PEARL_ERR_CUDA;
-    h->launches += 5;
-    h->main_touched = true; h->main_last_gather = 0; h->after_forked_tree = 0;
+    h->launches += (uint64_t)k + 4u;
+    h->main_touched = true; h->main_last_gather = 0; h->after_rows = false;
     // (the cursor comes back with the batch: into the handle's pinned buffer where there is one -- no call
     // leaves its second half in use -- so that the copy call itself does not wait for the stream)
     unsigned long long cursor_here = 0;
@@ -884,9 +876,9 @@ int step_host_duplex(pearl_prb* h, uint32_t B_upd, const int32_t* h_upd_idx, con
 }  // namespace
 
 // One iteration through host buffers as one call.  A small step (all inputs, and all outputs, within 256 KB
-// each) makes no copy call at all: the inputs are gathered in the handle's pinned buffer, which the device
-// sees mapped, the kernels read them from there and write the sampled batch into its second half, and the
-// one synchronisation of the step is the wait for that.  A larger step with long rows both ways (8 KB and
+// each) makes no copy call (one, of the indices and TD errors, from 1025 updates on): the inputs are gathered
+// in the handle's pinned buffer, which the device sees mapped, the kernels read them from there and write the
+// sampled batch into its second half, and the one synchronisation of the step is the wait for that.  A larger step with long rows both ways (8 KB and
 // more, plain layout, at most PEARL_UPDATE_SUBBATCH updates) runs with both directions of the host link busy
 // at once (step_host_duplex above); any other is the three host calls.
 int pearl_prb_step_host(pearl_prb_t* h, uint32_t B_upd, const int32_t* h_upd_idx, const float* h_td, float alpha, float eps,
@@ -931,6 +923,7 @@ int pearl_prb_step_host(pearl_prb_t* h, uint32_t B_upd, const int32_t* h_upd_idx
     if (!guard.ok) return PEARL_ERR_CUDA;
     // the pinned buffer may still be the source of a copy an earlier *_host call left on the stream
     if (cudaEventSynchronize(h->pin_read) != cudaSuccess) return PEARL_ERR_CUDA;
+    const bool many = B_upd > kPrbTreeEntries;
     void* din[PRB_NUM_FIELDS + 3];
     void* dout[PRB_NUM_FIELDS + 2];
     for (int i = 0; i < PRB_NUM_FIELDS + 3; ++i) {
@@ -940,6 +933,13 @@ int pearl_prb_step_host(pearl_prb_t* h, uint32_t B_upd, const int32_t* h_upd_idx
         din[i] = h->pin_dev + in.off[i];
     }
     for (int i = 0; i < PRB_NUM_FIELDS + 2; ++i) dout[i] = (dst[i] && out.bytes[i]) ? h->pin_dev + kPackBytes + out.off[i] : nullptr;
+    if (many) {
+        // (every CTA of a large update looks at the whole batch: its indices and TD errors go to the device first)
+        const uint64_t from = in.off[PRB_NUM_FIELDS + 1];
+        unsigned char* arena = at(h, h->lay.off_stage_in[0]);
+        if (cudaMemcpyAsync(arena + from, h->pin + from, in.total - from, cudaMemcpyHostToDevice, h->stream) != cudaSuccess) return PEARL_ERR_CUDA;
+        for (int i = PRB_NUM_FIELDS + 1; i < PRB_NUM_FIELDS + 3; ++i) din[i] = arena + in.off[i];
+    }
     int rc = pearl_prb_step(h, B_upd, (const int32_t*)din[PRB_NUM_FIELDS + 1], (const float*)din[PRB_NUM_FIELDS + 2], alpha, eps, n,
                             din[F_OBS], din[F_ACT], (const float*)din[F_REW], din[F_NEXT_OBS], (const uint8_t*)din[F_DONE],
                             (const float*)din[PRB_NUM_FIELDS], B, beta, seed, (int32_t*)dout[PRB_NUM_FIELDS],
@@ -997,7 +997,7 @@ int pearl_prb_sample_static_scratch(pearl_prb_t* h, uint32_t B, float beta, uint
     const int k = prb_launch_sample(v, B, beta, seed, d_idx, d_w, b, h->stream);
     if (k < 0) return PEARL_ERR_CUDA;
     h->launches += (uint64_t)k;
-    h->main_touched = true; h->main_last_gather = 0; h->after_forked_tree = 0;
+    h->main_touched = true; h->main_last_gather = 0; h->after_rows = false;
     return PEARL_OK;
 }
 
@@ -1011,7 +1011,7 @@ int pearl_prb_sync(pearl_prb_t* h, uint32_t* status_bits)
     uint32_t st = 0;
     if (cudaMemcpyAsync(&st, &h->view.state->status, 4, cudaMemcpyDeviceToHost, h->stream) != cudaSuccess) return PEARL_ERR_CUDA;
     if (cudaMemsetAsync(&h->view.state->status, 0, 4, h->stream) != cudaSuccess) return PEARL_ERR_CUDA;
-    h->main_touched = true; h->main_last_gather = 0; h->after_forked_tree = 0;
+    h->main_touched = true; h->main_last_gather = 0; h->after_rows = false;
     if (cudaStreamSynchronize(h->stream) != cudaSuccess) return PEARL_ERR_CUDA;
     if (status_bits) *status_bits = st;
     return PEARL_OK;
@@ -1199,7 +1199,7 @@ int image_transfer(pearl_prb* h, uint64_t offset, unsigned char* host, uint64_t 
     if (rc == PEARL_OK)
         rc = copy_image_part(h, offset, host, bytes, kImageHeaderBytes + tree_bytes, store_bytes, h->lay.off_zero_end, to_host);
     if (rc != PEARL_OK) return rc;
-    if (!to_host) { h->main_touched = true; h->main_last_gather = 0; h->after_forked_tree = 0; }
+    if (!to_host) { h->main_touched = true; h->main_last_gather = 0; h->after_rows = false; }
     return cudaStreamSynchronize(h->stream) == cudaSuccess ? PEARL_OK : PEARL_ERR_CUDA;
 }
 

@@ -3,16 +3,14 @@
 // priority retrieval followed by priority update; Listing 2: experiences are added to the
 // Data Storage and insertion requests go to the Replay Manager).
 //
-// One kernel per call, in one of two shapes.
-//   Short rows: CTA 0 owns the tree, the other CTAs copy tiles of the dense batch to ring slots
-//   through registers.
-//   Long rows (at least 8 KB of 16-byte granules, Atari-shaped): one CTA per SM; warp 0 of
-//   every CTA drives bulk asynchronous copies global -> shared -> global through a ~200 KB
-//   ring (row chunks of <= 8 KB, one lane per stage), issuing its loads before the cursor has
-//   even arrived; the other warps copy the short fields.  CTA 0 does the tree and moves no rows;
-//   with a priority update in the same call the tree work is a kernel of its own on a second
-//   stream (prb_update.cu) and every CTA here copies.
-// Tree work: write the n leaves, then re-sum the dirty parents level by level (a contiguous
+// Short rows: one launch of the tree kernel (prb_tree.cu), whose spare CTAs copy them.
+// Long rows (at least 8 KB of 16-byte granules, Atari-shaped): the kernel below, one CTA per SM; warp 0 of
+// every CTA drives bulk asynchronous copies global -> shared -> global through a ~200 KB
+// ring (row chunks of <= 8 KB, one lane per stage), issuing its loads before the cursor has
+// even arrived; the other warps copy the short fields.  CTA 0 does the tree and moves no rows;
+// with a priority update in the same call the tree work is the tree kernel's, beside this one, and every
+// CTA here copies.
+// Tree work here: write the n leaves, then re-sum the dirty parents level by level (a contiguous
 // slot range dirties a contiguous parent range on every level, so no sorting is needed).
 // The CTA that is last to have read the cursor advances it (and the fill count) while the copies
 // are still running.  No CTA waits on another.
@@ -21,13 +19,13 @@
 namespace {
 
 constexpr int kWorkers = 256;                // threads that copy short rows / do the tree work
-constexpr int kThreadsShort = kWorkers + 32;     // short-row kernel: workers, then the warp whose lane 0 publishes the cursor
 constexpr int kThreadsRows = 32 + kWorkers + 32; // long-row kernel: ring warp, workers, publishing warp
 constexpr uint32_t kChunk = 512;             // upper bound on granules per chunk of a long row (8 KB)
 constexpr uint32_t kTile = kWorkers * 8;     // granules per tile of short rows
 constexpr uint32_t kRowMode = 512;           // rows of at least this many 16-byte granules are split into chunks
 constexpr uint32_t kRingBytes = 198 * 1024;  // bulk-copy ring (dynamic shared memory), <= 32 stages
 constexpr uint32_t kRingBarBytes = 1024;     // room for the ring's mbarriers in front of its buffers
+constexpr uint64_t kForkFrom = 4ull << 20;   // bytes of long rows from which the tree work goes to the side stream
 
 struct InsertPlan {
     // short-row tiles, numbered field by field: tiles of field f are [first_tile[f], first_tile[f+1])
@@ -76,66 +74,6 @@ __device__ __forceinline__ void copy_tile(const PrbView& v, const InsertPlan& pl
     case 4: copy_flat_tile<uint32_t>(v, f, src, n, cursor, local, rank, nthreads); break;
     case 2: copy_flat_tile<uint16_t>(v, f, src, n, cursor, local, rank, nthreads); break;
     default: copy_flat_tile<uint8_t>(v, f, src, n, cursor, local, rank, nthreads); break;
-    }
-}
-
-// A priority update to run before the insertion's tree work, by the same team (B == 0: none).
-struct FusedUpdate {
-    uint32_t B, n2;
-    const int32_t* idx;
-    const float* val;
-    int raw;
-    float alpha, eps;
-};
-
-// Short rows only: CTA 0 = tree (after the optional update), CTAs 1.. = a contiguous range of tiles
-// each.  Threads 0..kWorkers-1 work; thread kWorkers reads the cursor for the CTA and takes the ticket.
-template <bool kFrames, bool kMin>
-__global__ void __launch_bounds__(kThreadsShort, 2)
-prb_insert_kernel(const __grid_constant__ PrbView v, uint32_t n, const __grid_constant__ PrbBatch src,
-                  const float* __restrict__ prio, const __grid_constant__ InsertPlan plan,
-                  const __grid_constant__ FusedUpdate upd)
-{
-    extern __shared__ __align__(16) unsigned char s_dyn[];
-    __shared__ unsigned long long s_cursor, s_fill;     // read once per CTA, before anything is published
-    __shared__ unsigned int s_maxp;                     // running maximum of priorities at kernel start
-    const uint32_t tid = threadIdx.x;
-    // (the kernel after this one on the stream, if it was launched as a programmatic dependent, may be made
-    // resident now; it waits for this kernel's completion before it reads anything)
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (tid == kWorkers) { s_cursor = v.state->cursor; s_fill = v.state->fill; s_maxp = v.state->max_prio_bits; }
-    // the tree CTA fetches its first inputs now, while the cursor is on its way
-    // (and starts the copy of the tree's top into shared memory, behind the update's keys)
-    PrbPreloaded pre = PrbPreloaded{false, false, 0, 0.0f, 0.0f};
-    PrbTop top;
-    if (blockIdx.x == 0 && tid < kWorkers) {
-        if (tid < upd.B) { pre.has_update = true; pre.idx = upd.idx[tid]; pre.val = upd.val[tid]; }
-        if (tid < n && prio != nullptr) { pre.has_prio = true; pre.prio = prio[tid]; }
-        if (v.top_levels) top.mem = reinterpret_cast<float*>(s_dyn + (upd.B ? prb_update_smem_bytes(upd.n2) : 0));
-        if (kMin && v.top_levels) top.mem_min = top.mem + v.top_floats;
-        prb_top_begin(v, top, tid, kWorkers);
-    }
-    __syncthreads();
-    const uint64_t cursor = s_cursor;
-    if (tid == kWorkers) {
-        prb_publish_if_last(v, n, cursor, s_fill, gridDim.x);
-    } else if (tid < kWorkers) {
-        if (blockIdx.x == 0) {
-            PrbTeam team;
-            team.rank = tid; team.size = kWorkers; team.whole_cta = false;
-            if (kMin) team.min_off = v.min_off;
-            if (upd.B)      // update and insertion share one re-sum pass per level
-                prb_update_team(v, team, upd.B, upd.n2, upd.idx, upd.val, upd.raw, upd.alpha, upd.eps, s_fill, s_dyn, n, prio, cursor, pre, 0, top,
-                                src.ptr[F_DONE], kFrames ? v.stack : 0u);
-            else
-                prb_insert_tree_team(v, team, n, prio, cursor, pre, s_maxp, top, src.ptr[F_DONE], kFrames ? v.stack : 0u);
-        } else {
-            const uint32_t n_tiles = plan.first_tile[PRB_NUM_FIELDS];
-            const uint32_t copy_ctas = gridDim.x - 1, c = blockIdx.x - 1;
-            const uint32_t t_lo = (uint32_t)(((uint64_t)c * n_tiles) / copy_ctas);
-            const uint32_t t_hi = (uint32_t)(((uint64_t)(c + 1) * n_tiles) / copy_ctas);
-            for (uint32_t t = t_lo; t < t_hi; ++t) copy_tile(v, plan, src, n, cursor, t, tid, kWorkers);
-        }
     }
 }
 
@@ -212,26 +150,29 @@ prb_insert_rows_kernel(const __grid_constant__ PrbView v, uint32_t n, const __gr
         team.rank = tid - 32u; team.size = kWorkers; team.whole_cta = false;
         if (kMin) team.min_off = v.min_off;
         if (blockIdx.x == 0 && plan.tree_ctas == 0)
-            prb_insert_tree_team(v, team, n, prio, cursor, PrbPreloaded{false, false, 0, 0.0f, 0.0f}, s_maxp, PrbTop{}, src.ptr[F_DONE],
+            prb_insert_tree_team(v, team, n, prio, cursor, s_maxp, src.ptr[F_DONE],
                                  kFrames ? v.stack : 0u);
         const uint32_t n_tiles = plan.first_tile[PRB_NUM_FIELDS];
         for (uint32_t tile = (blockIdx.x + gridDim.x - 1) % gridDim.x; tile < n_tiles; tile += gridDim.x)
             copy_tile(v, plan, src, n, cursor, tile, team.rank, team.size);
     }
+    // Launched as a programmatic dependent of the tree kernel: this kernel is complete only when that one is.
+    prb_dep_wait();
 }
 
 }  // namespace
 
 int prb_launch_insert(const PrbView& v, uint32_t n, const PrbBatch& src, const float* d_prio, cudaStream_t s,
                       uint32_t upd_B, const int32_t* upd_idx, const float* upd_val, int upd_raw, float alpha, float eps,
-                      const PrbFork* fork, bool* forked_out, bool rows_only)
+                      const PrbFork* fork, bool* beside_out, bool rows_only)
 {
-    if (forked_out) *forked_out = false;
+    if (beside_out) *beside_out = false;
     if (rows_only && upd_B) return -1;
     const int sm_count = prb_sm_count();
     const int dev = prb_current_device();
-    FusedUpdate upd;
-    upd.B = upd_B; upd.n2 = prb_update_n2(upd_B); upd.idx = upd_idx; upd.val = upd_val; upd.raw = upd_raw; upd.alpha = alpha; upd.eps = eps;
+    PrbTreeArgs tree;
+    tree.B = upd_B; tree.idx = upd_idx; tree.val = upd_val; tree.raw = upd_raw; tree.alpha = alpha; tree.eps = eps;
+    tree.n = n; tree.prio = d_prio; tree.done = src.ptr[F_DONE];
 
     InsertPlan plan;
     uint32_t tiles = 0, tasks = 0, stage = 0;
@@ -252,89 +193,73 @@ int prb_launch_insert(const PrbView& v, uint32_t n, const PrbBatch& src, const f
             tiles += (uint32_t)((total + kTile - 1) / kTile);
         }
     }
+    if (tasks == 0) {
+        // short rows: one launch does the update, the insertion's tree work and the row copy
+        if (rows_only) return -1;
+        tree.rows = &src;
+        return prb_launch_tree(v, tree, s, true);
+    }
     plan.first_tile[PRB_NUM_FIELDS] = tiles;
     plan.first_task[PRB_NUM_FIELDS] = tasks;
-    plan.ring_stages = 0;
-    plan.ring_stage_bytes = 0;
     plan.tree_ctas = 0;
+    stage = (stage + 127u) / 128u * 128u;
+    plan.ring_stage_bytes = stage;
+    plan.ring_stages = kRingBytes / stage;
+    if (plan.ring_stages > 32) plan.ring_stages = 32;
     int launches = 1;
+    const bool beside = upd_B != 0;
     bool forked = false;
-    uint32_t rows_grid = 0;
-    if (rows_only && tasks == 0) return -1;
-    const bool fork_tree = upd.B && tasks > 0 && upd.B <= PEARL_UPDATE_SUBBATCH && fork != nullptr;
-    if (tasks > 0) {
-        stage = (stage + 127u) / 128u * 128u;
-        plan.ring_stage_bytes = stage;
-        plan.ring_stages = kRingBytes / stage;
-        if (plan.ring_stages > 32) plan.ring_stages = 32;
-    }
-    if (tasks > 0) {
-        // Without a tree kernel CTA 0 does the tree work and no copies; with one, its CTAs get SMs of
-        // their own: a copy CTA takes an SM's whole shared memory and would wait for them to leave.
-        const uint32_t want = tasks + ((fork_tree || rows_only) ? 0u : 1u);
-        uint32_t room = (uint32_t)sm_count;
-        if (fork_tree && room > 2u * prb_update_ctas(v, upd.B)) room -= prb_update_ctas(v, upd.B);
-        rows_grid = want < room ? want : room;
-    }
+    // Without a tree kernel CTA 0 does the tree work and no copies; with one, its CTAs get SMs of
+    // their own: a copy CTA takes an SM's whole shared memory and would wait for them to leave.
+    const uint32_t want = tasks + ((beside || rows_only) ? 0u : 1u);
+    uint32_t room = (uint32_t)sm_count;
     if (rows_only) {
         plan.tree_ctas = 1;       // (CTA 0 copies like the others and the row cursor is published by itself)
-    } else if (fork_tree) {
-        // Long rows: the update and the insertion's tree work are one kernel on the side stream, the
-        // row copy another on the caller's stream; neither waits for the other (each advances a
-        // cursor of its own), and the caller's stream goes on when both are done.  (In one kernel the tree's chain of dependent reads, slowed by the
-        // copy's traffic, was measured to outlast the copy by far.)
-        plan.tree_ctas = prb_update_ctas(v, upd.B);
-        if (cudaEventRecord(fork->fork, s) != cudaSuccess || cudaStreamWaitEvent(fork->side, fork->fork, 0) != cudaSuccess)
-            return -1;
-        const int k = prb_launch_update(v, upd_B, upd_idx, upd_val, upd_raw, alpha, eps, fork->side, 0, n, d_prio, src.ptr[F_DONE]);
-        if (k != 1 || cudaEventRecord(fork->join, fork->side) != cudaSuccess) return -1;
-        upd.B = 0;
-        launches = 2;
-        forked = true;
-        if (forked_out) *forked_out = true;
-    } else if (upd.B && (tasks > 0 || upd.B >= kPrbWideFrom)) {
-        // (a batch for the many-CTA update, or no side stream: the update goes first, in launches of its
-        // own; so does a batch of exactly one entry per thread, measured 14-25 us as two launches against
-        // 15-33 us fused at 1024 entries + 1024 insertions)
-        const int k = prb_launch_update(v, upd_B, upd_idx, upd_val, upd_raw, alpha, eps, s);
-        if (k < 0) return -1;
-        upd.B = 0;
+    } else if (beside) {
+        // The update and the insertion's tree work are one kernel, the row copy another beside it; neither waits for
+        // the other (each advances a cursor of its own).  (In one kernel the tree's chain of dependent reads, slowed
+        // by the copy's traffic, was measured to outlast the copy by far.)
+        // Few rows: both on the caller's stream, the copy a programmatic dependent that does not wait: it starts as
+        // soon as the tree kernel's CTAs have (they have waited for what came before) and waits for the tree only
+        // before it ends, so that what follows has both behind it.  No fork, no join: 4 rows of 56 KB, 18.6 ->
+        // 16.9 us a step.  Many rows: the tree kernel on the side stream, so that the copy, the longer of the two,
+        // does not start behind the tree kernel's start (512 rows of 56 KB: 33.5 us a step the first way).
+        forked = fork != nullptr && (uint64_t)tasks * stage > kForkFrom;
+        tree.most_ctas = kPrbTreeBesideRows;
+        plan.tree_ctas = prb_tree_ctas(v, upd_B, n, tree.most_ctas);
+        if (room > 2u * kPrbTreeBesideRows) room -= kPrbTreeBesideRows;
+        if (forked && (cudaEventRecord(fork->fork, s) != cudaSuccess || cudaStreamWaitEvent(fork->side, fork->fork, 0) != cudaSuccess)) return -1;
+        const int k = prb_launch_tree(v, tree, forked ? fork->side : s, !forked);
+        if (k < 1 || (forked && cudaEventRecord(fork->join, fork->side) != cudaSuccess)) return -1;
         launches = 1 + k;
+        if (beside_out) *beside_out = true;
     }
-    const uint32_t upd_smem = upd.B ? (uint32_t)prb_update_smem_bytes(upd.n2) : 0u;
-    if (tasks == 0) {
-        static bool big_smem[kPrbMaxDevices];
-        if (!big_smem[dev]) {
-            const int most = (int)(prb_update_smem_bytes(PEARL_UPDATE_SUBBATCH) + 2 * kPrbTopFloats * sizeof(float));
-            bool ok = true;
-#define PRB_ALLOW_SMEM(FF, MM) ok = ok && cudaFuncSetAttribute(prb_insert_kernel<FF, MM>, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess
-            PRB_ALLOW_SMEM(false, false); PRB_ALLOW_SMEM(true, false); PRB_ALLOW_SMEM(false, true); PRB_ALLOW_SMEM(true, true);
-#undef PRB_ALLOW_SMEM
-            if (!ok) return -1;
-            big_smem[dev] = true;
-        }
-        const uint32_t one_wave = (uint32_t)sm_count * 2 - 1;     // CTA 0 is the tree CTA
-        const uint32_t copy_ctas = tiles < one_wave ? tiles : one_wave;
-        const uint32_t smem = upd_smem + v.top_floats * (uint32_t)sizeof(float) * (v.min_off ? 2u : 1u);
-#define PRB_LAUNCH_INSERT_AS(FF, MM) prb_insert_kernel<FF, MM><<<copy_ctas + 1, kThreadsShort, smem, s>>>(v, n, src, d_prio, plan, upd)
-        PRB_WITH_TREE_OPTIONS(v, PRB_LAUNCH_INSERT_AS);
-#undef PRB_LAUNCH_INSERT_AS
-    } else {
-        const uint32_t smem = kRingBarBytes + plan.ring_stages * plan.ring_stage_bytes;
-        static bool big_rows[kPrbMaxDevices];
-        if (!big_rows[dev]) {
-            bool ok = true;
+    const uint32_t rows_grid = want < room ? want : room;
+    const uint32_t smem = kRingBarBytes + plan.ring_stages * plan.ring_stage_bytes;
+    static bool big_rows[kPrbMaxDevices];
+    if (!big_rows[dev]) {
+        bool ok = true;
 #define PRB_ALLOW_SMEM(FF, MM) \
     ok = ok && cudaFuncSetAttribute(prb_insert_rows_kernel<FF, MM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kRingBarBytes + kRingBytes)) == cudaSuccess
-            PRB_ALLOW_SMEM(false, false); PRB_ALLOW_SMEM(true, false); PRB_ALLOW_SMEM(false, true); PRB_ALLOW_SMEM(true, true);
+        PRB_ALLOW_SMEM(false, false); PRB_ALLOW_SMEM(true, false); PRB_ALLOW_SMEM(false, true); PRB_ALLOW_SMEM(true, true);
 #undef PRB_ALLOW_SMEM
-            if (!ok) return -1;
-            big_rows[dev] = true;
-        }
-#define PRB_LAUNCH_ROWS_AS(FF, MM) prb_insert_rows_kernel<FF, MM><<<rows_grid, kThreadsRows, smem, s>>>(v, n, src, d_prio, plan)
-        PRB_WITH_TREE_OPTIONS(v, PRB_LAUNCH_ROWS_AS);
-#undef PRB_LAUNCH_ROWS_AS
-        if (forked && cudaStreamWaitEvent(s, fork->join, 0) != cudaSuccess) return -1;
+        if (!ok) return -1;
+        big_rows[dev] = true;
     }
-    return cudaGetLastError() == cudaSuccess ? launches : -1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(rows_grid);
+    cfg.blockDim = dim3(kThreadsRows);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = beside && !forked ? 1 : 0;
+    cudaError_t e = cudaSuccess;
+#define PRB_LAUNCH_ROWS_AS(FF, MM) e = cudaLaunchKernelEx(&cfg, prb_insert_rows_kernel<FF, MM>, v, n, src, d_prio, plan)
+    PRB_WITH_TREE_OPTIONS(v, PRB_LAUNCH_ROWS_AS);
+#undef PRB_LAUNCH_ROWS_AS
+    if (e != cudaSuccess || (forked && cudaStreamWaitEvent(s, fork->join, 0) != cudaSuccess)) return -1;
+    return launches;
 }

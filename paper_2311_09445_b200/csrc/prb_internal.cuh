@@ -33,17 +33,16 @@ struct PrbState {
     unsigned int insert_ticket;       // CTAs of the running insert kernel that have finished
     unsigned int sample_ticket;       // CTAs of the running sample kernel that have finished
     unsigned int max_prio_bits;       // bits of the largest priority written so far (0: none yet)
-    unsigned int wide_arrived;        // grid barrier of the running many-CTA update: arrivals so far (0 between launches that ended well)
-    unsigned int wide_done;           // its CTAs that have passed their last barrier
-    unsigned long long wide_wmax_bits; // largest raw weight of the running large-batch sample (bits of a binary64; 0 between calls)
+    unsigned int unused[2];
+    unsigned long long wide_wmax_bits; // smallest priority of the running large-batch sample, complemented (0 between calls)
     // The ring cursor as the kernels that copy rows see it.  An insertion whose tree work and row copy are
     // two kernels on two streams advances `cursor` (and `fill`) from the tree kernel and `row_cursor` from
     // the row kernel, each with a ticket of its own, so that neither kernel's bookkeeping waits for, or
     // races with, the other's; a one-kernel insertion advances both.  Equal whenever no insertion is running.
     unsigned long long row_cursor;
     unsigned int row_ticket;          // CTAs of the running row kernel that have read row_cursor
-    unsigned int wide_poisoned;       // a many-CTA update gave up at its barrier once: the barrier's state is not to be trusted, and
-                                      // neither is the tree; every later many-CTA update raises INTERNAL and does nothing
+    unsigned int wide_poisoned;       // a sample of many co-resident CTAs gave up waiting once: its ticket is not to be trusted, and every
+                                      // later one raises INTERNAL and does nothing
 };
 
 // Geometry and device addresses, passed to kernels by value.
@@ -94,8 +93,9 @@ struct PrbBatch {
     unsigned char* ptr[PRB_NUM_FIELDS];
 };
 
-// A second stream of the handle and the two events that fork it off the caller's stream and join it
-// again: with long rows the tree work of an update + insertion runs there, beside the row copy.
+// A second stream of the handle and the two events that fork it off the caller's stream and join it again: the tree
+// work of an update + insertion of many long rows runs there, beside the row copy, and the descents of a two-kernel
+// sample.
 struct PrbFork {
     cudaStream_t side;
     cudaEvent_t fork, join;
@@ -103,14 +103,12 @@ struct PrbFork {
 
 // Kernel launchers; each returns the number of kernels launched, or -1 on a launch error.
 // (upd_B > 0 runs a priority update of that batch before the insertion's tree work: in the same
-// kernel for short rows; for long rows in a tree kernel of its own on fork->side, or, without a
-// fork, in launches of its own before the insertion's)
+// kernel for short rows; for long rows in a tree kernel beside the row copy: *beside_out)
 int prb_launch_insert(const PrbView& v, uint32_t n, const PrbBatch& src, const float* d_prio, cudaStream_t s,
                       uint32_t upd_B = 0, const int32_t* upd_idx = nullptr, const float* upd_val = nullptr,
                       int upd_raw = 0, float alpha = 0.0f, float eps = 0.0f, const PrbFork* fork = nullptr,
-                      bool* forked_out = nullptr, bool rows_only = false);
-// (rows_only: long rows, and the insertion's tree work is some other launch's -- a prb_launch_update with
-// ins_n = n: this one copies the rows and advances the row cursor, nothing else)
+                      bool* beside_out = nullptr, bool rows_only = false);
+// (rows_only: long rows, and the insertion's tree work is some other launch's: this one copies the rows and advances the row cursor, nothing else)
 // Streams and events of a sample call that is issued as sub-batches (the paper's sub-batch
 // streaming, Section IV-C): sub-batch i runs on stream[i]; done[i] fires when its rows are in place.
 constexpr uint32_t kPrbMaxSubBatches = 4;
@@ -165,17 +163,30 @@ int prb_launch_relay(cudaStream_t s);
 // true if a sample that writes these fields moves rows long enough for the bulk-copy ring
 bool prb_sample_has_long_rows(const PrbView& v, const PrbBatch& dst);
 // (stale > 0: skip entries that name one of the `stale` most recently written ring slots)
-// (ins_n > 0, B within one sub-batch: the tree part of an insertion of ins_n transitions follows
-// the update in the same kernel, which advances the tree's cursor and the fill count)
+// (values or TD errors: prb_launch_tree; changes, raw == 2, keep their batch order and go sub-batch by sub-batch)
 int prb_launch_update(const PrbView& v, uint32_t B, const int32_t* d_idx, const float* d_val, int raw,
-                      float alpha, float eps, cudaStream_t s, uint32_t stale = 0,
-                      uint32_t ins_n = 0, const float* ins_prio = nullptr, const unsigned char* ins_done = nullptr);
-// (ins_done: the done bytes of the inserted batch; read with the frame-deduplicated layout only)
-// Update batches above this many entries (one per thread of a CTA) go to one launch of many
-// co-resident CTAs instead (measured: 11-20 us for 16384 entries against 15-29 us for 4096 in one CTA);
-// an update + insertion of short rows is then two launches, the update's and the insertion's.
-constexpr uint32_t kPrbWideFrom = 1024;
-// CTAs (one cluster) of the kernel that updates a batch (or sub-batch) of b entries
+                      float alpha, float eps, cudaStream_t s, uint32_t stale = 0);
+// Tree work (prb_tree.cu): a priority update of B entries (values or TD errors; B may be 0), then the tree part of an
+// insertion of n transitions (may be 0), and with `rows` the insertion's short rows, in one launch.
+struct PrbTreeArgs {
+    uint32_t B = 0;
+    const int32_t* idx = nullptr;
+    const float* val = nullptr;
+    int raw = 0;                          // 0: val holds TD errors, 1: priorities
+    float alpha = 0.0f, eps = 0.0f;
+    uint32_t stale = 0;                   // see prb_launch_update
+    uint32_t n = 0;
+    const float* prio = nullptr;          // nullptr: the running maximum
+    const unsigned char* done = nullptr;
+    const PrbBatch* rows = nullptr;
+    uint32_t most_ctas = 0;               // a limit on the CTAs that do the tree work (0: none)
+};
+constexpr uint32_t kPrbTreeEntries = 1024;      // update entries one CTA (or cluster) takes, one per thread; more go to a grid
+constexpr uint32_t kPrbTreeBesideRows = 8;      // CTAs of the tree work beside a row copy of long rows, at most
+uint32_t prb_tree_ctas(const PrbView& v, uint32_t b, uint32_t n, uint32_t most);
+// (dependent: as a programmatic dependent of the kernel before it on the stream)
+int prb_launch_tree(const PrbView& v, const PrbTreeArgs& t, cudaStream_t s, bool dependent);
+// CTAs (one cluster) of the kernel that adds b changes
 uint32_t prb_update_ctas(const PrbView& v, uint32_t b);
 int prb_launch_get_priorities(const PrbView& v, uint32_t B, const int32_t* d_idx, float* d_out, cudaStream_t s);
 

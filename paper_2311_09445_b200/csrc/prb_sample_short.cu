@@ -21,6 +21,7 @@
 // memory.  More: a cooperative grid; p_min by an atomic per CTA, and a CTA waits (bounded) for the others only
 // after its rows are copied.
 #include "prb_descend.cuh"
+#include "prb_rows.cuh"
 
 namespace {
 
@@ -42,14 +43,6 @@ struct __align__(16) ShortStep {
     uint32_t levels;
 };
 
-// One field of the row: words of 1, 2 or 4 bytes, numbered from `first` over all fields.
-struct ShortField {
-    const unsigned char* src;     // slot 0
-    unsigned char* dst;           // row 0 of the batch
-    uint32_t first, log2;
-    uint32_t src_pitch, dst_pitch;
-};
-
 struct ShortPlan {
     PrbState* state;
     const float* level0;
@@ -60,31 +53,45 @@ struct ShortPlan {
     uint32_t B, capacity;
     float beta;
     uint32_t uniform, buffer_norm;
-    uint32_t n_steps, n_words, chunks, lane_words;      // chunks of 32 words; words a warp's row part holds (8, 16 or 32)
+    uint32_t n_steps;
     ShortStep step[kMaxSteps];
-    ShortField field[PRB_NUM_FIELDS];
+    PrbWords words;
 };
 
 // ---- steps of the walk -----------------------------------------------------------------------------------
 // (the child entered is the first whose prefix exceeds the target; a target that has passed every prefix --
 // possible by binary32 rounding only -- takes the last positive child and raises CLAMPED)
 
+// kWide (many strata per SM): prefixes are compared in binary32 with the largest binary32 not above the target --
+// the same answer, and one conversion of the target in place of one per prefix, whose rate bounds the walk there;
+// otherwise in binary64, whose conversions are off the chain that bounds a small batch.
+template <bool kWide>
+struct Target {
+    double x;
+    float below;
+    __device__ __forceinline__ explicit Target(double t) : x(t), below(0.0f) { if (kWide) below = __double2float_rd(t); }
+    __device__ __forceinline__ bool past(float prefix) const { return kWide ? prefix <= below : x >= (double)prefix; }
+};
+
 // Fanout 2: children c0, c1.
+template <bool kWide>
 __device__ __forceinline__ bool pick2(double& x, float c0, float c1, unsigned& flags)
 {
-    const double s0 = (double)c0, s1 = (double)__fadd_rn(c0, c1);
-    const bool past0 = x >= s0, past1 = x >= s1;
+    const Target<kWide> t(x);
+    const bool past0 = t.past(c0), past1 = t.past(__fadd_rn(c0, c1));
     const bool right = past0 && !(past1 && !(c1 > 0.0f));
     if (past1) flags |= (c0 > 0.0f || c1 > 0.0f) ? PEARL_ST_CLAMPED : (PEARL_ST_CLAMPED | PEARL_ST_INTERNAL);
-    if (right) x = __dsub_rn(x, s0);
+    if (right) x = __dsub_rn(x, (double)c0);
     return right;
 }
 
 // Fanout 4.
+template <bool kWide>
 __device__ __forceinline__ uint32_t pick4(double& x, const float (&c)[4], unsigned& flags)
 {
     const float a1 = __fadd_rn(c[0], c[1]), a2 = __fadd_rn(a1, c[2]), a3 = __fadd_rn(a2, c[3]);
-    uint32_t j = (x >= (double)c[0] ? 1u : 0u) + (x >= (double)a1 ? 1u : 0u) + (x >= (double)a2 ? 1u : 0u) + (x >= (double)a3 ? 1u : 0u);
+    const Target<kWide> t(x);
+    uint32_t j = (t.past(c[0]) ? 1u : 0u) + (t.past(a1) ? 1u : 0u) + (t.past(a2) ? 1u : 0u) + (t.past(a3) ? 1u : 0u);
     if (j == 4u) {
         j = c[3] > 0.0f ? 3u : c[2] > 0.0f ? 2u : c[1] > 0.0f ? 1u : 0u;
         flags |= (j > 0u || c[0] > 0.0f) ? PEARL_ST_CLAMPED : (PEARL_ST_CLAMPED | PEARL_ST_INTERNAL);
@@ -94,7 +101,7 @@ __device__ __forceinline__ uint32_t pick4(double& x, const float (&c)[4], unsign
 }
 
 // The 16 entries four levels (fanout 2) or two levels (fanout 4) below a node.
-template <int K>
+template <int K, bool kWide>
 __device__ __forceinline__ uint32_t step16(const float* row, double& x, float& chosen, unsigned& flags)
 {
     float e[16];
@@ -109,48 +116,48 @@ __device__ __forceinline__ uint32_t step16(const float* row, double& x, float& c
         for (int i = 0; i < 8; ++i) p8[i] = __fadd_rn(e[2 * i], e[2 * i + 1]);
 #pragma unroll
         for (int i = 0; i < 4; ++i) p4[i] = __fadd_rn(p8[2 * i], p8[2 * i + 1]);
-        const bool r0 = pick2(x, __fadd_rn(p4[0], p4[1]), __fadd_rn(p4[2], p4[3]), flags);
+        const bool r0 = pick2<kWide>(x, __fadd_rn(p4[0], p4[1]), __fadd_rn(p4[2], p4[3]), flags);
         const float a0 = r0 ? p4[2] : p4[0], a1 = r0 ? p4[3] : p4[1];
 #pragma unroll
         for (int i = 0; i < 4; ++i) p8[i] = r0 ? p8[4 + i] : p8[i];
 #pragma unroll
         for (int i = 0; i < 8; ++i) e[i] = r0 ? e[8 + i] : e[i];
-        const bool r1 = pick2(x, a0, a1, flags);
+        const bool r1 = pick2<kWide>(x, a0, a1, flags);
         const float b0 = r1 ? p8[2] : p8[0], b1 = r1 ? p8[3] : p8[1];
 #pragma unroll
         for (int i = 0; i < 4; ++i) e[i] = r1 ? e[4 + i] : e[i];
-        const bool r2 = pick2(x, b0, b1, flags);
+        const bool r2 = pick2<kWide>(x, b0, b1, flags);
         const float d0 = r2 ? e[2] : e[0], d1 = r2 ? e[3] : e[1];
-        const bool r3 = pick2(x, d0, d1, flags);
+        const bool r3 = pick2<kWide>(x, d0, d1, flags);
         chosen = r3 ? d1 : d0;
         return (r0 ? 8u : 0u) + (r1 ? 4u : 0u) + (r2 ? 2u : 0u) + (r3 ? 1u : 0u);
     } else {
         float s[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) s[i] = __fadd_rn(__fadd_rn(__fadd_rn(e[4 * i], e[4 * i + 1]), e[4 * i + 2]), e[4 * i + 3]);
-        const uint32_t j = pick4(x, s, flags);
+        const uint32_t j = pick4<kWide>(x, s, flags);
         float c[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) c[i] = j == 0u ? e[i] : j == 1u ? e[4 + i] : j == 2u ? e[8 + i] : e[12 + i];
-        const uint32_t j2 = pick4(x, c, flags);
+        const uint32_t j2 = pick4<kWide>(x, c, flags);
         chosen = j2 == 0u ? c[0] : j2 == 1u ? c[1] : j2 == 2u ? c[2] : c[3];
         return 4u * j + j2;
     }
 }
 
 // One level: the K children of a node.  (From fanout 8 on the chosen child's value is left to the caller.)
-template <int K>
+template <int K, bool kWide>
 __device__ __forceinline__ uint32_t step1(const float* row, double& x, float& chosen, unsigned& flags)
 {
     if constexpr (K == 2) {
         const float2 c = *reinterpret_cast<const float2*>(row);
-        const bool r = pick2(x, c.x, c.y, flags);
+        const bool r = pick2<kWide>(x, c.x, c.y, flags);
         chosen = r ? c.y : c.x;
         return r ? 1u : 0u;
     } else if constexpr (K == 4) {
         const float4 t = *reinterpret_cast<const float4*>(row);
         const float c[4] = { t.x, t.y, t.z, t.w };
-        const uint32_t j = pick4(x, c, flags);
+        const uint32_t j = pick4<kWide>(x, c, flags);
         chosen = j == 0u ? c[0] : j == 1u ? c[1] : j == 2u ? c[2] : c[3];
         return j;
     } else {
@@ -194,7 +201,7 @@ __device__ __forceinline__ uint32_t step1(const float* row, double& x, float& ch
     }
 }
 
-template <int K>
+template <int K, bool kWide>
 __device__ __forceinline__ void walk(const ShortPlan& plan, const ShortStep* steps, const float* s_top, double x, uint32_t& leaf, float& p, unsigned& flags)
 {
     constexpr uint32_t lg = K == 2 ? 1u : K == 4 ? 2u : K == 8 ? 3u : K == 16 ? 4u : 5u;
@@ -211,91 +218,13 @@ __device__ __forceinline__ void walk(const ShortPlan& plan, const ShortStep* ste
         // (a generic address: staged level or global memory, one code path)
         row = (st.top != kNotStaged ? s_top + st.top : plan.level0 + ((uint64_t)st.off << 6)) + first;
         uint32_t j;
-        if (many) { if constexpr (K <= 4) j = step16<K>(row, x, chosen, flags); }
-        else j = step1<K>(row, x, chosen, flags);
+        if (many) { if constexpr (K <= 4) j = step16<K, kWide>(row, x, chosen, flags); }
+        else j = step1<K, kWide>(row, x, chosen, flags);
         if (K > 4) row += j;
         g = (uint32_t)first + j;
     }
     leaf = g;
     p = K > 4 ? *row : chosen;
-}
-
-// ---- rows --------------------------------------------------------------------------------------------------
-// Where word `w` of a transition lies in the store and in the batch.
-struct ShortWord {
-    const unsigned char* src;
-    unsigned char* dst;
-    uint32_t src_pitch, dst_pitch, log2;
-};
-__device__ __forceinline__ ShortWord find_word(const ShortPlan& plan, uint32_t w)
-{
-    ShortWord o = ShortWord{nullptr, nullptr, 0u, 0u, 0u};
-#pragma unroll
-    for (int f = 0; f < PRB_NUM_FIELDS; ++f) {
-        const ShortField& fd = plan.field[f];
-        if (w >= fd.first) {
-            o.log2 = fd.log2; o.src_pitch = fd.src_pitch; o.dst_pitch = fd.dst_pitch;
-            o.src = fd.src + ((uint64_t)(w - fd.first) << fd.log2);
-            o.dst = fd.dst + ((uint64_t)(w - fd.first) << fd.log2);
-        }
-    }
-    return o;
-}
-
-// The `warps` copying warps of a CTA share the rows: a warp takes a chunk of 32 words (or, with short rows, a whole
-// row per `lane_words` lanes) and every `groups`-th of the CTA's rows; `first` is where the first chunk's word lies,
-// looked up ahead of time.
-struct GatherShare {
-    uint32_t chunk, grp, groups;
-    ShortWord first;
-};
-__device__ __forceinline__ GatherShare gather_share(const ShortPlan& plan, uint32_t warp, uint32_t warps)
-{
-    GatherShare g;
-    g.groups = warps > plan.chunks ? warps / plan.chunks : 1u;
-    g.grp = warp / plan.chunks;
-    g.chunk = warp - g.grp * plan.chunks;
-    if (g.grp >= g.groups) g.chunk = plan.chunks;              // (a warp left over)
-    g.first = find_word(plan, g.chunk * 32u + (threadIdx.x & (plan.lane_words - 1u)));
-    return g;
-}
-
-// Rows of strata [k0, k0 + n): up to eight loads of a thread in flight.
-__device__ __forceinline__ void gather_words(const ShortPlan& plan, const GatherShare& g, uint32_t warps, uint32_t k0, uint32_t n, const uint32_t* s_idx)
-{
-    const uint32_t lane = threadIdx.x & 31u, per_row = plan.lane_words, at_once = 32u / per_row;
-    const uint32_t stride = g.groups * at_once, r_first = g.grp * at_once + lane / per_row;
-    ShortWord o = g.first;
-    for (uint32_t c = g.chunk; c < plan.chunks; c += warps) {
-        const uint32_t w = c * 32u + (lane & (per_row - 1u));
-        if (c != g.chunk) o = find_word(plan, w);
-        if (w >= plan.n_words) continue;
-        unsigned char* const dst = o.dst + (uint64_t)k0 * o.dst_pitch;
-        constexpr int U = 8;
-        for (uint32_t r0 = r_first; r0 < n; r0 += stride * U) {
-            uint32_t v[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const uint32_t r = r0 + u * stride;
-                if (r < n && PRB_IN_BOUNDS(plan, s_idx[r] < plan.capacity)) {
-                    const unsigned char* at = o.src + (uint64_t)s_idx[r] * o.src_pitch;
-                    if (o.log2 == 2u) v[u] = *reinterpret_cast<const uint32_t*>(at);
-                    else if (o.log2 == 1u) v[u] = *reinterpret_cast<const uint16_t*>(at);
-                    else v[u] = *at;
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const uint32_t r = r0 + u * stride;
-                if (r < n) {
-                    unsigned char* at = dst + (uint64_t)r * o.dst_pitch;
-                    if (o.log2 == 2u) *reinterpret_cast<uint32_t*>(at) = v[u];
-                    else if (o.log2 == 1u) *reinterpret_cast<uint16_t*>(at) = (uint16_t)v[u];
-                    else *at = (unsigned char)v[u];
-                }
-            }
-        }
-    }
 }
 
 // ---- weights -----------------------------------------------------------------------------------------------
@@ -344,7 +273,7 @@ __device__ __forceinline__ float weight_of(const ShortPlan& plan, double log_p, 
 }
 
 // Index (and, with uniform replay, all there is to the draw) of stratum k.
-template <int K>
+template <int K, bool kWide>
 __device__ __forceinline__ uint32_t draw(const ShortPlan& plan, const ShortStep* steps, const float* s_top, uint32_t k, double x,
                                          unsigned long long calls, unsigned long long fill, float& p, unsigned& flags)
 {
@@ -353,8 +282,14 @@ __device__ __forceinline__ uint32_t draw(const ShortPlan& plan, const ShortStep*
         return (uint32_t)(((unsigned long long)r0 * fill) >> 32);       // floor(u * fill)
     }
     uint32_t leaf;
-    walk<K>(plan, steps, s_top, x, leaf, p, flags);
+    walk<K, kWide>(plan, steps, s_top, x, leaf, p, flags);
     return leaf;
+}
+
+// Rows of strata [k0, k0 + n).
+__device__ __forceinline__ void gather(const ShortPlan& plan, const PrbWordShare& share, uint32_t warps, uint32_t k0, uint32_t n, const uint32_t* s_idx)
+{
+    prb_copy_words<false>(plan.words, share, warps, k0, n, [&](uint32_t r) { return PRB_IN_BOUNDS(plan, s_idx[r] < plan.capacity) ? s_idx[r] : 0u; });
 }
 
 // What a CTA stages: 16-byte unit `q` of the staged levels, taken one after another (from: nullptr beyond the last).
@@ -417,8 +352,8 @@ prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)sizeof(SmallestSeen) * gridDim.x * strata_warps) : "memory");
     }
-    GatherShare share = {};
-    if (copies) share = gather_share(plan, warp - first_copier, warps - first_copier);
+    PrbWordShare share = {};
+    if (copies) share = prb_word_share(plan.words, warp - first_copier, warps - first_copier);
     StagedUnit unit[kStagedUnits];
 #pragma unroll
     for (uint32_t i = 0; i < kStagedUnits; ++i) unit[i] = plan.uniform ? StagedUnit{nullptr, 0u} : staged_unit(plan, s_top, tid + i * blockDim.x);
@@ -428,8 +363,8 @@ prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
     }
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");      // (every CTA's s_bar can be signalled)
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     prb_dep_wait();
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const unsigned long long calls = plan.state->sample_calls;
     const unsigned long long fill = plan.state->fill;
     const float total32 = *plan.level0;
@@ -453,14 +388,14 @@ prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
     uint32_t leaf = 0;
     if (warp < strata_warps) {
         unsigned flags = 0u;
-        if (mine) { leaf = draw<K>(plan, s_step, s_top, k, x, calls, fill, p, flags); s_idx[tid] = leaf; }
+        if (mine) { leaf = draw<K, false>(plan, s_step, s_top, k, x, calls, fill, p, flags); s_idx[tid] = leaf; }
         __syncwarp();
         if (split) asm volatile("bar.arrive 1, %0;" ::"r"(blockDim.x) : "memory");      // the copying warps may go on
         if (flags) atomicOr(&plan.state->status, flags);
     }
     if (copies) {
         asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");
-        if (split) { gather_words(plan, share, warps - first_copier, k_lo, n, s_idx); return; }
+        if (split) { gather(plan, share, warps - first_copier, k_lo, n, s_idx); return; }
     }
     double log_p = 0.0;
     if (warp < strata_warps) {
@@ -479,7 +414,7 @@ prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
         }
         if (mine) plan.out_idx[k] = (int32_t)leaf;
     }
-    if (!split) gather_words(plan, share, warps, k_lo, n, s_idx);
+    if (!split) gather(plan, share, warps, k_lo, n, s_idx);
     // (the first warp always gets here: it keeps the CTA's shared memory until every value has come)
     if (warp >= strata_warps) return;
     bool there = false;
@@ -542,7 +477,7 @@ prb_sample_grid_kernel(const __grid_constant__ ShortPlan plan)
     }
     if (tid < plan.n_steps) s_step[tid] = plan.step[tid];
     if (tid == 0) { s_min = 0xFFFFFFFFu; s_flags = 0u; }
-    const GatherShare share = gather_share(plan, tid >> 5, warps);
+    const PrbWordShare share = prb_word_share(plan.words, tid >> 5, warps);
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     if (poisoned) {
@@ -565,7 +500,7 @@ prb_sample_grid_kernel(const __grid_constant__ ShortPlan plan)
         const uint32_t n = min(kShortThreads, k_hi - kb), k = kb + tid;
         if (tid < n) {
             const double x = plan.uniform ? 0.0 : prb_stratum_target(k, plan.B, (double)total32, calls, plan.seed);
-            const uint32_t leaf = draw<K>(plan, s_step, s_top, k, x, calls, fill, p, flags);
+            const uint32_t leaf = draw<K, true>(plan, s_step, s_top, k, x, calls, fill, p, flags);
             s_idx[tid] = leaf;
             plan.out_idx[k] = (int32_t)leaf;
             best = min(best, __float_as_uint(p));
@@ -588,7 +523,7 @@ prb_sample_grid_kernel(const __grid_constant__ ShortPlan plan)
             if (exchange) atomicMax(&plan.state->wide_wmax_bits, (unsigned long long)(~s_min));
             asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&plan.state->sample_ticket) : "memory");
         }
-        gather_words(plan, share, warps, kb, n, s_idx);
+        gather(plan, share, warps, kb, n, s_idx);
         if (!last) __syncthreads();           // s_idx is rewritten by the next pass
     }
     if (tid == kShortThreads - 1u) {
@@ -704,22 +639,7 @@ int prb_launch_sample_short(const PrbView& v, uint32_t B, float beta, uint64_t s
         if (staging) at += entries;
     }
     plan.n_steps = n;
-    uint32_t words = 0;
-    for (int f = 0; f < PRB_NUM_FIELDS; ++f) {
-        ShortField& fd = plan.field[f];
-        fd = ShortField{nullptr, nullptr, 0xFFFFFFFFu, 0u, 0u, 0u};
-        if (dst.ptr[f] == nullptr || v.field_bytes[f] == 0) continue;
-        fd.src = v.store[f];
-        fd.dst = dst.ptr[f];
-        fd.log2 = v.field_vec[f] >= 4u ? 2u : v.field_vec[f] == 2u ? 1u : 0u;
-        fd.first = words;
-        fd.src_pitch = v.field_pitch[f];
-        fd.dst_pitch = v.field_bytes[f];
-        words += v.field_bytes[f] >> fd.log2;
-    }
-    plan.n_words = words;
-    plan.chunks = words ? (words + 31u) / 32u : 1u;
-    plan.lane_words = words <= 8u ? 8u : words <= 16u ? 16u : 32u;
+    plan.words = prb_plan_words(v, dst);
     cudaLaunchConfig_t cfg = {};
     cfg.stream = s;
     cudaLaunchAttribute a[2];

@@ -9,14 +9,6 @@
 
 #ifdef __CUDACC__
 
-// Inputs of entry `rank` that a kernel may have fetched before the team's work starts (so that the
-// fetch overlaps an earlier wait); valid only where the matching flag is set.
-struct PrbPreloaded {
-    bool has_update, has_prio;
-    int32_t idx;
-    float val, prio;
-};
-
 struct PrbTeam {
     uint32_t rank, size;     // this thread's rank in the team, number of threads (multiple of 32)
     bool whole_cta;          // the team is the whole CTA: plain __syncthreads; otherwise named barrier 1
@@ -394,69 +386,44 @@ __host__ __device__ inline size_t prb_update_smem_bytes(uint32_t n2)
     return (size_t)n2 * (sizeof(unsigned long long) + sizeof(float));
 }
 
-// Batched priority update by one team (PEARL Section V-A, "priority update", read as set +
-// re-sum).  Entries are keyed (index, batch position) and sorted -- with one entry per thread by
-// warp-wide sorting networks and a merge by rank, each thread then holding its place's index and
-// its neighbours' in registers; with more, by a bitonic network in shared memory.  The last entry
-// of every run of equal indices wins and writes its leaf (raw == 2: adds the run's changes to the
-// leaf in batch order); then, level by level from the deepest down to the staged top, the first
-// entry of every run of equal ancestors re-sums that ancestor from its children in left-to-right
-// order, and the staged levels are re-summed whole (prb_top_passes).  Sorted order survives
-// dropping low digits of the index, so no list is compacted and no lock is taken.
-// raw: 0 = val holds TD errors (transformed), 1 = priorities, 2 = changes of priorities.
-// n2 = prb_update_n2(B); smem holds
-// prb_update_smem_bytes(n2) bytes; fill = the fill count before this launch (indices must be below it).
-// With stale > 0 (and n == 0) entries that name one of the `stale` ring slots before `cursor` are
-// skipped: they were overwritten after they had been sampled.
-// With n > 0 the tree part of an insertion of n transitions at `cursor` follows in the same
-// passes: the inserted leaves are written after the update's (an updated leaf that is also
-// inserted keeps the inserted priority), and every level is re-summed once for both, the
-// insertion's parents being the contiguous range(s) above its slots.  A parent reached both ways
-// is computed twice with the same result.
-__device__ __forceinline__ void prb_update_team(const PrbView& v, const PrbTeam& team, uint32_t B, uint32_t n2,
-                                                const int32_t* __restrict__ idx, const float* __restrict__ val, int raw,
-                                                float alpha, float eps, unsigned long long fill, unsigned char* smem,
-                                                uint32_t n = 0, const float* __restrict__ prio = nullptr,
-                                                uint64_t cursor = 0, PrbPreloaded pre = PrbPreloaded{false, false, 0, 0.0f, 0.0f},
-                                                uint32_t stale = 0, PrbTop top = PrbTop{}, const unsigned char* __restrict__ ins_done = nullptr,
-                                                uint32_t stack = 0)
+// A batch of changes by one team (PEARL Section V-A's interface).  Entries are keyed (index, batch position) and
+// sorted -- with one entry per thread by warp-wide sorting networks and a merge by rank, each thread then holding
+// its place's index and its neighbours' in registers; with more, by a bitonic network in shared memory.  The
+// last entry of every run of equal indices adds the run's changes to the leaf one by one in batch order -- the
+// order of the sorted run -- skipping a sum that is not a valid priority; then, level by level from the deepest
+// down to the staged top, the first entry of every run of equal ancestors re-sums that ancestor from its
+// children in left-to-right order, and the staged levels are re-summed whole (prb_top_passes).  Sorted order
+// survives dropping low digits of the index, so no list is compacted and no lock is taken.
+// n2 = prb_update_n2(B); smem holds prb_update_smem_bytes(n2) bytes; fill = the fill count before this launch
+// (indices must be below it).
+__device__ __forceinline__ void prb_delta_team(const PrbView& v, const PrbTeam& team, uint32_t B, uint32_t n2,
+                                               const int32_t* __restrict__ idx, const float* __restrict__ val,
+                                               unsigned long long fill, unsigned char* smem, uint64_t cursor, PrbTop top, uint32_t stack)
 {
-    // (frames: the insertion's dirty leaves reach past its n transitions; cursor, fill and priorities do not)
-    const uint32_t n_leaves = n + prb_cleared_after(v, n, stack);
     unsigned long long* keys = reinterpret_cast<unsigned long long*>(smem);
     float* vals = reinterpret_cast<float*>(smem + (size_t)n2 * sizeof(unsigned long long));
     const uint32_t rank = team.rank, nt = team.size;
     const bool one_each = n2 <= nt;        // every thread holds one entry, in registers from the sort on
     const uint64_t N = v.capacity;
 
-    // transform and validate; vals[b] = the priority entry b would write
+    // validate; vals[b] = the change of entry b
     unsigned flags = 0;
-    float wmax = 0.0f;                 // largest priority this thread accepted
     bool my_valid = false;
     uint32_t my_idx = 0;
     for (uint32_t b = rank; b < n2; b += nt) {
         unsigned long long key = 0xFFFFFFFF00000000ull | b;
         if (b < B) {
-            const bool mine = pre.has_update && b == rank;
-            const int32_t i = mine ? pre.idx : idx[b];
-            const float x = mine ? pre.val : val[b];
-            float p = 0.0f;
-            bool ok_p;
-            if (raw == 2) { p = x; ok_p = fabsf(x) <= 3.402823466e+38f; }      // a change: any finite value
-            else if (raw) { p = x; ok_p = prb_valid_priority(p); }
-            else ok_p = prb_priority_pow(x, eps, alpha, p);
-            // stale: one of the `stale` slots written most recently, i.e. overwritten since it was sampled
-            const uint64_t back = (i >= 0 && stale) ? (cursor + N - 1 - (uint64_t)i) % N : ~0ull;
+            const int32_t i = idx[b];
+            const float x = val[b];
             if (i < 0 || (unsigned long long)i >= fill) flags |= PEARL_ST_BAD_INDEX;
-            else if (back < stale || prb_history_less(v, cursor, (uint64_t)i, stack)) flags |= PEARL_ST_STALE;
-            else if (!ok_p) flags |= PEARL_ST_BAD_PRIORITY;
-            else { key = ((unsigned long long)(uint32_t)i << 32) | b; if (raw != 2) wmax = fmaxf(wmax, p); my_valid = true; my_idx = (uint32_t)i; }
-            vals[b] = p;
+            else if (prb_history_less(v, cursor, (uint64_t)i, stack)) flags |= PEARL_ST_STALE;
+            else if (!(fabsf(x) <= 3.402823466e+38f)) flags |= PEARL_ST_BAD_PRIORITY;
+            else { key = ((unsigned long long)(uint32_t)i << 32) | b; my_valid = true; my_idx = (uint32_t)i; }
+            vals[b] = x;
         }
         if (!one_each) keys[b] = key;
     }
     if (flags && team.part == 0) atomicOr(&v.state->status, flags);
-    prb_note_priorities(v.state, wmax, team.part == 0);
     prb_top_wait();                // (the staged top of the tree, if the kernel started a copy)
 
     PrbSlot slot = PrbSlot{0xFFFFFFFFu, 0u, 0xFFFFFFFFu, 0xFFFFFFFFu};
@@ -507,91 +474,48 @@ __device__ __forceinline__ void prb_update_team(const PrbView& v, const PrbTeam&
         else team.phase_sync();
     };
     float* leaves = v.level[v.depth];
-    if (raw == 2) {
-        // Changes instead of values (n == 0): the last entry of a run of equal indices adds the run's
-        // changes to the leaf one by one in batch order -- the order of the sorted run -- skipping a
-        // sum that is not a valid priority.
-        float dmax = 0.0f;
-        bool refused = false;
-        auto add_change = [&](float& p, float change) {
-            const float q = __fadd_rn(p, change);
-            if (prb_valid_priority(q)) { p = q; dmax = fmaxf(dmax, q); }
-            else refused = true;
-        };
-        if (one_each) {
-            // the sorted indices and positions of all slots, in place of the keys
-            uint32_t* sidx = reinterpret_cast<uint32_t*>(smem);
-            uint32_t* spos = sidx + n2;
-            team.sync();
-            if (rank < n2) { sidx[rank] = slot.idx; spos[rank] = slot.pos; }
-            team.sync();
-            if (slot.idx != 0xFFFFFFFFu && slot.next != slot.idx && mine(slot.idx, rank)) {
-                uint32_t s0 = rank;
-                while (s0 > 0 && sidx[s0 - 1] == slot.idx) --s0;
-                if (PRB_IN_BOUNDS(v, slot.idx < v.level_alloc[v.depth])) {
-                    float p = __ldcg(leaves + slot.idx);
-                    for (uint32_t s2 = s0; s2 <= rank; ++s2) add_change(p, vals[spos[s2]]);
-                    leaves[slot.idx] = p;
-                }
-            }
-        } else {
-            for (uint32_t s1 = rank; s1 < n2; s1 += nt) {
-                const unsigned long long key = keys[s1];
-                if (prb_key_invalid(key) || !mine(key >> 32, s1)) continue;
-                const uint32_t i = (uint32_t)(key >> 32);
-                if (s1 + 1 < n2 && (uint32_t)(keys[s1 + 1] >> 32) == i) continue;      // not the last of its run
-                uint32_t s0 = s1;
-                while (s0 > 0 && (uint32_t)(keys[s0 - 1] >> 32) == i) --s0;
-                float p = __ldcg(leaves + i);
-                for (uint32_t s2 = s0; s2 <= s1; ++s2) add_change(p, vals[(uint32_t)keys[s2]]);
-                leaves[i] = p;
-            }
-        }
-        if (refused) atomicOr(&v.state->status, PEARL_ST_BAD_PRIORITY);
-        prb_note_priorities(v.state, dmax, true);
-    } else if (one_each) {
+    float dmax = 0.0f;
+    bool refused = false;
+    auto add_change = [&](float& p, float change) {
+        const float q = __fadd_rn(p, change);
+        if (prb_valid_priority(q)) { p = q; dmax = fmaxf(dmax, q); }
+        else refused = true;
+    };
+    if (one_each) {
+        // the sorted indices and positions of all slots, in place of the keys
+        uint32_t* sidx = reinterpret_cast<uint32_t*>(smem);
+        uint32_t* spos = sidx + n2;
+        team.sync();
+        if (rank < n2) { sidx[rank] = slot.idx; spos[rank] = slot.pos; }
+        team.sync();
         if (slot.idx != 0xFFFFFFFFu && slot.next != slot.idx && mine(slot.idx, rank)) {
-            const uint64_t ahead = slot.idx >= cursor ? slot.idx - cursor : slot.idx + N - cursor;   // distance from the cursor along the ring
-            if (!(ahead < n_leaves) && PRB_IN_BOUNDS(v, slot.idx < v.level_alloc[v.depth] && slot.pos < n2)) leaves[slot.idx] = vals[slot.pos];
+            uint32_t s0 = rank;
+            while (s0 > 0 && sidx[s0 - 1] == slot.idx) --s0;
+            if (PRB_IN_BOUNDS(v, slot.idx < v.level_alloc[v.depth])) {
+                float p = __ldcg(leaves + slot.idx);
+                for (uint32_t s2 = s0; s2 <= rank; ++s2) add_change(p, vals[spos[s2]]);
+                leaves[slot.idx] = p;
+            }
         }
     } else {
-        for (uint32_t s = rank; s < n2; s += nt) {
-            const unsigned long long key = keys[s];
-            if (prb_key_invalid(key) || !mine(key >> 32, s)) continue;
+        for (uint32_t s1 = rank; s1 < n2; s1 += nt) {
+            const unsigned long long key = keys[s1];
+            if (prb_key_invalid(key) || !mine(key >> 32, s1)) continue;
             const uint32_t i = (uint32_t)(key >> 32);
-            const bool last = (s + 1 == n2) || ((uint32_t)(keys[s + 1] >> 32) != i);
-            const uint64_t ahead = i >= cursor ? i - cursor : i + N - cursor;
-            if (last && !(ahead < n_leaves) && PRB_IN_BOUNDS(v, i < v.level_alloc[v.depth] && (uint32_t)key < n2)) leaves[i] = vals[(uint32_t)key];
+            if (s1 + 1 < n2 && (uint32_t)(keys[s1 + 1] >> 32) == i) continue;      // not the last of its run
+            uint32_t s0 = s1;
+            while (s0 > 0 && (uint32_t)(keys[s0 - 1] >> 32) == i) --s0;
+            float p = __ldcg(leaves + i);
+            for (uint32_t s2 = s0; s2 <= s1; ++s2) add_change(p, vals[(uint32_t)keys[s2]]);
+            leaves[i] = p;
         }
     }
-    bool bad = false;
-    float imax = 0.0f;
-    // without priorities the new transitions take the running maximum, this update's writes included
-    // (reported by CTA 0: in a cluster the others read it after a barrier)
-    if (n && prio == nullptr && team.parts > 1) { __threadfence(); team.phase_sync(); }
-    const float dflt = (n && prio == nullptr) ? prb_default_priority(__ldcg(&v.state->max_prio_bits)) : 0.0f;
-    for (uint32_t t = rank; t < n_leaves; t += nt) {
-        uint64_t at = cursor + t;
-        if (at >= N) at -= N;
-        if (!mine(at, t)) continue;
-        float p = 0.0f;
-        if (t < n && !(stack && (ins_done[t] & kPrbEpisodeStart))) {
-            p = prio == nullptr ? dflt : ((pre.has_prio && t == rank) ? pre.prio : prio[t]);
-            if (!prb_valid_priority(p)) { p = 0.0f; bad = true; }
-            else imax = fmaxf(imax, p);
-        }
-        if (PRB_IN_BOUNDS(v, at < N)) leaves[at] = p;
-    }
-    if (bad) atomicOr(&v.state->status, PEARL_ST_BAD_PRIORITY);
-    if (n) prb_note_priorities(v.state, imax, true);      // (every CTA of a cluster wrote leaves of its own; a first default insertion writes 1)
+    if (refused) atomicOr(&v.state->status, PEARL_ST_BAD_PRIORITY);
+    prb_note_priorities(v.state, dmax, true);
     pass_sync(false);
 
     // re-sum the ancestors below the staged levels, deepest level first: the first entry of every run
-    // of equal ancestors does it; the insertion dirties parent range A = [a0, a1] >> sh and, if the
-    // ring wrapped, B = [0, b1] >> sh
-    const uint64_t a0 = cursor, a1 = (n ? min(cursor + n_leaves, N) : cursor + 1) - 1;
-    const bool wrapped = cursor + n_leaves > N;
-    const uint64_t b1 = wrapped ? cursor + n_leaves - N - 1 : 0;
+    // of equal ancestors does it
     for (int l = (int)v.depth - 1; l >= (int)T; --l) {
         const uint32_t sh = min(lg * (v.depth - (uint32_t)l), 31u);      // (indices are below 2^31)
         if (one_each) {
@@ -607,15 +531,6 @@ __device__ __forceinline__ void prb_update_team(const PrbView& v, const PrbTeam&
                 if (first) prb_resum(v, top, team, T, (uint32_t)l, a);
             }
         }
-        if (n) {
-            const uint64_t pa0 = a0 >> sh, cntA = (a1 >> sh) - pa0 + 1;
-            uint64_t cntB = 0;
-            if (wrapped) cntB = (pa0 == 0) ? 0 : min(b1 >> sh, pa0 - 1) + 1;     // parents of B not already in A
-            for (uint64_t i = rank; i < cntA + cntB; i += nt) {
-                const uint64_t a = (i < cntA) ? pa0 + i : i - cntA;
-                if (mine_node(a, (uint32_t)l, (uint32_t)i)) prb_resum(v, top, team, T, (uint32_t)l, a);
-            }
-        }
         pass_sync((uint32_t)l == T);
     }
     // the staged levels: CTA 0 alone
@@ -627,13 +542,11 @@ __device__ __forceinline__ void prb_update_team(const PrbView& v, const PrbTeam&
 // a contiguous parent range on every level (two ranges if the ring wrapped), so nothing is sorted.
 __device__ __forceinline__ void prb_insert_tree_team(const PrbView& v, const PrbTeam& team, uint32_t n,
                                                      const float* __restrict__ prio, uint64_t cursor,
-                                                     PrbPreloaded pre = PrbPreloaded{false, false, 0, 0.0f, 0.0f},
-                                                     unsigned max_bits = 0, PrbTop top = PrbTop{},
-                                                     const unsigned char* __restrict__ ins_done = nullptr, uint32_t stack = 0)
+                                                     unsigned max_bits, const unsigned char* __restrict__ ins_done, uint32_t stack)
 {
     const uint64_t N = v.capacity;
     const uint32_t n_leaves = n + prb_cleared_after(v, n, stack);
-    const uint32_t D = v.depth, lg = v.log2_fanout, T = prb_top_levels(v, top);
+    const uint32_t D = v.depth, lg = v.log2_fanout;
     float* leaves = v.level[D];
     bool bad = false;
     float imax = 0.0f;
@@ -643,7 +556,7 @@ __device__ __forceinline__ void prb_insert_tree_team(const PrbView& v, const Prb
         if (slot >= N) slot -= N;
         float p = 0.0f;
         if (t < n && !(stack && (ins_done[t] & kPrbEpisodeStart))) {
-            p = prio == nullptr ? dflt : ((pre.has_prio && t == team.rank) ? pre.prio : prio[t]);
+            p = prio == nullptr ? dflt : prio[t];
             if (!prb_valid_priority(p)) { p = 0.0f; bad = true; }
             else imax = fmaxf(imax, p);
         }
@@ -651,14 +564,13 @@ __device__ __forceinline__ void prb_insert_tree_team(const PrbView& v, const Prb
     }
     if (bad) atomicOr(&v.state->status, PEARL_ST_BAD_PRIORITY);
     prb_note_priorities(v.state, imax, true);                       // (a first default insertion writes 1)
-    prb_top_wait();
     team.sync();
     // dirty leaf ranges: A = [a0, a1]; if the ring wrapped also B = [0, b1]
     const uint64_t a0 = cursor;
     const uint64_t a1 = min(cursor + n_leaves, N) - 1;
     const bool wrapped = cursor + n_leaves > N;
     const uint64_t b1 = wrapped ? cursor + n_leaves - N - 1 : 0;
-    for (int l = (int)D - 1; l >= (int)T; --l) {
+    for (int l = (int)D - 1; l >= 0; --l) {
         const uint32_t sh = lg * (D - (uint32_t)l);
         const uint64_t pa0 = a0 >> sh, pa1 = a1 >> sh;
         const uint64_t cntA = pa1 - pa0 + 1;
@@ -668,10 +580,9 @@ __device__ __forceinline__ void prb_insert_tree_team(const PrbView& v, const Prb
             cntB = (pa0 == 0) ? 0 : min(pb1, pa0 - 1) + 1;   // parents of B not already in A
         }
         for (uint64_t i = team.rank; i < cntA + cntB; i += team.size)
-            prb_resum(v, top, team, T, (uint32_t)l, (i < cntA) ? pa0 + i : i - cntA);
+            prb_resum(v, PrbTop{}, team, 0u, (uint32_t)l, (i < cntA) ? pa0 + i : i - cntA);
         team.sync();
     }
-    prb_top_passes(v, top, team, T);
 }
 
 #endif  // __CUDACC__

@@ -1,0 +1,65 @@
+"""The tree kernel (update, insertion, both) at the sizes where its form changes: one CTA, clusters, the grid; several
+levels per pass (fanouts 2 and 4), trees too shallow for that, levels that end inside a group; batches that fall to one
+subtree; insertions that wrap; and what an update and an insertion both write."""
+import numpy as np
+import pytest
+
+from prb_harness import Pair
+
+pytestmark = pytest.mark.gpu
+
+
+def _batch(rng, n, obs_bytes, act_bytes):
+    prio = np.exp(rng.standard_normal(n)).astype(np.float32)
+    prio[rng.random(n) < 0.05] = np.nan
+    return dict(obs=rng.integers(0, 256, size=(n, obs_bytes), dtype=np.uint8), act=rng.integers(0, 256, size=(n, act_bytes), dtype=np.uint8),
+                rew=rng.standard_normal(n).astype(np.float32), next_obs=rng.integers(0, 256, size=(n, obs_bytes), dtype=np.uint8),
+                done=rng.integers(0, 2, size=n, dtype=np.uint8), prio=prio)
+
+
+def _check(pr, min_tree):
+    pr.compare_tree()
+    if min_tree:
+        pr.compare_min_tree()
+    pr.compare_status()
+    pr.compare_state()
+
+
+@pytest.mark.parametrize("min_tree", [False, True])
+@pytest.mark.parametrize("K,N", [(2, 3), (2, 33), (2, 70), (2, 40_001), (4, 17), (4, 30_000), (8, 9000), (16, 70_001), (32, 31), (32, 40_000)])
+def test_forms(oracle_mod, K, N, min_tree):
+    rng = np.random.default_rng(K * 100 + N)
+    pr = Pair(oracle_mod, N, K, 12, 4, 70_000, min_tree=min_tree)
+    pr.insert(_batch(rng, N - N // 4, 12, 4))                                 # (a quarter of the ring stays unwritten)
+    _check(pr, min_tree)
+    for B, n in [(1, 1), (33, 5), (64, 64), (65, 300), (257, 0), (512, 777), (1000, 31), (1024, 4097), (1025, 1), (4099, 100), (20_000, 17)]:
+        n = min(n, N)
+        fill = pr.gpu.info()[0]
+        idx = rng.integers(-1, fill + 1, size=B).astype(np.int32)             # (some out of range)
+        if B > 40:
+            idx[B // 2:] = np.where(rng.random(B - B // 2) < 0.5, idx[:B - B // 2], idx[B // 2:])     # repeats, the later one wins
+        td = rng.standard_normal(B).astype(np.float32)
+        td[rng.random(B) < 0.02] = np.inf
+        if n:
+            pr.update_insert(idx, td, 0.6, 1e-6, _batch(rng, n, 12, 4))
+        else:
+            pr.update(idx, td, 0.6, 1e-6)
+        _check(pr, min_tree)
+    pr.compare_rows(np.arange(pr.gpu.info()[0], dtype=np.int32))
+    pr.close()
+
+
+@pytest.mark.parametrize("K,N", [(2, 1 << 16), (4, 1 << 18), (32, 1 << 19)])
+def test_batch_in_one_subtree(oracle_mod, K, N):
+    # all entries fall to the leaves of one CTA: more than its list holds at a time, worked off in batch order
+    rng = np.random.default_rng(K)
+    pr = Pair(oracle_mod, N, K, 0, 0, 30_000)
+    for at in range(0, N, 30_000):
+        pr.insert(dict(prio=np.exp(rng.standard_normal(min(30_000, N - at))).astype(np.float32)))
+    for span in (1, 30, 5000):
+        for B in (1500, 9000, 30_000):
+            idx = (N // 2 + rng.integers(0, span, size=B)).astype(np.int32)
+            pr.update_priorities(idx, np.exp(rng.standard_normal(B)).astype(np.float32))
+            pr.compare_tree()
+    pr.compare_status()
+    pr.close()
