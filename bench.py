@@ -552,7 +552,7 @@ def run_ours(args, wl, rank, world):
                          "value_from": "median" if len(m["region_ms"]) > 1 else "the one region"},
         "rates": rates,
         "roofline": {"kernel": "prb_gather_rows_kernel (+ prb_descend_kernel beside the copy before it)" if long_rows and not args.no_graph
-                     else "prb_sample_kernel",
+                     else ("prb_sample_kernel" if long_rows else "prb_sample_cluster_kernel"),
                      "bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "peak_kind": "%s copy bandwidth" % peak_kind,
                      "frac_of_8TBs_nominal": achieved / 8000.0, "bytes_per_launch": sample_bytes,
@@ -574,7 +574,7 @@ def run_ours(args, wl, rank, world):
                              "peak": peak, "unit": "GB/s", "frac": step_bytes / (ms / args.steps * 1e-3) / 1e9 / peak}
     if n_ins:
         ins_bytes = n_ins * (2 * E + 4)
-        line["roofline_insert"] = {"kernel": "prb_insert_rows_kernel" if long_rows else "prb_insert_kernel", "bound": "hbm",
+        line["roofline_insert"] = {"kernel": "prb_insert_rows_kernel" if long_rows else "prb_tree_kernel", "bound": "hbm",
                                    "bytes_per_launch": ins_bytes,
                                    "achieved": ins_bytes / (m["ms_insert"] * 1e-3) / 1e9, "peak": peak, "unit": "GB/s",
                                    "frac": ins_bytes / (m["ms_insert"] * 1e-3) / 1e9 / peak}

@@ -55,24 +55,21 @@ typedef struct pearl_layout {
 #define PEARL_ST_EMPTY 4u          /* sample on an empty buffer or a non-positive total; outputs untouched */
 #define PEARL_ST_CLAMPED 8u        /* a descent met residual >= last prefix sum and took the last positive child */
 #define PEARL_ST_INTERNAL 16u      /* inconsistent tree met during a descent, or a bounded wait ran out.
-                                      Every wait on the device (a bulk copy's completion, the grid barrier of
-                                      a large update) gives up after a fixed number of polls instead of
-                                      hanging.  After a copy that gave up, rows of that call are missing or
-                                      partial.  After an update of more than 1024 entries that gave up, the
-                                      tree is not consistent: leaves named by the batch may hold the marker
-                                      bit pattern 0x80000000|entry instead of a priority, and parents may not
-                                      equal the sum of their children; every later update of more than 1024
-                                      entries on that buffer raises the bit again and does nothing.  Treat the
-                                      buffer as lost: destroy it and build a new one.  No correct run raises
-                                      this bit. */
+                                      Every wait on the device (a bulk copy's completion, one thread block's
+                                      wait for the others of its call) gives up after a fixed number of polls
+                                      instead of hanging.  After a copy that gave up, rows of that call are
+                                      missing or partial; after an update or insertion, nodes of the tree's
+                                      top may not equal the sum of their children; after a sample of short
+                                      rows, weights are missing, and every later sample of more than 1536
+                                      strata of short rows on that buffer raises the bit again and does
+                                      nothing.  Treat the buffer as lost: destroy it and build a new one.  No
+                                      correct run raises this bit. */
 #define PEARL_ST_STALE 32u         /* update_after_insert: the index was overwritten since it was sampled; entry skipped */
 
-/* The largest update batch one thread block handles.  A batch of more than 1024 priorities or TD
- * errors is applied by one launch of many co-resident thread blocks (a cooperative launch; the last
- * valid entry of a repeated index still wins); a batch of changes (pearl_prb_update_delta) of any
- * size, or any batch on a device without cooperative launches, by one thread block per sub-batch of
- * at most this many entries, sub-batches in batch order, one launch each.  The result is that of
- * the whole batch either way. */
+/* The largest batch of changes (pearl_prb_update_delta) one launch handles: a larger one is applied as
+ * sub-batches of at most this many entries, in batch order, one launch each, with the result of the whole
+ * batch.  A batch of priorities or TD errors of any size is one launch; the last valid entry of a repeated
+ * index wins. */
 #define PEARL_UPDATE_SUBBATCH 4096u
 
 /* Bytes of device memory a buffer of this geometry needs (tree, storage, scratch and the
@@ -227,10 +224,11 @@ int pearl_prb_get_priorities(pearl_prb_t* prb, uint32_t B, const int32_t* d_idx,
  * pearl_prb_update(prb, B, d_idx, d_td, alpha, eps) followed by pearl_prb_insert(prb, n, ...): the
  * update's tree work is done first, the insertion's tree work after it, by the same thread blocks,
  * while other thread blocks already copy the new rows into the Data Storage (an update touches
- * the tree only, so the two do not conflict).  Short rows: one launch (update batches of 1024 entries
- * and more: the update's launch, then the insertion's).  Rows of 8 KB and more: the
- * tree work is a kernel of its own on a second stream of the handle, beside the kernel that copies
- * the rows; the handle's stream continues when both are done (capturable in a CUDA graph).  This
+ * the tree only, so the two do not conflict).  Short rows: one launch (two if d_prio is NULL and the update is
+ * more than one thread block's work).  Rows of 8 KB and more: the
+ * tree work is a kernel of its own beside the kernel that copies the rows -- on a second stream of the
+ * handle when the rows come to more than 4 MB -- and the handle's stream continues when both are done
+ * (capturable in a CUDA graph).  This
  * is the overlap of the paper's training
  * protocol, where insertion runs beside the priority update (Section IV-C; Eq. 7:
  * T_itr = T_samp + max(T_ins, T_upd + T_learner)).  Arguments and errors as for the two calls. */
@@ -302,7 +300,7 @@ int pearl_prb_update_host(pearl_prb_t* prb, uint32_t B, const int32_t* h_idx, co
  * transitions and the sample of the next batch, with every array in host memory (Section IV-A: the host
  * runtime exchanges requests and data with the Replay Manager over PCIe).  Returns when the sampled batch is
  * in the caller's arrays.  A step whose inputs and whose outputs come to at most 256 KB each makes no copy
- * call: the inputs are gathered in a pinned buffer of the handle that the device reads in place, the kernels
+ * call (one, of the indices and TD errors, from 1025 updates on): the inputs are gathered in a pinned buffer of the handle that the device reads in place, the kernels
  * write the batch into that buffer, and the step's one synchronisation is the wait for them.  A larger step
  * that inserts and samples rows of 8 KB and more (plain layout, n >= 1, B_upd <= PEARL_UPDATE_SUBBATCH) keeps
  * both directions of the host link busy at once: the new rows travel to the device on a stream of the handle
@@ -329,8 +327,8 @@ int pearl_prb_step_host(pearl_prb_t* prb, uint32_t B_upd, const int32_t* h_upd_i
  * framework whose memory pool has already claimed the whole GPU, so that a cudaMalloc would fail
  * or fragment it; a real-time control or serving loop whose rules forbid allocator calls after
  * start-up.  Such a caller hands in the same inputs and outputs as pearl_prb_sample, and the
- * kernel's scratch (the batch's raw, un-normalised importance-sampling weights, one binary64 per
- * stratum) lives in a fixed 32 KiB array that is part of the library image: every GPU on which
+ * kernel's scratch (rows of 8 KB and more: the batch's raw, un-normalised importance-sampling weights, one
+ * binary64 per stratum) lives in a fixed 32 KiB array that is part of the library image: every GPU on which
  * the library runs this call holds that array until the process exits, whether or not it is used
  * again.  The call itself performs no cudaMalloc/cudaFree and calls no allocating routine.
  *

@@ -125,7 +125,8 @@ struct PrbSubStreams {
 int prb_launch_sample(const PrbView& v, uint32_t B, float beta, uint64_t seed, int32_t* d_idx, float* d_w,
                       const PrbBatch& dst, cudaStream_t s, int uniform = 0, uint32_t n_sub = 1,
                       const PrbSubStreams* subs = nullptr, int buffer_norm = 0);
-// The same for short rows of a buffer without frames, in one launch (prb_sample_short.cu).
+// The same for short rows of a buffer without frames, in one launch (prb_sample_short.cu); 0: this device has no
+// cooperative launches and the batch needs one.
 int prb_launch_sample_short(const PrbView& v, uint32_t B, float beta, uint64_t seed, int32_t* d_idx, float* d_w, const PrbBatch& dst,
                             cudaStream_t s, int uniform, int buffer_norm);
 // The scan of the leaves for their smallest positive one, into PrbState::pmin_bits.
@@ -316,24 +317,6 @@ __device__ __forceinline__ float prb_default_priority(unsigned max_bits)
 __device__ __forceinline__ bool prb_valid_priority(float p)
 {
     return (p >= 0.0f) && (p <= 3.402823466e+38f);   // false for NaN, negative, +Inf
-}
-
-// Contiguous copy of n 16-byte granules by all threads of the CTA (the bandwidth-critical path:
-// one chunk of a long row).  Each thread issues up to U independent loads before its stores;
-// consecutive threads touch consecutive granules.
-template <int U>
-__device__ __forceinline__ void prb_copy_span16(uint4* __restrict__ dst, const uint4* __restrict__ src, uint32_t n)
-{
-    const uint32_t stride = blockDim.x;
-    for (uint32_t base = threadIdx.x; base < n; base += stride * U) {
-        uint4 tmp[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (base + u * stride < n) tmp[u] = __ldcs(src + base + u * stride);
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (base + u * stride < n) __stcs(dst + base + u * stride, tmp[u]);
-    }
 }
 
 // Copy of short rows: granule e of [e_begin, e_end) is read from src[src_at(e)] and written to

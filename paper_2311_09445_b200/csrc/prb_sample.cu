@@ -1,5 +1,6 @@
 // Stratified priority sampling, importance-sampling weights and the gather of the sampled
-// transitions, in one kernel.
+// transitions, in one kernel: long rows, rebuilt observations (frames) and the sub-batches of a streamed
+// call (short rows otherwise: prb_sample_short.cu).
 //
 // Priority sampling is Eq. 1 of PEARL (Section II-A) carried out as Section V-A describes it:
 // "traversing the tree performing prefix sum from root to leaf".  A group of K lanes (K = the
@@ -795,7 +796,10 @@ int prb_launch_sample(const PrbView& v, uint32_t B, float beta, uint64_t seed, i
     const bool row_mode = plan_row_mode(v, dst, plan);
     // Short rows in one piece have a kernel of their own (prb_sample_short.cu); here: long rows, rebuilt
     // observations, and the sub-batches of a streamed call.
-    if (!row_mode && n_sub == 1 && v.stack == 0) return prb_launch_sample_short(v, B, beta, seed, d_idx, d_w, dst, s, uniform, buffer_norm);
+    if (!row_mode && n_sub == 1 && v.stack == 0) {
+        const int k = prb_launch_sample_short(v, B, beta, seed, d_idx, d_w, dst, s, uniform, buffer_norm);
+        if (k != 0) return k;
+    }
     plan.n_tasks = B * plan.tps;
     plan.first_task = 0;
     plan.ticket_total = 0;

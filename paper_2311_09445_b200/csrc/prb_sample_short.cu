@@ -593,7 +593,7 @@ const ShortLimits* short_limits(uint32_t fanout, int ki, int dev)
     if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kg, (int)kShortThreads, 0) != cudaSuccess || nb < 1) {
         cudaGetLastError();
-        return nullptr;
+        nb = 0;                                          // (no grid form here)
     }
     l.per_sm = nb > 2 ? 2u : (uint32_t)nb;
     l.cluster = cluster;
@@ -607,7 +607,7 @@ int prb_launch_sample_short(const PrbView& v, uint32_t B, float beta, uint64_t s
 {
     const int dev = prb_current_device();
     const ShortLimits* lim = short_limits(v.fanout, (int)v.log2_fanout, dev);
-    if (lim == nullptr) return -1;
+    if (B > kClusterStrata && lim->per_sm == 0) return 0;
     ShortPlan plan;
     plan.state = v.state;
     plan.level0 = v.level[0];

@@ -1,8 +1,7 @@
-// Sum-tree maintenance shared by the update and insert kernels: the priority transform, the
-// batched leaf update with last-writer-wins deduplication, and the re-sum of a contiguous range
-// of inserted leaves.  All of it is written for a "team": a whole number of warps of one CTA
-// that synchronise on their own barrier, so that the same code runs as a full CTA (the update
-// kernel) or as a few warps beside the copy warps of an insert kernel.
+// Sum-tree maintenance: the priority transform (shared with the tree kernel, prb_tree.cu), a batch of changes of
+// priorities, and the re-sum of a contiguous range of inserted leaves.  The last two are written for a "team": a
+// whole number of warps of one CTA that synchronise on their own barrier, so that the same code runs as a full
+// CTA (the kernel of changes) or as a few warps beside the copy warps of the long-row insertion.
 #pragma once
 #include "prb_internal.cuh"
 #include "../../include/pearl_prb.h"
@@ -14,7 +13,7 @@ struct PrbTeam {
     bool whole_cta;          // the team is the whole CTA: plain __syncthreads; otherwise named barrier 1
     // Several CTAs of one thread-block cluster may share the tree work: each holds the full sorted
     // key list and CTA `part` of `parts` takes its share -- by subtree where the tree has staged levels
-    // (see prb_update_team), else the slots whose warp-sized group number is congruent to it, the
+    // (see prb_delta_team), else the slots whose warp-sized group number is congruent to it, the
     // phases then separated by the cluster's hardware barrier.  parts == 1: one CTA.
     uint32_t part = 0, parts = 1;
     // PrbView::min_off in the kernels instantiated for a buffer with a min-tree, the constant 0 in the others
