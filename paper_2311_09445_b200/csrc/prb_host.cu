@@ -170,6 +170,7 @@ struct pearl_prb {
     bool main_touched = true;                    // since fork.side last waited for the caller's stream, that stream
                                                  // has been given work that reads or writes the tree or the state
     uint32_t handoff_next = 0;
+    bool linked_inputs = false;                  // the running call's inputs lie in mapped host memory (pearl_prb_step_host)
     bool after_rows = false;                     // the last call was an update + insertion of long rows: a tree kernel beside a row copy
     unsigned long long main_last_gather = 0;     // the capture in which the last kernel given to the caller's stream was such a row copy (0: it was not)
     ~pearl_prb()
@@ -546,7 +547,7 @@ static int update_common(pearl_prb_t* h, uint32_t B, const int32_t* d_idx, const
     DeviceGuard guard(h->device);
     if (!guard.ok) return PEARL_ERR_CUDA;
     if (stale > h->view.capacity) return PEARL_ERR_BAD_ARG;
-    const int k = prb_launch_update(h->view, B, d_idx, d_val, raw, alpha, eps, h->stream, stale);
+    const int k = prb_launch_update(h->view, B, d_idx, d_val, raw, alpha, eps, h->stream, stale, h->linked_inputs);
     if (k < 0) return PEARL_ERR_CUDA;
     h->launches += (uint64_t)k;
     h->main_touched = true; h->main_last_gather = 0; h->after_rows = false;
@@ -615,7 +616,8 @@ int pearl_prb_update_insert(pearl_prb_t* h, uint32_t B, const int32_t* d_idx, co
     PrbBatch b;
     for (int f = 0; f < PRB_NUM_FIELDS; ++f) b.ptr[f] = (unsigned char*)ptrs[f];
     bool beside = false;
-    const int k = prb_launch_insert(h->view, n, b, d_prio, h->stream, B, d_idx, d_td, 0, alpha, eps, &h->fork, &beside);
+    const int k = prb_launch_insert(h->view, n, b, d_prio, h->stream, B, d_idx, d_td, 0, alpha, eps, &h->fork, &beside, false,
+                                    h->linked_inputs);
     if (k < 0) return PEARL_ERR_CUDA;
     h->launches += (uint64_t)k;
     h->main_touched = true; h->main_last_gather = 0; h->after_rows = beside;
@@ -940,11 +942,13 @@ int pearl_prb_step_host(pearl_prb_t* h, uint32_t B_upd, const int32_t* h_upd_idx
         if (cudaMemcpyAsync(arena + from, h->pin + from, in.total - from, cudaMemcpyHostToDevice, h->stream) != cudaSuccess) return PEARL_ERR_CUDA;
         for (int i = PRB_NUM_FIELDS + 1; i < PRB_NUM_FIELDS + 3; ++i) din[i] = arena + in.off[i];
     }
+    h->linked_inputs = true;
     int rc = pearl_prb_step(h, B_upd, (const int32_t*)din[PRB_NUM_FIELDS + 1], (const float*)din[PRB_NUM_FIELDS + 2], alpha, eps, n,
                             din[F_OBS], din[F_ACT], (const float*)din[F_REW], din[F_NEXT_OBS], (const uint8_t*)din[F_DONE],
                             (const float*)din[PRB_NUM_FIELDS], B, beta, seed, (int32_t*)dout[PRB_NUM_FIELDS],
                             (float*)dout[PRB_NUM_FIELDS + 1], dout[F_OBS], dout[F_ACT], (float*)dout[F_REW], dout[F_NEXT_OBS],
                             (uint8_t*)dout[F_DONE]);
+    h->linked_inputs = false;
     if (rc != PEARL_OK) return rc;
     if (cudaStreamSynchronize(h->stream) != cudaSuccess) return PEARL_ERR_CUDA;
     for (int i = 0; i < PRB_NUM_FIELDS + 2; ++i)

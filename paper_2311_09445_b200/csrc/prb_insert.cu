@@ -164,7 +164,7 @@ prb_insert_rows_kernel(const __grid_constant__ PrbView v, uint32_t n, const __gr
 
 int prb_launch_insert(const PrbView& v, uint32_t n, const PrbBatch& src, const float* d_prio, cudaStream_t s,
                       uint32_t upd_B, const int32_t* upd_idx, const float* upd_val, int upd_raw, float alpha, float eps,
-                      const PrbFork* fork, bool* beside_out, bool rows_only)
+                      const PrbFork* fork, bool* beside_out, bool rows_only, bool linked)
 {
     if (beside_out) *beside_out = false;
     if (rows_only && upd_B) return -1;
@@ -197,6 +197,7 @@ int prb_launch_insert(const PrbView& v, uint32_t n, const PrbBatch& src, const f
         // short rows: one launch does the update, the insertion's tree work and the row copy
         if (rows_only) return -1;
         tree.rows = &src;
+        if (linked) tree.most_ctas = 4u;      // (every CTA reads the batch over the link: 256 + 256 entries 39.2 us a step with 4, 44.9 with 16)
         return prb_launch_tree(v, tree, s, true);
     }
     plan.first_tile[PRB_NUM_FIELDS] = tiles;

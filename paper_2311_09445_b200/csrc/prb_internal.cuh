@@ -107,7 +107,8 @@ struct PrbFork {
 int prb_launch_insert(const PrbView& v, uint32_t n, const PrbBatch& src, const float* d_prio, cudaStream_t s,
                       uint32_t upd_B = 0, const int32_t* upd_idx = nullptr, const float* upd_val = nullptr,
                       int upd_raw = 0, float alpha = 0.0f, float eps = 0.0f, const PrbFork* fork = nullptr,
-                      bool* beside_out = nullptr, bool rows_only = false);
+                      bool* beside_out = nullptr, bool rows_only = false, bool linked = false);
+// (linked: the inputs lie in mapped host memory -- short rows: few CTAs read them)
 // (rows_only: long rows, and the insertion's tree work is some other launch's: this one copies the rows and advances the row cursor, nothing else)
 // Streams and events of a sample call that is issued as sub-batches (the paper's sub-batch
 // streaming, Section IV-C): sub-batch i runs on stream[i]; done[i] fires when its rows are in place.
@@ -166,7 +167,7 @@ bool prb_sample_has_long_rows(const PrbView& v, const PrbBatch& dst);
 // (stale > 0: skip entries that name one of the `stale` most recently written ring slots)
 // (values or TD errors: prb_launch_tree; changes, raw == 2, keep their batch order and go sub-batch by sub-batch)
 int prb_launch_update(const PrbView& v, uint32_t B, const int32_t* d_idx, const float* d_val, int raw,
-                      float alpha, float eps, cudaStream_t s, uint32_t stale = 0);
+                      float alpha, float eps, cudaStream_t s, uint32_t stale = 0, bool linked = false);
 // Tree work (prb_tree.cu): a priority update of B entries (values or TD errors; B may be 0), then the tree part of an
 // insertion of n transitions (may be 0), and with `rows` the insertion's short rows, in one launch.
 struct PrbTreeArgs {

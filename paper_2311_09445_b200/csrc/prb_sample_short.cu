@@ -29,7 +29,9 @@ constexpr uint32_t kShortThreads = 512;
 constexpr uint32_t kShortTopFloats = 5120;           // tree entries staged in shared memory
 constexpr uint32_t kMaxSteps = 16;
 constexpr uint32_t kMaxCluster = 16;
-constexpr uint32_t kClusterStrata = 1536;            // batches of at most this many strata run as one cluster
+// Batches of at most this many strata run as one cluster: three warps of strata per CTA.  (The grid form costs a
+// cooperative launch, no programmatic one, and a round through global memory for the smallest priority.)
+constexpr uint32_t kClusterStrata = 1536;
 constexpr uint32_t kMaxSeen = 64;                    // strata warps of a cluster: 8 CTAs x 6 warps, 16 x 3
 constexpr uint32_t kGridStrata = 32;                 // strata per CTA of the cooperative grid, at least
 constexpr uint32_t kShortSpinLimit = 1u << 22;
@@ -325,6 +327,9 @@ __device__ __forceinline__ void stage(const StagedUnit (&u)[kStagedUnits])
 // written, and all that depends on the arguments alone is done -- where every thread's words and staged units
 // lie, and a dry run of the arithmetic, which fetches its constants (the first use of a binary64 constant was
 // measured at 430 cycles, each further line of them at 84).
+// From that wait to the last store, fanout 16, 2^20 slots, 64 strata: 7000 cycles; the kernel before it (a lane group
+// per stratum over 32 CTAs, raw weights through global memory and a ticket, rows field by field) took 16000, 5400 of
+// them the last CTA's division.  CTAs: 2, 4, 8 or 16 strata each measured the same within 1 %; 4.
 struct __align__(16) SmallestSeen { double log_p; unsigned long long p_bits; };
 
 template <int K>

@@ -640,16 +640,19 @@ constexpr uint32_t kTreeSmem = 2u * kPrbTopFloats * 4u + 2u * 2u * kGridList * 4
 
 }  // namespace
 
-// Which form: one CTA up to a few thousand children per level to read, a cluster (by subtree) beyond -- many wide
-// child groups are more L2 misses than one SM keeps in flight -- and the grid beyond one entry per thread, or for an
-// insertion that one CTA would take many turns to write.
+// Which form.  One CTA while the entries' groups of a pass come to at most 2 K entries (8 KB); a cluster of 16 CTAs
+// beyond -- one SM pulls and stores scattered groups so slowly that they outlast the round trip.  us per 8 steps with
+// 1 / 4 / 8 / 16 CTAs: fanout 16, 256 + 256 entries 93.3 / 83.5 / 84.0 / 80.9; fanout 2, 1000 + 777 entries 271 / 149 /
+// 128 / 119; fanout 32, 512 + 512 (frames) 219 / 188 / 183 / 184; us per step at fanout 16, 64 + 64 entries 12.2 /
+// 12.7 / 13.1 / 12.5, at fanout 2, 32 entries 10.9 / 11.3 / 11.7 / 11.1.  A grid beyond one entry per thread, or for an
+// insertion that one CTA would take many turns to write (before it one cooperative launch with a barrier per pass and
+// a launch for the insertion: 4096 + 16384 entries 56.6 -> 31.2 us a step, 4096 + 1024 41.0 -> 24.9).
 static bool tree_grid_form(uint32_t b, uint32_t n) { return b > kPrbTreeEntries || n > 4u * kPrbTreeEntries; }
 uint32_t prb_tree_ctas(const PrbView& v, uint32_t b, uint32_t n, uint32_t most)
 {
-    // (bytes that the entries' groups of a pass span: 4 KB and more keep one SM busy for longer than a round trip)
     const uint32_t group = v.fanout == 2u ? 32u : v.fanout == 4u ? 16u : v.fanout;
     const uint64_t work = (uint64_t)group * b + 4ull * n;
-    const uint32_t want = tree_grid_form(b, n) ? 128u : work <= 2048u ? 1u : work <= 8192u ? 4u : work <= 16384u ? 8u : 16u;
+    const uint32_t want = tree_grid_form(b, n) ? 128u : work <= 2048u ? 1u : 16u;
     return most && want > most ? most : want;
 }
 

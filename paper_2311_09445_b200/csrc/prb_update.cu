@@ -59,11 +59,12 @@ uint32_t prb_update_ctas(const PrbView& v, uint32_t b)
 }
 
 int prb_launch_update(const PrbView& v, uint32_t B, const int32_t* d_idx, const float* d_val, int raw,
-                      float alpha, float eps, cudaStream_t s, uint32_t stale)
+                      float alpha, float eps, cudaStream_t s, uint32_t stale, bool linked)
 {
     if (raw != 2) {
         PrbTreeArgs t;
         t.B = B; t.idx = d_idx; t.val = d_val; t.raw = raw; t.alpha = alpha; t.eps = eps; t.stale = stale;
+        if (linked) t.most_ctas = 4u;      // (see prb_launch_insert)
         return prb_launch_tree(v, t, s, true);
     }
     static bool big_smem[kPrbMaxDevices];
