@@ -197,7 +197,8 @@ int prb_launch_insert(const PrbView& v, uint32_t n, const PrbBatch& src, const f
         // short rows: one launch does the update, the insertion's tree work and the row copy
         if (rows_only) return -1;
         tree.rows = &src;
-        if (linked) tree.most_ctas = 4u;      // (every CTA reads the batch over the link: 256 + 256 entries 39.2 us a step with 4, 44.9 with 16)
+        tree.linked = linked;
+        if (linked) tree.most_ctas = 4u;      // (every CTA reads the indices over the link)
         return prb_launch_tree(v, tree, s, true);
     }
     plan.first_tile[PRB_NUM_FIELDS] = tiles;

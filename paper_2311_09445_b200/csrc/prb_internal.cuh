@@ -181,6 +181,7 @@ struct PrbTreeArgs {
     const float* prio = nullptr;          // nullptr: the running maximum
     const unsigned char* done = nullptr;
     const PrbBatch* rows = nullptr;
+    bool linked = false;                  // the inputs lie in mapped host memory
     uint32_t most_ctas = 0;               // a limit on the CTAs that do the tree work (0: none)
 };
 constexpr uint32_t kPrbTreeEntries = 1024;      // update entries one CTA (or cluster) takes, one per thread; more go to a grid

@@ -118,4 +118,50 @@ __device__ __forceinline__ void prb_copy_words(const PrbWords& p, const PrbWordS
     }
 }
 
+// The same copy to the store, all n rows of a batch that lies in mapped host memory: 32 consecutive words of one field
+// at a time, whatever rows they belong to, so that the link carries whole sectors (row by row, a sector of rewards
+// or done bytes crossed it once per row).  256 rows of 165 bytes: 43.3 -> 41.2 us a step through host buffers.  `warp` of `warps` over all copying CTAs; four loads of a thread in flight.
+template <typename SlotOf>
+__device__ __forceinline__ void prb_copy_flat(const PrbWords& p, uint32_t warp, uint32_t warps, uint32_t n, SlotOf slot_of)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    uint32_t total = 0;
+#pragma unroll
+    for (int f = 0; f < PRB_NUM_FIELDS; ++f) if (p.field[f].batch) total += (n * (p.field[f].batch_pitch >> p.field[f].log2) + 31u) / 32u;
+    constexpr int U = 4;
+    for (uint32_t c0 = warp; c0 < total; c0 += warps * U) {
+        uint32_t v[U], lg[U], at[U], pitch[U], row[U];
+        unsigned char* store[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            uint32_t c = c0 + u * warps;
+            store[u] = nullptr;
+            v[u] = 0u;
+            if (c >= total) continue;
+#pragma unroll 1
+            for (int f = 0; f < PRB_NUM_FIELDS; ++f) {
+                const PrbWordField& fd = p.field[f];
+                if (!fd.batch) continue;
+                const uint32_t W = fd.batch_pitch >> fd.log2, words = n * W, here = (words + 31u) / 32u;
+                if (c >= here) { c -= here; continue; }
+                const uint32_t e = c * 32u + lane;
+                if (e < words) {
+                    row[u] = e / W; at[u] = (e - row[u] * W) << fd.log2; lg[u] = fd.log2; pitch[u] = fd.store_pitch; store[u] = fd.store;
+                    const unsigned char* from = fd.batch + ((uint64_t)e << fd.log2);
+                    v[u] = fd.log2 == 2u ? *reinterpret_cast<const uint32_t*>(from) : fd.log2 == 1u ? *reinterpret_cast<const uint16_t*>(from) : *from;
+                }
+                break;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (store[u] == nullptr) continue;
+            unsigned char* to = store[u] + (uint64_t)slot_of(row[u]) * pitch[u] + at[u];
+            if (lg[u] == 2u) *reinterpret_cast<uint32_t*>(to) = v[u];
+            else if (lg[u] == 1u) *reinterpret_cast<uint16_t*>(to) = (uint16_t)v[u];
+            else *to = (unsigned char)v[u];
+        }
+    }
+}
+
 #endif  // __CUDACC__

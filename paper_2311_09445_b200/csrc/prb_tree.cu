@@ -55,6 +55,7 @@ struct TreePlan {
     uint32_t list, hash_mask;                // capacity of the entry list, size of the hash table less one
     uint32_t copies;                         // CTAs that copy rows
     uint32_t dependent;                      // launched as a programmatic dependent
+    uint32_t linked;                         // the inputs lie in mapped host memory
     uint32_t off[PRB_MAX_LEVELS];            // level l starts off[l] * 64 entries behind level 0
     PrbWords words;
 };
@@ -301,6 +302,11 @@ prb_tree_kernel(const __grid_constant__ TreePlan plan)
         if (tid == nt - 1u && prb_ticket(&plan.state->row_ticket) == plan.copies - 1u) {
             plan.state->row_cursor = cursor + plan.n >= N ? cursor + plan.n - N : cursor + plan.n;
             plan.state->row_ticket = 0u;
+        }
+        if (plan.linked) {
+            prb_copy_flat(plan.words, c * (nt >> 5) + (tid >> 5), plan.copies * (nt >> 5), plan.n,
+                          [&](uint32_t r) { const uint32_t s = cursor + r; return s >= N ? s - N : s; });
+            return;
         }
         prb_copy_words<true>(plan.words, share, nt >> 5, r_lo, r_hi - r_lo,
                              [&](uint32_t r) { const uint32_t s = cursor + r_lo + r; return s >= N ? s - N : s; });
@@ -732,6 +738,7 @@ int prb_launch_tree(const PrbView& v, const PrbTreeArgs& t, cudaStream_t s, bool
     }
     p.copies = 0;
     p.dependent = dependent ? 1u : 0u;
+    p.linked = t.linked ? 1u : 0u;
     PrbBatch none;
     for (int f = 0; f < PRB_NUM_FIELDS; ++f) none.ptr[f] = nullptr;
     p.words = prb_plan_words(v, t.rows ? *t.rows : none);
