@@ -165,8 +165,9 @@ __device__ __forceinline__ uint32_t step1(const float* row, double& x, float& ch
     } else {
         // prefix <= x, a binary32 against a binary64, is prefix <= (the largest binary32 not above x).
         // All prefixes first (one chain of additions), then the comparisons as masks, not predicates: counted
-        // for the child's number, and the largest prefix passed picked out of them (bits of non-negative
-        // values order like the values).
+        // for the child's number, and the largest prefix passed picked out of them: as signed integers, whose
+        // order is that of the values and which put -0.0 (a priority that is accepted; only the prefixes before the
+        // first positive child can be it) below every prefix not passed, so that +0.0 is subtracted then.
         const float xf = __double2float_rd(x);
         float r[K];
 #pragma unroll
@@ -176,18 +177,20 @@ __device__ __forceinline__ uint32_t step1(const float* row, double& x, float& ch
         }
 #pragma unroll
         for (int i = 1; i < K; ++i) r[i] = __fadd_rn(r[i - 1], r[i]);
-        uint32_t cnt[K], top[K];
+        uint32_t cnt[K];
+        int top[K];
 #pragma unroll
         for (int i = 0; i < K; ++i) {
             asm("set.le.u32.f32 %0, %1, %2;" : "=r"(cnt[i]) : "f"(r[i]), "f"(xf));      // (all ones where passed)
-            top[i] = cnt[i] & __float_as_uint(r[i]);
+            top[i] = (int)cnt[i] & __float_as_int(r[i]);
         }
 #pragma unroll
         for (int h = K / 2; h > 0; h /= 2) {
 #pragma unroll
             for (int i = 0; i < h; ++i) { cnt[i] += cnt[i + h]; top[i] = max(top[i], top[i + h]); }
         }
-        uint32_t j = 0u - cnt[0], before = top[0];
+        uint32_t j = 0u - cnt[0];
+        int before = top[0];
         if (j == (uint32_t)K) {
             flags |= PEARL_ST_CLAMPED;
             while (j > 0u && !(row[j - 1u] > 0.0f)) --j;
@@ -196,9 +199,9 @@ __device__ __forceinline__ uint32_t step1(const float* row, double& x, float& ch
             float run = 0.0f;
 #pragma unroll 1
             for (uint32_t i = 0; i < j; ++i) run = i ? __fadd_rn(run, row[i]) : row[0];
-            before = __float_as_uint(run);
+            before = __float_as_int(run);
         }
-        x = __dsub_rn(x, (double)__uint_as_float(before));              // (0 in front of the first child)
+        x = __dsub_rn(x, (double)__int_as_float(before));              // (0 in front of the first child)
         return j;
     }
 }

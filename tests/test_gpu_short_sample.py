@@ -58,3 +58,34 @@ def test_weights_against_binary64(oracle_mod, B):
             assert np.all(np.abs(got - want)[normal] <= want[normal] * (2.0 ** -24 + 1e-9))
             assert np.all(np.abs(got - want)[~normal] <= 2.0 ** -149)
     pr.close()
+
+
+@pytest.mark.parametrize("K", [2, 4, 8, 16, 32])
+def test_negative_zero_priorities(oracle_mod, K):
+    # -0.0 is a valid priority (p >= 0), stored as it is; a node whose leaves are all -0.0 sums to -0.0.  As the first
+    # child of its group it is passed by every target, and what is subtracted is still the prefix before the child
+    # entered, not the -0.0.  First by insertion, then by an update; the cluster's and the grid's form.
+    rng = np.random.default_rng(K)
+    N = K ** 3 if K > 4 else 512
+    pr = Pair(oracle_mod, N, K, 4, 4, 4096)
+    rows = lambda n: dict(obs=rng.integers(0, 256, size=(n, 4), dtype=np.uint8), act=rng.integers(0, 256, size=(n, 4), dtype=np.uint8),
+                          rew=rng.standard_normal(n).astype(np.float32), next_obs=rng.integers(0, 256, size=(n, 4), dtype=np.uint8),
+                          done=rng.integers(0, 2, size=n, dtype=np.uint8))
+    prio = np.exp(rng.standard_normal(N)).astype(np.float32)
+    for a in range(0, N, K * K):
+        prio[a:a + K] = -0.0                                   # the first leaf group under a node two levels up
+    prio[5 * K * K:5 * K * K + K * K] = -0.0                   # a whole node's leaves
+    prio[rng.random(N) < 0.1] = -0.0
+    for at in range(0, N, 4096):
+        b = rows(min(4096, N - at))
+        pr.insert(dict(b, prio=prio[at:at + 4096]))
+    for B in (64, 1500, 1537, 4000):
+        pr.sample(B, 0.7, 11 + B)
+    idx = np.arange(3 * K * K, min(N, 3 * K * K + 1000), dtype=np.int32)
+    pr.update_priorities(idx, np.where(rng.random(idx.size) < 0.7, -0.0, 2.5).astype(np.float32))
+    pr.compare_tree()
+    for B in (64, 1500, 1537, 4000):
+        pr.sample(B, 0.7, 17 + B)
+    pr.compare_state()
+    assert pr.compare_status() in (0, 8)
+    pr.close()
