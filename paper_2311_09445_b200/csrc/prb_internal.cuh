@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 #include "../../include/pearl_prb.h"
+#include "prb_arith.cuh"
 
 // The checked build (-DPEARL_CHECKED; build.py --checked): every index into a tree level, the Data Storage,
 // a batch or a staging area is compared with its extent before it is used; an index out of range raises

@@ -226,7 +226,7 @@ __device__ __forceinline__ void top_passes(const TreeCtx& c)
     for (uint32_t l = T; l > 0;) {
         // (where fewer than H levels are left a whole block is taken all the same, from levels re-summed already)
         const uint32_t h = T >= H ? H : 1u, child = max(l, h), lt = child - h;
-        const uint32_t blocks = ((c.plan.capacity - 1u) >> (kLog2<K> * (D - lt))) + 1u;
+        const uint32_t blocks = prb_nodes_covering(c.plan.capacity, kLog2<K> * (D - lt));
         for (uint32_t i = c.tid; i < blocks; i += c.nt) {
             if (h == H) top_block<K, (int)H>(c.top, c, child, i, 0);
             else top_block<K, 1>(c.top, c, child, i, 0);

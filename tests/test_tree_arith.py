@@ -1,0 +1,30 @@
+"""The tree work's index arithmetic, compiled for the host with the sanitizer for undefined behaviour."""
+import os
+import subprocess
+
+import pytest
+
+from conftest import ROOT
+
+
+@pytest.fixture(scope="module")
+def probe(tmp_path_factory):
+    exe = str(tmp_path_factory.mktemp("arith") / "tree_arith_probe")
+    subprocess.check_call(["g++", "-O1", "-std=c++17", "-fsanitize=undefined", "-fno-sanitize-recover=all",
+                           "-I", os.path.join(ROOT, "paper_2311_09445_b200", "csrc"), "-o", exe,
+                           os.path.join(ROOT, "tests", "tree_arith_probe.cpp")])
+    return lambda lines: subprocess.run([exe], input="".join(ln + "\n" for ln in lines), capture_output=True, text=True, check=True).stdout.split()
+
+
+def test_nodes_of_every_level(probe):
+    # capacities up to the largest a handle takes (2^30), about every power of the fanout; every level
+    ask = []
+    for lg in (1, 2, 3, 4, 5):
+        for cap in sorted({min(max(1, (1 << e) + d), 1 << 30) for e in range(0, 31) for d in (-1, 0, 1)}):
+            depth = 1
+            while (1 << (lg * depth)) < cap:
+                depth += 1
+            ask += [(cap, lg * up) for up in range(depth + 1)]
+    got = probe("nodes %d %d" % q for q in ask)
+    assert [int(g) for g in got] == [-((-cap) >> sh) for cap, sh in ask]
+    assert max(sh for _, sh in ask) >= 32
