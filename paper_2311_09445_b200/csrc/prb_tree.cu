@@ -287,6 +287,7 @@ prb_tree_kernel(const __grid_constant__ TreePlan plan)
     __shared__ uint32_t s_off[PRB_MAX_LEVELS];
     __shared__ __align__(8) unsigned long long s_bar;        // (cluster, CTA 0) level T is complete in the staged copy
     __shared__ unsigned s_max, s_count, s_sent, s_last, s_before;
+    __shared__ uint32_t s_row;                               // (copying CTAs) row_cursor
     const uint32_t tid = threadIdx.x, nt = blockDim.x;
     constexpr uint32_t lg = kLog2<K>;
 
@@ -296,9 +297,14 @@ prb_tree_kernel(const __grid_constant__ TreePlan plan)
         const PrbWordShare share = prb_word_share(plan.words, tid >> 5, nt >> 5);
         prb_dep_wait();
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-        const uint32_t cursor = (uint32_t)__ldcg(&plan.state->row_cursor), N = plan.capacity;
+        const uint32_t N = plan.capacity;
+        // (one thread reads the cursor for the CTA: it is in shared memory, so the load has answered, before the CTA
+        // draws its ticket -- a barrier alone would not say so of loads that other threads still have on their way --
+        // and only then may the last CTA move it)
+        if (tid == 0) s_row = (uint32_t)__ldcg(&plan.state->row_cursor);
         const uint32_t r_lo = (uint32_t)(((uint64_t)c * plan.n) / plan.copies), r_hi = (uint32_t)(((uint64_t)(c + 1) * plan.n) / plan.copies);
-        __syncthreads();                             // (the whole CTA holds the cursor)
+        __syncthreads();
+        const uint32_t cursor = s_row;
         if (tid == nt - 1u && prb_ticket(&plan.state->row_ticket) == plan.copies - 1u) {
             plan.state->row_cursor = cursor + plan.n >= N ? cursor + plan.n - N : cursor + plan.n;
             plan.state->row_ticket = 0u;

@@ -3,6 +3,7 @@ levels per pass (fanouts 2 and 4), trees too shallow for that, levels that end i
 subtree; insertions that wrap; and what an update and an insertion both write."""
 import numpy as np
 import pytest
+import torch
 
 from prb_harness import Pair
 
@@ -62,4 +63,20 @@ def test_batch_in_one_subtree(oracle_mod, K, N):
             pr.update_priorities(idx, np.exp(rng.standard_normal(B)).astype(np.float32))
             pr.compare_tree()
     pr.compare_status()
+    pr.close()
+
+
+@pytest.mark.parametrize("K,n", [(16, 1), (16, 300), (2, 777), (32, 1500)])
+def test_rows_of_many_insertions_in_a_row(oracle_mod, K, n):
+    # every insertion's copying CTAs read the row cursor that the last of the insertion before moved; rows of several
+    # CTAs' worth, a ring that wraps every few calls, nothing waited for in between
+    rng = np.random.default_rng(n)
+    N = 2 * n + 3
+    pr = Pair(oracle_mod, N, K, 40, 4, 1500)
+    batches = [_batch(rng, n, 40, 4) for _ in range(3)]
+    dev = [{k: torch.from_numpy(v).to(pr.dev) for k, v in b.items()} for b in batches]
+    for i in range(100):
+        pr.insert(batches[i % 3], dev_batch=dev[i % 3])
+    _check(pr, False)
+    pr.compare_rows(np.arange(N, dtype=np.int32))
     pr.close()
