@@ -360,6 +360,17 @@ __device__ __forceinline__ unsigned int prb_ticket(unsigned int* counter)
 #endif
 }
 
+// Arrival at the cluster's barrier (the wait that follows acquires): a release in the checked build, relaxed in the
+// ordinary one, for arrivals in front of which nothing is outstanding that the others read or overwrite.
+__device__ __forceinline__ void prb_cluster_arrive()
+{
+#ifdef PEARL_CHECKED
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+#else
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+#endif
+}
+
 // A kernel launched as a programmatic dependent waits here until the kernel before it on its stream has
 // completed and its writes are visible; a no-op for a kernel launched the ordinary way.
 __device__ __forceinline__ void prb_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
