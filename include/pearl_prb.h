@@ -60,9 +60,9 @@ typedef struct pearl_layout {
                                       instead of hanging.  After a copy that gave up, rows of that call are
                                       missing or partial; after an update or insertion, nodes of the tree's
                                       top may not equal the sum of their children; after a sample of short
-                                      rows, weights are missing, and every later sample of more than 1536
-                                      strata of short rows on that buffer raises the bit again and does
-                                      nothing.  Treat the buffer as lost: destroy it and build a new one.  No
+                                      rows, weights are missing.  After either of the last two every later
+                                      sample of more than 1536 strata of short rows on that buffer raises the
+                                      bit again and does nothing.  Treat the buffer as lost: destroy it and build a new one.  No
                                       correct run raises this bit. */
 #define PEARL_ST_STALE 32u         /* update_after_insert: the index was overwritten since it was sampled; entry skipped */
 

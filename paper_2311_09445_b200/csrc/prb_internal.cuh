@@ -5,6 +5,7 @@
 
 #include "../../include/pearl_prb.h"
 #include "prb_arith.cuh"
+#include "prb_wait.cuh"
 
 // The checked build (-DPEARL_CHECKED; build.py --checked): every index into a tree level, the Data Storage,
 // a batch or a staging area is compared with its extent before it is used; an index out of range raises
@@ -42,8 +43,8 @@ struct PrbState {
     // races with, the other's; a one-kernel insertion advances both.  Equal whenever no insertion is running.
     unsigned long long row_cursor;
     unsigned int row_ticket;          // CTAs of the running row kernel that have read row_cursor
-    unsigned int wide_poisoned;       // a sample of many co-resident CTAs gave up waiting once: its ticket is not to be trusted, and every
-                                      // later one raises INTERNAL and does nothing
+    unsigned int wide_poisoned;       // CTAs that wait for one another (a cluster, or a co-resident grid) gave up once: tickets are not to be
+                                      // trusted, and every later sample of many co-resident CTAs raises INTERNAL and does nothing
 };
 
 // Geometry and device addresses, passed to kernels by value.
@@ -390,6 +391,27 @@ __device__ __forceinline__ void prb_dep_wait() { asm volatile("griddepcontrol.wa
 constexpr uint32_t kBulkSpinLimit = 1u << 20;   // mbarrier polls before a wait gives up
 
 __device__ __forceinline__ uint32_t prb_smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// The wait for the first phase of a barrier that peers' transfers complete, by one thread, a warp or a CTA.  One that ran out
+// is raised and marks the buffer (see PrbState::wide_poisoned) -- out of line: in line it cost the sample of 64 strata
+// 0.1 us of 4.3.
+__device__ __forceinline__ bool prb_first_phase_over(uint32_t bar)
+{
+    uint32_t ok;
+    asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0; selp.u32 %0, 1, 0, p; }"
+                 : "=r"(ok) : "r"(bar) : "memory");
+    return ok != 0u;
+}
+static __noinline__ __device__ PrbWaited prb_first_phase_ran_out(PrbState* st, uint32_t bar)
+{
+    atomicOr(&st->status, PEARL_ST_INTERNAL);
+    atomicExch(&st->wide_poisoned, 1u);
+    return prb_poll([bar]() { return prb_first_phase_over(bar); }, kBulkSpinLimit) ? kPrbLate : kPrbNever;
+}
+__device__ __forceinline__ PrbWaited prb_wait_first_phase(PrbState* st, uint32_t bar)
+{
+    return prb_wait_bounded([bar]() { return prb_first_phase_over(bar); }, kBulkSpinLimit, [st, bar]() { return prb_first_phase_ran_out(st, bar); });
+}
 
 struct PrbBulkLane {
     uint32_t bar;        // shared address of this lane's mbarrier

@@ -425,13 +425,7 @@ prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
     if (!split) gather(plan, share, warps, k_lo, n, s_idx);
     // (the first warp always gets here: it keeps the CTA's shared memory until every value has come)
     if (warp >= strata_warps) return;
-    bool there = false;
-    for (uint32_t spins = 0; spins < kBulkSpinLimit && !there; ++spins) {
-        uint32_t ok;
-        asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0; selp.u32 %0, 1, 0, p; }" : "=r"(ok) : "r"(bar) : "memory");
-        there = ok != 0u;
-    }
-    if (!there) { atomicOr(&plan.state->status, PEARL_ST_INTERNAL); return; }
+    if (prb_wait_first_phase(plan.state, bar) == kPrbNever) return;
     if (blockIdx.x == 0 && tid == 0) {
         plan.state->sample_calls = calls + 1;                  // (every CTA has drawn)
         if (plan.buffer_norm) plan.state->pmin_bits = ~0ull;   // (ready for the next scan)

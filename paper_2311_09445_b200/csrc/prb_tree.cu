@@ -615,14 +615,7 @@ prb_tree_kernel(const __grid_constant__ TreePlan plan)
         if (tid == 0)
             asm volatile("mbarrier.arrive.expect_tx.relaxed.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(c.bar), "r"(s_sent * (kMin ? 8u : 4u)) : "memory");
         if (blockIdx.x != 0) return;
-        bool there = false;
-        for (uint32_t spins = 0; spins < kBulkSpinLimit && !there; ++spins) {
-            uint32_t ok;
-            asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0; selp.u32 %0, 1, 0, p; }"
-                         : "=r"(ok) : "r"(prb_smem_addr(&s_bar)) : "memory");
-            there = ok != 0u;
-        }
-        if (!there) atomicOr(&plan.state->status, PEARL_ST_INTERNAL);
+        prb_wait_first_phase(plan.state, prb_smem_addr(&s_bar));
         __syncthreads();
     }
     // every CTA of the tree work has read cursor and fill: they move on

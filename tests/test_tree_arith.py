@@ -1,4 +1,4 @@
-"""The tree work's index arithmetic, compiled for the host with the sanitizer for undefined behaviour."""
+"""The tree work's index arithmetic and the bounded wait, compiled for the host with the sanitizer for undefined behaviour."""
 import os
 import subprocess
 
@@ -28,3 +28,9 @@ def test_nodes_of_every_level(probe):
     got = probe("nodes %d %d" % q for q in ask)
     assert [int(g) for g in got] == [-((-cap) >> sh) for cap, sh in ask]
     assert max(sh for _, sh in ask) >= 32
+
+
+def test_a_wait_that_runs_out_is_reported_and_goes_on_for_what_is_in_flight(probe):
+    # limit 5: in time up to poll 5, late (reported, but waited for) up to poll 10, never beyond
+    got = probe("wait %d 5" % ready for ready in (1, 5, 6, 10, 11, 1000))
+    assert got == ["0:1", "0:5", "1:6", "1:10", "2:10", "2:10"]
