@@ -52,7 +52,7 @@ struct TreePlan {
     float alpha, eps;
     uint32_t parts, grid_form;               // CTAs of the tree work (the others copy rows)
     uint32_t many;                           // 1: passes of kPassLevels levels, 0: of one level
-    uint32_t list, hash_mask;                // capacity of the entry list, size of the hash table less one
+    uint32_t list, hash_mask, hash_shift;    // capacity of the entry list, size of the hash table less one, 32 - its log2
     uint32_t copies;                         // CTAs that copy rows
     uint32_t dependent;                      // launched as a programmatic dependent
     uint32_t linked;                         // the inputs lie in mapped host memory
@@ -269,9 +269,9 @@ __device__ __forceinline__ bool entry_ok(const TreePlan& plan, int32_t i, uint32
 }
 
 // The hash table: linear probing; returns where leaf i lies (the table has twice as many places as entries).
-__device__ __forceinline__ uint32_t hash_find(unsigned* key, uint32_t mask, uint32_t i)
+__device__ __forceinline__ uint32_t hash_find(unsigned* key, uint32_t mask, uint32_t shift, uint32_t i)
 {
-    uint32_t h = (i * 0x9E3779B1u) >> 8 & mask;
+    uint32_t h = prb_hash_place(i, shift);
     while (true) {
         const unsigned old = atomicCAS(key + h, kNone, i);
         if (old == kNone || old == i) return h;
@@ -387,7 +387,7 @@ prb_tree_kernel(const __grid_constant__ TreePlan plan)
         p = x;
         const bool ok = plan.raw ? prb_valid_priority(x) : prb_priority_pow(x, plan.eps, plan.alpha, p);
         if (!ok) { flags |= PEARL_ST_BAD_PRIORITY; return kNone; }
-        const uint32_t h = hash_find(key, plan.hash_mask, i);
+        const uint32_t h = hash_find(key, plan.hash_mask, plan.hash_shift, i);
         atomicMax(last + h, b + 1u);
         wmax = fmaxf(wmax, p);
         return h;
@@ -731,7 +731,8 @@ int prb_launch_tree(const PrbView& v, const PrbTreeArgs& t, cudaStream_t s, bool
     p.parts = parts;
     p.list = p.grid_form ? kGridList : t.B;
     uint32_t slots = 32;
-    while (slots < 2u * p.list) slots *= 2u;
+    p.hash_shift = 27;
+    while (slots < 2u * p.list) { slots *= 2u; --p.hash_shift; }
     p.hash_mask = t.B ? slots - 1u : 0u;
     if (t.B == 0) p.list = 0;
     uint32_t threads = t.B >= 16u * kPrbTreeEntries ? kTreeThreads : kGridThreads;

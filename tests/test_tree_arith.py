@@ -2,6 +2,7 @@
 import os
 import subprocess
 
+import numpy as np
 import pytest
 
 from conftest import ROOT
@@ -28,6 +29,28 @@ def test_nodes_of_every_level(probe):
     got = probe("nodes %d %d" % q for q in ask)
     assert [int(g) for g in got] == [-((-cap) >> sh) for cap, sh in ask]
     assert max(sh for _, sh in ask) >= 32
+
+
+def test_no_stride_of_indices_meets_in_one_line_of_probes(probe):
+    # full tables of the tree kernel (twice as many places as entries), linear probing: a random batch of 1024 needs some
+    # tens of probes at worst, so 64 is the line; one place for all would need 1024
+    rng = np.random.default_rng(0)
+    for bits in (11, 12):
+        n = 1 << (bits - 1)
+        batches = [(np.arange(n, dtype=np.int64) << k) & ((1 << 30) - 1) for k in range(0, 21)]
+        batches += [(np.arange(n) * step) % (1 << 30) for step in (3, 84, 1000, 4097, 999_983)] + [rng.integers(0, 1 << 30, n)]
+        for keys in batches:
+            keys = np.unique(keys)
+            at = [int(x) for x in probe("place %d %d" % (i, 32 - bits) for i in keys)]
+            assert max(at) < 1 << bits
+            taken, worst = set(), 0
+            for h in at:
+                probes = 1
+                while h in taken:
+                    h, probes = (h + 1) % (1 << bits), probes + 1
+                taken.add(h)
+                worst = max(worst, probes)
+            assert worst <= 64, (bits, keys[:3], worst)
 
 
 def test_a_wait_that_runs_out_is_reported_and_goes_on_for_what_is_in_flight(probe):
