@@ -349,7 +349,10 @@ prb_tree_kernel(const __grid_constant__ TreePlan plan)
                 asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             }
             asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(c.bar) : "r"(prb_smem_addr(&s_bar)), "r"(0u));
-            asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+            // (relaxed: the fence above releases the barrier's initialisation, and a release here would wait for the
+            // inputs' loads, slow beside a row copy: with the 512 threads below 230 -> 220 us per 8 steps of 512 rows of 56 KB)
+            __syncthreads();
+            asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
             asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
         } else {
             __syncthreads();
@@ -739,6 +742,10 @@ int prb_launch_tree(const PrbView& v, const PrbTreeArgs& t, cudaStream_t s, bool
     if (!p.grid_form) {
         threads = (t.B + 31u) / 32u * 32u + (t.n < 512u ? (t.n + 31u) / 32u * 32u : 512u);
         threads = threads < 256u ? 256u : threads > kTreeThreads ? kTreeThreads : threads;
+        // Beside a row copy no more than an entry each asks for: a copying CTA holds 20480 of an SM's 65536 registers, and
+        // 512 of these threads hold 32768, so that the cluster fits on SMs that copy too.  With 1024 it needed whole SMs, eight
+        // of them in one group (512 + 512 entries alone with their rows: 10.1 us, 9.85 this way).
+        if (t.most_ctas == kPrbTreeBesideRows && threads > 512u) threads = t.B <= 512u ? 512u : (t.B + 31u) / 32u * 32u;
     }
     p.copies = 0;
     p.dependent = dependent ? 1u : 0u;
