@@ -733,8 +733,10 @@ int prb_launch_tree(const PrbView& v, const PrbTreeArgs& t, cudaStream_t s, bool
     p.grid_form = tree_grid_form(t.B, t.n) ? 1u : 0u;
     p.parts = parts;
     p.list = p.grid_form ? kGridList : t.B;
-    uint32_t slots = 32;
-    p.hash_shift = 27;
+    // (at least 512 places, whatever the entries: probes are a chain of shared atomics; 32 entries in 64 places took 4.7 to
+    // 5.5 us a call, by the batch's luck)
+    uint32_t slots = 512;
+    p.hash_shift = 23;
     while (slots < 2u * p.list) { slots *= 2u; --p.hash_shift; }
     p.hash_mask = t.B ? slots - 1u : 0u;
     if (t.B == 0) p.list = 0;
