@@ -385,16 +385,20 @@ prb_tree_kernel(const __grid_constant__ TreePlan plan)
     unsigned flags = 0u;
     float wmax = 0.0f;
 
-    // An entry's priority and its place in the table (kNone: refused).
-    auto transform = [&](uint32_t i, uint32_t b, float x, float& p) {
+    // An entry's priority and, if the entry is this CTA's, its place in the table (kNone: refused).
+    auto transform = [&](uint32_t i, uint32_t b, float x, float& p, bool enter) {
         p = x;
         const bool ok = plan.raw ? prb_valid_priority(x) : prb_priority_pow(x, plan.eps, plan.alpha, p);
         if (!ok) { flags |= PEARL_ST_BAD_PRIORITY; return kNone; }
+        wmax = fmaxf(wmax, p);
+        if (!enter) return kNone;
         const uint32_t h = hash_find(key, plan.hash_mask, plan.hash_shift, i);
         atomicMax(last + h, b + 1u);
-        wmax = fmaxf(wmax, p);
         return h;
     };
+    // New transitions without priorities take the running maximum, this update's writes included: each of several CTAs
+    // then needs the whole batch's, and transforms all of it.
+    const bool whole_max = plan.n != 0u && plan.prio == nullptr && plan.parts > 1u;
     // The leaf, if the entry is the last to write it (every entry has its place in the table, a barrier ago).
     auto write_leaf = [&](uint32_t i, uint32_t b, uint32_t h, float p) {
         if (h != kNone && last[h] == b + 1u && !(plan.n && inserted(i)) && PRB_IN_BOUNDS(plan, i < N)) leaves[i] = p;
@@ -439,14 +443,14 @@ prb_tree_kernel(const __grid_constant__ TreePlan plan)
     uint32_t m = 0, my_i = kNone, my_b = 0, my_h = kNone;      // (one entry per thread) this thread's
     float my_p = 0.0f;
     if (!grid_form) {
-        bool take = false;
+        bool take = false, valid = false;
         if (tid < plan.B) {
             unsigned f = 0u;
-            const bool ok = entry_ok(plan, i0, fill, cursor, f);
+            valid = entry_ok(plan, i0, fill, cursor, f);
             if (blockIdx.x == 0) flags |= f;
-            take = ok && mine((uint32_t)i0);
+            take = valid && mine((uint32_t)i0);
         }
-        if (clustered) {
+        if (clustered && !whole_max) {
             // this CTA's entries to its first threads: the transform costs a warp the same for one entry as for 32
             const unsigned who = __ballot_sync(0xFFFFFFFFu, take);
             uint32_t base = 0;
@@ -454,18 +458,26 @@ prb_tree_kernel(const __grid_constant__ TreePlan plan)
             base = __shfl_sync(0xFFFFFFFFu, base, 0) + __popc(who & ((1u << (tid & 31u)) - 1u));
             if (take) { l_idx[base] = (uint32_t)i0; l_pos[base] = tid; l_val[base] = v0; }
             __syncthreads();
-            if (tid < s_count) { my_i = l_idx[tid]; my_b = l_pos[tid]; v0 = l_val[tid]; }
-        } else if (take) {
+            valid = take = tid < s_count;
+            if (take) { my_i = l_idx[tid]; my_b = l_pos[tid]; v0 = l_val[tid]; }
+        } else if (valid) {
             my_i = (uint32_t)i0;
             my_b = tid;
         }
-        if (my_i != kNone) my_h = transform(my_i, my_b, v0, my_p);
+        if (valid) my_h = transform(my_i, my_b, v0, my_p, take);
+        if (!take) my_i = kNone;
     } else if (plan.B) {
         // the whole batch, for the entries that are this CTA's
+        if (whole_max)
+            for (uint32_t b = tid; b < plan.B; b += nt) {
+                unsigned unused = 0u;
+                float p;
+                if (entry_ok(plan, plan.idx[b], fill, cursor, unused)) transform(0u, 0u, plan.val[b], p, false);
+            }
         auto work_off = [&]() {
             __syncthreads();
             const uint32_t k = s_count;
-            for (uint32_t e = tid; e < k; e += nt) { float p; l_place[e] = transform(l_idx[e], l_pos[e], plan.val[l_pos[e]], p); l_val[e] = p; }
+            for (uint32_t e = tid; e < k; e += nt) { float p; l_place[e] = transform(l_idx[e], l_pos[e], plan.val[l_pos[e]], p, true); l_val[e] = p; }
             __syncthreads();
             return k;
         };
@@ -538,8 +550,7 @@ prb_tree_kernel(const __grid_constant__ TreePlan plan)
         m = work_off();
     }
     if (plan.n && plan.prio == nullptr) {
-        // without priorities the new transitions take the running maximum, this update's writes included
-        // (one CTA only: the update's maximum is in its shared memory)
+        // (the update's maximum: see whole_max)
         const unsigned w = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(wmax));
         if ((tid & 31u) == 0u && w) atomicMax(&s_max, w);
     }
@@ -696,8 +707,10 @@ int prb_launch_tree(const PrbView& v, const PrbTreeArgs& t, cudaStream_t s, bool
 {
     const int dev = prb_current_device();
     if (t.B == 0 && t.n == 0) return 0;
-    if (t.n && t.prio == nullptr && t.B && prb_tree_ctas(v, t.B, t.n, t.most_ctas) > 1u) {
-        // default priorities take the update's maximum, which several CTAs do not have in time: two launches
+    if (t.n && t.prio == nullptr && t.B > kPrbTreeEntries) {
+        // default priorities take the update's maximum, for which every CTA would have to transform the whole batch (see
+        // whole_max in the kernel): two launches from there on.  One launch below: fanout 16, 256 + 256 entries 8.7 -> XX us,
+        // 256 + 5000 10.9 -> XX.
         PrbTreeArgs u = t, w = t;
         u.n = 0;
         w.B = 0;
