@@ -482,21 +482,34 @@ prb_sample_kernel(const __grid_constant__ PrbView v, uint32_t B, float beta, uin
 // The smallest positive leaf among the `fill` stored ones, into state->pmin_bits (all ones at creation and
 // again after every sample that used it): positive binary32 values order like their bit patterns.
 // Bound by L2 bandwidth (the leaves of up to 2^24 slots stay there): eight 16-byte loads in flight per thread.
-// (a slot beyond the fill count has leaf 0, and so has the padding behind the last one: neither counts)
+// Only the stored slots count: the rest of the level, zeros, is not read where it is more than the grid's first loads (a buffer
+// of 2^26 slots, 1/1000 full: 66 -> XX us a sample).  There the fill count arrives while two loads per thread are under
+// way; a level that all threads' first loads cover is read whole (a zero leaf never wins), without waiting for the count.
 __global__ void __launch_bounds__(256) prb_leaf_min_kernel(const __grid_constant__ PrbView v)
 {
     const float4* leaves = reinterpret_cast<const float4*>(v.level[v.depth]);
-    const uint64_t units = (v.level_alloc[v.depth] + 3u) / 4u, stride = (uint64_t)gridDim.x * blockDim.x;
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    uint64_t units = (v.level_alloc[v.depth] + 3u) / 4u, i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     unsigned best = 0xFFFFFFFFu;
     // (a zero leaf wraps to the largest value and never wins)
-    auto take = [&best](float p) { best = min(best, __float_as_uint(p) - 1u); };
+    auto take = [&best](const float4& t) {
+        best = min(min(best, __float_as_uint(t.x) - 1u), min(__float_as_uint(t.y) - 1u, min(__float_as_uint(t.z) - 1u, __float_as_uint(t.w) - 1u)));
+    };
     constexpr int U = 8;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < units; i += stride * U) {
+    if (units > stride * U) {
+        const uint64_t stored = (__ldg(&v.state->fill) + 3u) / 4u;
+        const float4 a = __ldg(leaves + i), b = __ldg(leaves + i + stride);
+        take(a);
+        take(b);
+        i += 2u * stride;
+        units = min(units, stored);
+    }
+    for (; i < units; i += stride * U) {
         float4 t[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) t[u] = i + u * stride < units ? __ldg(leaves + i + u * stride) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
-        for (int u = 0; u < U; ++u) { take(t[u].x); take(t[u].y); take(t[u].z); take(t[u].w); }
+        for (int u = 0; u < U; ++u) take(t[u]);
     }
     __shared__ unsigned s_best[8];
     best = __reduce_min_sync(0xFFFFFFFFu, best);

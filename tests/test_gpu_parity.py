@@ -1054,6 +1054,27 @@ def test_sample_normalised_over_the_buffer(oracle_mod, wl, N, B):
     pr.close()
 
 
+@pytest.mark.parametrize("N,fill", [(1 << 23, 5000), (1 << 23, 6_000_000), (20_000, 7)])
+def test_buffer_norm_reads_the_stored_slots(oracle_mod, N, fill):
+    # the scan for the smallest priority: levels larger than one round of the grid's loads and smaller ones, nearly empty
+    # and not; the smallest priority in the last stored slot
+    pr = Pair(oracle_mod, N, 16, 0, 0, 1 << 20, oracle_store=False)
+    rng = np.random.default_rng(fill)
+    for at in range(0, fill, 1 << 20):
+        p = (1.0 + rng.random(min(1 << 20, fill - at))).astype(np.float32)
+        if at + p.size == fill:
+            p[-1] = 0.125
+        pr.insert(dict(prio=p))
+    for call in range(2):
+        o = pr.ora.sample_buffer_norm(64, 0.7, 3, gather=False)
+        idx, w = torch.zeros(64, dtype=torch.int32, device=pr.dev), torch.zeros(64, device=pr.dev)
+        pr.gpu.sample_buffer_norm(64, 0.7, 3, idx, w)
+        assert np.array_equal(o["idx"], idx.cpu().numpy())
+        np.testing.assert_allclose(w.cpu().numpy(), o["w"], rtol=1e-5, atol=0)
+    pr.compare_status()
+    pr.close()
+
+
 @pytest.mark.parametrize("wl,N,B,n_sub", [(wk.CARTPOLE, 3000, 64, 2), (wk.DDPG, 100_000, 1000, 4), (wk.DDPG, 5000, 3, 3),
                                           (wk.ATARI, 700, 512, 4), (wk.ATARI, 700, 37, 3)])
 def test_sample_streamed_as_sub_batches(oracle_mod, wl, N, B, n_sub):
