@@ -64,7 +64,7 @@ int prb_launch_update(const PrbView& v, uint32_t B, const int32_t* d_idx, const 
     if (raw != 2) {
         PrbTreeArgs t;
         t.B = B; t.idx = d_idx; t.val = d_val; t.raw = raw; t.alpha = alpha; t.eps = eps; t.stale = stale;
-        if (linked) t.most_ctas = 4u;      // (see prb_launch_insert)
+        if (linked && B <= kPrbTreeEntries) t.most_ctas = 4u;      // (see prb_launch_insert)
         return prb_launch_tree(v, t, s, true);
     }
     static bool big_smem[kPrbMaxDevices];

@@ -468,6 +468,38 @@ def test_step_through_host_buffers(oracle_mod, wl, N, B, n):
     pr.close()
 
 
+@pytest.mark.parametrize("obs_bytes,act_bytes", [(16, 4), (6, 2), (7, 3)])
+@pytest.mark.parametrize("B_upd,n,B", [(1024, 777, 1536), (1025, 777, 1537), (2000, 1, 2000), (3000, 4097, 64), (4096, 0, 1025)])
+def test_host_step_of_many_short_rows(oracle_mod, obs_bytes, act_bytes, B_upd, n, B):
+    # within 256 KB each way, so through the mapped buffer: from 1025 updates on their indices and TD errors are copied to
+    # the device first, the new rows are read over the link all the same (rows of 4-, 2- and 1-byte words)
+    rng = np.random.default_rng(B_upd + obs_bytes)
+    N = 9000
+    pr = Pair(oracle_mod, N, 16, obs_bytes, act_bytes, 4200)
+    mk = lambda m: dict(raw_fields(rng, m, obs_bytes, act_bytes), prio=np.exp(rng.standard_normal(m)).astype(np.float32))
+    for at in range(0, N, 4000):
+        pr.insert(mk(min(4000, N - at)))
+    for step in range(3):
+        idx = rng.integers(-1, N, size=B_upd).astype(np.int32)
+        td = rng.standard_normal(B_upd).astype(np.float32)
+        b = mk(n)
+        assert pr.ora.update(idx, td, 0.6, 1e-6) == 0
+        if n:
+            assert pr.ora.insert(b["obs"], b["act"], b["rew"], b["next_obs"], b["done"], b["prio"]) == 0
+        o = pr.ora.sample(B, 0.4, 2 + step)
+        g = {"idx": np.full(B, -1, np.int32), "w": np.zeros(B, np.float32), "obs": np.zeros((B, obs_bytes), np.uint8),
+             "act": np.zeros((B, act_bytes), np.uint8), "rew": np.zeros(B, np.float32), "next_obs": np.zeros((B, obs_bytes), np.uint8),
+             "done": np.zeros(B, np.uint8)}
+        new = [np.ascontiguousarray(b[k]) for k in ("obs", "act", "rew", "next_obs", "done", "prio")] if n else [None] * 6
+        pr.gpu.step_host(idx, td, 0.6, 1e-6, *new, B, 0.4, 2 + step, g["idx"], g["w"], g["obs"], g["act"], g["rew"], g["next_obs"], g["done"])
+        pr.compare_sample(o, g)
+        pr.compare_tree()
+        pr.compare_state()
+    pr.compare_rows(np.arange(N, dtype=np.int32))
+    pr.compare_status()
+    pr.close()
+
+
 @pytest.mark.parametrize("wl,N,B,n", [(wk.CARTPOLE, 5000, 64, 64), (wk.DDPG, 70_000, 256, 256), (wk.DDPG, 3000, 1000, 777),
                                       (wk.ATARI, 1500, 512, 512), (wk.ATARI, 700, 37, 1), (wk.ATARI, 700, 4096, 300)])
 def test_fused_update_insert(oracle_mod, wl, N, B, n):
@@ -1066,7 +1098,7 @@ def test_buffer_norm_reads_the_stored_slots(oracle_mod, N, fill):
             p[-1] = 0.125
         pr.insert(dict(prio=p))
     for call in range(2):
-        o = pr.ora.sample_buffer_norm(64, 0.7, 3, gather=False)
+        o = pr.ora.sample(64, 0.7, 3, gather=False, buffer_norm=True)
         idx, w = torch.zeros(64, dtype=torch.int32, device=pr.dev), torch.zeros(64, device=pr.dev)
         pr.gpu.sample_buffer_norm(64, 0.7, 3, idx, w)
         assert np.array_equal(o["idx"], idx.cpu().numpy())
