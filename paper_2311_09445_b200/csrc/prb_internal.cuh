@@ -393,8 +393,8 @@ constexpr uint32_t kBulkSpinLimit = 1u << 20;   // mbarrier polls before a wait 
 __device__ __forceinline__ uint32_t prb_smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // The wait for the first phase of a barrier that peers' transfers complete, by one thread, a warp or a CTA.  One that ran out
-// is raised and marks the buffer (see PrbState::wide_poisoned) -- out of line: in line it cost the sample of 64 strata
-// 0.1 us of 4.3.
+// is raised and marks the buffer (see PrbState::wide_poisoned).  kOutOfLine: in line that cost the sample of 64 strata 0.1 us
+// of 4.3; in the tree kernel it is the call that costs (a stack).
 __device__ __forceinline__ bool prb_first_phase_over(uint32_t bar)
 {
     uint32_t ok;
@@ -402,15 +402,18 @@ __device__ __forceinline__ bool prb_first_phase_over(uint32_t bar)
                  : "=r"(ok) : "r"(bar) : "memory");
     return ok != 0u;
 }
-static __noinline__ __device__ PrbWaited prb_first_phase_ran_out(PrbState* st, uint32_t bar)
+__device__ __forceinline__ PrbWaited prb_first_phase_late(PrbState* st, uint32_t bar)
 {
     atomicOr(&st->status, PEARL_ST_INTERNAL);
     atomicExch(&st->wide_poisoned, 1u);
     return prb_poll([bar]() { return prb_first_phase_over(bar); }, kBulkSpinLimit) ? kPrbLate : kPrbNever;
 }
+static __noinline__ __device__ PrbWaited prb_first_phase_ran_out(PrbState* st, uint32_t bar) { return prb_first_phase_late(st, bar); }
+template <bool kOutOfLine>
 __device__ __forceinline__ PrbWaited prb_wait_first_phase(PrbState* st, uint32_t bar)
 {
-    return prb_wait_bounded([bar]() { return prb_first_phase_over(bar); }, kBulkSpinLimit, [st, bar]() { return prb_first_phase_ran_out(st, bar); });
+    return prb_wait_bounded([bar]() { return prb_first_phase_over(bar); }, kBulkSpinLimit,
+                            [st, bar]() { return kOutOfLine ? prb_first_phase_ran_out(st, bar) : prb_first_phase_late(st, bar); });
 }
 
 struct PrbBulkLane {

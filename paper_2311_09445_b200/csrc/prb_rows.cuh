@@ -1,7 +1,15 @@
-// Short rows as words: the copy between the Data Storage (slots) and a dense batch, in either direction, without
-// an index being divided.  A transition is numbered in words of 4 bytes (2 or 1 where a field's granule is
-// smaller) over all its fields; a lane's word is fixed, so where it lies in a slot and in a row of the batch is
-// looked up once, and consecutive lanes touch consecutive words.
+// The copy of rows between the Data Storage (slots) and a dense batch, through registers, in three ways.
+//
+// Words (rows of up to kPrbMostWords of them): no index is divided.  A transition is numbered in words of 4 bytes (2 or 1
+// where a field's granule is smaller) over all its fields; a lane's word is fixed, so where it lies in a slot and in a row of
+// the batch is looked up once, and consecutive lanes touch consecutive words.
+// Tiles (an insertion's longer rows): kPrbTile consecutive granules (the largest power of two up to 16 bytes that divides
+// the field) of one field, whatever rows they belong to; a division each.  A row is no unit of work, so one long row keeps
+// several CTAs busy and a thread moves up to 16 bytes at a time.
+// Units (a sample's longer rows): all the granules of a CTA's rows, field by field, dealt to its threads; a division each,
+// loads of several fields in flight at once.
+// us a call, as words / this way: insertion of 1 row of 14 KB 9.4 / 3.8, of 256 11.2 / 4.4, of one row of 56 KB of an odd size
+// 131 / 3.6; sample of 512 rows of 2 KB 19 / 7.0, of 8 KB 46 / 10, of 64 rows of 56 KB of an odd size 141 / 60.
 #pragma once
 #include "prb_internal.cuh"
 
@@ -9,30 +17,51 @@
 struct PrbWordField {
     unsigned char* store;         // slot 0
     unsigned char* batch;         // row 0 of the batch
-    uint32_t first, log2;
+    uint32_t first;
+    uint16_t log2, unit;                       // log2 of the word and of the granule (few bytes: a cold line of parameters is 84 cycles)
     uint32_t store_pitch, batch_pitch;
+    PRB_HD uint32_t units() const { return batch_pitch >> unit; }      // granules per row
 };
 struct PrbWords {
     uint32_t n_words, chunks, lane_words;      // chunks of 32 words; lanes that share a row (8, 16 or 32)
+    uint32_t units;                            // granules per row over all fields; 0: too many of them for 32 bits
+    uint32_t fine;                             // 1: most of the row is granules of up to 4 bytes (and all of it is copied as such)
     PrbWordField field[PRB_NUM_FIELDS];
 };
+constexpr uint32_t kPrbMostWords = 64;
+constexpr uint32_t kPrbTile = 2048;
 
 inline PrbWords prb_plan_words(const PrbView& v, const PrbBatch& batch)
 {
     PrbWords p;
-    uint32_t words = 0;
+    uint32_t words = 0, coarse = 0;
+    uint64_t units = 0;
     for (int f = 0; f < PRB_NUM_FIELDS; ++f) {
         PrbWordField& fd = p.field[f];
-        fd = PrbWordField{nullptr, nullptr, 0xFFFFFFFFu, 0u, 0u, 0u};
+        fd = PrbWordField{nullptr, nullptr, 0xFFFFFFFFu, 0, 0, 0u, 0u};
         if (batch.ptr[f] == nullptr || v.field_bytes[f] == 0) continue;
         fd.store = v.store[f];
         fd.batch = batch.ptr[f];
-        fd.log2 = v.field_vec[f] >= 4u ? 2u : v.field_vec[f] == 2u ? 1u : 0u;
+        fd.log2 = (uint16_t)(v.field_vec[f] >= 4u ? 2u : v.field_vec[f] == 2u ? 1u : 0u);
         fd.first = words;
         fd.store_pitch = v.field_pitch[f];
         fd.batch_pitch = v.field_bytes[f];
         words += v.field_bytes[f] >> fd.log2;
+        while ((1u << fd.unit) < v.field_vec[f]) ++fd.unit;
+        units += v.field_bytes[f] >> fd.unit;
+        if (fd.unit > 2u) coarse += v.field_bytes[f] >> fd.log2;
     }
+    p.fine = coarse < words - coarse ? 1u : 0u;
+    if (p.fine) {
+        // (then the other fields go as units of 4 bytes, too)
+        for (int f = 0; f < PRB_NUM_FIELDS; ++f) {
+            PrbWordField& fd = p.field[f];
+            if (fd.unit <= 2u) continue;
+            units += ((uint64_t)fd.units() << (fd.unit - 2u)) - fd.units();
+            fd.unit = 2u;
+        }
+    }
+    p.units = units * v.max_batch < (1ull << 31) ? (uint32_t)units : 0u;
     p.n_words = words;
     p.chunks = words ? (words + 31u) / 32u : 1u;
     p.lane_words = words <= 8u ? 8u : words <= 16u ? 16u : 32u;
@@ -113,6 +142,95 @@ __device__ __forceinline__ void prb_copy_words(const PrbWords& p, const PrbWordS
                     else if (o.log2 == 1u) *reinterpret_cast<uint16_t*>(at) = (uint16_t)v[u];
                     else *at = (unsigned char)v[u];
                 }
+            }
+        }
+    }
+}
+
+// Tile `tile` of the n rows of a batch, to the store, by the whole CTA.
+template <typename T, typename SlotOf>
+__device__ __forceinline__ void prb_copy_tile(const PrbWordField& fd, uint32_t n, uint32_t tile, SlotOf slot_of)
+{
+    const uint32_t W = fd.units(), e0 = tile * kPrbTile, e1 = (uint32_t)min((uint64_t)n * W, (uint64_t)e0 + kPrbTile);      // (n W is below 2^32)
+    const uint64_t Wp = fd.store_pitch / sizeof(T);
+    prb_copy_mapped<T>(reinterpret_cast<T*>(fd.store), reinterpret_cast<const T*>(fd.batch), e0, e1, [](uint32_t e) { return (uint64_t)e; },
+                       [=](uint32_t e) { const uint32_t r = e / W; return (uint64_t)slot_of(r) * Wp + (e - r * W); }, threadIdx.x, blockDim.x);
+}
+// All tiles, shared out over `ctas` CTAs of which this one is number `cta`.
+template <typename SlotOf>
+__device__ __forceinline__ void prb_copy_tiles(const PrbWords& p, uint32_t cta, uint32_t ctas, uint32_t n, SlotOf slot_of)
+{
+    auto tiles = [&](int f) { return (uint32_t)(((uint64_t)n * p.field[f].units() + kPrbTile - 1u) / kPrbTile); };
+    uint32_t total = 0;
+#pragma unroll
+    for (int f = 0; f < PRB_NUM_FIELDS; ++f) total += tiles(f);
+    const uint32_t t_lo = (uint32_t)(((uint64_t)cta * total) / ctas), t_hi = (uint32_t)(((uint64_t)(cta + 1u) * total) / ctas);
+    for (uint32_t t = t_lo; t < t_hi; ++t) {
+        uint32_t tile = t;
+        int f = 0;
+        for (; f + 1 < PRB_NUM_FIELDS; ++f) {
+            const uint32_t here = tiles(f);
+            if (tile < here) break;
+            tile -= here;
+        }
+        const PrbWordField& fd = p.field[f];
+        switch (fd.unit) {
+        case 4: prb_copy_tile<uint4>(fd, n, tile, slot_of); break;
+        case 3: prb_copy_tile<uint2>(fd, n, tile, slot_of); break;
+        case 2: prb_copy_tile<uint32_t>(fd, n, tile, slot_of); break;
+        case 1: prb_copy_tile<uint16_t>(fd, n, tile, slot_of); break;
+        default: prb_copy_tile<unsigned char>(fd, n, tile, slot_of); break;
+        }
+    }
+}
+
+// Rows [k0, k0 + n) of the batch as units, from the store, by `nthreads` threads of which this one has rank `rank`; four loads of
+// a thread in flight (65536 rows of 165 bytes 20.9 us; with eight 4-byte loads where no granule is larger 25.9, and with the field
+// looked up again for the store instead of kept 23.5).
+template <typename SlotOf>
+__device__ __forceinline__ void prb_copy_units(const PrbWords& p, uint32_t rank, uint32_t nthreads, uint32_t k0, uint32_t n, SlotOf slot_of)
+{
+    constexpr int U = 4;
+    const uint32_t total = p.units * n;
+    for (uint32_t e0 = rank; e0 < total; e0 += nthreads * U) {
+        uint4 v[U];
+        unsigned char* to[U];
+        uint32_t lg[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            uint32_t e = e0 + u * nthreads;
+            to[u] = nullptr;
+            lg[u] = 0u;
+            v[u] = make_uint4(0u, 0u, 0u, 0u);
+            if (e >= total) continue;
+            int f = 0;
+#pragma unroll
+            for (int g = 0; g + 1 < PRB_NUM_FIELDS; ++g) {
+                const uint32_t here = p.field[g].units() * n;
+                if (f == g && e >= here) { e -= here; f = g + 1; }
+            }
+            const PrbWordField& fd = p.field[f];
+            const uint32_t W = fd.units(), r = e / W, at = (e - r * W) << fd.unit;
+            const unsigned char* const from = fd.store + (uint64_t)slot_of(r) * fd.store_pitch + at;
+            to[u] = fd.batch + (uint64_t)(k0 + r) * fd.batch_pitch + at;
+            lg[u] = fd.unit;
+            switch (fd.unit) {
+            case 4: v[u] = *reinterpret_cast<const uint4*>(from); break;
+            case 3: { const uint2 t = *reinterpret_cast<const uint2*>(from); v[u].x = t.x; v[u].y = t.y; break; }
+            case 2: v[u].x = *reinterpret_cast<const uint32_t*>(from); break;
+            case 1: v[u].x = *reinterpret_cast<const uint16_t*>(from); break;
+            default: v[u].x = *from; break;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (to[u] == nullptr) continue;
+            switch (lg[u]) {
+            case 4: *reinterpret_cast<uint4*>(to[u]) = v[u]; break;
+            case 3: *reinterpret_cast<uint2*>(to[u]) = make_uint2(v[u].x, v[u].y); break;
+            case 2: *reinterpret_cast<uint32_t*>(to[u]) = v[u].x; break;
+            case 1: *reinterpret_cast<uint16_t*>(to[u]) = (uint16_t)v[u].x; break;
+            default: *to[u] = (unsigned char)v[u].x; break;
             }
         }
     }

@@ -14,7 +14,7 @@
 //    with p, so this is division by the batch's largest weight), one power per stratum and nothing to
 //    normalise afterwards.  p_min is exchanged while the rows are on their way.
 //  * Rows are copied word by word, a warp (or a part of one) per row: a lane's word of the row is fixed, so
-//    where it lies is looked up once and no index is divided.
+//    where it lies is looked up once and no index is divided; longer rows, and all rows of the grid, unit by unit.
 //
 // Two shapes, by batch size.  Up to kClusterStrata strata: one thread-block cluster of up to 16 CTAs; p_min goes
 // through distributed shared memory (each transfer signals the receiver's barrier), nothing through global
@@ -33,7 +33,10 @@ constexpr uint32_t kMaxCluster = 16;
 // cooperative launch, no programmatic one, and a round through global memory for the smallest priority.)
 constexpr uint32_t kClusterStrata = 1536;
 constexpr uint32_t kMaxSeen = 64;                    // strata warps of a cluster: 8 CTAs x 6 warps, 16 x 3
-constexpr uint32_t kGridStrata = 32;                 // strata per CTA of the cooperative grid, at least
+constexpr uint32_t kGridStrata = 32;                 // strata per CTA of the cooperative grid, at least (fewer where rows are long)
+constexpr uint32_t kClusterUnits = 1u << 16;         // a cluster copies at most this many units ...
+constexpr uint32_t kClusterWords = 400u << 10;       // ... or words
+constexpr uint32_t kLaneGroupUnits = 160;            // units of a row up to which the lane-group kernel comes next
 constexpr uint32_t kShortSpinLimit = 1u << 22;
 constexpr uint32_t kNotStaged = 0xFFFFFFFFu;
 
@@ -56,6 +59,7 @@ struct ShortPlan {
     float beta;
     uint32_t uniform, buffer_norm;
     uint32_t n_steps;
+    uint32_t as_units;            // rows are copied unit by unit
     ShortStep step[kMaxSteps];
     PrbWords words;
 };
@@ -291,10 +295,12 @@ __device__ __forceinline__ uint32_t draw(const ShortPlan& plan, const ShortStep*
     return leaf;
 }
 
-// Rows of strata [k0, k0 + n).
-__device__ __forceinline__ void gather(const ShortPlan& plan, const PrbWordShare& share, uint32_t warps, uint32_t k0, uint32_t n, const uint32_t* s_idx)
+// Rows of strata [k0, k0 + n), by `warps` warps; `rank`: this thread's among them.
+__device__ __forceinline__ void gather(const ShortPlan& plan, const PrbWordShare& share, uint32_t warps, uint32_t rank, uint32_t k0, uint32_t n, const uint32_t* s_idx)
 {
-    prb_copy_words<false>(plan.words, share, warps, k0, n, [&](uint32_t r) { return PRB_IN_BOUNDS(plan, s_idx[r] < plan.capacity) ? s_idx[r] : 0u; });
+    auto slot_of = [&](uint32_t r) { return PRB_IN_BOUNDS(plan, s_idx[r] < plan.capacity) ? s_idx[r] : 0u; };
+    if (plan.as_units == 0u) { prb_copy_words<false>(plan.words, share, warps, k0, n, slot_of); return; }
+    prb_copy_units(plan.words, rank, warps * 32u, k0, n, slot_of);
 }
 
 // What a CTA stages: 16-byte unit `q` of the staged levels, taken one after another (from: nullptr beyond the last).
@@ -403,7 +409,7 @@ prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
     }
     if (copies) {
         asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");
-        if (split) { gather(plan, share, warps - first_copier, k_lo, n, s_idx); return; }
+        if (split) { gather(plan, share, warps - first_copier, tid - first_copier * 32u, k_lo, n, s_idx); return; }
     }
     double log_p = 0.0;
     if (warp < strata_warps) {
@@ -422,10 +428,10 @@ prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
         }
         if (mine) plan.out_idx[k] = (int32_t)leaf;
     }
-    if (!split) gather(plan, share, warps, k_lo, n, s_idx);
+    if (!split) gather(plan, share, warps, tid, k_lo, n, s_idx);
     // (the first warp always gets here: it keeps the CTA's shared memory until every value has come)
     if (warp >= strata_warps) return;
-    if (prb_wait_first_phase(plan.state, bar) == kPrbNever) return;
+    if (prb_wait_first_phase<true>(plan.state, bar) == kPrbNever) return;
     if (blockIdx.x == 0 && tid == 0) {
         plan.state->sample_calls = calls + 1;                  // (every CTA has drawn)
         if (plan.buffer_norm) plan.state->pmin_bits = ~0ull;   // (ready for the next scan)
@@ -525,7 +531,7 @@ prb_sample_grid_kernel(const __grid_constant__ ShortPlan plan)
             if (exchange) atomicMax(&plan.state->wide_wmax_bits, (unsigned long long)(~s_min));
             asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&plan.state->sample_ticket) : "memory");
         }
-        gather(plan, share, warps, kb, n, s_idx);
+        gather(plan, share, warps, tid, kb, n, s_idx);
         if (!last) __syncthreads();           // s_idx is rewritten by the next pass
     }
     if (tid == kShortThreads - 1u) {
@@ -609,8 +615,21 @@ int prb_launch_sample_short(const PrbView& v, uint32_t B, float beta, uint64_t s
 {
     const int dev = prb_current_device();
     const ShortLimits* lim = short_limits(v.fanout, (int)v.log2_fanout, dev);
-    if (B > kClusterStrata && lim->per_sm == 0) return 0;
     ShortPlan plan;
+    plan.words = prb_plan_words(v, dst);
+    const PrbWords& rows = plan.words;
+    // Which kernel.  The cluster's 16 SMs while they have little to copy: up to kClusterUnits units (kClusterWords words where a
+    // row's granules are small).  Beyond, up to kClusterStrata strata: rows of medium length go to the lane-group kernel
+    // (prb_sample.cu: every SM copies, and no grid-wide minimum); longer ones, and more strata, to the grid, with fewer
+    // strata to a CTA where rows are long.  us a call, cluster / lane groups / grid, fanout 16: 512 rows of 1 KB 6.6 / 6.9 /
+    // 8.6, 1024 of 1 KB 8.7 / 8.4 / 9.3, 512 of 2 KB 7.7 / 7.0 / 8.5, 1024 of 2 KB 11.5 / 8.3 / 9.0; 256 of 4 KB 8.1 / 9.3 / 8.5,
+    // 512 of 4 KB 11.5 / 9.6 / 9.1, 256 of 14 KB 17 / 21 / 10.7, 1024 of 14 KB 57 / 22 / 13.5.
+    const bool longer = rows.n_words > kPrbMostWords;
+    const uint64_t units = (uint64_t)B * rows.units, words = (uint64_t)B * rows.n_words;
+    const bool cluster = B <= kClusterStrata && (!longer || rows.units == 0u || (rows.fine ? words <= kClusterWords : units <= kClusterUnits));
+    if (!cluster && B <= kClusterStrata && !rows.fine && rows.units <= kLaneGroupUnits) return 0;
+    if (!cluster && lim->per_sm == 0) return 0;
+    plan.as_units = rows.units != 0u && (!cluster || (longer && !rows.fine)) ? 1u : 0u;
     plan.state = v.state;
     plan.level0 = v.level[0];
     plan.out_idx = d_idx;
@@ -641,7 +660,6 @@ int prb_launch_sample_short(const PrbView& v, uint32_t B, float beta, uint64_t s
         if (staging) at += entries;
     }
     plan.n_steps = n;
-    plan.words = prb_plan_words(v, dst);
     cudaLaunchConfig_t cfg = {};
     cfg.stream = s;
     cudaLaunchAttribute a[2];
@@ -654,7 +672,7 @@ int prb_launch_sample_short(const PrbView& v, uint32_t B, float beta, uint64_t s
     }
     cudaError_t e;
     cfg.blockDim = dim3(kShortThreads);
-    if (B <= kClusterStrata) {
+    if (cluster) {
         // a few strata per CTA (their rows are copied by all its warps), up to the whole cluster
         uint32_t ctas = 1;
         while (ctas < lim->cluster && ctas * 4u < B) ctas *= 2u;
@@ -666,7 +684,8 @@ int prb_launch_sample_short(const PrbView& v, uint32_t B, float beta, uint64_t s
         cfg.numAttrs = 2;
         e = cudaLaunchKernelEx(&cfg, short_kernel<false>(v.fanout), plan);
     } else {
-        uint32_t grid = (B + kGridStrata - 1) / kGridStrata;
+        const uint32_t strata = rows.units >= 4000u ? 1u : rows.units >= 400u ? 4u : rows.units >= 100u ? 8u : kGridStrata;
+        uint32_t grid = (B + strata - 1) / strata;
         const uint32_t room = (uint32_t)prb_sm_count() * lim->per_sm;
         if (grid > room) grid = room;
         cfg.gridDim = dim3(grid);

@@ -56,6 +56,7 @@ struct TreePlan {
     uint32_t copies;                         // CTAs that copy rows
     uint32_t dependent;                      // launched as a programmatic dependent
     uint32_t linked;                         // the inputs lie in mapped host memory
+    uint32_t tiles;                          // rows are copied as tiles
     uint32_t off[PRB_MAX_LEVELS];            // level l starts off[l] * 64 entries behind level 0
     PrbWords words;
 };
@@ -287,7 +288,6 @@ prb_tree_kernel(const __grid_constant__ TreePlan plan)
     __shared__ uint32_t s_off[PRB_MAX_LEVELS];
     __shared__ __align__(8) unsigned long long s_bar;        // (cluster, CTA 0) level T is complete in the staged copy
     __shared__ unsigned s_max, s_count, s_sent, s_last, s_before;
-    __shared__ uint32_t s_row;                               // (copying CTAs) row_cursor
     const uint32_t tid = threadIdx.x, nt = blockDim.x;
     constexpr uint32_t lg = kLog2<K>;
 
@@ -297,25 +297,22 @@ prb_tree_kernel(const __grid_constant__ TreePlan plan)
         const PrbWordShare share = prb_word_share(plan.words, tid >> 5, nt >> 5);
         prb_dep_wait();
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-        const uint32_t N = plan.capacity;
-        // (one thread reads the cursor for the CTA: it is in shared memory, so the load has answered, before the CTA
-        // draws its ticket -- a barrier alone would not say so of loads that other threads still have on their way --
-        // and only then may the last CTA move it)
-        if (tid == 0) s_row = (uint32_t)__ldcg(&plan.state->row_cursor);
+        const uint32_t cursor = (uint32_t)__ldcg(&plan.state->row_cursor), N = plan.capacity;
         const uint32_t r_lo = (uint32_t)(((uint64_t)c * plan.n) / plan.copies), r_hi = (uint32_t)(((uint64_t)(c + 1) * plan.n) / plan.copies);
+        auto slot_from = [&](uint32_t first) {
+            return [cursor, first, N](uint32_t r) { const uint32_t s = cursor + first + r; return s >= N ? s - N : s; };
+        };
+        if (plan.linked) prb_copy_flat(plan.words, c * (nt >> 5) + (tid >> 5), plan.copies * (nt >> 5), plan.n, slot_from(0u));
+        else if (plan.tiles) prb_copy_tiles(plan.words, c, plan.copies, plan.n, slot_from(0u));
+        else prb_copy_words<true>(plan.words, share, nt >> 5, r_lo, r_hi - r_lo, slot_from(r_lo));
+        // The ticket comes last: whoever used the cursor has had its answer (the addresses it has stored to come from it), so
+        // the last CTA may move it.  (Drawn first, behind one thread's read, the rows' loads waited for the cursor, which they
+        // do not need: 0.3 us an insertion.)
         __syncthreads();
-        const uint32_t cursor = s_row;
         if (tid == nt - 1u && prb_ticket(&plan.state->row_ticket) == plan.copies - 1u) {
             plan.state->row_cursor = cursor + plan.n >= N ? cursor + plan.n - N : cursor + plan.n;
             plan.state->row_ticket = 0u;
         }
-        if (plan.linked) {
-            prb_copy_flat(plan.words, c * (nt >> 5) + (tid >> 5), plan.copies * (nt >> 5), plan.n,
-                          [&](uint32_t r) { const uint32_t s = cursor + r; return s >= N ? s - N : s; });
-            return;
-        }
-        prb_copy_words<true>(plan.words, share, nt >> 5, r_lo, r_hi - r_lo,
-                             [&](uint32_t r) { const uint32_t s = cursor + r_lo + r; return s >= N ? s - N : s; });
         return;
     }
 
@@ -629,7 +626,7 @@ prb_tree_kernel(const __grid_constant__ TreePlan plan)
         if (tid == 0)
             asm volatile("mbarrier.arrive.expect_tx.relaxed.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(c.bar), "r"(s_sent * (kMin ? 8u : 4u)) : "memory");
         if (blockIdx.x != 0) return;
-        prb_wait_first_phase(plan.state, prb_smem_addr(&s_bar));
+        prb_wait_first_phase<false>(plan.state, prb_smem_addr(&s_bar));
         __syncthreads();
     }
     // every CTA of the tree work has read cursor and fill: they move on
@@ -742,8 +739,15 @@ int prb_launch_tree(const PrbView& v, const PrbTreeArgs& t, cudaStream_t s, bool
         p.T = l;
         p.top_floats = (uint32_t)end;
     }
-    uint32_t parts = p.T ? prb_tree_ctas(v, t.B, t.n, t.most_ctas) : 1u;      // (no staged level: nothing to split by)
+    PrbBatch none;
+    for (int f = 0; f < PRB_NUM_FIELDS; ++f) none.ptr[f] = nullptr;
+    p.words = prb_plan_words(v, t.rows ? *t.rows : none);
+    p.tiles = p.words.n_words > kPrbMostWords && !t.linked ? 1u : 0u;
     p.grid_form = tree_grid_form(t.B, t.n) ? 1u : 0u;
+    uint32_t parts = p.T ? prb_tree_ctas(v, t.B, t.n, t.most_ctas) : 1u;      // (no staged level: nothing to split by)
+    // (an insertion of longer rows alone: its copying CTAs, which take longer than the tree work, would come in clusters, too,
+    // and leave SMs idle that no whole cluster fits on: 1024 rows of 14 KB 9.3 us with a cluster of 16, 6.8 with one CTA)
+    if (p.tiles && t.B == 0u && !p.grid_form) parts = 1u;
     p.parts = parts;
     p.list = p.grid_form ? kGridList : t.B;
     // (at least 512 places, whatever the entries: probes are a chain of shared atomics; 32 entries in 64 places took 4.7 to
@@ -765,16 +769,18 @@ int prb_launch_tree(const PrbView& v, const PrbTreeArgs& t, cudaStream_t s, bool
     p.copies = 0;
     p.dependent = dependent ? 1u : 0u;
     p.linked = t.linked ? 1u : 0u;
-    PrbBatch none;
-    for (int f = 0; f < PRB_NUM_FIELDS; ++f) none.ptr[f] = nullptr;
-    p.words = prb_plan_words(v, t.rows ? *t.rows : none);
     if (t.rows && t.n) {
-        // a few rows' words per warp, on the SMs the tree work leaves
-        const uint64_t items = (uint64_t)t.n * p.words.chunks * p.words.lane_words / 32u, per_cta = threads / 32u * 4u;
-        uint64_t ctas = (items + per_cta - 1) / per_cta;
+        // a few rows' words per warp, or a tile per CTA, on the SMs the tree work leaves
+        uint64_t ctas = 0;
+        if (p.tiles) {
+            for (int f = 0; f < PRB_NUM_FIELDS; ++f) ctas += ((uint64_t)t.n * p.words.field[f].units() + kPrbTile - 1) / kPrbTile;
+        } else {
+            const uint64_t items = (uint64_t)t.n * p.words.chunks * p.words.lane_words / 32u, per_cta = threads / 32u * 4u;
+            ctas = (items + per_cta - 1) / per_cta;
+            if (ctas > t.n) ctas = t.n;
+        }
         const uint64_t room = (uint64_t)prb_sm_count() * (threads <= 512u ? 2u : 1u) - parts;
         if (ctas > room) ctas = room;
-        if (ctas > t.n) ctas = t.n;
         p.copies = ctas ? (uint32_t)ctas : 1u;
     }
     if (!p.grid_form && parts > 8u && !tree_cluster_of_16(v, k, dev)) p.parts = parts = 8u;

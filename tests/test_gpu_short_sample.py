@@ -35,6 +35,26 @@ def test_batch_sizes(oracle_mod, K, N, obs_bytes, act_bytes):
     pr.close()
 
 
+@pytest.mark.parametrize("K", [2, 16, 32])
+@pytest.mark.parametrize("obs_bytes,act_bytes", [(128, 4), (132, 4), (1024, 16), (4104, 4), (7056, 8), (8190, 4), (9001, 3)])
+def test_longer_rows(oracle_mod, K, obs_bytes, act_bytes):
+    # rows on either side of the line between words and larger granules (16, 8, 4, 2 and 1 bytes), inserted in batches that
+    # end inside a tile and wrap, sampled by each of the three kernels: the cluster (few, or little to copy), the lane
+    # groups (medium rows), the grid
+    rng = np.random.default_rng(obs_bytes + K)
+    N = 701
+    pr = Pair(oracle_mod, N, K, obs_bytes, act_bytes, 1600)
+    _fill(pr, rng, N, obs_bytes, act_bytes, 333)
+    for n in (1, 2, 17, 256, 700):
+        _fill(pr, rng, n, obs_bytes, act_bytes, n)
+    pr.compare_rows(np.arange(N, dtype=np.int32))
+    for call, B in enumerate([1, 31, 33, 64, 65, 300, 1000, 1600]):
+        pr.sample(B, 0.4, 7 + call)
+        pr.compare_state()
+    assert pr.compare_status() in (0, 8)
+    pr.close()
+
+
 @pytest.mark.parametrize("B", [48, 3000, 200_000])
 def test_weights_against_binary64(oracle_mod, B):
     # (p / p_min)^-beta is formed in binary64 and rounded once to binary32: half a unit in the last place, 2^-24
