@@ -58,11 +58,14 @@ typedef struct pearl_layout {
                                       Every wait on the device (a bulk copy's completion, one thread block's
                                       wait for the others of its call) gives up after a fixed number of polls
                                       instead of hanging.  After a copy that gave up, rows of that call are
-                                      missing or partial; after an update or insertion, nodes of the tree's
-                                      top may not equal the sum of their children; after a sample of short
-                                      rows, weights are missing.  After either of the last two every later
-                                      sample of more than 1536 strata of short rows on that buffer raises the
-                                      bit again and does nothing.  Treat the buffer as lost: destroy it and build a new one.  No
+                                      missing or partial; after an update or insertion, nodes of the tree may
+                                      not equal the sum of their children, and leaves named by an update of
+                                      more than 16384 entries may hold the marker bit pattern 0x80000000|entry
+                                      instead of a priority; after a sample of short rows, weights are
+                                      missing.  After either of the last two every later call on that buffer
+                                      that runs as a grid of co-resident thread blocks (updates of more than
+                                      16384 to 32768 entries, by fanout; samples of more than 1536 strata, or
+                                      of long rows below 8 KB) raises the bit again and does nothing.  Treat the buffer as lost: destroy it and build a new one.  No
                                       correct run raises this bit. */
 #define PEARL_ST_STALE 32u         /* update_after_insert: the index was overwritten since it was sampled; entry skipped */
 

@@ -36,7 +36,7 @@ struct InsertPlan {
     uint32_t chunk[PRB_NUM_FIELDS];           // granules per chunk
     uint32_t ring_stages, ring_stage_bytes;
     // CTAs of a tree kernel that runs beside this one and does the insertion's tree work (0: this
-    // kernel does it); they share the cursor ticket
+    // kernel does it); this kernel then keeps the row cursor, with a ticket of its own
     uint32_t tree_ctas;
 };
 
@@ -193,15 +193,24 @@ int prb_launch_insert(const PrbView& v, uint32_t n, const PrbBatch& src, const f
             tiles += (uint32_t)((total + kTile - 1) / kTile);
         }
     }
+    if (rows_only && tasks == 0) return -1;
+    int ahead = 0;      // launches ahead of the insertion's
+    // a very large update goes first, in a launch of its own: also one that is two launches anyway (no priorities, see
+    // prb_launch_tree) or that eight CTAs beside a copy of long rows would work on (16384 entries, 32 rows: 26 us a call, 14 this way)
+    if (upd_B && (prb_update_is_wide(v, upd_B, d_prio != nullptr) || (tasks && upd_B > 4u * kPrbTreeEntries))) {
+        ahead = prb_launch_update_wide(v, upd_B, upd_idx, upd_val, upd_raw, alpha, eps, s, 0u);
+        if (ahead < 0) return -1;
+        if (ahead) tree.B = upd_B = 0;
+    }
     if (tasks == 0) {
         // short rows: one launch does the update, the insertion's tree work and the row copy
-        if (rows_only) return -1;
         tree.rows = &src;
         tree.linked = linked;
         // (every CTA reads the indices over the link; a larger update's have been copied to the device: with 4 CTAs all the
         // same, a host step of 4000 updates and 64 insertions took 70 us and one of 5000 updates 78, 61 and 65 without the limit)
         if (linked && upd_B <= kPrbTreeEntries) tree.most_ctas = 4u;
-        return prb_launch_tree(v, tree, s, true);
+        const int k = prb_launch_tree(v, tree, s, true);
+        return k < 0 ? -1 : ahead + k;
     }
     plan.first_tile[PRB_NUM_FIELDS] = tiles;
     plan.first_task[PRB_NUM_FIELDS] = tasks;
@@ -265,5 +274,5 @@ int prb_launch_insert(const PrbView& v, uint32_t n, const PrbBatch& src, const f
     PRB_WITH_TREE_OPTIONS(v, PRB_LAUNCH_ROWS_AS);
 #undef PRB_LAUNCH_ROWS_AS
     if (e != cudaSuccess || (forked && cudaStreamWaitEvent(s, fork->join, 0) != cudaSuccess)) return -1;
-    return launches;
+    return ahead + launches;
 }

@@ -35,7 +35,8 @@ struct PrbState {
     unsigned int insert_ticket;       // CTAs of the running insert kernel that have finished
     unsigned int sample_ticket;       // CTAs of the running sample kernel that have finished
     unsigned int max_prio_bits;       // bits of the largest priority written so far (0: none yet)
-    unsigned int unused[2];
+    unsigned int wide_arrived;        // grid barrier of the running many-CTA update: arrivals so far (0 between launches that ended well)
+    unsigned int wide_done;           // its CTAs that have passed their last barrier
     unsigned long long wide_wmax_bits; // smallest priority of the running large-batch sample, complemented (0 between calls)
     // The ring cursor as the kernels that copy rows see it.  An insertion whose tree work and row copy are
     // two kernels on two streams advances `cursor` (and `fill`) from the tree kernel and `row_cursor` from
@@ -43,8 +44,9 @@ struct PrbState {
     // races with, the other's; a one-kernel insertion advances both.  Equal whenever no insertion is running.
     unsigned long long row_cursor;
     unsigned int row_ticket;          // CTAs of the running row kernel that have read row_cursor
-    unsigned int wide_poisoned;       // CTAs that wait for one another (a cluster, or a co-resident grid) gave up once: tickets are not to be
-                                      // trusted, and every later sample of many co-resident CTAs raises INTERNAL and does nothing
+    unsigned int wide_poisoned;       // CTAs that wait for one another (a cluster, or a co-resident grid) gave up once: tickets and the grid
+                                      // barrier's state are not to be trusted, and every later update or sample of many co-resident CTAs
+                                      // raises INTERNAL and does nothing
 };
 
 // Geometry and device addresses, passed to kernels by value.
@@ -191,6 +193,11 @@ constexpr uint32_t kPrbTreeBesideRows = 8;      // CTAs of the tree work beside 
 uint32_t prb_tree_ctas(const PrbView& v, uint32_t b, uint32_t n, uint32_t most);
 // (dependent: as a programmatic dependent of the kernel before it on the stream)
 int prb_launch_tree(const PrbView& v, const PrbTreeArgs& t, cudaStream_t s, bool dependent);
+// A large batch of priorities or TD errors (prb_update_wide.cu): 1 launch, or 0 if this device cannot run it (no cooperative
+// launch), or -1 on a launch error.  prb_update_is_wide: the line between it and the tree kernel.
+int prb_launch_update_wide(const PrbView& v, uint32_t B, const int32_t* d_idx, const float* d_val, int raw, float alpha, float eps,
+                           cudaStream_t s, uint32_t stale);
+bool prb_update_is_wide(const PrbView& v, uint32_t B, bool with_insertion);
 // CTAs (one cluster) of the kernel that adds b changes
 uint32_t prb_update_ctas(const PrbView& v, uint32_t b);
 int prb_launch_get_priorities(const PrbView& v, uint32_t B, const int32_t* d_idx, float* d_out, cudaStream_t s);

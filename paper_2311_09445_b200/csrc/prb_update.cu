@@ -62,6 +62,10 @@ int prb_launch_update(const PrbView& v, uint32_t B, const int32_t* d_idx, const 
                       float alpha, float eps, cudaStream_t s, uint32_t stale, bool linked)
 {
     if (raw != 2) {
+        if (prb_update_is_wide(v, B, false)) {
+            const int k = prb_launch_update_wide(v, B, d_idx, d_val, raw, alpha, eps, s, stale);
+            if (k != 0) return k;
+        }
         PrbTreeArgs t;
         t.B = B; t.idx = d_idx; t.val = d_val; t.raw = raw; t.alpha = alpha; t.eps = eps; t.stale = stale;
         if (linked && B <= kPrbTreeEntries) t.most_ctas = 4u;      // (see prb_launch_insert)

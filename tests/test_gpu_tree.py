@@ -104,3 +104,31 @@ def test_default_priorities_with_an_update(oracle_mod, K, N):
         assert pr.gpu.kernel_launches() - before == (1 if B <= 1024 else 2)
         _check(pr, False)
     pr.close()
+
+
+@pytest.mark.parametrize("min_tree", [False, True])
+@pytest.mark.parametrize("K,N,B", [(2, 90_001, 32_769), (2, 200_000, 100_000), (4, 70_000, 24_577), (8, 40_000, 33_000), (16, 100_001, 16_385), (32, 60_000, 50_000)])
+def test_very_large_updates(oracle_mod, K, N, B, min_tree):
+    # beyond the line where the batch is shared out over co-resident CTAs: repeats (the last valid entry wins), refused
+    # entries, leaves of -0.0; alone, after an insertion, and with one (one launch, or two beyond three times the line)
+    rng = np.random.default_rng(K + B)
+    pr = Pair(oracle_mod, N, K, 4, 4, 100_000, min_tree=min_tree)
+    for at in range(0, N - N // 8, 50_000):
+        b = _batch(rng, min(50_000, N - N // 8 - at), 4, 4)
+        b["prio"][rng.random(b["prio"].size) < 0.05] = -0.0
+        pr.insert(b)
+    fill = pr.gpu.info()[0]
+    for call in range(3):
+        idx = rng.integers(-1, fill + 1, size=B).astype(np.int32)
+        if call:
+            idx = np.sort(idx)
+        td = rng.standard_normal(B).astype(np.float32)
+        td[rng.random(B) < 0.02] = np.inf
+        if call == 0:
+            pr.update(idx, td, 0.6, 1e-6)
+        elif call == 1:
+            pr.update_after_insert(idx, td, 0.6, 1e-6, 100)
+        else:
+            pr.update_insert(idx, td, 0.6, 1e-6, _batch(rng, 1000, 4, 4))
+        _check(pr, min_tree)
+    pr.close()
