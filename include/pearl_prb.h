@@ -228,7 +228,7 @@ int pearl_prb_get_priorities(pearl_prb_t* prb, uint32_t B, const int32_t* d_idx,
  * update's tree work is done first, the insertion's tree work after it, by the same thread blocks,
  * while other thread blocks already copy the new rows into the Data Storage (an update touches
  * the tree only, so the two do not conflict).  Short rows: one launch (two if d_prio is NULL and the update has
- * more than 1024 entries).  Rows of 8 KB and more: the
+ * more than 2048 entries, or if the update is very large).  Rows of 8 KB and more: the
  * tree work is a kernel of its own beside the kernel that copies the rows -- on a second stream of the
  * handle when the rows come to more than 4 MB -- and the handle's stream continues when both are done
  * (capturable in a CUDA graph).  This

@@ -239,7 +239,7 @@ int prb_launch_insert(const PrbView& v, uint32_t n, const PrbBatch& src, const f
         // does not start behind the tree kernel's start (512 rows of 56 KB: 33.5 us a step the first way).
         forked = fork != nullptr && (uint64_t)tasks * stage > kForkFrom;
         tree.most_ctas = kPrbTreeBesideRows;
-        plan.tree_ctas = prb_tree_ctas(v, upd_B, n, tree.most_ctas);
+        plan.tree_ctas = prb_tree_ctas(v, upd_B, n, d_prio != nullptr, tree.most_ctas);
         if (room > 2u * kPrbTreeBesideRows) room -= kPrbTreeBesideRows;
         if (forked && (cudaEventRecord(fork->fork, s) != cudaSuccess || cudaStreamWaitEvent(fork->side, fork->fork, 0) != cudaSuccess)) return -1;
         const int k = prb_launch_tree(v, tree, forked ? fork->side : s, !forked);

@@ -190,7 +190,7 @@ struct PrbTreeArgs {
 };
 constexpr uint32_t kPrbTreeEntries = 1024;      // update entries one CTA (or cluster) takes, one per thread; more go to a grid
 constexpr uint32_t kPrbTreeBesideRows = 8;      // CTAs of the tree work beside a row copy of long rows, at most
-uint32_t prb_tree_ctas(const PrbView& v, uint32_t b, uint32_t n, uint32_t most);
+uint32_t prb_tree_ctas(const PrbView& v, uint32_t b, uint32_t n, bool prio, uint32_t most);
 // (dependent: as a programmatic dependent of the kernel before it on the stream)
 int prb_launch_tree(const PrbView& v, const PrbTreeArgs& t, cudaStream_t s, bool dependent);
 // A large batch of priorities or TD errors (prb_update_wide.cu): 1 launch, or 0 if this device cannot run it (no cooperative

@@ -666,13 +666,16 @@ constexpr uint32_t kTreeSmem = 2u * kPrbTopFloats * 4u + 2u * 2u * kGridList * 4
 // 128 / 119; fanout 32, 512 + 512 (frames) 219 / 188 / 183 / 184; us per step at fanout 16, 64 + 64 entries 12.2 /
 // 12.7 / 13.1 / 12.5, at fanout 2, 32 entries 10.9 / 11.3 / 11.7 / 11.1.  A grid beyond one entry per thread, or for an
 // insertion that one CTA would take many turns to write (before it one cooperative launch with a barrier per pass and
-// a launch for the insertion: 4096 + 16384 entries 56.6 -> 31.2 us a step, 4096 + 1024 41.0 -> 24.9).
-static bool tree_grid_form(uint32_t b, uint32_t n) { return b > kPrbTreeEntries || n > 4u * kPrbTreeEntries; }
-uint32_t prb_tree_ctas(const PrbView& v, uint32_t b, uint32_t n, uint32_t most)
+// a launch for the insertion: 4096 + 16384 entries 56.6 -> 31.2 us a step, 4096 + 1024 41.0 -> 24.9).  An insertion alone
+// dirties few groups: one CTA up to 1024 (fanout 32, 2^20 slots, 1024 5.1 -> 4.9 us; 2048 5.5 with 16, 5.6 with one), and
+// without priorities to read a cluster up to 16384 (5000 6.4 -> 5.0, 16384 6.7 -> 6.1; with priorities 5000 6.5 and 6.7, 16384
+// 6.8 and 11).
+static bool tree_grid_form(uint32_t b, uint32_t n, bool prio) { return b > kPrbTreeEntries || n > (prio ? 4u : 16u) * kPrbTreeEntries; }
+uint32_t prb_tree_ctas(const PrbView& v, uint32_t b, uint32_t n, bool prio, uint32_t most)
 {
     const uint32_t group = v.fanout == 2u ? 32u : v.fanout == 4u ? 16u : v.fanout;
     const uint64_t work = (uint64_t)group * b + 4ull * n;
-    const uint32_t want = tree_grid_form(b, n) ? 128u : work <= 2048u ? 1u : 16u;
+    const uint32_t want = tree_grid_form(b, n, prio) ? 128u : work <= (b ? 2048u : 4096u) ? 1u : 16u;
     return most && want > most ? most : want;
 }
 
@@ -704,10 +707,10 @@ int prb_launch_tree(const PrbView& v, const PrbTreeArgs& t, cudaStream_t s, bool
 {
     const int dev = prb_current_device();
     if (t.B == 0 && t.n == 0) return 0;
-    if (t.n && t.prio == nullptr && t.B > kPrbTreeEntries) {
+    if (t.n && t.prio == nullptr && t.B > 2u * kPrbTreeEntries) {
         // default priorities take the update's maximum, for which every CTA would have to transform the whole batch (see
-        // whole_max in the kernel): two launches from there on.  One launch below: fanout 16, 256 + 256 entries 8.7 -> 5.3 us,
-        // 1000 + 777 10.1 -> 7.4, 256 + 5000 11.0 -> 9.2.
+        // whole_max in the kernel): two launches from there on (4096 updates, 64 long rows: 16.3 us, 19.6 with one launch).  One launch
+        // below: fanout 16, 256 + 256 entries 8.7 -> 5.3 us, 1000 + 777 10.1 -> 7.4; 2048 updates, 256 long rows 14.7 -> 13.9.
         PrbTreeArgs u = t, w = t;
         u.n = 0;
         w.B = 0;
@@ -743,8 +746,8 @@ int prb_launch_tree(const PrbView& v, const PrbTreeArgs& t, cudaStream_t s, bool
     for (int f = 0; f < PRB_NUM_FIELDS; ++f) none.ptr[f] = nullptr;
     p.words = prb_plan_words(v, t.rows ? *t.rows : none);
     p.tiles = p.words.n_words > kPrbMostWords && !t.linked ? 1u : 0u;
-    p.grid_form = tree_grid_form(t.B, t.n) ? 1u : 0u;
-    uint32_t parts = p.T ? prb_tree_ctas(v, t.B, t.n, t.most_ctas) : 1u;      // (no staged level: nothing to split by)
+    p.grid_form = tree_grid_form(t.B, t.n, t.prio != nullptr) ? 1u : 0u;
+    uint32_t parts = p.T ? prb_tree_ctas(v, t.B, t.n, t.prio != nullptr, t.most_ctas) : 1u;      // (no staged level: nothing to split by)
     // (an insertion of longer rows alone: its copying CTAs, which take longer than the tree work, would come in clusters, too,
     // and leave SMs idle that no whole cluster fits on: 1024 rows of 14 KB 9.3 us with a cluster of 16, 6.8 with one CTA)
     if (p.tiles && t.B == 0u && !p.grid_form) parts = 1u;

@@ -85,12 +85,12 @@ def test_rows_of_many_insertions_in_a_row(oracle_mod, K, n):
 @pytest.mark.parametrize("K,N", [(2, 5000), (4, 30_000), (16, 70_001), (32, 40_000)])
 def test_default_priorities_with_an_update(oracle_mod, K, N):
     # new transitions without priorities take the running maximum, the very update's writes included, whichever CTA
-    # made them: one launch up to 1024 update entries (one CTA, a cluster, the grid of a large insertion), two beyond
+    # made them: one launch up to 2048 update entries (one CTA, a cluster, the grid), two beyond
     rng = np.random.default_rng(K)
     pr = Pair(oracle_mod, N, K, 12, 4, 5000)
     for at in range(0, N, 4000):
         pr.insert(_batch(rng, min(4000, N - at), 12, 4))
-    for step, (B, n) in enumerate([(1, 1), (40, 3), (64, 64), (256, 256), (1000, 777), (1024, 4096), (300, 4097), (1025, 20), (4000, 4900)]):
+    for step, (B, n) in enumerate([(1, 1), (40, 3), (64, 64), (256, 256), (1000, 777), (1024, 4096), (300, 4097), (1025, 20), (2048, 300), (2049, 300), (4000, 4900)]):
         idx = rng.integers(-1, N + 1, size=B).astype(np.int32)
         td = (rng.standard_normal(B) * 3.0 ** step).astype(np.float32)        # (the largest so far, somewhere in the batch)
         td[rng.random(B) < 0.05] = np.nan
@@ -101,7 +101,7 @@ def test_default_priorities_with_an_update(oracle_mod, K, N):
         before = pr.gpu.kernel_launches()
         pr.gpu.update_insert(torch.from_numpy(idx).to(pr.dev), torch.from_numpy(td).to(pr.dev), 0.6, 1e-6, d["obs"], d["act"], d["rew"],
                              d["next_obs"], d["done"], None, n=n)
-        assert pr.gpu.kernel_launches() - before == (1 if B <= 1024 else 2)
+        assert pr.gpu.kernel_launches() - before == (1 if B <= 2048 else 2)
         _check(pr, False)
     pr.close()
 
