@@ -25,7 +25,10 @@ constexpr uint32_t kTile = kWorkers * 8;     // granules per tile of short rows
 constexpr uint32_t kRowMode = 512;           // rows of at least this many 16-byte granules are split into chunks
 constexpr uint32_t kRingBytes = 198 * 1024;  // bulk-copy ring (dynamic shared memory), <= 32 stages
 constexpr uint32_t kRingBarBytes = 1024;     // room for the ring's mbarriers in front of its buffers
-constexpr uint64_t kForkFrom = 4ull << 20;   // bytes of long rows from which the tree work goes to the side stream
+// Bytes of long rows from which the tree work goes to the side stream.  Rows of 56 KB, us a call / a step with the fork and
+// without: 32 6.4 / 14.5 and 6.4 / 14.3, 128 6.5 / 15.4 and 6.6 / 15.2, 256 7.1 / 17.1 and 7.2 / 17.2, 512 9.3 / 25.6 and 12.4 / 29.6:
+// the same up to 256, and called eagerly the fork costs two events (4 rows: 18.6 -> 16.9 us a step without).
+constexpr uint64_t kForkFrom = 4ull << 20;
 
 struct InsertPlan {
     // short-row tiles, numbered field by field: tiles of field f are [first_tile[f], first_tile[f+1])

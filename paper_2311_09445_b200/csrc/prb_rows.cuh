@@ -185,8 +185,7 @@ __device__ __forceinline__ void prb_copy_tiles(const PrbWords& p, uint32_t cta, 
 }
 
 // Rows [k0, k0 + n) of the batch as units, from the store, by `nthreads` threads of which this one has rank `rank`; four loads of
-// a thread in flight (65536 rows of 165 bytes 20.9 us; with eight 4-byte loads where no granule is larger 25.9, and with the field
-// looked up again for the store instead of kept 23.5).
+// a thread in flight.
 template <typename SlotOf>
 __device__ __forceinline__ void prb_copy_units(const PrbWords& p, uint32_t rank, uint32_t nthreads, uint32_t k0, uint32_t n, SlotOf slot_of)
 {

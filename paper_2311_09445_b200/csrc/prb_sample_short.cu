@@ -14,7 +14,8 @@
 //    with p, so this is division by the batch's largest weight), one power per stratum and nothing to
 //    normalise afterwards.  p_min is exchanged while the rows are on their way.
 //  * Rows are copied word by word, a warp (or a part of one) per row: a lane's word of the row is fixed, so
-//    where it lies is looked up once and no index is divided; longer rows, and all rows of the grid, unit by unit.
+//    where it lies is looked up once and no index is divided; longer rows unit by unit, by instances of their own (with
+//    both copies in one kernel the grid's registers spilled: 65536 rows of 165 bytes 20.6 -> 28.7 us).
 //
 // Two shapes, by batch size.  Up to kClusterStrata strata: one thread-block cluster of up to 16 CTAs; p_min goes
 // through distributed shared memory (each transfer signals the receiver's barrier), nothing through global
@@ -59,7 +60,6 @@ struct ShortPlan {
     float beta;
     uint32_t uniform, buffer_norm;
     uint32_t n_steps;
-    uint32_t as_units;            // rows are copied unit by unit
     ShortStep step[kMaxSteps];
     PrbWords words;
 };
@@ -296,11 +296,12 @@ __device__ __forceinline__ uint32_t draw(const ShortPlan& plan, const ShortStep*
 }
 
 // Rows of strata [k0, k0 + n), by `warps` warps; `rank`: this thread's among them.
+template <bool kUnits>
 __device__ __forceinline__ void gather(const ShortPlan& plan, const PrbWordShare& share, uint32_t warps, uint32_t rank, uint32_t k0, uint32_t n, const uint32_t* s_idx)
 {
     auto slot_of = [&](uint32_t r) { return PRB_IN_BOUNDS(plan, s_idx[r] < plan.capacity) ? s_idx[r] : 0u; };
-    if (plan.as_units == 0u) { prb_copy_words<false>(plan.words, share, warps, k0, n, slot_of); return; }
-    prb_copy_units(plan.words, rank, warps * 32u, k0, n, slot_of);
+    if constexpr (kUnits) prb_copy_units(plan.words, rank, warps * 32u, k0, n, slot_of);
+    else prb_copy_words<false>(plan.words, share, warps, k0, n, slot_of);
 }
 
 // What a CTA stages: 16-byte unit `q` of the staged levels, taken one after another (from: nullptr beyond the last).
@@ -341,7 +342,7 @@ __device__ __forceinline__ void stage(const StagedUnit (&u)[kStagedUnits])
 // them the last CTA's division.  CTAs: 2, 4, 8 or 16 strata each measured the same within 1 %; 4.
 struct __align__(16) SmallestSeen { double log_p; unsigned long long p_bits; };
 
-template <int K>
+template <int K, bool kUnits>
 __global__ void __launch_bounds__(kShortThreads, K == 32 ? 1 : 2)
 prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
 {
@@ -409,7 +410,7 @@ prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
     }
     if (copies) {
         asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");
-        if (split) { gather(plan, share, warps - first_copier, tid - first_copier * 32u, k_lo, n, s_idx); return; }
+        if (split) { gather<kUnits>(plan, share, warps - first_copier, tid - first_copier * 32u, k_lo, n, s_idx); return; }
     }
     double log_p = 0.0;
     if (warp < strata_warps) {
@@ -428,7 +429,7 @@ prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
         }
         if (mine) plan.out_idx[k] = (int32_t)leaf;
     }
-    if (!split) gather(plan, share, warps, tid, k_lo, n, s_idx);
+    if (!split) gather<kUnits>(plan, share, warps, tid, k_lo, n, s_idx);
     // (the first warp always gets here: it keeps the CTA's shared memory until every value has come)
     if (warp >= strata_warps) return;
     if (prb_wait_first_phase<true>(plan.state, bar) == kPrbNever) return;
@@ -459,7 +460,7 @@ prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
 // Every CTA takes a contiguous range of strata, kShortThreads at a time; all its threads copy.  The smallest priority
 // is raised (complemented: the word is 0 between calls) with one atomic per CTA, and sample_ticket counts the
 // CTAs that have given theirs, then those that have read the answer.
-template <int K>
+template <int K, bool kUnits>
 __global__ void __launch_bounds__(kShortThreads, 2)
 prb_sample_grid_kernel(const __grid_constant__ ShortPlan plan)
 {
@@ -531,7 +532,7 @@ prb_sample_grid_kernel(const __grid_constant__ ShortPlan plan)
             if (exchange) atomicMax(&plan.state->wide_wmax_bits, (unsigned long long)(~s_min));
             asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&plan.state->sample_ticket) : "memory");
         }
-        gather(plan, share, warps, tid, kb, n, s_idx);
+        gather<kUnits>(plan, share, warps, tid, kb, n, s_idx);
         if (!last) __syncthreads();           // s_idx is rewritten by the next pass
     }
     if (tid == kShortThreads - 1u) {
@@ -562,27 +563,32 @@ prb_sample_grid_kernel(const __grid_constant__ ShortPlan plan)
 }
 
 using ShortKernel = void (*)(ShortPlan);
-template <bool kGrid>
-ShortKernel short_kernel(uint32_t fanout)
+template <int K>
+ShortKernel short_kernel_k(bool grid, bool units)
+{
+    if (grid) return units ? prb_sample_grid_kernel<K, true> : prb_sample_grid_kernel<K, false>;
+    return units ? prb_sample_cluster_kernel<K, true> : prb_sample_cluster_kernel<K, false>;
+}
+ShortKernel short_kernel(uint32_t fanout, bool grid, bool units)
 {
     switch (fanout) {
-    case 2: return kGrid ? prb_sample_grid_kernel<2> : prb_sample_cluster_kernel<2>;
-    case 4: return kGrid ? prb_sample_grid_kernel<4> : prb_sample_cluster_kernel<4>;
-    case 8: return kGrid ? prb_sample_grid_kernel<8> : prb_sample_cluster_kernel<8>;
-    case 16: return kGrid ? prb_sample_grid_kernel<16> : prb_sample_cluster_kernel<16>;
-    default: return kGrid ? prb_sample_grid_kernel<32> : prb_sample_cluster_kernel<32>;
+    case 2: return short_kernel_k<2>(grid, units);
+    case 4: return short_kernel_k<4>(grid, units);
+    case 8: return short_kernel_k<8>(grid, units);
+    case 16: return short_kernel_k<16>(grid, units);
+    default: return short_kernel_k<32>(grid, units);
     }
 }
 
 // What this device runs: CTAs a cluster may have (16 needs the opt-in and an SM group that holds it), and
 // co-resident CTAs of the grid form per SM.
 struct ShortLimits { uint32_t cluster, per_sm; };
-const ShortLimits* short_limits(uint32_t fanout, int ki, int dev)
+const ShortLimits* short_limits(uint32_t fanout, int ki, int dev, bool units)
 {
-    static ShortLimits cache[kPrbMaxDevices][6];
-    ShortLimits& l = cache[dev][ki];
+    static ShortLimits cache[kPrbMaxDevices][6][2];
+    ShortLimits& l = cache[dev][ki][units ? 1 : 0];
     if (l.cluster) return &l;
-    ShortKernel kc = short_kernel<false>(fanout), kg = short_kernel<true>(fanout);
+    ShortKernel kc = short_kernel(fanout, false, units), kg = short_kernel(fanout, true, units);
     uint32_t cluster = 8;
     if (cudaFuncSetAttribute(kc, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
         cudaLaunchConfig_t cfg = {};
@@ -614,7 +620,6 @@ int prb_launch_sample_short(const PrbView& v, uint32_t B, float beta, uint64_t s
                             cudaStream_t s, int uniform, int buffer_norm)
 {
     const int dev = prb_current_device();
-    const ShortLimits* lim = short_limits(v.fanout, (int)v.log2_fanout, dev);
     ShortPlan plan;
     plan.words = prb_plan_words(v, dst);
     const PrbWords& rows = plan.words;
@@ -628,8 +633,9 @@ int prb_launch_sample_short(const PrbView& v, uint32_t B, float beta, uint64_t s
     const uint64_t units = (uint64_t)B * rows.units, words = (uint64_t)B * rows.n_words;
     const bool cluster = B <= kClusterStrata && (!longer || rows.units == 0u || (rows.fine ? words <= kClusterWords : units <= kClusterUnits));
     if (!cluster && B <= kClusterStrata && !rows.fine && rows.units <= kLaneGroupUnits) return 0;
+    const bool as_units = rows.units != 0u && longer && (!cluster || !rows.fine);
+    const ShortLimits* lim = short_limits(v.fanout, (int)v.log2_fanout, dev, as_units);
     if (!cluster && lim->per_sm == 0) return 0;
-    plan.as_units = rows.units != 0u && (!cluster || (longer && !rows.fine)) ? 1u : 0u;
     plan.state = v.state;
     plan.level0 = v.level[0];
     plan.out_idx = d_idx;
@@ -682,9 +688,9 @@ int prb_launch_sample_short(const PrbView& v, uint32_t B, float beta, uint64_t s
         a[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         a[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.numAttrs = 2;
-        e = cudaLaunchKernelEx(&cfg, short_kernel<false>(v.fanout), plan);
+        e = cudaLaunchKernelEx(&cfg, short_kernel(v.fanout, false, as_units), plan);
     } else {
-        const uint32_t strata = rows.units >= 4000u ? 1u : rows.units >= 400u ? 4u : rows.units >= 100u ? 8u : kGridStrata;
+        const uint32_t strata = !as_units ? kGridStrata : rows.units >= 4000u ? 1u : rows.units >= 400u ? 4u : rows.units >= 100u ? 8u : kGridStrata;
         uint32_t grid = (B + strata - 1) / strata;
         const uint32_t room = (uint32_t)prb_sm_count() * lim->per_sm;
         if (grid > room) grid = room;
@@ -692,7 +698,7 @@ int prb_launch_sample_short(const PrbView& v, uint32_t B, float beta, uint64_t s
         a[0].id = cudaLaunchAttributeCooperative;
         a[0].val.cooperative = 1;
         cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, short_kernel<true>(v.fanout), plan);
+        e = cudaLaunchKernelEx(&cfg, short_kernel(v.fanout, true, as_units), plan);
     }
     return e == cudaSuccess ? launches : -1;
 }

@@ -56,7 +56,6 @@ struct TreePlan {
     uint32_t copies;                         // CTAs that copy rows
     uint32_t dependent;                      // launched as a programmatic dependent
     uint32_t linked;                         // the inputs lie in mapped host memory
-    uint32_t tiles;                          // rows are copied as tiles
     uint32_t off[PRB_MAX_LEVELS];            // level l starts off[l] * 64 entries behind level 0
     PrbWords words;
 };
@@ -280,7 +279,8 @@ __device__ __forceinline__ uint32_t hash_find(unsigned* key, uint32_t mask, uint
     }
 }
 
-template <int K, bool kFrames, bool kMin>
+// (kTiles: longer rows are copied as tiles; an instance of its own, so that the short rows' kernel carries none of that code)
+template <int K, bool kFrames, bool kMin, bool kTiles>
 __global__ void __launch_bounds__(kTreeThreads, 1)
 prb_tree_kernel(const __grid_constant__ TreePlan plan)
 {
@@ -302,8 +302,8 @@ prb_tree_kernel(const __grid_constant__ TreePlan plan)
         auto slot_from = [&](uint32_t first) {
             return [cursor, first, N](uint32_t r) { const uint32_t s = cursor + first + r; return s >= N ? s - N : s; };
         };
-        if (plan.linked) prb_copy_flat(plan.words, c * (nt >> 5) + (tid >> 5), plan.copies * (nt >> 5), plan.n, slot_from(0u));
-        else if (plan.tiles) prb_copy_tiles(plan.words, c, plan.copies, plan.n, slot_from(0u));
+        if constexpr (kTiles) prb_copy_tiles(plan.words, c, plan.copies, plan.n, slot_from(0u));
+        else if (plan.linked) prb_copy_flat(plan.words, c * (nt >> 5) + (tid >> 5), plan.copies * (nt >> 5), plan.n, slot_from(0u));
         else prb_copy_words<true>(plan.words, share, nt >> 5, r_lo, r_hi - r_lo, slot_from(r_lo));
         // The ticket comes last: whoever used the cursor has had its answer (the addresses it has stored to come from it), so
         // the last CTA may move it.  (Drawn first, behind one thread's read, the rows' loads waited for the cursor, which they
@@ -638,21 +638,22 @@ prb_tree_kernel(const __grid_constant__ TreePlan plan)
 }
 
 using TreeKernel = void (*)(TreePlan);
-template <int K>
+template <int K, bool kTiles>
 TreeKernel tree_kernel_k(bool frames, bool with_min)
 {
-    if (frames) return with_min ? prb_tree_kernel<K, true, true> : prb_tree_kernel<K, true, false>;
-    return with_min ? prb_tree_kernel<K, false, true> : prb_tree_kernel<K, false, false>;
+    if (frames) return with_min ? prb_tree_kernel<K, true, true, kTiles> : prb_tree_kernel<K, true, false, kTiles>;
+    return with_min ? prb_tree_kernel<K, false, true, kTiles> : prb_tree_kernel<K, false, false, kTiles>;
 }
+template <bool kTiles>
 TreeKernel tree_kernel(const PrbView& v)
 {
     const bool fr = v.stack != 0, mn = v.min_off != 0;
     switch (v.fanout) {
-    case 2: return tree_kernel_k<2>(fr, mn);
-    case 4: return tree_kernel_k<4>(fr, mn);
-    case 8: return tree_kernel_k<8>(fr, mn);
-    case 16: return tree_kernel_k<16>(fr, mn);
-    default: return tree_kernel_k<32>(fr, mn);
+    case 2: return tree_kernel_k<2, kTiles>(fr, mn);
+    case 4: return tree_kernel_k<4, kTiles>(fr, mn);
+    case 8: return tree_kernel_k<8, kTiles>(fr, mn);
+    case 16: return tree_kernel_k<16, kTiles>(fr, mn);
+    default: return tree_kernel_k<32, kTiles>(fr, mn);
     }
 }
 
@@ -661,29 +662,31 @@ constexpr uint32_t kTreeSmem = 2u * kPrbTopFloats * 4u + 2u * 2u * kGridList * 4
 }  // namespace
 
 // Which form.  One CTA while the entries' groups of a pass come to at most 2 K entries (8 KB); a cluster of 16 CTAs
-// beyond -- one SM pulls and stores scattered groups so slowly that they outlast the round trip.  us per 8 steps with
+// beyond -- one SM pulls and stores scattered groups so slowly that they outlast the round trip.  us a call in a graph, one CTA /
+// 16: fanout 16, 48 + 48 entries 5.25 / 5.23, 96 + 96 5.5 / 5.3, 112 + 112 5.9 / 5.4; fanout 32, 48 + 48 5.6 / 5.3, 64 + 64 5.8 /
+// 5.4; fanout 4, 112 + 112 6.8 / 6.5; fanout 2, 48 + 48 7.5 / 7.0, 64 + 64 7.7 / 7.0; called eagerly a single CTA is the
+// cheaper launch (64 + 64: below).  us per 8 steps with
 // 1 / 4 / 8 / 16 CTAs: fanout 16, 256 + 256 entries 93.3 / 83.5 / 84.0 / 80.9; fanout 2, 1000 + 777 entries 271 / 149 /
 // 128 / 119; fanout 32, 512 + 512 (frames) 219 / 188 / 183 / 184; us per step at fanout 16, 64 + 64 entries 12.2 /
 // 12.7 / 13.1 / 12.5, at fanout 2, 32 entries 10.9 / 11.3 / 11.7 / 11.1.  A grid beyond one entry per thread, or for an
 // insertion that one CTA would take many turns to write (before it one cooperative launch with a barrier per pass and
-// a launch for the insertion: 4096 + 16384 entries 56.6 -> 31.2 us a step, 4096 + 1024 41.0 -> 24.9).  An insertion alone
-// dirties few groups: one CTA up to 1024 (fanout 32, 2^20 slots, 1024 5.1 -> 4.9 us; 2048 5.5 with 16, 5.6 with one), and
-// without priorities to read a cluster up to 16384 (5000 6.4 -> 5.0, 16384 6.7 -> 6.1; with priorities 5000 6.5 and 6.7, 16384
-// 6.8 and 11).
+// a launch for the insertion: 4096 + 16384 entries 56.6 -> 31.2 us a step, 4096 + 1024 41.0 -> 24.9).  Without
+// priorities to read a cluster inserts up to 16384 (5000 6.4 -> 5.0 us, 16384 6.7 -> 6.1; with priorities 5000 6.5 and 6.7,
+// 16384 6.8 and 11).
 static bool tree_grid_form(uint32_t b, uint32_t n, bool prio) { return b > kPrbTreeEntries || n > (prio ? 4u : 16u) * kPrbTreeEntries; }
 uint32_t prb_tree_ctas(const PrbView& v, uint32_t b, uint32_t n, bool prio, uint32_t most)
 {
     const uint32_t group = v.fanout == 2u ? 32u : v.fanout == 4u ? 16u : v.fanout;
     const uint64_t work = (uint64_t)group * b + 4ull * n;
-    const uint32_t want = tree_grid_form(b, n, prio) ? 128u : work <= (b ? 2048u : 4096u) ? 1u : 16u;
+    const uint32_t want = tree_grid_form(b, n, prio) ? 128u : work <= 2048u ? 1u : 16u;
     return most && want > most ? most : want;
 }
 
 // Clusters beyond eight CTAs need the opt-in and a group of SMs that holds one.
-static bool tree_cluster_of_16(const PrbView& v, TreeKernel k, int dev)
+static bool tree_cluster_of_16(const PrbView& v, TreeKernel k, bool tiles, int dev)
 {
-    static int known[kPrbMaxDevices][6][2][2];      // 0: not asked yet, 1: yes, 2: no
-    int& y = known[dev][v.log2_fanout][v.stack ? 1 : 0][v.min_off ? 1 : 0];
+    static int known[kPrbMaxDevices][6][2][2][2];      // 0: not asked yet, 1: yes, 2: no
+    int& y = known[dev][v.log2_fanout][v.stack ? 1 : 0][v.min_off ? 1 : 0][tiles ? 1 : 0];
     if (y == 0) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(16);
@@ -718,7 +721,6 @@ int prb_launch_tree(const PrbView& v, const PrbTreeArgs& t, cudaStream_t s, bool
         const int b = a < 0 ? -1 : prb_launch_tree(v, w, s, dependent);
         return b < 0 ? -1 : a + b;
     }
-    const TreeKernel k = tree_kernel(v);
     TreePlan p;
     p.state = v.state;
     p.level0 = v.level[0];
@@ -745,12 +747,13 @@ int prb_launch_tree(const PrbView& v, const PrbTreeArgs& t, cudaStream_t s, bool
     PrbBatch none;
     for (int f = 0; f < PRB_NUM_FIELDS; ++f) none.ptr[f] = nullptr;
     p.words = prb_plan_words(v, t.rows ? *t.rows : none);
-    p.tiles = p.words.n_words > kPrbMostWords && !t.linked ? 1u : 0u;
+    const bool tiles = p.words.n_words > kPrbMostWords && !t.linked;
+    const TreeKernel k = tiles ? tree_kernel<true>(v) : tree_kernel<false>(v);
     p.grid_form = tree_grid_form(t.B, t.n, t.prio != nullptr) ? 1u : 0u;
     uint32_t parts = p.T ? prb_tree_ctas(v, t.B, t.n, t.prio != nullptr, t.most_ctas) : 1u;      // (no staged level: nothing to split by)
     // (an insertion of longer rows alone: its copying CTAs, which take longer than the tree work, would come in clusters, too,
     // and leave SMs idle that no whole cluster fits on: 1024 rows of 14 KB 9.3 us with a cluster of 16, 6.8 with one CTA)
-    if (p.tiles && t.B == 0u && !p.grid_form) parts = 1u;
+    if (tiles && t.B == 0u && !p.grid_form) parts = 1u;
     p.parts = parts;
     p.list = p.grid_form ? kGridList : t.B;
     // (at least 512 places, whatever the entries: probes are a chain of shared atomics; 32 entries in 64 places took 4.7 to
@@ -760,7 +763,9 @@ int prb_launch_tree(const PrbView& v, const PrbTreeArgs& t, cudaStream_t s, bool
     while (slots < 2u * p.list) { slots *= 2u; --p.hash_shift; }
     p.hash_mask = t.B ? slots - 1u : 0u;
     if (t.B == 0) p.list = 0;
-    uint32_t threads = t.B >= 16u * kPrbTreeEntries ? kTreeThreads : kGridThreads;
+    // (grid: what a large batch costs is that every CTA looks at all of it.  fanout 16, with 1024 insertions, 512 / 1024 threads:
+    // 4096 entries 9.7 / 10.4 us a call, 8192 11.4 / 10.4, 16384 15.1 / 12.3, 49000 28.7 / 19.8)
+    uint32_t threads = t.B >= 8u * kPrbTreeEntries ? kTreeThreads : kGridThreads;
     if (!p.grid_form) {
         threads = (t.B + 31u) / 32u * 32u + (t.n < 512u ? (t.n + 31u) / 32u * 32u : 512u);
         threads = threads < 256u ? 256u : threads > kTreeThreads ? kTreeThreads : threads;
@@ -775,7 +780,7 @@ int prb_launch_tree(const PrbView& v, const PrbTreeArgs& t, cudaStream_t s, bool
     if (t.rows && t.n) {
         // a few rows' words per warp, or a tile per CTA, on the SMs the tree work leaves
         uint64_t ctas = 0;
-        if (p.tiles) {
+        if (tiles) {
             for (int f = 0; f < PRB_NUM_FIELDS; ++f) ctas += ((uint64_t)t.n * p.words.field[f].units() + kPrbTile - 1) / kPrbTile;
         } else {
             const uint64_t items = (uint64_t)t.n * p.words.chunks * p.words.lane_words / 32u, per_cta = threads / 32u * 4u;
@@ -786,11 +791,11 @@ int prb_launch_tree(const PrbView& v, const PrbTreeArgs& t, cudaStream_t s, bool
         if (ctas > room) ctas = room;
         p.copies = ctas ? (uint32_t)ctas : 1u;
     }
-    if (!p.grid_form && parts > 8u && !tree_cluster_of_16(v, k, dev)) p.parts = parts = 8u;
+    if (!p.grid_form && parts > 8u && !tree_cluster_of_16(v, k, tiles, dev)) p.parts = parts = 8u;
     const uint32_t cluster = p.grid_form ? 1u : parts;
     p.copies = p.copies ? (p.copies + cluster - 1u) / cluster * cluster : 0u;      // (whole clusters)
-    static bool ready[kPrbMaxDevices][6][2][2];
-    bool& rd = ready[dev][v.log2_fanout][v.stack ? 1 : 0][v.min_off ? 1 : 0];
+    static bool ready[kPrbMaxDevices][6][2][2][2];
+    bool& rd = ready[dev][v.log2_fanout][v.stack ? 1 : 0][v.min_off ? 1 : 0][tiles ? 1 : 0];
     if (!rd) {
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTreeSmem) != cudaSuccess) return -1;
         rd = true;
