@@ -110,6 +110,20 @@ class Pair:
             self.compare_sample(o, g)
         return o, g
 
+    def sample_streamed(self, B, beta, seed, n_sub):
+        """A streamed sample (n_sub sub-batches): the kernel with a group of lanes per stratum, whatever the rows."""
+        o = self.ora.sample(B, beta, seed, gather=self.oracle_store)
+        z = lambda *s: torch.zeros(s, dtype=torch.uint8, device=self.dev)
+        t = {"idx": torch.full((B,), -1, dtype=torch.int32, device=self.dev), "w": torch.zeros(B, dtype=torch.float32, device=self.dev),
+             "obs": z(B, self.obs_bytes), "act": z(B, self.act_bytes), "rew": torch.zeros(B, dtype=torch.float32, device=self.dev),
+             "next_obs": z(B, self.obs_bytes), "done": z(B)}
+        torch.cuda.synchronize()
+        self.gpu.sample_streamed(B, beta, seed, n_sub, t["idx"], t["w"], t["obs"], t["act"], t["rew"], t["next_obs"], t["done"])
+        torch.cuda.synchronize()
+        g = {k: v.cpu().numpy() for k, v in t.items()}
+        self.compare_sample(o, g)
+        return o, g
+
     def compare_sample(self, o, g):
         assert np.array_equal(o["idx"], g["idx"]), "sampled indices differ"
         np.testing.assert_allclose(g["w"], o["w"], rtol=W_RTOL, atol=0)

@@ -298,10 +298,28 @@ def test_sample_with_a_ragged_last_warp(oracle_mod, K, N, B):
     pr.close()
 
 
+@pytest.mark.parametrize("K,N,B,n_sub", [(2, 1 << 16, 4096, 2), (2, 5000, 5, 2), (4, 5000, 5, 3), (4, 20_000, 2001, 2), (8, 40_000, 3, 2),
+                                         (8, 40_000, 1100, 4), (16, 70_000, 3, 3), (16, 70_000, 777, 2), (32, 100_000, 3333, 4)])
+def test_lane_groups_with_a_ragged_last_warp(oracle_mod, K, N, B, n_sub):
+    # The same in the kernel whose warps hold several lane groups (prb_sample_kernel<K>), which short rows reach as the
+    # sub-batches of a streamed call only.
+    rng = np.random.default_rng(K + N + B)
+    pr = Pair(oracle_mod, N, K, 8, 4, max(B, 4096))
+    for first in range(0, N, 4096):
+        n = min(4096, N - first)
+        b = raw_fields(rng, n, 8, 4)
+        b["prio"] = rng.uniform(0.01, 1, n).astype(np.float32)
+        pr.insert(b)
+    for _ in range(3):
+        pr.sample_streamed(B, 0.4, 3, n_sub)
+    pr.compare_status()
+    pr.close()
+
+
 @pytest.mark.parametrize("K", FANOUTS)
 @pytest.mark.parametrize("B", [2048, 4099, 20_000])
 def test_large_batch_sample_cases(oracle_mod, K, B):
-    # Large batches of short rows take the one-stratum-per-thread kernel: most leaves zero, the rest
+    # Large batches of short rows run as a grid, a thread per stratum: most leaves zero, the rest
     # spread over many orders of magnitude (prefix sums that round), every beta, weights optional.
     rng = np.random.default_rng(K * 31 + B)
     N = 50_000
@@ -327,11 +345,11 @@ def test_large_batch_sample_cases(oracle_mod, K, B):
 
 
 @pytest.mark.parametrize("K,D,lift,B", [
-    # a lane group per stratum (prb_sample_kernel<K>): the group falls off in a staged level, in a level
-    # read from global memory, in prefetched leaves, and at an inner level
+    # one cluster (prb_sample_cluster_kernel<K>): the walk falls off in a staged level, in a level read from global
+    # memory, in the leaves, and at an inner level
     (2, 10, 0, 1024), (2, 14, 0, 1024), (2, 9, 2, 1024), (4, 6, 1, 1024), (8, 4, 0, 1024), (16, 3, 0, 1024),
     (16, 5, 0, 1024), (16, 3, 1, 1024), (32, 3, 0, 1024), (32, 4, 0, 1024), (32, 2, 1, 512),
-    # a thread per stratum (prb_sample_wide_kernel<K>, from 2048 strata of short rows)
+    # a grid (prb_sample_grid_kernel<K>, from 1537 strata on)
     (2, 14, 0, 4096), (2, 9, 2, 2048), (4, 6, 1, 4096), (8, 4, 0, 4096), (16, 5, 0, 4096), (16, 3, 1, 65536),
     (32, 3, 0, 2048), (32, 2, 1, 4096)])
 def test_descent_falls_off_a_child_group(oracle_mod, K, D, lift, B):
@@ -355,6 +373,26 @@ def test_descent_falls_off_a_child_group(oracle_mod, K, D, lift, B):
         o, g = pr.sample(B, 0.4, seed)
         assert o["idx"][-1] == leaf
         assert pr.compare_status() == 8      # CLAMPED on both sides, nothing else
+    pr.compare_state()
+    pr.close()
+
+
+@pytest.mark.parametrize("K,D,lift,B", [(2, 10, 0, 1024), (2, 14, 0, 1024), (2, 9, 2, 1024), (4, 6, 1, 1024), (8, 4, 0, 1024), (16, 3, 0, 1024),
+                                        (16, 5, 0, 1024), (16, 3, 1, 1024), (32, 3, 0, 1024), (32, 4, 0, 1024), (32, 2, 1, 512)])
+def test_lane_group_falls_off_a_child_group(oracle_mod, K, D, lift, B):
+    # The same sliver in the kernel with a lane group per stratum (prb_sample_kernel<K>), through a streamed call: the
+    # group falls off in a staged level, in a level read from global memory, in prefetched leaves, and at an inner level.
+    p, leaf = sliver_leaves(K, D, lift)
+    N = p.shape[0]
+    rng = np.random.default_rng(K * 100 + D)
+    pr = Pair(oracle_mod, N, K, 12, 4, max(B, 4096))
+    for first in range(0, N, 4096):
+        n = min(4096, N - first)
+        pr.insert(dict(raw_fields(rng, n, 12, 4), prio=p[first:first + n]))
+    for call in range(2):
+        o, g = pr.sample_streamed(B, 0.4, seed_for_sliver(oracle_mod, B, call=call), 2)
+        assert o["idx"][-1] == leaf
+        assert pr.compare_status() == 8
     pr.compare_state()
     pr.close()
 

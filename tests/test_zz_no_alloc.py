@@ -7,9 +7,9 @@ array inside the library.  This test drives it through the C ABI on a buffer tha
 mirrors, next to the ordinary pearl_prb_sample on a second buffer with identical contents, and
 requires identical indices and gathered bytes, and weights within the suite's tolerance, against
 both, on two calls in a row (the second call finds the array as the first left it).  The cases
-cover the three shapes the call can take: a lane group per stratum with short rows, with long
-rows (the bulk-copy ring), and the largest batch it accepts, which runs as a thread per stratum
-with a second launch that reads the static array.  It is collected last so that a
+cover the three shapes the call can take: short rows in one cluster and the largest batch it accepts,
+as a grid (neither needs scratch), and long rows (a lane group per stratum and the bulk-copy ring), whose
+raw weights go through the static array.  It is collected last so that a
 stop-at-first-failure run has already run every other test.
 """
 import numpy as np
