@@ -7,9 +7,9 @@
 #include "prb_arith.cuh"
 #include "prb_wait.cuh"
 
-// The checked build (-DPEARL_CHECKED; build.py --checked): every index into a tree level, the Data Storage,
-// a batch or a staging area is compared with its extent before it is used; an index out of range raises
-// PEARL_ST_INTERNAL and the access is skipped, nothing traps.  The test suite runs against that library
+// The checked build (-DPEARL_CHECKED; build.py --checked): every index into a tree level (staged or not), the Data
+// Storage, a bulk copy's batch and stage, or a list of entries is compared with its extent before it is used; an index out of
+// range raises PEARL_ST_INTERNAL and the access is skipped or made at 0, nothing traps.  The test suite runs against that library
 // too: a bit that no test expects is a finding.  In the ordinary build the checks compile to nothing.
 #ifdef PEARL_CHECKED
 #define PRB_IN_BOUNDS(v, cond) ((cond) ? true : (atomicOr(&(v).state->status, PEARL_ST_INTERNAL), false))

@@ -62,6 +62,9 @@ struct ShortPlan {
     uint32_t n_steps;
     ShortStep step[kMaxSteps];
     PrbWords words;
+#ifdef PEARL_CHECKED
+    uint32_t entries[kMaxSteps];  // of the level a step reads, whole 16-entry groups
+#endif
 };
 
 // ---- steps of the walk -----------------------------------------------------------------------------------
@@ -224,6 +227,10 @@ __device__ __forceinline__ void walk(const ShortPlan& plan, const ShortStep* ste
         if (s + 1 < plan.n_steps) next = steps[s + 1];
         const bool many = K <= 4 && st.levels > 1u;
         const uint64_t first = (uint64_t)g << (lg * st.levels);
+#ifdef PEARL_CHECKED
+        const uint64_t beyond = first + (1ull << (lg * st.levels));
+        if (!PRB_IN_BOUNDS(plan, beyond <= plan.entries[s] && (st.top == kNotStaged || st.top + beyond <= kShortTopFloats))) { leaf = 0u; p = 1.0f; return; }
+#endif
         // (a generic address: staged level or global memory, one code path)
         row = (st.top != kNotStaged ? s_top + st.top : plan.level0 + ((uint64_t)st.off << 6)) + first;
         uint32_t j;
@@ -331,8 +338,8 @@ __device__ __forceinline__ void stage(const StagedUnit (&u)[kStagedUnits])
 }
 
 // ---- up to kClusterStrata strata: one cluster -----------------------------------------------------------------
-// The first warps of a CTA hold its strata, a thread each, and look after the weights; the others copy the rows
-// as soon as the indices are known (all do both where that would leave fewer than half of them to copy).
+// The first warps of a CTA hold its strata, a thread each, and look after the weights; the others, at least half of them,
+// copy the rows as soon as the indices are known.
 // Launched as a programmatic dependent: until the wait the kernel before it may still be running, nothing is read or
 // written, and all that depends on the arguments alone is done -- where every thread's words and staged units
 // lie, and a dry run of the arithmetic, which fetches its constants (the first use of a binary64 constant was
@@ -357,9 +364,8 @@ prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
     const uint32_t n = k_hi - k_lo, k = k_lo + tid;
     const bool mine = tid < n;
     const uint32_t strata_warps = ((plan.B + gridDim.x - 1) / gridDim.x + 31u) / 32u;      // the same in every CTA
-    const bool split = strata_warps * 2u <= warps;
-    const uint32_t first_copier = split ? strata_warps : 0u;
-    const bool copies = warp >= first_copier;
+    static_assert(kClusterStrata / 8u / 32u * 2u <= kShortThreads / 32u, "half a CTA's warps copy, whatever the cluster");
+    const bool copies = warp >= strata_warps;
     const uint32_t bar = prb_smem_addr(&s_bar);
     if (tid < plan.n_steps) s_step[tid] = plan.step[tid];
     if (tid == 0) {
@@ -368,7 +374,7 @@ prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)sizeof(SmallestSeen) * gridDim.x * strata_warps) : "memory");
     }
     PrbWordShare share = {};
-    if (copies) share = prb_word_share(plan.words, warp - first_copier, warps - first_copier);
+    if (copies) share = prb_word_share(plan.words, warp - strata_warps, warps - strata_warps);
     StagedUnit unit[kStagedUnits];
 #pragma unroll
     for (uint32_t i = 0; i < kStagedUnits; ++i) unit[i] = plan.uniform ? StagedUnit{nullptr, 0u} : staged_unit(plan, s_top, tid + i * blockDim.x);
@@ -401,22 +407,20 @@ prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
     __syncthreads();                                           // the staged levels are in place
     float p = 1.0f;
     uint32_t leaf = 0;
-    if (warp < strata_warps) {
-        unsigned flags = 0u;
-        if (mine) { leaf = draw<K, false>(plan, s_step, s_top, k, x, calls, fill, p, flags); s_idx[tid] = leaf; }
-        __syncwarp();
-        if (split) asm volatile("bar.arrive 1, %0;" ::"r"(blockDim.x) : "memory");      // the copying warps may go on
-        if (flags) atomicOr(&plan.state->status, flags);
-    }
     if (copies) {
-        asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");
-        if (split) { gather<kUnits>(plan, share, warps - first_copier, tid - first_copier * 32u, k_lo, n, s_idx); return; }
+        asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");      // the indices are there
+        gather<kUnits>(plan, share, warps - strata_warps, tid - strata_warps * 32u, k_lo, n, s_idx);
+        return;
     }
-    double log_p = 0.0;
-    if (warp < strata_warps) {
-        // the warp's smallest priority and its logarithm go to every CTA of the cluster; a transfer signals the
-        // receiver's barrier  (priorities are not negative: they order like their bits)
-        log_p = log2_of(p);
+    unsigned flags = 0u;
+    if (mine) { leaf = draw<K, false>(plan, s_step, s_top, k, x, calls, fill, p, flags); s_idx[tid] = leaf; }
+    __syncwarp();
+    asm volatile("bar.arrive 1, %0;" ::"r"(blockDim.x) : "memory");        // the copying warps may go on
+    if (flags) atomicOr(&plan.state->status, flags);
+    // the warp's smallest priority and its logarithm go to every CTA of the cluster; a transfer signals the
+    // receiver's barrier  (priorities are not negative: they order like their bits)
+    const double log_p = log2_of(p);
+    {
         const unsigned bits = mine ? __float_as_uint(p) : 0x7F800000u;
         const unsigned least = __reduce_min_sync(0xFFFFFFFFu, bits);
         const double log_least = __shfl_sync(0xFFFFFFFFu, log_p, __ffs(__ballot_sync(0xFFFFFFFFu, bits == least)) - 1);
@@ -429,9 +433,7 @@ prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
         }
         if (mine) plan.out_idx[k] = (int32_t)leaf;
     }
-    if (!split) gather<kUnits>(plan, share, warps, tid, k_lo, n, s_idx);
     // (the first warp always gets here: it keeps the CTA's shared memory until every value has come)
-    if (warp >= strata_warps) return;
     if (prb_wait_first_phase<true>(plan.state, bar) == kPrbNever) return;
     if (blockIdx.x == 0 && tid == 0) {
         plan.state->sample_calls = calls + 1;                  // (every CTA has drawn)
@@ -660,6 +662,9 @@ int prb_launch_sample_short(const PrbView& v, uint32_t B, float beta, uint64_t s
         st.levels = h;
         // whole 16-entry groups (a level's end is padded with zeros to a 256-byte boundary)
         const uint32_t entries = (v.level_alloc[l] + 15u) / 16u * 16u;
+#ifdef PEARL_CHECKED
+        plan.entries[n - 1] = entries;
+#endif
         staging = staging && entries <= kShortTopFloats && at + entries <= kShortTopFloats;
         st.top = staging ? at : kNotStaged;
         st.vec4 = staging ? entries / 4u : 0u;

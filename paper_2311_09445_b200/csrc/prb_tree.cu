@@ -157,7 +157,7 @@ __device__ __forceinline__ void resum(const TreeCtx& c, uint32_t lt, uint32_t a,
     load_entries<M>(from, e);
     if constexpr (kMin) load_entries<M>(child == c.plan.depth ? from : from + c.plan.min_off, m);
     climb<K, H, 0, kMin>(c, child, a, e, m);
-    if (staged) {
+    if (staged && PRB_IN_BOUNDS(c.plan, c.top_at(lt) + a < c.plan.top_floats)) {
         const uint32_t at = c.top_at(lt) + a;
         if (c.plan.parts == 1u) {
             c.top[at] = e[0];
@@ -202,6 +202,7 @@ template <int K, int H>
 __device__ __forceinline__ void top_block(float* top, const TreeCtx& c, uint32_t child, uint32_t i, uint64_t min_off)
 {
     constexpr int M = ipow(K, H);
+    if (!PRB_IN_BOUNDS(c.plan, c.top_at(child) + (i + 1u) * M <= c.plan.top_floats)) return;
     float e[M];
     const float* from = top + c.top_at(child) + i * M;
     if constexpr (M == 2) {
@@ -300,7 +301,10 @@ prb_tree_kernel(const __grid_constant__ TreePlan plan)
         const uint32_t cursor = (uint32_t)__ldcg(&plan.state->row_cursor), N = plan.capacity;
         const uint32_t r_lo = (uint32_t)(((uint64_t)c * plan.n) / plan.copies), r_hi = (uint32_t)(((uint64_t)(c + 1) * plan.n) / plan.copies);
         auto slot_from = [&](uint32_t first) {
-            return [cursor, first, N](uint32_t r) { const uint32_t s = cursor + first + r; return s >= N ? s - N : s; };
+            return [&plan, cursor, first, N](uint32_t r) {
+                const uint32_t s = cursor + first + r, slot = s >= N ? s - N : s;
+                return PRB_IN_BOUNDS(plan, slot < N && first + r < plan.n) ? slot : 0u;
+            };
         };
         if constexpr (kTiles) prb_copy_tiles(plan.words, c, plan.copies, plan.n, slot_from(0u));
         else if (plan.linked) prb_copy_flat(plan.words, c * (nt >> 5) + (tid >> 5), plan.copies * (nt >> 5), plan.n, slot_from(0u));
@@ -453,7 +457,7 @@ prb_tree_kernel(const __grid_constant__ TreePlan plan)
             uint32_t base = 0;
             if (who && (tid & 31u) == 0u) base = atomicAdd(&s_count, (unsigned)__popc(who));
             base = __shfl_sync(0xFFFFFFFFu, base, 0) + __popc(who & ((1u << (tid & 31u)) - 1u));
-            if (take) { l_idx[base] = (uint32_t)i0; l_pos[base] = tid; l_val[base] = v0; }
+            if (take && PRB_IN_BOUNDS(plan, base < plan.list)) { l_idx[base] = (uint32_t)i0; l_pos[base] = tid; l_val[base] = v0; }
             __syncthreads();
             valid = take = tid < s_count;
             if (take) { my_i = l_idx[tid]; my_b = l_pos[tid]; v0 = l_val[tid]; }
@@ -537,7 +541,7 @@ prb_tree_kernel(const __grid_constant__ TreePlan plan)
                     uint32_t base = 0;
                     if (who && lane == 0u) base = atomicAdd(&s_count, (unsigned)__popc(who));
                     base = __shfl_sync(0xFFFFFFFFu, base, 0) + __popc(who & ((1u << lane) - 1u));
-                    if ((take >> u) & 1u) { l_idx[base] = (uint32_t)cur[u]; l_pos[base] = b0 + tid + u * nt; }
+                    if (((take >> u) & 1u) && PRB_IN_BOUNDS(plan, base < plan.list)) { l_idx[base] = (uint32_t)cur[u]; l_pos[base] = b0 + tid + u * nt; }
                 }
                 __syncthreads();
             }
