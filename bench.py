@@ -552,7 +552,8 @@ def run_ours(args, wl, rank, world):
                          "value_from": "median" if len(m["region_ms"]) > 1 else "the one region"},
         "rates": rates,
         "roofline": {"kernel": "prb_gather_rows_kernel (+ prb_descend_kernel beside the copy before it)" if long_rows and not args.no_graph
-                     else ("prb_sample_kernel" if long_rows else "prb_sample_cluster_kernel"),
+                     else "prb_sample_kernel" if long_rows or wl.frame_stack
+                     else "prb_sample_cluster_kernel" if B <= 1536 else "prb_sample_grid_kernel",
                      "bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "peak_kind": "%s copy bandwidth" % peak_kind,
                      "frac_of_8TBs_nominal": achieved / 8000.0, "bytes_per_launch": sample_bytes,

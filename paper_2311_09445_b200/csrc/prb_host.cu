@@ -1,6 +1,6 @@
 // Host side of libpearl_prb: handle, device-memory layout, argument checks and the C ABI.
-// Every step of the replay path runs in the kernels of prb_insert.cu / prb_sample.cu /
-// prb_update.cu; this file only places memory and enqueues.
+// Every step of the replay path runs in the kernels of prb_tree.cu, prb_insert.cu, prb_update.cu, prb_update_wide.cu,
+// prb_sample.cu and prb_sample_short.cu; this file only places memory and enqueues.
 #include <math.h>
 #include <new>
 #include <stdlib.h>
