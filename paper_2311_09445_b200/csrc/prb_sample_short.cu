@@ -338,8 +338,8 @@ __device__ __forceinline__ void stage(const StagedUnit (&u)[kStagedUnits])
 }
 
 // ---- up to kClusterStrata strata: one cluster -----------------------------------------------------------------
-// The first warps of a CTA hold its strata, a thread each, and look after the weights; the others, at least half of them,
-// copy the rows as soon as the indices are known.
+// The first warps of a CTA hold its strata, a thread each, and look after the weights; the others copy the rows
+// as soon as the indices are known (all do both where that would leave fewer than half of them to copy).
 // Launched as a programmatic dependent: until the wait the kernel before it may still be running, nothing is read or
 // written, and all that depends on the arguments alone is done -- where every thread's words and staged units
 // lie, and a dry run of the arithmetic, which fetches its constants (the first use of a binary64 constant was
@@ -364,8 +364,9 @@ prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
     const uint32_t n = k_hi - k_lo, k = k_lo + tid;
     const bool mine = tid < n;
     const uint32_t strata_warps = ((plan.B + gridDim.x - 1) / gridDim.x + 31u) / 32u;      // the same in every CTA
-    static_assert(kClusterStrata / 8u / 32u * 2u <= kShortThreads / 32u, "half a CTA's warps copy, whatever the cluster");
-    const bool copies = warp >= strata_warps;
+    const bool split = strata_warps * 2u <= warps;
+    const uint32_t first_copier = split ? strata_warps : 0u;
+    const bool copies = warp >= first_copier;
     const uint32_t bar = prb_smem_addr(&s_bar);
     if (tid < plan.n_steps) s_step[tid] = plan.step[tid];
     if (tid == 0) {
@@ -374,7 +375,7 @@ prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)sizeof(SmallestSeen) * gridDim.x * strata_warps) : "memory");
     }
     PrbWordShare share = {};
-    if (copies) share = prb_word_share(plan.words, warp - strata_warps, warps - strata_warps);
+    if (copies) share = prb_word_share(plan.words, warp - first_copier, warps - first_copier);
     StagedUnit unit[kStagedUnits];
 #pragma unroll
     for (uint32_t i = 0; i < kStagedUnits; ++i) unit[i] = plan.uniform ? StagedUnit{nullptr, 0u} : staged_unit(plan, s_top, tid + i * blockDim.x);
@@ -407,20 +408,22 @@ prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
     __syncthreads();                                           // the staged levels are in place
     float p = 1.0f;
     uint32_t leaf = 0;
-    if (copies) {
-        asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");      // the indices are there
-        gather<kUnits>(plan, share, warps - strata_warps, tid - strata_warps * 32u, k_lo, n, s_idx);
-        return;
+    if (warp < strata_warps) {
+        unsigned flags = 0u;
+        if (mine) { leaf = draw<K, false>(plan, s_step, s_top, k, x, calls, fill, p, flags); s_idx[tid] = leaf; }
+        __syncwarp();
+        if (split) asm volatile("bar.arrive 1, %0;" ::"r"(blockDim.x) : "memory");      // the copying warps may go on
+        if (flags) atomicOr(&plan.state->status, flags);
     }
-    unsigned flags = 0u;
-    if (mine) { leaf = draw<K, false>(plan, s_step, s_top, k, x, calls, fill, p, flags); s_idx[tid] = leaf; }
-    __syncwarp();
-    asm volatile("bar.arrive 1, %0;" ::"r"(blockDim.x) : "memory");        // the copying warps may go on
-    if (flags) atomicOr(&plan.state->status, flags);
-    // the warp's smallest priority and its logarithm go to every CTA of the cluster; a transfer signals the
-    // receiver's barrier  (priorities are not negative: they order like their bits)
-    const double log_p = log2_of(p);
-    {
+    if (copies) {
+        asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");
+        if (split) { gather<kUnits>(plan, share, warps - first_copier, tid - first_copier * 32u, k_lo, n, s_idx); return; }
+    }
+    double log_p = 0.0;
+    if (warp < strata_warps) {
+        // the warp's smallest priority and its logarithm go to every CTA of the cluster; a transfer signals the
+        // receiver's barrier  (priorities are not negative: they order like their bits)
+        log_p = log2_of(p);
         const unsigned bits = mine ? __float_as_uint(p) : 0x7F800000u;
         const unsigned least = __reduce_min_sync(0xFFFFFFFFu, bits);
         const double log_least = __shfl_sync(0xFFFFFFFFu, log_p, __ffs(__ballot_sync(0xFFFFFFFFu, bits == least)) - 1);
@@ -433,7 +436,9 @@ prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
         }
         if (mine) plan.out_idx[k] = (int32_t)leaf;
     }
+    if (!split) gather<kUnits>(plan, share, warps, tid, k_lo, n, s_idx);
     // (the first warp always gets here: it keeps the CTA's shared memory until every value has come)
+    if (warp >= strata_warps) return;
     if (prb_wait_first_phase<true>(plan.state, bar) == kPrbNever) return;
     if (blockIdx.x == 0 && tid == 0) {
         plan.state->sample_calls = calls + 1;                  // (every CTA has drawn)
