@@ -9,7 +9,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libpearl_prb.so")
 LIB_CHECKED = os.path.join(HERE, "libpearl_prb_checked.so")     # every index checked against its extent (-DPEARL_CHECKED)
-SOURCES = ["prb_host.cu", "prb_insert.cu", "prb_sample.cu", "prb_sample_short.cu", "prb_tree.cu", "prb_update.cu", "prb_update_wide.cu"]
+SOURCES = ["prb_host.cu", "prb_insert.cu", "prb_sample.cu", "prb_sample_short.cu", "prb_step.cu", "prb_tree.cu", "prb_update.cu", "prb_update_wide.cu"]
 
 NVCC_FLAGS = [
     "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",

@@ -23,6 +23,15 @@ __device__ __forceinline__ uint32_t philox4x32_10_word0(uint32_t c0, uint32_t c1
     return c0;
 }
 
+// a / b rounded to nearest, from y = 1 / b rounded to nearest: one correction of a y by its exact remainder gives the correctly rounded
+// quotient (P. W. Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", IBM J. Res. Dev. 34 (1990),
+// theorem 8.3; no overflow or underflow here: a is a binary32 sum, b a batch size).  Three dependent operations where y is known ahead.
+__device__ __forceinline__ double prb_quotient(double a, double b, double y)
+{
+    const double q = __dmul_rn(a, y);
+    return __fma_rn(__fma_rn(-q, b, a), y, q);
+}
+
 // Eq. 1's target of stratum k of B (one draw per equal segment of [0, total), Schaul et al.):
 // x_k = (k + u_k) * (total / B) in binary64, two rounded operations, clamped to the binary64 just below
 // total; u_k = word 0 of Philox4x32-10(counter = (k, 0, call_lo, call_hi), key = (seed_lo, seed_hi)) * 2^-32.

@@ -624,19 +624,64 @@ int pearl_prb_update_insert(pearl_prb_t* h, uint32_t B, const int32_t* d_idx, co
     return PEARL_OK;
 }
 
+// The iteration in one launch (prb_step.cu), where it takes it: short rows, a batch that a cluster takes, and no array that is read
+// overlapping one that is written -- sampled rows may be read from the insertion's batch while others are written already.
+// (The update's indices may be the very array that the sampled ones go to: every CTA has read them before any is written.)
+static constexpr int PEARL_STEP_IN_PARTS = 1;
+static int step_in_one(pearl_prb_t* h, uint32_t B_upd, const int32_t* d_upd_idx, const float* d_td, float alpha, float eps, uint32_t n,
+                       const void* const in[PRB_NUM_FIELDS], const float* d_new_prio, uint32_t B, float beta, uint64_t seed, int32_t* d_idx,
+                       float* d_w, void* const out[PRB_NUM_FIELDS])
+{
+    if (h->view.stack || h->view.min_off || (n && !d_new_prio)) return PEARL_STEP_IN_PARTS;
+    struct Range { uintptr_t at, end; };
+    Range reads[PRB_NUM_FIELDS + 3], writes[PRB_NUM_FIELDS + 2];
+    uint32_t nr = 0, nw = 0;
+    auto add = [](Range* to, uint32_t& count, const void* p, uint64_t bytes) { if (p && bytes) to[count++] = Range{(uintptr_t)p, (uintptr_t)p + bytes}; };
+    for (int f = 0; f < PRB_NUM_FIELDS; ++f) {
+        add(reads, nr, in[f], (uint64_t)n * h->view.field_bytes[f]);
+        add(writes, nw, out[f], (uint64_t)B * h->lay.out_bytes[f]);
+    }
+    add(reads, nr, d_new_prio, (uint64_t)n * 4);
+    add(reads, nr, d_td, (uint64_t)B_upd * 4);
+    add(reads, nr, d_upd_idx, (uint64_t)B_upd * 4);
+    const uint32_t upd = nr - 1u;
+    add(writes, nw, d_w, (uint64_t)B * 4);
+    add(writes, nw, d_idx, (uint64_t)B * 4);
+    for (uint32_t r = 0; r < nr; ++r)
+        for (uint32_t w = 0; w < nw; ++w)
+            if (reads[r].at < writes[w].end && writes[w].at < reads[r].end && !(r == upd && w == nw - 1u && reads[r].at == writes[w].at)) return PEARL_STEP_IN_PARTS;
+    DeviceGuard guard(h->device);
+    if (!guard.ok) return PEARL_ERR_CUDA;
+    PrbBatch src;
+    PrbSampleArgs sample;
+    for (int f = 0; f < PRB_NUM_FIELDS; ++f) { src.ptr[f] = n ? (unsigned char*)in[f] : nullptr; sample.dst.ptr[f] = (unsigned char*)out[f]; }
+    PrbTreeArgs t;
+    t.B = B_upd; t.idx = d_upd_idx; t.val = d_td; t.alpha = alpha; t.eps = eps;
+    t.n = n; t.prio = d_new_prio; t.rows = &src; t.linked = h->linked_inputs;
+    sample.B = B; sample.beta = beta; sample.seed = seed; sample.idx = d_idx; sample.w = d_w;
+    const int k = prb_launch_step(h->view, t, &sample, h->stream);
+    if (k == 0) return PEARL_STEP_IN_PARTS;
+    if (k < 0) return PEARL_ERR_CUDA;
+    h->launches += (uint64_t)k;
+    h->main_touched = true; h->main_last_gather = 0; h->after_rows = false;
+    return PEARL_OK;
+}
+
 int pearl_prb_step(pearl_prb_t* h, uint32_t B_upd, const int32_t* d_upd_idx, const float* d_td, float alpha, float eps,
                    uint32_t n, const void* d_new_obs, const void* d_new_act, const float* d_new_rew, const void* d_new_next_obs,
                    const uint8_t* d_new_done, const float* d_new_prio, uint32_t B, float beta, uint64_t seed, int32_t* d_idx,
                    float* d_w, void* d_obs, void* d_act, float* d_rew, void* d_next_obs, uint8_t* d_done)
 {
     const void* in[PRB_NUM_FIELDS] = { d_new_obs, d_new_next_obs, d_new_act, d_new_rew, d_new_done };
-    const void* out[PRB_NUM_FIELDS] = { d_obs, d_next_obs, d_act, d_rew, d_done };
+    void* out[PRB_NUM_FIELDS] = { d_obs, d_next_obs, d_act, d_rew, d_done };
     // (n == 0: an iteration without new transitions -- update, then sample)
     int rc = check_update_insert_args(h, B_upd, d_upd_idx, d_td, alpha, eps, n ? n : 1u, in, d_new_prio);
     if (rc != PEARL_OK) return rc;
     rc = check_sample_args(h, B, beta, d_idx, d_w, out);
     if (rc != PEARL_OK) return rc;
     // (both calls' arguments have been checked: nothing is enqueued unless both go through)
+    rc = step_in_one(h, B_upd, d_upd_idx, d_td, alpha, eps, n, in, d_new_prio, B, beta, seed, d_idx, d_w, out);
+    if (rc != PEARL_STEP_IN_PARTS) return rc;
     rc = n ? pearl_prb_update_insert(h, B_upd, d_upd_idx, d_td, alpha, eps, n, d_new_obs, d_new_act, d_new_rew, d_new_next_obs,
                                      d_new_done, d_new_prio)
            : pearl_prb_update(h, B_upd, d_upd_idx, d_td, alpha, eps);

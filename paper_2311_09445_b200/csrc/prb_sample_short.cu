@@ -21,7 +21,7 @@
 // through distributed shared memory (each transfer signals the receiver's barrier), nothing through global
 // memory.  More: a cooperative grid; p_min by an atomic per CTA, and a CTA waits (bounded) for the others only
 // after its rows are copied.
-#include "prb_descend.cuh"
+#include "prb_walk.cuh"
 #include "prb_rows.cuh"
 
 namespace {
@@ -32,7 +32,7 @@ constexpr uint32_t kMaxSteps = 16;
 constexpr uint32_t kMaxCluster = 16;
 // Batches of at most this many strata run as one cluster: three warps of strata per CTA.  (The grid form costs a
 // cooperative launch, no programmatic one, and a round through global memory for the smallest priority.)
-constexpr uint32_t kClusterStrata = 1536;
+constexpr uint32_t kClusterStrata = kPrbClusterStrata;
 constexpr uint32_t kMaxSeen = 64;                    // strata warps of a cluster: 8 CTAs x 6 warps, 16 x 3
 constexpr uint32_t kGridStrata = 32;                 // strata per CTA of the cooperative grid, at least (fewer where rows are long)
 constexpr uint32_t kClusterUnits = 1u << 16;         // a cluster copies at most this many units ...
@@ -67,152 +67,6 @@ struct ShortPlan {
 #endif
 };
 
-// ---- steps of the walk -----------------------------------------------------------------------------------
-// (the child entered is the first whose prefix exceeds the target; a target that has passed every prefix --
-// possible by binary32 rounding only -- takes the last positive child and raises CLAMPED)
-
-// kWide (many strata per SM): prefixes are compared in binary32 with the largest binary32 not above the target --
-// the same answer, and one conversion of the target in place of one per prefix, whose rate bounds the walk there;
-// otherwise in binary64, whose conversions are off the chain that bounds a small batch.
-template <bool kWide>
-struct Target {
-    double x;
-    float below;
-    __device__ __forceinline__ explicit Target(double t) : x(t), below(0.0f) { if (kWide) below = __double2float_rd(t); }
-    __device__ __forceinline__ bool past(float prefix) const { return kWide ? prefix <= below : x >= (double)prefix; }
-};
-
-// Fanout 2: children c0, c1.
-template <bool kWide>
-__device__ __forceinline__ bool pick2(double& x, float c0, float c1, unsigned& flags)
-{
-    const Target<kWide> t(x);
-    const bool past0 = t.past(c0), past1 = t.past(__fadd_rn(c0, c1));
-    const bool right = past0 && !(past1 && !(c1 > 0.0f));
-    if (past1) flags |= (c0 > 0.0f || c1 > 0.0f) ? PEARL_ST_CLAMPED : (PEARL_ST_CLAMPED | PEARL_ST_INTERNAL);
-    if (right) x = __dsub_rn(x, (double)c0);
-    return right;
-}
-
-// Fanout 4.
-template <bool kWide>
-__device__ __forceinline__ uint32_t pick4(double& x, const float (&c)[4], unsigned& flags)
-{
-    const float a1 = __fadd_rn(c[0], c[1]), a2 = __fadd_rn(a1, c[2]), a3 = __fadd_rn(a2, c[3]);
-    const Target<kWide> t(x);
-    uint32_t j = (t.past(c[0]) ? 1u : 0u) + (t.past(a1) ? 1u : 0u) + (t.past(a2) ? 1u : 0u) + (t.past(a3) ? 1u : 0u);
-    if (j == 4u) {
-        j = c[3] > 0.0f ? 3u : c[2] > 0.0f ? 2u : c[1] > 0.0f ? 1u : 0u;
-        flags |= (j > 0u || c[0] > 0.0f) ? PEARL_ST_CLAMPED : (PEARL_ST_CLAMPED | PEARL_ST_INTERNAL);
-    }
-    if (j > 0u) x = __dsub_rn(x, (double)(j == 1u ? c[0] : j == 2u ? a1 : a2));
-    return j;
-}
-
-// The 16 entries four levels (fanout 2) or two levels (fanout 4) below a node.
-template <int K, bool kWide>
-__device__ __forceinline__ uint32_t step16(const float* row, double& x, float& chosen, unsigned& flags)
-{
-    float e[16];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const float4 t = reinterpret_cast<const float4*>(row)[q];
-        e[4 * q] = t.x; e[4 * q + 1] = t.y; e[4 * q + 2] = t.z; e[4 * q + 3] = t.w;
-    }
-    if constexpr (K == 2) {
-        float p8[8], p4[4];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) p8[i] = __fadd_rn(e[2 * i], e[2 * i + 1]);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) p4[i] = __fadd_rn(p8[2 * i], p8[2 * i + 1]);
-        const bool r0 = pick2<kWide>(x, __fadd_rn(p4[0], p4[1]), __fadd_rn(p4[2], p4[3]), flags);
-        const float a0 = r0 ? p4[2] : p4[0], a1 = r0 ? p4[3] : p4[1];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) p8[i] = r0 ? p8[4 + i] : p8[i];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) e[i] = r0 ? e[8 + i] : e[i];
-        const bool r1 = pick2<kWide>(x, a0, a1, flags);
-        const float b0 = r1 ? p8[2] : p8[0], b1 = r1 ? p8[3] : p8[1];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) e[i] = r1 ? e[4 + i] : e[i];
-        const bool r2 = pick2<kWide>(x, b0, b1, flags);
-        const float d0 = r2 ? e[2] : e[0], d1 = r2 ? e[3] : e[1];
-        const bool r3 = pick2<kWide>(x, d0, d1, flags);
-        chosen = r3 ? d1 : d0;
-        return (r0 ? 8u : 0u) + (r1 ? 4u : 0u) + (r2 ? 2u : 0u) + (r3 ? 1u : 0u);
-    } else {
-        float s[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) s[i] = __fadd_rn(__fadd_rn(__fadd_rn(e[4 * i], e[4 * i + 1]), e[4 * i + 2]), e[4 * i + 3]);
-        const uint32_t j = pick4<kWide>(x, s, flags);
-        float c[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) c[i] = j == 0u ? e[i] : j == 1u ? e[4 + i] : j == 2u ? e[8 + i] : e[12 + i];
-        const uint32_t j2 = pick4<kWide>(x, c, flags);
-        chosen = j2 == 0u ? c[0] : j2 == 1u ? c[1] : j2 == 2u ? c[2] : c[3];
-        return 4u * j + j2;
-    }
-}
-
-// One level: the K children of a node.  (From fanout 8 on the chosen child's value is left to the caller.)
-template <int K, bool kWide>
-__device__ __forceinline__ uint32_t step1(const float* row, double& x, float& chosen, unsigned& flags)
-{
-    if constexpr (K == 2) {
-        const float2 c = *reinterpret_cast<const float2*>(row);
-        const bool r = pick2<kWide>(x, c.x, c.y, flags);
-        chosen = r ? c.y : c.x;
-        return r ? 1u : 0u;
-    } else if constexpr (K == 4) {
-        const float4 t = *reinterpret_cast<const float4*>(row);
-        const float c[4] = { t.x, t.y, t.z, t.w };
-        const uint32_t j = pick4<kWide>(x, c, flags);
-        chosen = j == 0u ? c[0] : j == 1u ? c[1] : j == 2u ? c[2] : c[3];
-        return j;
-    } else {
-        // prefix <= x, a binary32 against a binary64, is prefix <= (the largest binary32 not above x).
-        // All prefixes first (one chain of additions), then the comparisons as masks, not predicates: counted
-        // for the child's number, and the largest prefix passed picked out of them: as signed integers, whose
-        // order is that of the values and which put -0.0 (a priority that is accepted; only the prefixes before the
-        // first positive child can be it) below every prefix not passed, so that +0.0 is subtracted then.
-        const float xf = __double2float_rd(x);
-        float r[K];
-#pragma unroll
-        for (int q = 0; q < K / 4; ++q) {
-            const float4 t = reinterpret_cast<const float4*>(row)[q];
-            r[4 * q] = t.x; r[4 * q + 1] = t.y; r[4 * q + 2] = t.z; r[4 * q + 3] = t.w;
-        }
-#pragma unroll
-        for (int i = 1; i < K; ++i) r[i] = __fadd_rn(r[i - 1], r[i]);
-        uint32_t cnt[K];
-        int top[K];
-#pragma unroll
-        for (int i = 0; i < K; ++i) {
-            asm("set.le.u32.f32 %0, %1, %2;" : "=r"(cnt[i]) : "f"(r[i]), "f"(xf));      // (all ones where passed)
-            top[i] = (int)cnt[i] & __float_as_int(r[i]);
-        }
-#pragma unroll
-        for (int h = K / 2; h > 0; h /= 2) {
-#pragma unroll
-            for (int i = 0; i < h; ++i) { cnt[i] += cnt[i + h]; top[i] = max(top[i], top[i + h]); }
-        }
-        uint32_t j = 0u - cnt[0];
-        int before = top[0];
-        if (j == (uint32_t)K) {
-            flags |= PEARL_ST_CLAMPED;
-            while (j > 0u && !(row[j - 1u] > 0.0f)) --j;
-            if (j > 0u) --j;
-            else flags |= PEARL_ST_INTERNAL;
-            float run = 0.0f;
-#pragma unroll 1
-            for (uint32_t i = 0; i < j; ++i) run = i ? __fadd_rn(run, row[i]) : row[0];
-            before = __float_as_int(run);
-        }
-        x = __dsub_rn(x, (double)__int_as_float(before));              // (0 in front of the first child)
-        return j;
-    }
-}
-
 template <int K, bool kWide>
 __device__ __forceinline__ void walk(const ShortPlan& plan, const ShortStep* steps, const float* s_top, double x, uint32_t& leaf, float& p, unsigned& flags)
 {
@@ -234,8 +88,8 @@ __device__ __forceinline__ void walk(const ShortPlan& plan, const ShortStep* ste
         // (a generic address: staged level or global memory, one code path)
         row = (st.top != kNotStaged ? s_top + st.top : plan.level0 + ((uint64_t)st.off << 6)) + first;
         uint32_t j;
-        if (many) { if constexpr (K <= 4) j = step16<K, kWide>(row, x, chosen, flags); }
-        else j = step1<K, kWide>(row, x, chosen, flags);
+        if (many) { if constexpr (K <= 4) j = step16<K, kWide>(PrbRowAt{row}, x, chosen, flags); }
+        else j = step1<K, kWide, false>(PrbRowAt{row}, x, chosen, flags);
         if (K > 4) row += j;
         g = (uint32_t)first + j;
     }
@@ -244,42 +98,6 @@ __device__ __forceinline__ void walk(const ShortPlan& plan, const ShortStep* ste
 }
 
 // ---- weights -----------------------------------------------------------------------------------------------
-// log2 of a positive binary32, in binary64: p = m 2^E with m in (sqrt(1/2), sqrt(2)], t = (m-1)/(m+1),
-// ln m = 2 t (1 + t^2/3 + t^4/5 + ...); |t| < 0.172, so the terms left out are below 2^-53 of the sum.
-__device__ __forceinline__ double log2_of(float p)
-{
-    const long long bits = __double_as_longlong((double)p);
-    int E = (int)(bits >> 52) - 1023;
-    double m = __longlong_as_double((bits & 0x000FFFFFFFFFFFFFll) | 0x3FF0000000000000ll);
-    if (m > 1.4142135623730951) { m *= 0.5; E += 1; }
-    const double t = __ddiv_rn(m - 1.0, m + 1.0), t2 = t * t, t4 = t2 * t2;
-    // (two chains, in t^4: even and odd terms)
-    double a = 1.0 / 17.0, b = 1.0 / 19.0;
-    a = __fma_rn(a, t4, 1.0 / 13.0); b = __fma_rn(b, t4, 1.0 / 15.0);
-    a = __fma_rn(a, t4, 1.0 / 9.0);  b = __fma_rn(b, t4, 1.0 / 11.0);
-    a = __fma_rn(a, t4, 1.0 / 5.0);  b = __fma_rn(b, t4, 1.0 / 7.0);
-    a = __fma_rn(a, t4, 1.0);        b = __fma_rn(b, t4, 1.0 / 3.0);
-    const double S = __fma_rn(b, t2, a);
-    return __fma_rn(2.0 * 1.4426950408889634 * t, S, (double)E);
-}
-
-// 2^z for z <= 0, rounded to binary32: k = rint(z), 2^z = 2^k e^r with r = (z - k) ln 2 (|r| < 0.35), the
-// exponential's series to r^13.  (Below 2^-200 the binary32 is 0 anyway.)
-__device__ __forceinline__ float exp2_of(double z)
-{
-    if (!(z > -200.0)) return 0.0f;
-    const double k = rint(z), r = (z - k) * 0.6931471805599453, r2 = r * r;
-    double a = 1.0 / 479001600.0, b = 1.0 / 6227020800.0;                                // 1/12!, 1/13!
-    a = __fma_rn(a, r2, 1.0 / 3628800.0); b = __fma_rn(b, r2, 1.0 / 39916800.0);
-    a = __fma_rn(a, r2, 1.0 / 40320.0);   b = __fma_rn(b, r2, 1.0 / 362880.0);
-    a = __fma_rn(a, r2, 1.0 / 720.0);     b = __fma_rn(b, r2, 1.0 / 5040.0);
-    a = __fma_rn(a, r2, 1.0 / 24.0);      b = __fma_rn(b, r2, 1.0 / 120.0);
-    a = __fma_rn(a, r2, 0.5);             b = __fma_rn(b, r2, 1.0 / 6.0);
-    a = __fma_rn(a, r2, 1.0);             b = __fma_rn(b, r2, 1.0);
-    const double e = __fma_rn(b, r, a);
-    return (float)(e * __longlong_as_double(((long long)k + 1023ll) << 52));
-}
-
 // (p / p_min)^-beta from the two logarithms: 1 where p is the smallest.
 // Fewer dependent operations than a general power; against 64-bit references the weights are as close as they
 // were with one (the rounding to binary32 is all there is to see).
