@@ -195,6 +195,7 @@ uint32_t prb_tree_ctas(const PrbView& v, uint32_t b, uint32_t n, bool prio, uint
 int prb_launch_tree(const PrbView& v, const PrbTreeArgs& t, cudaStream_t s, bool dependent);
 // A whole iteration of short rows in one launch (prb_step.cu): the tree work t -- with t.rows, the insertion's rows, too -- and the sample
 // of the next batch; without `sample` the tree work alone.  1, or 0 where another route has to be taken, or -1 on a launch error.
+// (dependent: as a programmatic dependent of what precedes it.)
 // (No array of t may overlap one that the sample writes, t.idx and sample->idx excepted.)
 struct PrbSampleArgs {
     uint32_t B = 0;
@@ -205,7 +206,7 @@ struct PrbSampleArgs {
     PrbBatch dst;
 };
 constexpr uint32_t kPrbClusterStrata = 1536;    // strata of a sample that one cluster takes
-int prb_launch_step(const PrbView& v, const PrbTreeArgs& t, const PrbSampleArgs* sample, cudaStream_t s);
+int prb_launch_step(const PrbView& v, const PrbTreeArgs& t, const PrbSampleArgs* sample, cudaStream_t s, bool dependent = true);
 // A large batch of priorities or TD errors (prb_update_wide.cu): 1 launch, or 0 if this device cannot run it (no cooperative
 // launch), or -1 on a launch error.  prb_update_is_wide: the line between it and the tree kernel.
 int prb_launch_update_wide(const PrbView& v, uint32_t B, const int32_t* d_idx, const float* d_val, int raw, float alpha, float eps,

@@ -58,7 +58,7 @@ struct StepPlan {
     const unsigned char* done;
     int32_t* out_idx;
     float* out_w;
-    uint64_t seed;
+    uint64_t seed, min_off;
     uint32_t capacity, depth, B_upd, n, B;
     float alpha, eps, beta;
     uint32_t raw, stale, stack;
@@ -68,7 +68,7 @@ struct StepPlan {
     uint32_t n_u, own, own4;                  // nodes of level U; of them a CTA's, at most, and in units of four
     uint32_t log_parts;
     uint32_t rows, list;                      // groups held at a time (per step); entries: positions of the batch, or capacity of the list
-    uint32_t portion_units;
+    uint32_t portion_units, portion_floats;
     uint32_t leaf_mask, leaf_shift, node_mask, node_shift;       // hash tables: places less one, 32 - log2 of the places
     uint32_t up_floats;
     // byte offsets in dynamic shared memory
@@ -98,31 +98,43 @@ struct StepCtx {
 };
 
 // The levels between a group of level `child` and its node a, kSpan levels up, and that node: summed up in registers and stored.
-template <int K, int S>
-__device__ __forceinline__ void sum_up(const StepCtx& c, uint32_t child, uint32_t a, float (&e)[kGroup<K>])
+// (kLeast: the min-tree's nodes, min_off behind the sum tree's)
+template <int K, bool kLeast, int S>
+__device__ __forceinline__ void sum_up(const StepCtx& c, uint64_t min_off, uint32_t child, uint32_t a, float (&e)[kGroup<K>])
 {
     if constexpr (S < kSpan<K>) {
         constexpr int N = ipow(K, kSpan<K> - 1 - S);
-        sum_groups<K, N>(e);
-        store_entries<N>(c.level(child - 1 - S) + (uint64_t)a * N, e);
-        sum_up<K, S + 1>(c, child, a, e);
+        if constexpr (kLeast) min_groups<K, N>(e);
+        else sum_groups<K, N>(e);
+        store_entries<N>(c.level(child - 1 - S) + min_off + (uint64_t)a * N, e);
+        sum_up<K, kLeast, S + 1>(c, min_off, child, a, e);
+    }
+}
+template <int M>
+__device__ __forceinline__ void load_group(const float* from, float (&e)[M])
+{
+#pragma unroll
+    for (int q = 0; q < M / 4; ++q) {
+        const float4 t = reinterpret_cast<const float4*>(from)[q];
+        e[4 * q] = t.x; e[4 * q + 1] = t.y; e[4 * q + 2] = t.z; e[4 * q + 3] = t.w;
     }
 }
 
 // Upper levels: node i of level l - H and what lies between, from the entries of level l (which starts at `at`) under it.
-template <int K, int H, int S>
-__device__ __forceinline__ void sum_up_top(const StepCtx& c, float* up, bool store, uint32_t l, uint32_t i, float (&e)[ipow(K, H)])
+template <int K, bool kLeast, int H, int S>
+__device__ __forceinline__ void sum_up_top(const StepCtx& c, float* up, uint64_t min_off, bool store, uint32_t l, uint32_t i, float (&e)[ipow(K, H)])
 {
     if constexpr (S < H) {
         constexpr int N = ipow(K, H - 1 - S);
-        sum_groups<K, N>(e);
+        if constexpr (kLeast) min_groups<K, N>(e);
+        else sum_groups<K, N>(e);
         store_entries<N>(up + c.plan.up[l - 1 - S] + i * N, e);
-        if (store) store_entries<N>(c.level(l - 1 - S) + (uint64_t)i * N, e);
-        sum_up_top<K, H, S + 1>(c, up, store, l, i, e);
+        if (store) store_entries<N>(c.level(l - 1 - S) + min_off + (uint64_t)i * N, e);
+        sum_up_top<K, kLeast, H, S + 1>(c, up, min_off, store, l, i, e);
     }
 }
-template <int K, int H>
-__device__ __forceinline__ void top_group(const StepCtx& c, float* up, bool store, uint32_t l, uint32_t at, uint32_t i)
+template <int K, bool kLeast, int H>
+__device__ __forceinline__ void top_group(const StepCtx& c, float* up, uint64_t min_off, bool store, uint32_t l, uint32_t at, uint32_t i)
 {
     constexpr int M = ipow(K, H);
     float e[M];
@@ -132,13 +144,9 @@ __device__ __forceinline__ void top_group(const StepCtx& c, float* up, bool stor
         const float2 t = *reinterpret_cast<const float2*>(from);
         e[0] = t.x; e[1] = t.y;
     } else {
-#pragma unroll
-        for (int q = 0; q < M / 4; ++q) {
-            const float4 t = reinterpret_cast<const float4*>(from)[q];
-            e[4 * q] = t.x; e[4 * q + 1] = t.y; e[4 * q + 2] = t.z; e[4 * q + 3] = t.w;
-        }
+        load_group<M>(from, e);
     }
-    sum_up_top<K, H, 0>(c, up, store, l, i, e);
+    sum_up_top<K, kLeast, H, 0>(c, up, min_off, store, l, i, e);
 }
 
 // Rows of the walk: a group in a peer's portion, a group in L2.
@@ -180,7 +188,7 @@ __device__ __forceinline__ uint32_t global_of(uint32_t j, uint32_t lp, uint32_t 
 // for a unit beyond the level's end, which is zeroed here instead.)
 struct PortionUnit { const float* from; uint32_t to; };
 template <int K>
-__device__ __forceinline__ PortionUnit portion_unit(const StepPlan& plan, float* portion, uint32_t rank, uint32_t q)
+__device__ __forceinline__ PortionUnit portion_unit(const StepPlan& plan, float* portion, uint64_t min_off, uint32_t rank, uint32_t q)
 {
     constexpr uint32_t lgM = kLogGroup<K>;
     PortionUnit o = PortionUnit{nullptr, 0u};
@@ -192,7 +200,7 @@ __device__ __forceinline__ PortionUnit portion_unit(const StepPlan& plan, float*
         const uint32_t stored = (prb_nodes_covering(plan.capacity, kLog2<K> * (plan.depth - l)) + 63u) & ~63u;
         float* const to = portion + plan.portion_at[s] + padded<K>(f);
         o.to = prb_smem_addr(to);
-        if (a < stored) o.from = plan.level0 + ((uint64_t)plan.off[l] << 6) + a;
+        if (a < stored) o.from = plan.level0 + min_off + ((uint64_t)plan.off[l] << 6) + a;
         else *reinterpret_cast<float4*>(to) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         break;
     }
@@ -260,9 +268,10 @@ __device__ __forceinline__ void gather_rows(const StepPlan& plan, const PrbWordS
 }
 
 // kSample: the whole iteration; otherwise the tree work (and the rows of the insertion, if they are short) alone, which only
-// CTA 0 has to see the end of.  kFrames: the frame-deduplicated layout (tree work only).  kEach: entries of the batch, and inserted leaves, per
+// CTA 0 has to see the end of.  kFrames: the frame-deduplicated layout, kMin: a buffer with a
+// min-tree, whose nodes go through the same steps as the sum tree's (both: tree work only).  kEach: entries of the batch, and inserted leaves, per
 // thread that looks at them.
-template <int K, bool kSample, bool kFrames, uint32_t kEach>
+template <int K, bool kSample, bool kFrames, bool kMin, uint32_t kEach>
 __global__ void __launch_bounds__(kStepThreads<kEach>, 1)
 prb_step_kernel(const __grid_constant__ StepPlan plan)
 {
@@ -282,6 +291,10 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
     float* const portion = reinterpret_cast<float*>(s_dyn + plan.o_portion);
     unsigned char* const dirty = s_dyn + plan.o_dirty;
     float* const rows = reinterpret_cast<float*>(s_dyn + plan.o_rows);
+    // (the min-tree's, each as far behind the sum tree's as that is long)
+    float* const up_min = up + plan.up_floats;
+    float* const own_min = s_own + plan.own4 * 4u;
+    float* const portion_min = portion + plan.portion_floats;
     unsigned* const nodes = reinterpret_cast<unsigned*>(s_dyn + plan.o_nodes);                 // per step: keys, then the rows they have
     uint32_t* const s_place = reinterpret_cast<uint32_t*>(s_dyn + plan.o_place);               // per step and entry in hand: its group's place
     unsigned* const leaf_key = reinterpret_cast<unsigned*>(s_dyn + plan.o_leaf);
@@ -294,7 +307,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
     const uint32_t N = plan.capacity, D = plan.depth;
     // strata of this CTA: its first warps', a thread each
     const uint32_t k_lo = (uint32_t)(((uint64_t)rank * plan.B) >> lp), k_hi = (uint32_t)(((uint64_t)(rank + 1u) * plan.B) >> lp);
-    const uint32_t strata_warps = kSample ? (((plan.B + mask) >> lp) + 31u) / 32u : 0u;         // the same in every CTA
+    const uint32_t strata_warps = (((plan.B + mask) >> lp) + 31u) / 32u;         // the same in every CTA
 
     // ---- until the kernel before this one is complete: what depends on the arguments alone ----
     if (tid == 0) {
@@ -303,7 +316,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar_vis), "r"(parts));
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar_seen));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        if (receives) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_up), "r"((plan.n_u + 3u) / 4u * 16u) : "memory");
+        if (receives) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_up), "r"((plan.n_u + 3u) / 4u * (kMin ? 32u : 16u)) : "memory");
         if (kSample) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_seen), "r"((uint32_t)sizeof(SeenLeast) * strata_warps * parts) : "memory");
         s_count = 0u; s_found = 1u; s_refused = 0u;
     }
@@ -312,8 +325,8 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
         auto fill = [&](unsigned char* at, uint32_t bytes, uint32_t x) {      // (whole 16-byte units)
             for (uint32_t q = tid; q < bytes / 16u; q += kThreads) reinterpret_cast<uint4*>(at)[q] = make_uint4(x, x, x, x);
         };
-        fill(s_dyn, plan.up_floats * 4u, 0u);
-        fill(reinterpret_cast<unsigned char*>(s_own), plan.own4 * 16u, 0u);
+        fill(s_dyn, plan.up_floats * (kMin ? 8u : 4u), 0u);
+        fill(reinterpret_cast<unsigned char*>(s_own), plan.own4 * (kMin ? 32u : 16u), 0u);
         fill(dirty, plan.dirty_bytes, 0u);
         fill(reinterpret_cast<unsigned char*>(nodes), plan.passes * (plan.node_mask + 1u) * 4u, kNone);
         if (plan.B_upd) {
@@ -337,7 +350,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
     // (where this thread's first units of the staged levels lie)
     PortionUnit unit[kUnits];
 #pragma unroll
-    for (uint32_t q = 0; q < kUnits; ++q) unit[q] = warp < kTreeWarps ? portion_unit<K>(plan, portion, rank, tid + q * kTreeThreads) : PortionUnit{nullptr, 0u};
+    for (uint32_t q = 0; q < kUnits; ++q) unit[q] = warp < kTreeWarps ? portion_unit<K>(plan, portion, 0, rank, tid + q * kTreeThreads) : PortionUnit{nullptr, 0u};
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");      // (every CTA's barriers can be signalled, every CTA has cleared its own memory)
     prb_dep_wait();
@@ -350,6 +363,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
     auto holders_of = [&](uint32_t p) { return nodes + (plan.passes + p) * (plan.node_mask + 1u); };
     const uint32_t R = plan.rows;
     auto row_at = [&](uint32_t p, uint32_t r) { return rows + (p * R + r) * kPitch<K>; };
+    auto min_row_at = [&](uint32_t p, uint32_t r) { return rows + ((plan.passes + p - 1u) * R + r) * kPitch<K>; };      // (p >= 1: the leaves serve both trees)
     float* const leaves = c.level(D);
     const uint32_t n_leaves = plan.n + ((kFrames && plan.n) ? min(plan.stack, N - plan.n) : 0u);
     // group `j` of leaves that the insertion falls into, if there is such a one and it is this CTA's (else kNone); `from`: the cursor
@@ -379,6 +393,12 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
 #pragma unroll
                 for (uint32_t q = 0; q < (uint32_t)M / 4u; ++q)
                     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + q * 16u), "l"(from + q * 4u) : "memory");
+                if (kMin && p) {
+                    const uint32_t to_min = prb_smem_addr(min_row_at(p, r));
+#pragma unroll
+                    for (uint32_t q = 0; q < (uint32_t)M / 4u; ++q)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to_min + q * 16u), "l"(from + plan.min_off + q * 4u) : "memory");
+                }
             }
         }
     };
@@ -392,17 +412,20 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
     // the entry in row r, leaf i: step p's group, if it has fetched it, summed up into the next step's
     auto sum = [&](uint32_t p, uint32_t r, uint32_t i, const Last& last) {
         if (holders_of(p)[s_place[p * R + r]] != r) return;
-        const uint32_t a = i >> (lgM * (p + 1u));
-        const float* const row = row_at(p, r);
+        const uint32_t a = i >> (lgM * (p + 1u)), at = a & (uint32_t)(M - 1);
+        const uint32_t next = p + 1u < plan.passes ? holders_of(p + 1u)[s_place[(p + 1u) * R + r]] : 0u;
         float e[M];
-#pragma unroll
-        for (int q = 0; q < M / 4; ++q) {
-            const float4 t = reinterpret_cast<const float4*>(row)[q];
-            e[4 * q] = t.x; e[4 * q + 1] = t.y; e[4 * q + 2] = t.z; e[4 * q + 3] = t.w;
+        load_group<M>(row_at(p, r), e);
+        if constexpr (kMin) {
+            float m[M];
+            load_group<M>(p ? min_row_at(p, r) : row_at(p, r), m);
+            sum_up<K, true, 0>(c, plan.min_off, D - p * S, a, m);
+            if (p + 1u < plan.passes) min_row_at(p + 1u, next)[at] = m[0];
+            else last.node[plan.staged ? plan.portion_floats : plan.own4 * 4u] = m[0];
         }
-        sum_up<K, 0>(c, D - p * S, a, e);
+        sum_up<K, false, 0>(c, 0, D - p * S, a, e);
         if (p + 1u < plan.passes) {
-            row_at(p + 1u, holders_of(p + 1u)[s_place[(p + 1u) * R + r]])[a & (uint32_t)(M - 1)] = e[0];
+            row_at(p + 1u, next)[at] = e[0];
         } else {
             *last.node = e[0];
             *last.mark = 1;
@@ -577,8 +600,16 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
         for (uint32_t q = 0; q < kUnits; ++q)
             if (unit[q].from != nullptr) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(unit[q].to), "l"(unit[q].from) : "memory");
         for (uint32_t q = t256 + kUnits * kTreeThreads; q < plan.portion_units; q += kTreeThreads) {
-            const PortionUnit v = portion_unit<K>(plan, portion, rank, q);
+            const PortionUnit v = portion_unit<K>(plan, portion, 0, rank, q);
             if (v.from != nullptr) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(v.to), "l"(v.from) : "memory");
+        }
+        float least = 0.0f;
+        if constexpr (kMin) {
+            if (t256 < plan.own && global_of(t256, lp, rank) < plan.n_u) least = __ldcg(c.level(plan.U) + plan.min_off + global_of(t256, lp, rank));
+            for (uint32_t q = t256; q < plan.portion_units; q += kTreeThreads) {
+                const PortionUnit v = portion_unit<K>(plan, portion_min, plan.min_off, rank, q);
+                if (v.from != nullptr) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(v.to), "l"(v.from) : "memory");
+            }
         }
         auto inserted = [&](uint32_t leaf) { return (leaf >= cursor ? leaf - cursor : leaf + N - cursor) < n_leaves; };
         unsigned flags = 0u;
@@ -616,6 +647,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
             }
         };
         if (t256 < plan.own) s_own[t256] = own;
+        if (kMin && t256 < plan.own) own_min[t256] = least;
         asm volatile("cp.async.wait_all;" ::: "memory");
 #pragma unroll 1
         for (uint32_t e0 = 0;;) {
@@ -659,7 +691,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
             }
             if constexpr (kEach == 1) break;
             e0 += R;
-            if (e0 >= m) break;
+            if (kEach == 1 || e0 >= m) break;
             asm volatile("bar.arrive 6, %0;" ::"n"(kTreeThreads + kCopyThreads) : "memory");
         }
         asm volatile("bar.arrive 3, %0;" ::"n"(kThreads) : "memory");
@@ -675,13 +707,16 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
             for (uint32_t g = tid; g < plan.own << sh; g += kTreeThreads) {
                 const uint32_t a = (global_of(g >> sh, lp, rank) << sh) | (g & ((1u << sh) - 1u));
                 float e[M];
-#pragma unroll
-                for (int q = 0; q < M / 4; ++q) {
-                    const float4 t = reinterpret_cast<const float4*>(portion + plan.portion_at[s] + g * kPitch<K>)[q];
-                    e[4 * q] = t.x; e[4 * q + 1] = t.y; e[4 * q + 2] = t.z; e[4 * q + 3] = t.w;
-                }
+                load_group<M>(portion + plan.portion_at[s] + g * kPitch<K>, e);
                 if (!dirty[plan.dirty_at[s] + g]) continue;
-                sum_up<K, 0>(c, plan.U + s * S, a, e);
+                if constexpr (kMin) {
+                    float m[M];
+                    load_group<M>(portion_min + plan.portion_at[s] + g * kPitch<K>, m);
+                    sum_up<K, true, 0>(c, plan.min_off, plan.U + s * S, a, m);
+                    if (s > 1u) portion_min[plan.portion_at[s - 1u] + padded<K>(g)] = m[0];
+                    else own_min[g] = m[0];
+                }
+                sum_up<K, false, 0>(c, 0, plan.U + s * S, a, e);
                 if (s > 1u) {
                     portion[plan.portion_at[s - 1u] + padded<K>(g)] = e[0];
                     dirty[plan.dirty_at[s - 1u] + (g >> lgM)] = 1;
@@ -701,6 +736,11 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
             const uint4 x = reinterpret_cast<const uint4*>(s_own)[j];
             asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
                          ::"r"(at_rank(prb_smem_addr(up + plan.up[plan.U] + u), peer)), "r"(x.x), "r"(x.y), "r"(x.z), "r"(x.w), "r"(at_rank(bar_up, peer)) : "memory");
+            if constexpr (kMin) {
+                const uint4 y = reinterpret_cast<const uint4*>(own_min)[j];
+                asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                             ::"r"(at_rank(prb_smem_addr(up_min + plan.up[plan.U] + u), peer)), "r"(y.x), "r"(y.y), "r"(y.z), "r"(y.w), "r"(at_rank(bar_up, peer)) : "memory");
+            }
         }
         if (!kSample && rank != 0u) return;
         double ku = 0.0, per_b = 0.0;
@@ -722,8 +762,12 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
             while (true) {
                 if (!alone || warp == 0u)
                     for (uint32_t i = tid; i < count; i += kTreeThreads) {
-                        if (h == (uint32_t)S) top_group<K, S>(c, up, rank == 0u, l, from, i);
-                        else top_group<K, 1>(c, up, rank == 0u, l, from, i);
+                        if (h == (uint32_t)S) top_group<K, false, S>(c, up, 0, rank == 0u, l, from, i);
+                        else top_group<K, false, 1>(c, up, 0, rank == 0u, l, from, i);
+                        if constexpr (kMin) {
+                            if (h == (uint32_t)S) top_group<K, true, S>(c, up_min, plan.min_off, rank == 0u, l, from, i);
+                            else top_group<K, true, 1>(c, up_min, plan.min_off, rank == 0u, l, from, i);
+                        }
                     }
                 alone = alone || count <= 32u;
                 l -= h;
@@ -833,28 +877,34 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
 }
 
 using StepKernel = void (*)(StepPlan);
-template <bool kSample, bool kFrames, uint32_t kEach>
-StepKernel step_kernel_of(uint32_t fanout)
+template <bool kSample, bool kFrames, bool kMin>
+StepKernel step_kernel_of(uint32_t fanout, bool many)
 {
     switch (fanout) {
-    case 2: return prb_step_kernel<2, kSample, kFrames, kEach>;
-    case 4: return prb_step_kernel<4, kSample, kFrames, kEach>;
-    case 8: return prb_step_kernel<8, kSample, kFrames, kEach>;
-    case 16: return prb_step_kernel<16, kSample, kFrames, kEach>;
-    default: return prb_step_kernel<32, kSample, kFrames, kEach>;
+    case 2: return many ? prb_step_kernel<2, kSample, kFrames, kMin, kMostEach> : prb_step_kernel<2, kSample, kFrames, kMin, 1>;
+    case 4: return many ? prb_step_kernel<4, kSample, kFrames, kMin, kMostEach> : prb_step_kernel<4, kSample, kFrames, kMin, 1>;
+    case 8: return many ? prb_step_kernel<8, kSample, kFrames, kMin, kMostEach> : prb_step_kernel<8, kSample, kFrames, kMin, 1>;
+    case 16: return many ? prb_step_kernel<16, kSample, kFrames, kMin, kMostEach> : prb_step_kernel<16, kSample, kFrames, kMin, 1>;
+    default: return many ? prb_step_kernel<32, kSample, kFrames, kMin, kMostEach> : prb_step_kernel<32, kSample, kFrames, kMin, 1>;
     }
 }
-// (form: 0 an iteration, 1 tree work alone, 2 with frames)
+// form: 0 an iteration; the tree work alone: 1, with frames 2, with a min-tree 3, with both 4
+constexpr uint32_t kForms = 5;
 StepKernel step_kernel(uint32_t fanout, uint32_t form, bool many)
 {
-    if (many) return form == 0u ? step_kernel_of<true, false, kMostEach>(fanout) : form == 1u ? step_kernel_of<false, false, kMostEach>(fanout) : step_kernel_of<false, true, kMostEach>(fanout);
-    return form == 0u ? step_kernel_of<true, false, 1>(fanout) : form == 1u ? step_kernel_of<false, false, 1>(fanout) : step_kernel_of<false, true, 1>(fanout);
+    switch (form) {
+    case 0: return step_kernel_of<true, false, false>(fanout, many);
+    case 1: return step_kernel_of<false, false, false>(fanout, many);
+    case 2: return step_kernel_of<false, true, false>(fanout, many);
+    case 3: return step_kernel_of<false, false, true>(fanout, many);
+    default: return step_kernel_of<false, true, true>(fanout, many);
+    }
 }
 
 // CTAs a cluster of this kernel may have here: 16 needs the opt-in and a group of SMs that holds it.
 uint32_t most_parts(StepKernel k, uint32_t ki, uint32_t form, bool many, int dev)
 {
-    static uint32_t known[kPrbMaxDevices][6][3][2];
+    static uint32_t known[kPrbMaxDevices][6][kForms][2];
     uint32_t& y = known[dev][ki][form][many ? 1 : 0];
     if (y) return y;
     uint32_t most = 0;
@@ -900,13 +950,14 @@ bool plan_step(const PrbView& v, uint32_t parts, bool many, StepPlan& p, uint32_
     }
     p.up_floats = at;
     // (the staged steps stop above the leaves' own)
+    const uint32_t trees = p.min_off ? 2u : 1u;
     uint32_t floats = 0, groups = 0;
     p.staged = 0;
     for (uint32_t s = 0; s <= kMostStaged; ++s) p.portion_at[s] = p.dirty_at[s] = 0;
     const uint32_t steps = (D - p.U) / S;
     for (uint32_t s = 1; s < steps && s <= kMostStaged; ++s) {
         const uint64_t here = (uint64_t)p.own << (lgM * (s - 1u));      // groups
-        if (floats + here * (M + 4u) > kPortionFloats) break;
+        if ((floats + here * (M + 4u)) * trees > kPortionFloats) break;
         p.portion_at[s] = floats;
         p.dirty_at[s] = groups;
         floats += (uint32_t)here * (M + 4u);
@@ -935,12 +986,13 @@ bool plan_step(const PrbView& v, uint32_t parts, bool many, StepPlan& p, uint32_
     for (;; p.rows /= 2u) {
         // (fewer rows where many steps need them: what does not fit goes in rounds)
         table(many ? p.rows : p.B_upd + groups_in, 256u, p.node_mask, p.node_shift);
-        uint32_t o = aligned(p.up_floats * 4u, 16u);
-        p.o_own = o; o = aligned(o + p.own4 * 16u, 128u);
-        p.o_portion = o; o += floats * 4u;
+        uint32_t o = p.up_floats * 4u * trees;
+        p.o_own = o; o = aligned(o + p.own4 * 16u * trees, 128u);
+        p.portion_floats = floats;
+        p.o_portion = o; o += floats * 4u * trees;
         p.dirty_bytes = aligned(groups + 1u, 16u);
         p.o_dirty = o; o += p.dirty_bytes;
-        p.o_rows = o; o += p.passes * p.rows * (M + 4u) * 4u;
+        p.o_rows = o; o += (p.passes + (trees - 1u) * (p.passes - 1u)) * p.rows * (M + 4u) * 4u;
         p.o_nodes = o; o += p.passes * 2u * (p.node_mask + 1u) * 4u;
         p.o_place = o; o += p.passes * p.rows * 4u;
         p.o_leaf = o; o += p.B_upd ? 2u * (p.leaf_mask + 1u) * 4u : 0u;
@@ -953,9 +1005,9 @@ bool plan_step(const PrbView& v, uint32_t parts, bool many, StepPlan& p, uint32_
 
 }  // namespace
 
-int prb_launch_step(const PrbView& v, const PrbTreeArgs& t, const PrbSampleArgs* sample, cudaStream_t s)
+int prb_launch_step(const PrbView& v, const PrbTreeArgs& t, const PrbSampleArgs* sample, cudaStream_t s, bool dependent)
 {
-    if (v.min_off || (sample && v.stack) || (t.n && t.prio == nullptr) || (t.B == 0 && t.n == 0)) return 0;
+    if ((sample && (v.stack || v.min_off)) || (t.n && t.prio == nullptr) || (t.B == 0 && t.n == 0)) return 0;
     PrbBatch none;
     for (int f = 0; f < PRB_NUM_FIELDS; ++f) none.ptr[f] = nullptr;
     StepPlan p;
@@ -963,7 +1015,7 @@ int prb_launch_step(const PrbView& v, const PrbTreeArgs& t, const PrbSampleArgs*
     p.out = prb_plan_words(v, sample ? sample->dst : none);
     if (p.in.n_words > kPrbMostWords || p.out.n_words > kPrbMostWords) return 0;
     const int dev = prb_current_device();
-    const uint32_t form = sample ? 0u : v.stack ? 2u : 1u;
+    const uint32_t form = sample ? 0u : v.min_off ? (v.stack ? 4u : 3u) : v.stack ? 2u : 1u;
     bool many = t.B > kTreeThreads || (t.n && t.n + v.stack > kTreeThreads);
     // (as many CTAs as there may be, whatever the batch: 4 / 8 / 16, us a step: 32 entries 7.4 / 7.2 / 7.2, 256 + 256 10.2 / 9.5 / 8.3,
     // 1000 + 777 34 / 16.8 / 12.6; through host buffers, every CTA reading the batch over the link, 40.6 / 39.1 / 37.6)
@@ -971,6 +1023,7 @@ int prb_launch_step(const PrbView& v, const PrbTreeArgs& t, const PrbSampleArgs*
     if (parts == 1u || (sample && (sample->B > parts * kTreeThreads || sample->B > kPrbClusterStrata))) return 0;
     p.state = v.state;
     p.level0 = v.level[0];
+    p.min_off = v.min_off;
     p.idx = t.idx; p.val = t.val; p.prio = t.prio; p.done = t.done;
     p.out_idx = sample ? sample->idx : nullptr;
     p.out_w = sample ? sample->w : nullptr;
@@ -1002,6 +1055,6 @@ int prb_launch_step(const PrbView& v, const PrbTreeArgs& t, const PrbSampleArgs*
     a[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     a[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = a;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = dependent ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, step_kernel(v.fanout, form, many), p) == cudaSuccess ? 1 : -1;
 }

@@ -648,6 +648,13 @@ int prb_launch_tree(const PrbView& v, const PrbTreeArgs& t, cudaStream_t s, bool
         const int b = a < 0 ? -1 : prb_launch_tree(v, w, s, dependent);
         return b < 0 ? -1 : a + b;
     }
+    if (t.most_ctas == 0 && !t.linked && (t.B || t.n <= kTreeThreads / 2u)) {
+        // up to one cluster's worth of entries in a tree that it takes (prb_step.cu).  us a call in a graph, this file's cluster / that one: fanout
+        // 16, 2^20 slots, 256 entries 5.1 / 4.1, 256 + 256 5.6 / 4.4, 64 + 64 5.4 / 4.1, 256 insertions 4.1 / 3.9; fanout 2, 1000 + 777 8.9 / 6.2;
+        // fanout 32, 2^22 slots, 1024 + 1024 7.7 / 6.4 -- and 1024 insertions alone 5.4 / 5.9: their rows are better copied by CTAs of their own
+        const int k = prb_launch_step(v, t, nullptr, s, dependent);
+        if (k != 0) return k;
+    }
     TreePlan p;
     p.state = v.state;
     p.level0 = v.level[0];
