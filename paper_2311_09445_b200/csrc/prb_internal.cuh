@@ -33,7 +33,7 @@ struct PrbState {
     unsigned long long pmin_bits;     // smallest positive leaf (bits of a binary32), filled in before a sample that normalises over the buffer
     unsigned int status;              // PEARL_ST_* bits
     unsigned int insert_ticket;       // CTAs of the running insert kernel that have finished
-    unsigned int sample_ticket;       // CTAs of the running sample kernel that have finished
+    unsigned int sample_ticket;       // CTAs of the running sample kernel that have finished (large batches: that have given their smallest priority)
     unsigned int max_prio_bits;       // bits of the largest priority written so far (0: none yet)
     unsigned int wide_arrived;        // grid barrier of the running many-CTA update: arrivals so far (0 between launches that ended well)
     unsigned int wide_done;           // its CTAs that have passed their last barrier
@@ -47,6 +47,7 @@ struct PrbState {
     unsigned int wide_poisoned;       // CTAs that wait for one another (a cluster, or a co-resident grid) gave up once: tickets and the grid
                                       // barrier's state are not to be trusted, and every later update or sample of many co-resident CTAs
                                       // raises INTERNAL and does nothing
+    unsigned int sample_done;         // CTAs of the running large-batch sample that have read the smallest priority (0 between calls)
 };
 
 // Geometry and device addresses, passed to kernels by value.
@@ -130,8 +131,8 @@ struct PrbSubStreams {
 int prb_launch_sample(const PrbView& v, uint32_t B, float beta, uint64_t seed, int32_t* d_idx, float* d_w,
                       const PrbBatch& dst, cudaStream_t s, int uniform = 0, uint32_t n_sub = 1,
                       const PrbSubStreams* subs = nullptr, int buffer_norm = 0);
-// The same for short rows of a buffer without frames, in one launch (prb_sample_short.cu); 0: this device has no
-// cooperative launches and the batch needs one.
+// The same for short rows of a buffer without frames, in one launch (prb_sample_short.cu); 0: rows of medium length, which the lane-group
+// kernel takes.
 int prb_launch_sample_short(const PrbView& v, uint32_t B, float beta, uint64_t seed, int32_t* d_idx, float* d_w, const PrbBatch& dst,
                             cudaStream_t s, int uniform, int buffer_norm);
 // The scan of the leaves for their smallest positive one, into PrbState::pmin_bits.

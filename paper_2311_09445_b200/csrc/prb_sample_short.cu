@@ -19,8 +19,9 @@
 //
 // Two shapes, by batch size.  Up to kClusterStrata strata: one thread-block cluster of up to 16 CTAs; p_min goes
 // through distributed shared memory (each transfer signals the receiver's barrier), nothing through global
-// memory.  More: a cooperative grid; p_min by an atomic per CTA, and a CTA waits (bounded) for the others only
-// after its rows are copied.
+// memory.  More: a grid; p_min by an atomic per CTA, and no CTA waits for another: one that has copied its rows before all
+// have given theirs leaves its weights to the last that does.  (As a cooperative launch whose CTAs waited for the others it could be no
+// programmatic dependent: 4096 strata 24.6 -> 22.6 us a step with its tree kernel, 65536 55.4 -> 53.9.)
 #include "prb_walk.cuh"
 #include "prb_rows.cuh"
 
@@ -30,15 +31,14 @@ constexpr uint32_t kShortThreads = 512;
 constexpr uint32_t kShortTopFloats = 5120;           // tree entries staged in shared memory
 constexpr uint32_t kMaxSteps = 16;
 constexpr uint32_t kMaxCluster = 16;
-// Batches of at most this many strata run as one cluster: three warps of strata per CTA.  (The grid form costs a
-// cooperative launch, no programmatic one, and a round through global memory for the smallest priority.)
+// Batches of at most this many strata run as one cluster: three warps of strata per CTA.  (The grid form costs a round
+// through global memory for the smallest priority.)
 constexpr uint32_t kClusterStrata = kPrbClusterStrata;
 constexpr uint32_t kMaxSeen = 64;                    // strata warps of a cluster: 8 CTAs x 6 warps, 16 x 3
-constexpr uint32_t kGridStrata = 32;                 // strata per CTA of the cooperative grid, at least (fewer where rows are long)
+constexpr uint32_t kGridStrata = 32;                 // strata per CTA of the grid, at least (fewer where rows are long)
 constexpr uint32_t kClusterUnits = 1u << 16;         // a cluster copies at most this many units ...
 constexpr uint32_t kClusterWords = 400u << 10;       // ... or words
 constexpr uint32_t kLaneGroupUnits = 160;            // units of a row up to which the lane-group kernel comes next
-constexpr uint32_t kShortSpinLimit = 1u << 22;
 constexpr uint32_t kNotStaged = 0xFFFFFFFFu;
 
 // One step of the walk: from a node to one of its descendants `levels` levels down.
@@ -55,6 +55,7 @@ struct ShortPlan {
     const float* min_root;        // the min-tree's root, if the buffer keeps one and the weights want it
     int32_t* out_idx;
     float* out_w;
+    float* kept;                  // (grid) priorities that wait for their weight: B of them, then a word per CTA
     uint64_t seed;
     uint32_t B, capacity;
     float beta;
@@ -281,10 +282,13 @@ prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
     if (mine) plan.out_w[k] = plan.uniform ? 1.0f : weight_of(plan, log_p, log_pmin);
 }
 
-// ---- more strata: a cooperative grid ---------------------------------------------------------------------------
+// ---- more strata: a grid -------------------------------------------------------------------------------------------
 // Every CTA takes a contiguous range of strata, kShortThreads at a time; all its threads copy.  The smallest priority
-// is raised (complemented: the word is 0 between calls) with one atomic per CTA, and sample_ticket counts the
-// CTAs that have given theirs, then those that have read the answer.
+// is raised (complemented: the word is 0 between calls) with one atomic per CTA, and sample_ticket counts the CTAs that have given
+// theirs.  A CTA whose rows are copied forms its weights if all have; otherwise it leaves its priorities in `kept`, raises its word there
+// and looks once more: either it sees now that all have given theirs, or the last one to do so, which looks for raised words when its own
+// rows are copied, finds it (a sequentially consistent fence on either side; both may, and write the same).  So no CTA waits, the grid
+// need not be co-resident, and the launch is a programmatic dependent like the others.
 template <int K, bool kUnits>
 __global__ void __launch_bounds__(kShortThreads, 2)
 prb_sample_grid_kernel(const __grid_constant__ ShortPlan plan)
@@ -292,26 +296,29 @@ prb_sample_grid_kernel(const __grid_constant__ ShortPlan plan)
     __shared__ __align__(16) float s_top[kShortTopFloats];
     __shared__ uint32_t s_idx[kShortThreads];
     __shared__ ShortStep s_step[kMaxSteps];
-    __shared__ unsigned s_min, s_flags;
-    __shared__ int s_ok;
+    __shared__ unsigned s_min, s_flags, s_late;
+    __shared__ bool s_all, s_last;
     const uint32_t tid = threadIdx.x, warps = kShortThreads / 32u;
     const uint32_t k_lo = (uint32_t)(((uint64_t)blockIdx.x * plan.B) / gridDim.x);
     const uint32_t k_hi = (uint32_t)(((uint64_t)(blockIdx.x + 1) * plan.B) / gridDim.x);
+    const bool exchange = plan.out_w != nullptr && !plan.buffer_norm && !plan.uniform;
+    uint32_t* const raised = reinterpret_cast<uint32_t*>(plan.kept + plan.B);      // (a word per CTA)
+    StagedUnit unit[kStagedUnits];
+#pragma unroll
+    for (uint32_t i = 0; i < kStagedUnits; ++i) unit[i] = plan.uniform ? StagedUnit{nullptr, 0u} : staged_unit(plan, s_top, tid + i * kShortThreads);
+    if (tid < plan.n_steps) s_step[tid] = plan.step[tid];
+    if (tid == 0) { s_min = 0xFFFFFFFFu; s_flags = 0u; s_late = 0u; }
+    const PrbWordShare share = prb_word_share(plan.words, tid >> 5, warps);
+    prb_dep_wait();
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const unsigned long long calls = plan.state->sample_calls;
     const unsigned long long fill = plan.state->fill;
     const float total32 = *plan.level0;
     const bool poisoned = __ldcg(&plan.state->wide_poisoned) != 0u;
     float pmin = 0.0f;
     if (plan.buffer_norm) pmin = plan.min_root ? *plan.min_root : __uint_as_float((unsigned)plan.state->pmin_bits);
-    if (!plan.uniform) {
-        StagedUnit unit[kStagedUnits];
-#pragma unroll
-        for (uint32_t i = 0; i < kStagedUnits; ++i) unit[i] = staged_unit(plan, s_top, tid + i * kShortThreads);
-        stage(unit);
-    }
-    if (tid < plan.n_steps) s_step[tid] = plan.step[tid];
-    if (tid == 0) { s_min = 0xFFFFFFFFu; s_flags = 0u; }
-    const PrbWordShare share = prb_word_share(plan.words, tid >> 5, warps);
+    stage(unit);
+    if (tid == 0 && exchange) raised[blockIdx.x] = 0u;
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     if (poisoned) {
@@ -326,10 +333,9 @@ prb_sample_grid_kernel(const __grid_constant__ ShortPlan plan)
         }
         return;
     }
-    const bool exchange = plan.out_w != nullptr && !plan.buffer_norm && !plan.uniform;
-    const bool kept = k_hi - k_lo > kShortThreads && plan.out_w != nullptr;       // more than one pass: priorities wait in out_w for the weight
+    const bool kept = k_hi - k_lo > kShortThreads && plan.out_w != nullptr;       // more than one pass: priorities wait for the weight
     float p = 1.0f;
-    unsigned flags = 0u, best = 0xFFFFFFFFu;
+    unsigned flags = 0u, best = 0xFFFFFFFFu, given = 0u;
     for (uint32_t kb = k_lo; kb < k_hi; kb += kShortThreads) {
         const uint32_t n = min(kShortThreads, k_hi - kb), k = kb + tid;
         if (tid < n) {
@@ -338,7 +344,7 @@ prb_sample_grid_kernel(const __grid_constant__ ShortPlan plan)
             s_idx[tid] = leaf;
             plan.out_idx[k] = (int32_t)leaf;
             best = min(best, __float_as_uint(p));
-            if (kept) plan.out_w[k] = p;
+            if (kept) plan.kept[k] = p;
         }
         const bool last = kb + kShortThreads >= k_hi;
         __syncwarp();
@@ -352,39 +358,71 @@ prb_sample_grid_kernel(const __grid_constant__ ShortPlan plan)
         }
         __syncthreads();
         if (last && tid == kShortThreads - 1u) {
-            // this CTA's smallest priority goes out; the answer is looked at when the rows have been copied
+            // this CTA's smallest priority goes out; who else has given one is looked at when the rows have been copied
             if (s_flags) atomicOr(&plan.state->status, s_flags);
-            if (exchange) atomicMax(&plan.state->wide_wmax_bits, (unsigned long long)(~s_min));
-            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&plan.state->sample_ticket) : "memory");
+            if (exchange) {
+                atomicMax(&plan.state->wide_wmax_bits, (unsigned long long)(~s_min));
+                asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(given) : "l"(&plan.state->sample_ticket) : "memory");
+            }
         }
         gather<kUnits>(plan, share, warps, tid, kb, n, s_idx);
         if (!last) __syncthreads();           // s_idx is rewritten by the next pass
     }
-    if (tid == kShortThreads - 1u) {
-        // (bounded wait; the grid is co-resident)
-        int ok = 0;
-        for (uint32_t spins = 0; spins < kShortSpinLimit && !ok; ++spins) {
-            uint32_t seen;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&plan.state->sample_ticket) : "memory");
-            ok = seen >= gridDim.x;
+    auto all_given = [&]() {
+        uint32_t seen;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&plan.state->sample_ticket) : "memory");
+        return seen >= gridDim.x;
+    };
+    if (exchange) {
+        if (tid == kShortThreads - 1u) {
+            s_last = given == gridDim.x - 1u;
+            s_all = s_last || all_given();
         }
-        s_ok = ok;
-        s_min = ~(unsigned)__ldcg(&plan.state->wide_wmax_bits);
-        if (!ok) { atomicOr(&plan.state->status, PEARL_ST_INTERNAL); atomicExch(&plan.state->wide_poisoned, 1u); }
-        else if (prb_ticket(&plan.state->sample_ticket) == 2u * gridDim.x - 1u) {
-            // the last CTA to have read the minimum: the call's bookkeeping
-            plan.state->wide_wmax_bits = 0ull;
-            plan.state->sample_ticket = 0u;
-            plan.state->sample_calls = calls + 1;
-            if (plan.buffer_norm) plan.state->pmin_bits = ~0ull;      // (ready for the next scan)
+        __syncthreads();
+        if (!s_all) {
+            if (!kept && k_lo + tid < k_hi) plan.kept[k_lo + tid] = p;
+            __syncthreads();
+            if (tid == kShortThreads - 1u) {
+                __threadfence();
+                atomicExch(raised + blockIdx.x, 1u);
+                asm volatile("fence.sc.gpu;" ::: "memory");
+                s_all = all_given();
+            }
+            __syncthreads();
         }
     }
+    if (tid == kShortThreads - 1u) {
+        s_min = ~(unsigned)__ldcg(&plan.state->wide_wmax_bits);
+        if (exchange && s_last) asm volatile("fence.sc.gpu;" ::: "memory");
+    }
     __syncthreads();
-    if (!s_ok || plan.out_w == nullptr) return;
     if (exchange) pmin = __uint_as_float(s_min);
     const double log_pmin = plan.uniform ? 0.0 : log2_of(pmin);
-    for (uint32_t k = k_lo + tid; k < k_hi; k += kShortThreads)
-        plan.out_w[k] = plan.uniform ? 1.0f : weight_of(plan, log2_of(kept ? plan.out_w[k] : p), log_pmin);
+    if (plan.out_w != nullptr && (!exchange || s_all))
+        for (uint32_t k = k_lo + tid; k < k_hi; k += kShortThreads)
+            plan.out_w[k] = plan.uniform ? 1.0f : weight_of(plan, log2_of(kept ? plan.kept[k] : p), log_pmin);
+    if (exchange && s_last) {
+        // the CTAs that could not wait for this one
+        for (uint32_t c = tid; c < gridDim.x; c += kShortThreads) {
+            uint32_t up;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(up) : "l"(raised + c) : "memory");
+            if (up) s_idx[atomicAdd(&s_late, 1u)] = c;
+        }
+        __syncthreads();
+        for (uint32_t e = 0; e < s_late; ++e) {
+            const uint32_t c = s_idx[e], hi = (uint32_t)(((uint64_t)(c + 1u) * plan.B) / gridDim.x);
+            for (uint32_t k = (uint32_t)(((uint64_t)c * plan.B) / gridDim.x) + tid; k < hi; k += kShortThreads)
+                plan.out_w[k] = weight_of(plan, log2_of(__ldcg(plan.kept + k)), log_pmin);
+        }
+    }
+    if (tid == kShortThreads - 1u && prb_ticket(&plan.state->sample_done) == gridDim.x - 1u) {
+        // the last CTA to have read what the others have given: the call's bookkeeping
+        plan.state->wide_wmax_bits = 0ull;
+        plan.state->sample_ticket = 0u;
+        plan.state->sample_done = 0u;
+        plan.state->sample_calls = calls + 1;
+        if (plan.buffer_norm) plan.state->pmin_bits = ~0ull;      // (ready for the next scan)
+    }
 }
 
 using ShortKernel = void (*)(ShortPlan);
@@ -428,9 +466,8 @@ const ShortLimits* short_limits(uint32_t fanout, int ki, int dev, bool units)
         if (cudaOccupancyMaxActiveClusters(&fits, kc, &cfg) == cudaSuccess && fits >= 1) cluster = kMaxCluster;
     }
     cudaGetLastError();
-    int nb = 0, coop = 0;
-    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kg, (int)kShortThreads, 0) != cudaSuccess || nb < 1) {
+    int nb = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kg, (int)kShortThreads, 0) != cudaSuccess || nb < 1) {
         cudaGetLastError();
         nb = 0;                                          // (no grid form here)
     }
@@ -466,6 +503,7 @@ int prb_launch_sample_short(const PrbView& v, uint32_t B, float beta, uint64_t s
     plan.out_idx = d_idx;
     plan.out_w = d_w;
     plan.seed = seed;
+    plan.kept = reinterpret_cast<float*>(v.wraw);            // (eight bytes a stratum)
     plan.B = B;
     plan.capacity = (uint32_t)v.capacity;
     plan.beta = beta;
@@ -523,8 +561,8 @@ int prb_launch_sample_short(const PrbView& v, uint32_t B, float beta, uint64_t s
         const uint32_t room = (uint32_t)prb_sm_count() * lim->per_sm;
         if (grid > room) grid = room;
         cfg.gridDim = dim3(grid);
-        a[0].id = cudaLaunchAttributeCooperative;
-        a[0].val.cooperative = 1;
+        a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        a[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.numAttrs = 1;
         e = cudaLaunchKernelEx(&cfg, short_kernel(v.fanout, true, as_units), plan);
     }

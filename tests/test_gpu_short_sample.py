@@ -1,4 +1,4 @@
-"""The short-row sample at the sizes where its two shapes (one cluster, a cooperative grid) and its copy of rows
+"""The short-row sample at the sizes where its two shapes (one cluster, a grid) and its copy of rows
 change: batches around a warp, a CTA's share and the line between the shapes; rows of 1-, 2- and 4-byte words, shorter
 than half a warp's words and longer than a CTA's; and its weights against binary64."""
 import numpy as np
@@ -108,4 +108,24 @@ def test_negative_zero_priorities(oracle_mod, K):
         pr.sample(B, 0.7, 17 + B)
     pr.compare_state()
     assert pr.compare_status() in (0, 8)
+    pr.close()
+
+
+@pytest.mark.parametrize("K,B", [(4, 20_000), (16, 4096)])
+def test_large_batch_beside_other_work(oracle_mod, K, B):
+    # the grid's CTAs get their SMs one by one while another stream holds most of them: no CTA may count on the others being there
+    rng = np.random.default_rng(B)
+    pr = Pair(oracle_mod, 1 << 18, K, 68, 24, 65_536, oracle_store=False)
+    for _ in range(4):
+        pr.insert(dict(prio=np.exp(rng.standard_normal(65_536)).astype(np.float32)))
+    side = torch.cuda.Stream()
+    a = torch.randn(8192, 8192, device=pr.dev, dtype=torch.bfloat16)
+    torch.cuda.synchronize()
+    for i in range(6):
+        with torch.cuda.stream(side):
+            for _ in range(3):
+                a @ a
+        pr.sample(B, 0.4, i)
+    pr.compare_state()
+    pr.compare_status()
     pr.close()
