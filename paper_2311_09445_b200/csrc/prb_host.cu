@@ -633,6 +633,9 @@ static int step_in_one(pearl_prb_t* h, uint32_t B_upd, const int32_t* d_upd_idx,
                        float* d_w, void* const out[PRB_NUM_FIELDS])
 {
     if (h->view.stack || h->view.min_off || (n && !d_new_prio)) return PEARL_STEP_IN_PARTS;
+    // (inputs over the link, which every CTA reads: 256 + 256 entries 37.9 -> 36.4 us, but a larger batch is better read by the four CTAs of the other
+    // route)
+    if (h->linked_inputs && (B_upd > 256u || n > 256u)) return PEARL_STEP_IN_PARTS;
     struct Range { uintptr_t at, end; };
     Range reads[PRB_NUM_FIELDS + 3], writes[PRB_NUM_FIELDS + 2];
     uint32_t nr = 0, nw = 0;
