@@ -19,8 +19,8 @@
 //
 // Two shapes, by batch size.  Up to kClusterStrata strata: one thread-block cluster of up to 16 CTAs; p_min goes
 // through distributed shared memory (each transfer signals the receiver's barrier), nothing through global
-// memory.  More: a grid; p_min by an atomic per CTA, and no CTA waits for another: one that has copied its rows before all
-// have given theirs leaves its weights to the last that does.  (As a cooperative launch whose CTAs waited for the others it could be no
+// memory.  More: a grid; p_min by an atomic per CTA, and no CTA depends on another's being there: one that has copied its rows and does not
+// soon see that all have given theirs leaves its weights to the last that does.  (As a cooperative launch whose CTAs waited for the others it could be no
 // programmatic dependent: 4096 strata 24.6 -> 22.6 us a step with its tree kernel, 65536 55.4 -> 53.9.)
 #include "prb_walk.cuh"
 #include "prb_rows.cuh"
@@ -38,6 +38,7 @@ constexpr uint32_t kMaxSeen = 64;                    // strata warps of a cluste
 constexpr uint32_t kGridStrata = 32;                 // strata per CTA of the grid, at least (fewer where rows are long)
 constexpr uint32_t kClusterUnits = 1u << 16;         // a cluster copies at most this many units ...
 constexpr uint32_t kClusterWords = 400u << 10;       // ... or words
+constexpr uint32_t kGridPolls = 64;                  // looks of a CTA of the grid at whether all have given their smallest priority
 constexpr uint32_t kLaneGroupUnits = 160;            // units of a row up to which the lane-group kernel comes next
 constexpr uint32_t kNotStaged = 0xFFFFFFFFu;
 
@@ -285,9 +286,9 @@ prb_sample_cluster_kernel(const __grid_constant__ ShortPlan plan)
 // ---- more strata: a grid -------------------------------------------------------------------------------------------
 // Every CTA takes a contiguous range of strata, kShortThreads at a time; all its threads copy.  The smallest priority
 // is raised (complemented: the word is 0 between calls) with one atomic per CTA, and sample_ticket counts the CTAs that have given
-// theirs.  A CTA whose rows are copied forms its weights if all have; otherwise it leaves its priorities in `kept`, raises its word there
+// theirs.  A CTA whose rows are copied forms its weights if all have, or have after a few looks; otherwise it leaves its priorities in `kept`, raises its word there
 // and looks once more: either it sees now that all have given theirs, or the last one to do so, which looks for raised words when its own
-// rows are copied, finds it (a sequentially consistent fence on either side; both may, and write the same).  So no CTA waits, the grid
+// rows are copied, finds it (a sequentially consistent fence on either side; both may, and write the same).  So no CTA waits for long, the grid
 // need not be co-resident, and the launch is a programmatic dependent like the others.
 template <int K, bool kUnits>
 __global__ void __launch_bounds__(kShortThreads, 2)
@@ -376,7 +377,11 @@ prb_sample_grid_kernel(const __grid_constant__ ShortPlan plan)
     if (exchange) {
         if (tid == kShortThreads - 1u) {
             s_last = given == gridDim.x - 1u;
-            s_all = s_last || all_given();
+            // (a while, some 20 us, is waited all the same: CTAs whose SMs the kernel before this one held start later, and what is left to the
+            // last one it does alone)
+            bool all = s_last;
+            for (uint32_t spins = 0; spins < kGridPolls && !all; ++spins) all = all_given();
+            s_all = all;
         }
         __syncthreads();
         if (!s_all) {
