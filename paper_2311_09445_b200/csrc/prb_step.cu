@@ -13,8 +13,8 @@
 //    runs -- into rows of shared memory, which a hash table per step finds.  New values are written into the rows and summed up
 //    from row to row, from staged level to staged level: what separates the steps is a barrier of eight warps, not
 //    a round trip;
-//  * level U goes from every CTA to every CTA through distributed shared memory (each transfer signals the receiver's barrier),
-//    and every CTA sums up the few levels above it;
+//  * level U goes from every CTA to every CTA through distributed shared memory (each transfer signals the receiver's barrier; so does an
+//    arrival that releases the staged levels), and every CTA sums up the few levels above it;
 //  * a descent walks those in its own shared memory, the staged levels in their owners' (distributed shared memory), and only the
 //    last steps in L2, where a fence off the chain has made them visible;
 //  * rows of the insertion are copied by warps of their own meanwhile, and a sampled slot that this very call inserts is
@@ -312,7 +312,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
     // ---- until the kernel before this one is complete: what depends on the arguments alone ----
     if (tid == 0) {
         const bool receives = kSample || rank == 0u;
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar_up));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar_up), "r"(kSample ? parts + 1u : 1u));
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar_vis), "r"(parts));
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar_seen));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -561,6 +561,9 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
         cursor = __shfl_sync(0xFFFFFFFFu, cursor, 0);
         if (warp == kTreeWarps) {
             asm volatile("bar.sync 3, %0;" ::"n"(kThreads) : "memory");
+            // (Without the sample CTA 0 is told only that the others hold cursor and fill: what they have read decided their branches and
+            // addresses, so it has come.  The memory model asks for a release there, too; it would wait for the leaves' stores: update and
+            // insertion of 64 + 64 entries 3.60 -> 3.96 us, of 1000 + 777 5.80 -> 6.26, fanouts 2 and 16.)
             if (kSample) asm volatile("fence.acq_rel.cluster;" ::: "memory");
             if (lane < (kSample ? parts : 1u)) asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(at_rank(bar_vis, lane)) : "memory");
         } else {
@@ -726,10 +729,16 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
             }
             tree_sync();
         }
+        // The staged levels, which descents of the other CTAs read in this one's memory: one warp, behind the barrier that all who wrote them
+        // have passed, releases them to every CTA's barrier.  (The transfers below do not: an asynchronous store releases
+        // nothing that was written before it.)  The fence orders shared memory alone, which is all that is read before
+        // bar_vis; one that waits for the stores to L2 too costs a step 0.35 us, this one less than 0.06: fanout 16, 2^20 slots, 64 + 64 entries
+        // 7.69 / 7.36 / 7.35 us with it / with this one / without, 256 + 256 8.09 / 7.86 / 7.72.
+        if (kSample && warp == kTreeWarps - 1u && lane < parts) {
+            asm volatile("fence.release.sync_restrict::shared::cta.cluster;" ::: "memory");
+            asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(at_rank(bar_up, lane)) : "memory");
+        }
         // level U: to every CTA that goes on
-#ifdef PEARL_CHECKED
-        asm volatile("fence.acq_rel.cluster;" ::: "memory");
-#endif
         for (uint32_t t = tid; t < (kSample ? plan.own4 << lp : plan.own4); t += kTreeThreads) {
             const uint32_t peer = kSample ? t & mask : 0u, j = kSample ? t >> lp : t, u = ((j << lp) + rank) << 2;
             if (u >= plan.n_u) continue;
