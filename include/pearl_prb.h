@@ -62,10 +62,12 @@ typedef struct pearl_layout {
                                       not equal the sum of their children, and leaves named by an update of
                                       more than 16384 entries may hold the marker bit pattern 0x80000000|entry
                                       instead of a priority; after a sample of short rows, weights are
-                                      missing.  After either of the last two every later call on that buffer
-                                      that runs as a grid of co-resident thread blocks (updates of more than
-                                      16384 to 32768 entries, by fanout; samples of more than 1536 strata, or
-                                      of long rows below 8 KB) raises the bit again and does nothing.  Treat the buffer as lost: destroy it and build a new one.  No
+                                      missing; after a step of short rows, nodes of the tree may be stale, the
+                                      new transitions may not count (cursor and fill as before), and indices,
+                                      weights and rows of the sampled batch may be missing.  After any of the
+                                      last three every later call on that buffer that needs its bookkeeping
+                                      (updates of more than 16384 to 32768 entries, by fanout; samples of short
+                                      rows of more than 1536 strata) raises the bit again and does nothing.  Treat the buffer as lost: destroy it and build a new one.  No
                                       correct run raises this bit. */
 #define PEARL_ST_STALE 32u         /* update_after_insert: the index was overwritten since it was sampled; entry skipped */
 

@@ -45,8 +45,8 @@ struct PrbState {
     unsigned long long row_cursor;
     unsigned int row_ticket;          // CTAs of the running row kernel that have read row_cursor
     unsigned int wide_poisoned;       // CTAs that wait for one another (a cluster, or a co-resident grid) gave up once: tickets and the grid
-                                      // barrier's state are not to be trusted, and every later update or sample of many co-resident CTAs
-                                      // raises INTERNAL and does nothing
+                                      // barrier's state are not to be trusted, and every later very large update and sample of more strata than
+                                      // a cluster takes raises INTERNAL and does nothing
     unsigned int sample_done;         // CTAs of the running large-batch sample that have read the smallest priority (0 between calls)
 };
 

@@ -283,7 +283,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
     __shared__ uint32_t s_idx[kTreeThreads];
     __shared__ SeenLeast s_seen[kSample ? kMostSeen : 1];
     __shared__ __align__(8) unsigned long long s_bar_up, s_bar_vis, s_bar_seen;
-    __shared__ unsigned s_count, s_found, s_refused;
+    __shared__ unsigned s_count, s_found, s_refused, s_lost;
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, rank = blockIdx.x;
     const uint32_t parts = 1u << plan.log_parts, mask = parts - 1u, lp = plan.log_parts;
     float* const up = reinterpret_cast<float*>(s_dyn);
@@ -318,7 +318,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (receives) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_up), "r"((plan.n_u + 3u) / 4u * (kMin ? 32u : 16u)) : "memory");
         if (kSample) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_seen), "r"((uint32_t)sizeof(SeenLeast) * strata_warps * parts) : "memory");
-        s_count = 0u; s_found = 1u; s_refused = 0u;
+        s_count = 0u; s_found = 1u; s_refused = 0u; s_lost = 0u;
     }
     if (tid >= kThreads - PRB_MAX_LEVELS) s_off[tid - (kThreads - PRB_MAX_LEVELS)] = plan.off[tid - (kThreads - PRB_MAX_LEVELS)];
     {
@@ -761,21 +761,27 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
         }
         // the levels above U, S at a time while there are as many (what the next turn needs is looked up ahead of it); once a
         // level's nodes fit a warp the first warp goes on alone
+        // (a thread whose wait for level U ran out marks the CTA as lost, and after the next barrier no thread stores a sum: its own, in time,
+        // saw all of level U.  In time, not late: a walk that reads a peer's memory begins within one limit of polls, and the peer
+        // stays for two, see bar_seen)
+        bool sound;
+        auto still_sound = [&]() { return *const_cast<volatile unsigned*>(&s_lost) == 0u; };
         {
             uint32_t l = plan.U, h = 0, count = 0, from = 0;
             auto turn = [&]() { h = l >= (uint32_t)S ? (uint32_t)S : 1u; count = prb_nodes_covering(N, lg * (D - l + h)); from = plan.up[l]; };
             turn();
-            prb_wait_first_phase<true>(plan.state, bar_up);
+            sound = prb_wait_first_phase<true>(plan.state, bar_up) == kPrbInTime;
+            if (!sound) s_lost = 1u;
             bool alone = false;
 #pragma unroll 1
             while (true) {
                 if (!alone || warp == 0u)
                     for (uint32_t i = tid; i < count; i += kTreeThreads) {
-                        if (h == (uint32_t)S) top_group<K, false, S>(c, up, 0, rank == 0u, l, from, i);
-                        else top_group<K, false, 1>(c, up, 0, rank == 0u, l, from, i);
+                        if (h == (uint32_t)S) top_group<K, false, S>(c, up, 0, rank == 0u && sound, l, from, i);
+                        else top_group<K, false, 1>(c, up, 0, rank == 0u && sound, l, from, i);
                         if constexpr (kMin) {
-                            if (h == (uint32_t)S) top_group<K, true, S>(c, up_min, plan.min_off, rank == 0u, l, from, i);
-                            else top_group<K, true, 1>(c, up_min, plan.min_off, rank == 0u, l, from, i);
+                            if (h == (uint32_t)S) top_group<K, true, S>(c, up_min, plan.min_off, rank == 0u && sound, l, from, i);
+                            else top_group<K, true, 1>(c, up_min, plan.min_off, rank == 0u && sound, l, from, i);
                         }
                     }
                 alone = alone || count <= 32u;
@@ -784,8 +790,10 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
                 turn();
                 if (alone) __syncwarp();
                 else tree_sync();
+                sound = still_sound();
             }
             tree_sync();
+            sound = still_sound();
         }
         const uint64_t filled = min((uint64_t)fill + plan.n, (uint64_t)N);
         // (every CTA's warps have the cursor in hand once bar_vis is over)
@@ -797,14 +805,14 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
             if (plan.moves_rows) plan.state->row_cursor = moved;
         };
         if constexpr (!kSample) {
-            if (warp == 0u) { prb_wait_first_phase<true>(plan.state, bar_vis); move_cursor(); }
+            if (warp == 0u && prb_wait_first_phase<true>(plan.state, bar_vis) == kPrbInTime && sound) move_cursor();
             return;
         }
         if constexpr (kSample) {
             // ---- the sample ----
             const float total32 = up[plan.up[0]];
             const double total = (double)total32;
-            const bool empty = filled == 0u || !(total32 > 0.0f);
+            const bool empty = sound && (filled == 0u || !(total32 > 0.0f));
             const bool holds = k < k_hi;
             uint32_t leaf = 0;
             float p = 1.0f;
@@ -812,7 +820,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
                 unsigned wflags = 0u;
                 double x = __dmul_rn(ku, total32 <= 3.402823466e+38f ? prb_quotient(total, (double)plan.B, per_b) : total);
                 if (x >= total) x = __longlong_as_double(__double_as_longlong(total) - 1);
-                const bool walks = holds && !empty;
+                const bool walks = holds && !empty && sound;
                 uint32_t g = 0;
                 if (walks) {
 #pragma unroll 1
@@ -830,9 +838,9 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
                         g = (g << lgM) + step_of<K, false>(row, x, p, wflags);
                     }
                 }
-                prb_wait_first_phase<true>(plan.state, bar_vis);
-                move_cursor();
-                if (walks) {
+                sound = prb_wait_first_phase<true>(plan.state, bar_vis) == kPrbInTime && sound;
+                if (sound) move_cursor();
+                if (walks && sound) {
 #pragma unroll 1
                     for (uint32_t q = plan.passes; q > 0u; --q) {
                         const RowInL2 row = RowInL2{c.level(D - (q - 1u) * S) + ((uint64_t)g << lgM)};
@@ -842,7 +850,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
                     leaf = g;
                     s_idx[tid] = leaf;
                 }
-                if (tid == 0u && empty) s_found = 0u;
+                if ((tid == 0u && empty) || !sound) s_found = 0u;
                 __syncwarp();
                 asm volatile("bar.arrive 2, %0;" ::"n"(kThreads) : "memory");      // the copying warps may go on
                 if (wflags) atomicOr(&plan.state->status, wflags);
@@ -852,15 +860,17 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
                 }
                 // weights: as in the sample of short rows (prb_sample_short.cu)
                 const double log_p = log2_of(p);
-                const unsigned bits = holds ? __float_as_uint(p) : 0x7F800000u;
+                // (0, which no drawn leaf holds, from a thread that a wait has failed: then no CTA forms weights)
+                const unsigned bits = !sound ? 0u : holds ? __float_as_uint(p) : 0x7F800000u;
                 const unsigned least = __reduce_min_sync(0xFFFFFFFFu, bits);
                 const double log_least = __shfl_sync(0xFFFFFFFFu, log_p, __ffs(__ballot_sync(0xFFFFFFFFu, bits == least)) - 1);
                 if (lane < parts)
                     asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];"
                                  ::"r"(at_rank(prb_smem_addr(s_seen + rank * strata_warps + warp), lane)), "l"(__double_as_longlong(log_least)), "l"((unsigned long long)least),
                                  "r"(at_rank(bar_seen, lane)) : "memory");
-                if (holds) plan.out_idx[k] = (int32_t)leaf;
-                // (the first warp always gets here, and every walk is over when all values have come: no CTA leaves before)
+                if (holds && sound) plan.out_idx[k] = (int32_t)leaf;
+                // (the first warp always gets here, and every walk is over when all values have come: no CTA leaves before, unless it has waited for
+                // twice the limit, within which a peer that walks at all has done so)
                 if (prb_wait_first_phase<true>(plan.state, bar_seen) == kPrbNever) return;
                 if (rank == 0u && tid == 0u) plan.state->sample_calls = calls + 1;
                 if (plan.out_w == nullptr) return;
@@ -874,7 +884,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
                 __syncwarp();
                 const unsigned smallest = __reduce_min_sync(0xFFFFFFFFu, best);
                 const double log_pmin = __shfl_sync(0xFFFFFFFFu, log_best, __ffs(__ballot_sync(0xFFFFFFFFu, best == smallest)) - 1);
-                if (holds) plan.out_w[k] = exp2_of(-(double)plan.beta * (log_p - log_pmin));
+                if (holds && smallest != 0u) plan.out_w[k] = exp2_of(-(double)plan.beta * (log_p - log_pmin));
                 return;
             }
         }
