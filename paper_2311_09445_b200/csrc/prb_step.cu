@@ -199,6 +199,7 @@ __device__ __forceinline__ PortionUnit portion_unit(const StepPlan& plan, float*
         const uint32_t l = plan.U + s * (uint32_t)kSpan<K>, f = q * 4u, a = (global_of(f >> sh, plan.log_parts, rank) << sh) | (f & ((1u << sh) - 1u));
         const uint32_t stored = (prb_nodes_covering(plan.capacity, kLog2<K> * (plan.depth - l)) + 63u) & ~63u;
         float* const to = portion + plan.portion_at[s] + padded<K>(f);
+        if (!PRB_IN_BOUNDS(plan, plan.portion_at[s] + padded<K>(f) + 4u <= plan.portion_floats)) break;
         o.to = prb_smem_addr(to);
         if (a < stored) o.from = plan.level0 + min_off + ((uint64_t)plan.off[l] << 6) + a;
         else *reinterpret_cast<float4*>(to) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -377,6 +378,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
     const uint32_t t256 = tid & (kTreeThreads - 1u);
     // row r for leaf i: the places of the groups above it; the first to name a group fetches it
     auto fetch = [&](uint32_t r, uint32_t i) {
+        if (!PRB_IN_BOUNDS(plan, r < R && i < N)) return;
 #pragma unroll 1
         for (uint32_t p = 0; p < plan.passes; ++p) {
             const uint32_t a = i >> (lgM * (p + 1u));
@@ -406,14 +408,17 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
     struct Last { float* node; unsigned char* mark; };
     auto last_of = [&](uint32_t i) {
         const uint32_t a = i >> (lgM * plan.passes), sh = lgM * plan.staged, f = (local_of(a >> sh, lp) << sh) | (a & ((1u << sh) - 1u));
+        if (!PRB_IN_BOUNDS(plan, plan.staged ? plan.portion_at[plan.staged] + padded<K>(f) < plan.portion_floats && plan.dirty_at[plan.staged] + (f >> lgM) < plan.dirty_bytes
+                                             : f < plan.own4 * 4u)) return Last{s_own, dirty};
         if (plan.staged == 0u) return Last{s_own + f, dirty};
         return Last{portion + plan.portion_at[plan.staged] + padded<K>(f), dirty + plan.dirty_at[plan.staged] + (f >> lgM)};
     };
     // the entry in row r, leaf i: step p's group, if it has fetched it, summed up into the next step's
     auto sum = [&](uint32_t p, uint32_t r, uint32_t i, const Last& last) {
-        if (holders_of(p)[s_place[p * R + r]] != r) return;
+        if (!PRB_IN_BOUNDS(plan, r < R) || holders_of(p)[s_place[p * R + r]] != r) return;
         const uint32_t a = i >> (lgM * (p + 1u)), at = a & (uint32_t)(M - 1);
         const uint32_t next = p + 1u < plan.passes ? holders_of(p + 1u)[s_place[(p + 1u) * R + r]] : 0u;
+        if (!PRB_IN_BOUNDS(plan, next < R)) return;
         float e[M];
         load_group<M>(row_at(p, r), e);
         if constexpr (kMin) {
@@ -543,7 +548,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
                         if (!prb_valid_priority(p)) { p = 0.0f; flags |= PEARL_ST_BAD_PRIORITY; }
                         else wmax = fmaxf(wmax, p);
                     }
-                    if (!PRB_IN_BOUNDS(plan, slot < N)) continue;
+                    if (!PRB_IN_BOUNDS(plan, slot < N && holders_of(0u)[h] < R)) continue;
                     row_at(0u, holders_of(0u)[h])[slot & (uint32_t)(M - 1)] = p;
                     leaves[slot] = p;
                 }
@@ -590,7 +595,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
     } else {
         // ---- the tree ----
         float v0 = 0.0f;
-        int32_t i0 = -1;
+        int32_t i0 = 0;
         if (kEach == 1 && tid < plan.B_upd) { v0 = plan.val[tid]; i0 = plan.idx[tid]; }
         const uint32_t fill = (uint32_t)plan.state->fill;
         unsigned long long calls = 0;
@@ -644,7 +649,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
         auto write_leaf = [&](uint32_t r, uint32_t i, uint32_t pos, uint32_t place, float p) {
             const uint32_t holder = holders_of(0u)[s_place[r]];
             if (p >= 0.0f) wmax = fmaxf(wmax, p);
-            if (leaf_last[place] == pos + 1u && !(plan.n && inserted(i)) && PRB_IN_BOUNDS(plan, i < N)) {
+            if (leaf_last[place] == pos + 1u && !(plan.n && inserted(i)) && PRB_IN_BOUNDS(plan, i < N && holder < R)) {
                 row_at(0u, holder)[i & (uint32_t)(M - 1)] = p;
                 leaves[i] = p;
             }
@@ -709,9 +714,11 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
             const uint32_t sh = lgM * (s - 1u);
             for (uint32_t g = tid; g < plan.own << sh; g += kTreeThreads) {
                 const uint32_t a = (global_of(g >> sh, lp, rank) << sh) | (g & ((1u << sh) - 1u));
+                if (!PRB_IN_BOUNDS(plan, plan.portion_at[s] + g * kPitch<K> + M <= plan.portion_floats && plan.dirty_at[s] + g < plan.dirty_bytes)) continue;
                 float e[M];
                 load_group<M>(portion + plan.portion_at[s] + g * kPitch<K>, e);
                 if (!dirty[plan.dirty_at[s] + g]) continue;
+                if (!PRB_IN_BOUNDS(plan, (uint64_t)a << (sh_u - sh) < N)) continue;
                 if constexpr (kMin) {
                     float m[M];
                     load_group<M>(portion_min + plan.portion_at[s] + g * kPitch<K>, m);
@@ -741,7 +748,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
         // level U: to every CTA that goes on
         for (uint32_t t = tid; t < (kSample ? plan.own4 << lp : plan.own4); t += kTreeThreads) {
             const uint32_t peer = kSample ? t & mask : 0u, j = kSample ? t >> lp : t, u = ((j << lp) + rank) << 2;
-            if (u >= plan.n_u) continue;
+            if (u >= plan.n_u || !PRB_IN_BOUNDS(plan, plan.up[plan.U] + u + 4u <= plan.up_floats)) continue;
             const uint4 x = reinterpret_cast<const uint4*>(s_own)[j];
             asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
                          ::"r"(at_rank(prb_smem_addr(up + plan.up[plan.U] + u), peer)), "r"(x.x), "r"(x.y), "r"(x.z), "r"(x.w), "r"(at_rank(bar_up, peer)) : "memory");
@@ -827,13 +834,15 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
                     for (uint32_t l = 0; l < plan.U;) {
                         const uint32_t h = (plan.U - l) % (uint32_t)S ? 1u : (uint32_t)S;
                         l += h;
+                        if (!PRB_IN_BOUNDS(plan, plan.up[l] + ((g + 1u) << (lg * h)) <= plan.up_floats)) g = 0u;
                         const PrbRowAt row = PrbRowAt{up + plan.up[l] + (g << (lg * h))};
                         if (h == (uint32_t)S) g = (g << lgM) + step_of<K, false>(row, x, p, wflags);
                         else g = (g << lg) + step1<K, false, false>(row, x, p, wflags);
                     }
 #pragma unroll 1
                     for (uint32_t s = 1; s <= plan.staged; ++s) {
-                        const uint32_t sh = lgM * (s - 1u), u = g >> sh, local = (local_of(u, lp) << sh) | (g & ((1u << sh) - 1u));
+                        const uint32_t sh = lgM * (s - 1u), u = g >> sh, at_owner = (local_of(u, lp) << sh) | (g & ((1u << sh) - 1u));
+                        const uint32_t local = PRB_IN_BOUNDS(plan, plan.portion_at[s] + at_owner * kPitch<K> + M <= plan.portion_floats) ? at_owner : 0u;
                         const RowOfPeer row = RowOfPeer{at_rank(prb_smem_addr(portion + plan.portion_at[s] + local * kPitch<K>), owner_of(u, mask))};
                         g = (g << lgM) + step_of<K, false>(row, x, p, wflags);
                     }

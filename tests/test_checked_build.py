@@ -41,3 +41,13 @@ def test_tree_kernel_and_short_samples_against_the_checked_library():
     tail = r.stdout[-3000:] + r.stderr[-2000:]
     assert r.returncode == 0, tail
     assert " passed" in r.stdout and "failed" not in r.stdout, tail
+
+
+def test_iteration_in_one_launch_against_the_checked_library():
+    from paper_2311_09445_b200 import build
+    env = dict(os.environ, PEARL_PRB_LIB=build.build(checked=True))
+    r = subprocess.run([sys.executable, "-m", "pytest", os.path.join("tests", "test_gpu_step.py"), os.path.join("tests", "test_gpu_deep_trees.py"),
+                        "-x", "-q", "-m", "gpu"], cwd=ROOT, env=env, capture_output=True, text=True, timeout=1800)
+    tail = r.stdout[-3000:] + r.stderr[-2000:]
+    assert r.returncode == 0, tail
+    assert " passed" in r.stdout and "failed" not in r.stdout, tail

@@ -150,3 +150,76 @@ def test_overlapping_arrays_take_the_other_route(oracle_mod):
         assert np.array_equal(out.cpu().numpy(), np.asarray(o["obs"]).view(np.uint8).reshape(B, OBS))
         _check(pr)
     pr.close()
+
+
+@pytest.mark.parametrize("captured", [False, True])
+def test_long_rows_left_out(oracle_mod, captured):
+    # a buffer of long rows whose iteration leaves them out goes in one launch, between iterations that copy them on the handle's streams
+    rng = np.random.default_rng(5)
+    N, E, B, n = 2000, 16_384, 64, 48
+    stream = torch.cuda.Stream()
+    from paper_2311_09445_b200 import PrioritizedReplay
+    gpu = PrioritizedReplay(N, 16, E, 4, 1024, stream=stream)
+    ora = oracle_mod.OraclePRB(N, 16, E, 4)
+
+    def batch(k):
+        return dict(obs=rng.integers(0, 256, size=(k, E), dtype=np.uint8), act=rng.integers(0, 256, size=(k, 4), dtype=np.uint8),
+                    rew=rng.standard_normal(k).astype(np.float32), next_obs=rng.integers(0, 256, size=(k, E), dtype=np.uint8),
+                    done=rng.integers(0, 2, size=k, dtype=np.uint8), prio=np.exp(rng.standard_normal(k)).astype(np.float32))
+    def up(b):
+        return {k: torch.from_numpy(v).cuda() for k, v in b.items()}
+    for _ in range(2):
+        b = batch(900)
+        d = up(b)
+        torch.cuda.synchronize()
+        gpu.insert(d["obs"], d["act"], d["rew"], d["next_obs"], d["done"], d["prio"])
+        assert ora.insert(b["obs"], b["act"], b["rew"], b["next_obs"], b["done"], b["prio"]) == 0
+        torch.cuda.synchronize()
+    full = (True, False, True, False, False, True)
+    host = [batch(n) for _ in full]
+    for b, whole in zip(host, full):
+        if not whole:
+            b["obs"] = b["next_obs"] = None
+    new = [up({k: v for k, v in b.items() if v is not None}) for b in host]
+    idx = [rng.integers(0, 1800, size=B).astype(np.int32) for _ in full]
+    td = [rng.standard_normal(B).astype(np.float32) for _ in full]
+    d_idx, d_td = [torch.from_numpy(x).cuda() for x in idx], [torch.from_numpy(x).cuda() for x in td]
+    z = lambda *s: torch.zeros(s, dtype=torch.uint8, device="cuda")
+    out = [dict(idx=torch.zeros(B, dtype=torch.int32, device="cuda"), w=torch.zeros(B, device="cuda"), obs=z(B, E) if whole else None, act=z(B, 4),
+                rew=torch.zeros(B, device="cuda"), next_obs=z(B, E) if whole else None, done=z(B)) for whole in full]
+
+    def iterations():
+        for i in range(len(full)):
+            r, o = new[i], out[i]
+            gpu.step(d_idx[i], d_td[i], 0.6, 1e-6, r.get("obs"), r["act"], r["rew"], r.get("next_obs"), r["done"], r["prio"], B, 0.4, 7,
+                     o["idx"], o["w"], o["obs"], o["act"], o["rew"], o["next_obs"], o["done"])
+    torch.cuda.synchronize()
+    graph = None
+    if captured:
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            iterations()
+    for _ in range(3):
+        with torch.cuda.stream(stream):
+            if graph is not None:
+                graph.replay()
+            else:
+                iterations()
+        torch.cuda.synchronize()
+        for i, whole in enumerate(full):
+            b = host[i]
+            assert ora.update(idx[i], td[i], 0.6, 1e-6) == 0
+            assert ora.insert(b["obs"], b["act"], b["rew"], b["next_obs"], b["done"], b["prio"]) == 0
+            o = ora.sample(B, 0.4, 7)
+            assert np.array_equal(out[i]["idx"].cpu().numpy(), o["idx"])
+            np.testing.assert_allclose(out[i]["w"].cpu().numpy(), o["w"], rtol=1e-5)
+            for f in ("obs", "act", "rew", "next_obs", "done"):
+                if out[i][f] is not None:
+                    assert np.array_equal(out[i][f].cpu().numpy().view(np.uint8).reshape(-1), np.ascontiguousarray(o[f]).view(np.uint8).reshape(-1)), (i, f)
+    assert gpu.info() == ora.info() and gpu.sync() == ora.status()
+    keep = np.arange(0, 2000, 7, dtype=np.int32)
+    a, g = ora.read_rows(keep), gpu.read_rows(keep)
+    for f in ("obs", "act", "rew", "next_obs", "done"):
+        assert np.array_equal(np.ascontiguousarray(a[f]).view(np.uint8).reshape(-1), np.ascontiguousarray(g[f]).view(np.uint8).reshape(-1)), f
+    gpu.close()
+    ora.close()
