@@ -38,7 +38,13 @@ constexpr uint32_t kMaxSeen = 64;                    // strata warps of a cluste
 constexpr uint32_t kGridStrata = 32;                 // strata per CTA of the grid, at least (fewer where rows are long)
 constexpr uint32_t kClusterUnits = 1u << 16;         // a cluster copies at most this many units ...
 constexpr uint32_t kClusterWords = 400u << 10;       // ... or words
-constexpr uint32_t kGridPolls = 64;                  // looks of a CTA of the grid at whether all have given their smallest priority
+// Looks of a CTA of the grid at whether all have given their smallest priority.  (None in the checked build: there every CTA but the last takes
+// the way of those that come too early, which the others hardly ever do.)
+#ifdef PEARL_CHECKED
+constexpr uint32_t kGridPolls = 0;
+#else
+constexpr uint32_t kGridPolls = 64;
+#endif
 constexpr uint32_t kLaneGroupUnits = 160;            // units of a row up to which the lane-group kernel comes next
 constexpr uint32_t kNotStaged = 0xFFFFFFFFu;
 

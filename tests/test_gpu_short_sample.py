@@ -129,3 +129,18 @@ def test_large_batch_beside_other_work(oracle_mod, K, B):
     pr.compare_state()
     pr.compare_status()
     pr.close()
+
+
+@pytest.mark.parametrize("K,B", [(2, 1537), (8, 5000), (16, 160_000)])
+def test_weights_left_to_the_last_cta(oracle_mod, K, B):
+    # the checked library looks at no other CTA's progress: all CTAs but one leave their priorities behind, of one pass of strata or of
+    # several (160000: more than 512 strata a CTA)
+    rng = np.random.default_rng(B)
+    pr = Pair(oracle_mod, 1 << 18, K, 68, 24, 160_000, oracle_store=False)
+    for n in (160_000, 102_144):
+        pr.insert(dict(prio=np.exp(rng.standard_normal(n)).astype(np.float32)))
+    for i in range(8):
+        pr.sample(B, 0.4, i)
+    pr.compare_state()
+    pr.compare_status()
+    pr.close()
