@@ -8,7 +8,7 @@
 //  * the tree is cut at level U (at most kMostUpper nodes).  What lies below a node of level U belongs to one CTA (nodes
 //    dealt round-robin): it alone writes there, and no other CTA has to be waited for below level U;
 //  * levels go in steps of a group of 8, 16 or 32 entries (fanouts 2 and 4: four and two levels a step).  The CTA stages
-//    the levels of the first steps below U whole, as far as they fit (kPortionFloats); of the steps below those it fetches
+//    the levels of the first steps below U whole, as far as that pays (kPortionFloats); of the steps below those it fetches
 //    the groups that its entries fall into, all of them at once and as soon as the indices are known -- while the transform
 //    runs -- into rows of shared memory, which a hash table per step finds.  New values are written into the rows and summed up
 //    from row to row, from staged level to staged level: what separates the steps is a barrier of eight warps, not
@@ -40,7 +40,11 @@ constexpr uint32_t kMostEach = 4;                           // entries of the ba
 constexpr uint32_t kMostEntries = kTreeThreads * kMostEach; // update entries, and inserted leaves
 constexpr uint32_t kMostUpper = 1024;                       // nodes of level U
 constexpr uint32_t kUpperLevels = 12;
-constexpr uint32_t kPortionFloats = 14336;                  // staged entries below level U, per CTA
+// Staged entries below level U, per CTA: of a batch of one entry a thread, and of larger ones.  All of them are fetched and every staged group is looked
+// at whatever the batch, so a small batch rather works one more level off as groups of its own: us a call in a graph, 14336 / 8192: fanout 8, 2^20 slots, updates
+// of 32 5.67 / 4.08 (4.88 with prb_tree.cu), steps of 32 8.81 / 7.42; 2^23 slots 5.81 / 4.63; fanout 16, 2^21 slots 4.91 / 4.05, steps of 256 + 256
+// 8.79 / 8.20; fanout 32, 2^22 slots 4.75 / 3.99.  400 + 400 entries in the same trees: fanout 8 9.56 / 9.20, but 16 9.04 / 9.32, 32 9.19 / 9.58, 4 11.74 / 12.00.
+constexpr uint32_t kPortionFloats = 8192, kPortionFloatsMany = 14336;
 constexpr uint32_t kMostStaged = 4, kMostPasses = 8;
 constexpr uint32_t kMostSeen = 64;
 constexpr uint32_t kStepSmem = 200u * 1024u;
@@ -985,7 +989,7 @@ bool plan_step(const PrbView& v, uint32_t parts, bool many, StepPlan& p, uint32_
     const uint32_t steps = (D - p.U) / S;
     for (uint32_t s = 1; s < steps && s <= kMostStaged; ++s) {
         const uint64_t here = (uint64_t)p.own << (lgM * (s - 1u));      // groups
-        if ((floats + here * (M + 4u)) * trees > kPortionFloats) break;
+        if ((floats + here * (M + 4u)) * trees > (many && M > 8u ? kPortionFloatsMany : kPortionFloats)) break;
         p.portion_at[s] = floats;
         p.dirty_at[s] = groups;
         floats += (uint32_t)here * (M + 4u);

@@ -2,8 +2,9 @@
 those steps in L2, the tree work alone with a min-tree or with frames, batches that go in rounds, insertions beyond what the
 cluster takes -- against the oracle.
 
-Steps of groups, by the kernel's own cut: two from 2^21 + 1 slots on for fanouts 2, 4 and 16, from 2^20 + 1 for 8, from 2^22 + 1 for 32; three for fanout 8 from
-2^22 + 1; with a min-tree earlier by a factor of two."""
+Steps of groups, by the kernel's own cut: two from 2^20 + 1 slots on for fanouts 2, 4 and 16 (batches of more than 256: 2^21 + 1), from 2^19 + 1 for 8, from
+2^21 + 1 (2^22 + 1) for 32; three for fanout 8 from 2^22 + 1; with a min-tree earlier by a factor of two or more.  Fewer CTAs, which a small batch gets, stage
+less."""
 import numpy as np
 import pytest
 
