@@ -588,7 +588,7 @@ constexpr uint32_t kTreeSmem = 2u * kPrbTopFloats * 4u + 2u * 2u * kGridList * 4
 
 }  // namespace
 
-// Which form.  One CTA while the entries' groups of a pass come to at most 2 K entries (8 KB); a cluster of 16 CTAs
+// Which form, of the calls that prb_step.cu does not take.  One CTA while the entries' groups of a pass come to at most 2 K entries (8 KB); a cluster of 16 CTAs
 // beyond -- one SM pulls and stores scattered groups so slowly that they outlast the round trip.  us a call in a graph, one CTA /
 // 16: fanout 16, 48 + 48 entries 5.25 / 5.23, 96 + 96 5.5 / 5.3, 112 + 112 5.9 / 5.4; fanout 32, 48 + 48 5.6 / 5.3, 64 + 64 5.8 /
 // 5.4; fanout 4, 112 + 112 6.8 / 6.5; fanout 2, 48 + 48 7.5 / 7.0, 64 + 64 7.7 / 7.0; called eagerly a single CTA is the
@@ -648,10 +648,16 @@ int prb_launch_tree(const PrbView& v, const PrbTreeArgs& t, cudaStream_t s, bool
         const int b = a < 0 ? -1 : prb_launch_tree(v, w, s, dependent);
         return b < 0 ? -1 : a + b;
     }
-    if (t.most_ctas == 0 && !t.linked && (t.B || t.n <= kTreeThreads / 2u)) {
+    // (insertions alone that are more than a leaf a thread there: only where this file's cluster has many passes to make)
+    const bool alone = t.B == 0, few = t.n + v.stack <= 256u;
+    const bool deep = v.fanout == 2u || ((v.fanout == 4u || v.min_off) && v.capacity > 1u << 15);
+    if (t.most_ctas == 0 && !t.linked && (!alone || few || (deep && t.n <= kTreeThreads / 2u))) {
         // up to one cluster's worth of entries in a tree that it takes (prb_step.cu).  us a call in a graph, this file's cluster / that one: fanout
-        // 16, 2^20 slots, 256 entries 5.1 / 4.1, 256 + 256 5.6 / 4.4, 64 + 64 5.4 / 4.1, 256 insertions 4.1 / 3.9; fanout 2, 1000 + 777 8.9 / 6.2;
-        // fanout 32, 2^22 slots, 1024 + 1024 7.7 / 6.4 -- and 1024 insertions alone 5.4 / 5.9: their rows are better copied by CTAs of their own
+        // 16, 2^20 slots, 256 entries 5.1 / 4.1, 256 + 256 5.6 / 4.4, 64 + 64 5.4 / 4.1, 256 insertions 4.1 / 3.5; fanout 2, 1000 + 777 8.9 / 6.2;
+        // fanout 32, 2^22 slots, 1024 + 1024 7.7 / 6.4 -- and 1024 insertions alone 5.4 / 5.9: their rows are better copied by CTAs of their own.  400
+        // insertions alone: fanout 2, 2^15 slots 5.3 / 4.5; 4, 2^20 slots 5.0 / 4.3; 8, 2^20 slots 4.5 / 5.2; 16, 3000 slots 3.3 / 3.8; 32, 2^15 slots 3.65 / 4.06; with a
+        // min-tree 512 at fanout 8, 2^20 slots 5.6 / 5.1, at 32, 2^15 slots 4.65 / 4.83; 4, 3000 slots 3.63 / 3.84.  Fanouts 4 and 8, 2^18 slots, 64 + 64 entries:
+        // 5.6 / 3.9 and 5.0 / 4.1.
         const int k = prb_launch_step(v, t, nullptr, s, dependent);
         if (k != 0) return k;
     }
