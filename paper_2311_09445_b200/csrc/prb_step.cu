@@ -963,7 +963,7 @@ uint32_t most_parts(StepKernel k, uint32_t ki, uint32_t form, bool many, int dev
 // Cut, staged steps and shared memory of a launch; false: a tree or batch this kernel does not take.
 bool plan_step(const PrbView& v, uint32_t parts, bool many, StepPlan& p, uint32_t& smem)
 {
-    static_assert(kMostUpper / 8u <= kTreeThreads, "a thread each fetches a CTA's nodes of level U");
+    static_assert(kMostUpper / 4u <= kTreeThreads, "a thread each fetches a CTA's nodes of level U");
     const uint32_t S = v.fanout == 2 ? 4u : v.fanout == 4 ? 2u : 1u, lg = v.log2_fanout, lgM = lg * S, M = 1u << lgM, D = v.depth, N = (uint32_t)v.capacity;
     p.U = 0;
     for (uint32_t u = 1; u + S <= D && u < kUpperLevels; ++u)
@@ -1049,9 +1049,17 @@ int prb_launch_step(const PrbView& v, const PrbTreeArgs& t, const PrbSampleArgs*
     const int dev = prb_current_device();
     const uint32_t form = sample ? 0u : v.min_off ? (v.stack ? 4u : 3u) : v.stack ? 2u : 1u;
     bool many = t.B > kTreeThreads || (t.n && t.n + v.stack > kTreeThreads);
-    // (as many CTAs as there may be, whatever the batch: 4 / 8 / 16, us a step: 32 entries 7.4 / 7.2 / 7.2, 256 + 256 10.2 / 9.5 / 8.3,
-    // 1000 + 777 34 / 16.8 / 12.6; through host buffers, every CTA reading the batch over the link, 40.6 / 39.1 / 37.6)
+    // As many CTAs as there may be -- 4 / 8 / 16, us a step: 256 + 256 entries 10.2 / 9.5 / 8.3, 1000 + 777 34 / 16.8 / 12.6; through host buffers, every CTA
+    // reading the batch over the link, 40.6 / 39.1 / 37.6 -- but fewer for a small batch: the CTAs of a cluster start together, on SMs of one
+    // group, and beside a learner's kernels on another stream that is what a small call waits for.  us a call, 4 / 8 / 16 CTAs, fanout 16, 2^20 slots, alone (in a
+    // graph) and beside matrix products of 4096^3 in bfloat16: updates of 32 3.89 / 3.82 / 3.83 and 5.9 / 11.7 / 36; 64 + 64 4.08 / 3.95 / 3.96; steps of 32 6.76 / 6.73 /
+    // 6.82 and 12 / 21 / 38; of 64 + 64 7.06 / 7.00 / 7.00 and 14 / 22 / 45.  (As two kernels 6.6 beside them for the update, 25 and 94 for the steps.)  In larger trees
+    // eight CTAs have more of the tree each than they stage: fanout 4, 2^22 slots, steps of 32 10.4 / 9.9 / 9.2.
+    const uint32_t entries = t.n ? t.n + v.stack : 0u, largest = sample && sample->B > entries ? sample->B : entries;
+    const bool small = t.B <= 64u && largest <= 64u && v.capacity <= 1u << 20;
+    const uint32_t want = t.linked ? kStepParts : !sample && t.n == 0u && t.B <= 32u ? 4u : small ? 8u : kStepParts;
     uint32_t parts = most_parts(step_kernel(v.fanout, form, many), v.log2_fanout, form, many, dev);
+    if (parts > want) parts = want;
     if (parts == 1u || (sample && (sample->B > parts * kTreeThreads || sample->B > kPrbClusterStrata))) return 0;
     p.state = v.state;
     p.level0 = v.level[0];

@@ -107,3 +107,32 @@ def test_insertions_beyond_the_cluster_of_the_iteration(oracle_mod, K):
         _check(pr)
     pr.compare_rows(np.arange(0, pr.gpu.info()[0], 3, dtype=np.int32))
     pr.close()
+
+
+@pytest.mark.parametrize("K,N,kw", [(2, 4096, {}), (2, 1_000_003, {}), (4, 1000, {}), (4, 2_100_003, {}), (8, 100, {}), (8, 1 << 20, {}), (8, 1 << 21, {}), (16, 5000, {}),
+                                    (16, 1 << 20, {}), (32, 40_000, {}), (32, 1_100_000, {}), (2, 1 << 18, dict(min_tree=True)), (16, 1 << 20, dict(min_tree=True)),
+                                    (32, 1 << 20, dict(min_tree=True)), (4, 33_000, dict(min_tree=True)), (8, 300_007, dict(frame_stack=4, obs=32, store=True)),
+                                    (16, 1 << 20, dict(frame_stack=4, obs=32, store=True, min_tree=True))])
+def test_few_entries(oracle_mod, K, N, kw):
+    # around the lines at which a small batch gets fewer CTAs, and at which insertions alone go to the other kernel; with the same entries in one CTA's part
+    pr, rng = _filled(oracle_mod, N, K, **kw)
+    for B, n in [(1, 0), (31, 0), (32, 0), (33, 0), (64, 0), (65, 0), (32, 1), (64, 60), (64, 64), (65, 10), (10, 65),
+                 (0, 1), (0, 60), (0, 64), (0, 65), (0, 252), (0, 256), (0, 257), (0, 512), (0, 513)]:
+        if n > N // 2:
+            continue
+        new = _new(rng, n, pr) if n else None
+        fill = pr.gpu.info()[0]
+        for span in (0, min(5, fill // 2)) if B else (0,):
+            idx, td = _indices(rng, fill, B, span), rng.standard_normal(B).astype(np.float32)
+            if B and n:
+                pr.update_insert(idx, td, 0.6, 1e-6, new)
+            elif B:
+                pr.update(idx, td, 0.6, 1e-6)
+            else:
+                pr.insert(new)
+        if B in (1, 33, 64) or n in (65, 257, 513):
+            _check(pr, kw.get("min_tree", False))
+        if "frame_stack" not in kw and not kw.get("min_tree") and B and B <= 64 and n:
+            pr.step(_indices(rng, fill, B, 0), td, 0.6, 1e-6, _new(rng, n, pr), 64, 0.4, 3)
+    _check(pr, kw.get("min_tree", False))
+    pr.close()
