@@ -156,7 +156,7 @@ def test_overlapping_arrays_take_the_other_route(oracle_mod):
 def test_long_rows_left_out(oracle_mod, captured):
     # a buffer of long rows whose iteration leaves them out goes in one launch, between iterations that copy them on the handle's streams
     rng = np.random.default_rng(5)
-    N, E, B, n = 2000, 16_384, 64, 48
+    N, E, B, n = 1800, 16_384, 64, 48                                          # (the ring is full: every row that is compared has been written)
     stream = torch.cuda.Stream()
     from paper_2311_09445_b200 import PrioritizedReplay
     gpu = PrioritizedReplay(N, 16, E, 4, 1024, stream=stream)
@@ -217,7 +217,7 @@ def test_long_rows_left_out(oracle_mod, captured):
                 if out[i][f] is not None:
                     assert np.array_equal(out[i][f].cpu().numpy().view(np.uint8).reshape(-1), np.ascontiguousarray(o[f]).view(np.uint8).reshape(-1)), (i, f)
     assert gpu.info() == ora.info() and gpu.sync() == ora.status()
-    keep = np.arange(0, 2000, 7, dtype=np.int32)
+    keep = np.arange(0, 1800, 7, dtype=np.int32)
     a, g = ora.read_rows(keep), gpu.read_rows(keep)
     for f in ("obs", "act", "rew", "next_obs", "done"):
         assert np.array_equal(np.ascontiguousarray(a[f]).view(np.uint8).reshape(-1), np.ascontiguousarray(g[f]).view(np.uint8).reshape(-1)), f
