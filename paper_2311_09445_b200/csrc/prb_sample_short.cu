@@ -402,30 +402,13 @@ prb_sample_grid_kernel(const __grid_constant__ ShortPlan plan)
             __syncthreads();
         }
     }
-    if (tid == kShortThreads - 1u) {
-        s_min = ~(unsigned)__ldcg(&plan.state->wide_wmax_bits);
-        if (exchange && s_last) asm volatile("fence.sc.gpu;" ::: "memory");
-    }
+    // (what the last CTA does is the call's tail -- the fence, the looks for raised words and the bookkeeping's atomic each a round trip -- so the fence is
+    // another thread's than the read of the minimum, the looks are on their way while the weights are formed, and the atomic does not wait for them: us a
+    // sample of 4096 strata in a graph, fanout 8, 262144 slots, one after the other / with an ordinary kernel between them: 8.7 / 9.8 as a cooperative launch, 8.3 / 10.7 with one of
+    // these behind the other, 7.65 / 10.1 so; 65536 strata 15.8 / 17.5, 15.0 / 18.2, 14.4 / 17.4)
+    if (tid == kShortThreads - 1u) s_min = ~(unsigned)__ldcg(&plan.state->wide_wmax_bits);
+    if (tid == 0u && exchange && s_last) asm volatile("fence.sc.gpu;" ::: "memory");
     __syncthreads();
-    if (exchange) pmin = __uint_as_float(s_min);
-    const double log_pmin = plan.uniform ? 0.0 : log2_of(pmin);
-    if (plan.out_w != nullptr && (!exchange || s_all))
-        for (uint32_t k = k_lo + tid; k < k_hi; k += kShortThreads)
-            plan.out_w[k] = plan.uniform ? 1.0f : weight_of(plan, log2_of(kept ? plan.kept[k] : p), log_pmin);
-    if (exchange && s_last) {
-        // the CTAs that could not wait for this one
-        for (uint32_t c = tid; c < gridDim.x; c += kShortThreads) {
-            uint32_t up;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(up) : "l"(raised + c) : "memory");
-            if (up) s_idx[atomicAdd(&s_late, 1u)] = c;
-        }
-        __syncthreads();
-        for (uint32_t e = 0; e < s_late; ++e) {
-            const uint32_t c = s_idx[e], hi = (uint32_t)(((uint64_t)(c + 1u) * plan.B) / gridDim.x);
-            for (uint32_t k = (uint32_t)(((uint64_t)c * plan.B) / gridDim.x) + tid; k < hi; k += kShortThreads)
-                plan.out_w[k] = weight_of(plan, log2_of(__ldcg(plan.kept + k)), log_pmin);
-        }
-    }
     if (tid == kShortThreads - 1u && prb_ticket(&plan.state->sample_done) == gridDim.x - 1u) {
         // the last CTA to have read what the others have given: the call's bookkeeping
         plan.state->wide_wmax_bits = 0ull;
@@ -433,6 +416,26 @@ prb_sample_grid_kernel(const __grid_constant__ ShortPlan plan)
         plan.state->sample_done = 0u;
         plan.state->sample_calls = calls + 1;
         if (plan.buffer_norm) plan.state->pmin_bits = ~0ull;      // (ready for the next scan)
+    }
+    uint32_t up = 0u;
+    if (exchange && s_last && tid < gridDim.x) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(up) : "l"(raised + tid) : "memory");
+    if (exchange) pmin = __uint_as_float(s_min);
+    const double log_pmin = plan.uniform ? 0.0 : log2_of(pmin);
+    if (plan.out_w != nullptr && (!exchange || s_all))
+        for (uint32_t k = k_lo + tid; k < k_hi; k += kShortThreads)
+            plan.out_w[k] = plan.uniform ? 1.0f : weight_of(plan, log2_of(kept ? plan.kept[k] : p), log_pmin);
+    if (exchange && s_last) {
+        // the CTAs that could not wait for this one
+        if (up) {
+            asm volatile("fence.acq_rel.gpu;" ::: "memory");
+            s_idx[atomicAdd(&s_late, 1u)] = tid;
+        }
+        __syncthreads();
+        for (uint32_t e = 0; e < s_late; ++e) {
+            const uint32_t c = s_idx[e], hi = (uint32_t)(((uint64_t)(c + 1u) * plan.B) / gridDim.x);
+            for (uint32_t k = (uint32_t)(((uint64_t)c * plan.B) / gridDim.x) + tid; k < hi; k += kShortThreads)
+                plan.out_w[k] = weight_of(plan, log2_of(__ldcg(plan.kept + k)), log_pmin);
+        }
     }
 }
 
@@ -571,6 +574,7 @@ int prb_launch_sample_short(const PrbView& v, uint32_t B, float beta, uint64_t s
         uint32_t grid = (B + strata - 1) / strata;
         const uint32_t room = (uint32_t)prb_sm_count() * lim->per_sm;
         if (grid > room) grid = room;
+        if (grid > kShortThreads) grid = kShortThreads;      // (a thread looks at a CTA's word)
         cfg.gridDim = dim3(grid);
         a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         a[0].val.programmaticStreamSerializationAllowed = 1;
