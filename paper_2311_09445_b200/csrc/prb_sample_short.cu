@@ -315,7 +315,12 @@ prb_sample_grid_kernel(const __grid_constant__ ShortPlan plan)
     for (uint32_t i = 0; i < kStagedUnits; ++i) unit[i] = plan.uniform ? StagedUnit{nullptr, 0u} : staged_unit(plan, s_top, tid + i * kShortThreads);
     if (tid < plan.n_steps) s_step[tid] = plan.step[tid];
     if (tid == 0) { s_min = 0xFFFFFFFFu; s_flags = 0u; s_late = 0u; }
-    const PrbWordShare share = prb_word_share(plan.words, tid >> 5, warps);
+    // (Where a warp's words lie is looked up ahead -- or, at the fanouts whose walks need the registers, behind the walk, where most warps wait anyway: kept across it
+    // it was spilled, and every copy read it back.  us a sample in a graph, 262144 slots, 68-byte observations, ahead / behind: fanout 2, 4096 strata 8.99 / 8.18, 65536 17.7 / 15.4;
+    // 32, 4096 9.3 / 8.3, 65536 18.3 / 15.5; a step of 16384 27.9 / 26.0 and 24.7 / 23.4; but fanouts 4, 8 and 16, which spill nothing, 24.5 / 24.9, 22.4 / 22.6, 22.4 / 22.8.)
+    constexpr bool kBehind = K == 2 || K == 32;
+    PrbWordShare share = {};
+    if (!kBehind) share = prb_word_share(plan.words, tid >> 5, warps);
     prb_dep_wait();
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const unsigned long long calls = plan.state->sample_calls;
@@ -363,6 +368,7 @@ prb_sample_grid_kernel(const __grid_constant__ ShortPlan plan)
                 if (fl) atomicOr(&s_flags, fl);
             }
         }
+        if (kBehind) share = prb_word_share(plan.words, tid >> 5, warps);
         __syncthreads();
         if (last && tid == kShortThreads - 1u) {
             // this CTA's smallest priority goes out; who else has given one is looked at when the rows have been copied
