@@ -43,7 +43,7 @@ constexpr uint32_t kClusterWords = 400u << 10;       // ... or words
 #ifdef PEARL_CHECKED
 constexpr uint32_t kGridPolls = 0;
 #else
-constexpr uint32_t kGridPolls = 64;
+constexpr uint32_t kGridPolls = 512;
 #endif
 constexpr uint32_t kLaneGroupUnits = 160;            // units of a row up to which the lane-group kernel comes next
 constexpr uint32_t kNotStaged = 0xFFFFFFFFu;
@@ -389,8 +389,10 @@ prb_sample_grid_kernel(const __grid_constant__ ShortPlan plan)
     if (exchange) {
         if (tid == kShortThreads - 1u) {
             s_last = given == gridDim.x - 1u;
-            // (a while, some 20 us, is waited all the same: CTAs whose SMs the kernel before this one held start later, and what is left to the
-            // last one it does alone)
+            // (a while, some 150 us, is waited all the same: CTAs whose SMs other kernels hold start later, and what is left to the last one it does
+            // alone.  16384 strata beside matrix products of 4096^3 in bfloat16 on another stream, us a sample and a product, fanout 16: no look 262 and 200, 8 looks
+            // 147 and 165, 64 102 and 120, 512 74 and 92; a cooperative launch, whose CTAs all wait, 93 and 93; 2048 strata 61, 21, 25, 31 and 86.  Alone all numbers from 8 on measured
+            // the same.)
             bool all = s_last;
             for (uint32_t spins = 0; spins < kGridPolls && !all; ++spins) all = all_given();
             s_all = all;
