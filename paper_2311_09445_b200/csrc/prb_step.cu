@@ -92,6 +92,13 @@ template <int K> __device__ __forceinline__ uint32_t padded(uint32_t f) { return
 // Barriers: 1 the tree warps' own (8 with the insertion's groups), 4 the other warps'; 7 the list of entries, 5 their groups are there; 6 the
 // groups are done with; 3 everything below level U is stored; 2 the sampled indices are there.
 __device__ __forceinline__ void tree_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kTreeThreads) : "memory"); }
+// ... which says whether all its threads still hold sound sums
+__device__ __forceinline__ bool tree_sync_all(bool sound)
+{
+    uint32_t all;
+    asm volatile("{ .reg .pred p, q; setp.ne.u32 p, %1, 0; barrier.cta.red.and.pred q, 1, %2, p; selp.u32 %0, 1, 0, q; }" : "=r"(all) : "r"(sound ? 1u : 0u), "n"(kTreeThreads) : "memory");
+    return all != 0u;
+}
 template <uint32_t kEach> __device__ __forceinline__ void sum_sync() { asm volatile("bar.sync 8, %0;" ::"n"(kTreeThreads + kGroupThreads<kEach>) : "memory"); }
 template <uint32_t kEach> __device__ __forceinline__ void copy_sync() { asm volatile("bar.sync 4, %0;" ::"n"(kCopyThreads + kGroupThreads<kEach>) : "memory"); }
 
@@ -288,7 +295,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
     __shared__ uint32_t s_idx[kTreeThreads];
     __shared__ SeenLeast s_seen[kSample ? kMostSeen : 1];
     __shared__ __align__(8) unsigned long long s_bar_up, s_bar_vis, s_bar_seen;
-    __shared__ unsigned s_count, s_found, s_refused, s_lost;
+    __shared__ unsigned s_count, s_found, s_refused;
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, rank = blockIdx.x;
     const uint32_t parts = 1u << plan.log_parts, mask = parts - 1u, lp = plan.log_parts;
     float* const up = reinterpret_cast<float*>(s_dyn);
@@ -323,7 +330,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (receives) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_up), "r"((plan.n_u + 3u) / 4u * (kMin ? 32u : 16u)) : "memory");
         if (kSample) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_seen), "r"((uint32_t)sizeof(SeenLeast) * strata_warps * parts) : "memory");
-        s_count = 0u; s_found = 1u; s_refused = 0u; s_lost = 0u;
+        s_count = 0u; s_found = 1u; s_refused = 0u;
     }
     if (tid >= kThreads - PRB_MAX_LEVELS) s_off[tid - (kThreads - PRB_MAX_LEVELS)] = plan.off[tid - (kThreads - PRB_MAX_LEVELS)];
     {
@@ -772,17 +779,15 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
         }
         // the levels above U, S at a time while there are as many (what the next turn needs is looked up ahead of it); once a
         // level's nodes fit a warp the first warp goes on alone
-        // (a thread whose wait for level U ran out marks the CTA as lost, and after the next barrier no thread stores a sum: its own, in time,
-        // saw all of level U.  In time, not late: a walk that reads a peer's memory begins within one limit of polls, and the peer
-        // stays for two, see bar_seen)
+        // (A warp one of whose threads' wait for level U was not over in time stores no sum, nor does any that sums up what other warps have summed
+        // then: the barriers between them carry the answer, which as a word in shared memory cost a step 0.15 us.  In time, not late: a walk that reads
+        // a peer's memory begins within one limit of polls, and the peer stays for two, see bar_seen.)
         bool sound;
-        auto still_sound = [&]() { return *const_cast<volatile unsigned*>(&s_lost) == 0u; };
         {
             uint32_t l = plan.U, h = 0, count = 0, from = 0;
             auto turn = [&]() { h = l >= (uint32_t)S ? (uint32_t)S : 1u; count = prb_nodes_covering(N, lg * (D - l + h)); from = plan.up[l]; };
             turn();
-            sound = prb_wait_first_phase<true>(plan.state, bar_up) == kPrbInTime;
-            if (!sound) s_lost = 1u;
+            sound = __all_sync(0xFFFFFFFFu, prb_wait_first_phase<true>(plan.state, bar_up) == kPrbInTime);
             bool alone = false;
 #pragma unroll 1
             while (true) {
@@ -800,11 +805,9 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
                 if (l == 0u) break;
                 turn();
                 if (alone) __syncwarp();
-                else tree_sync();
-                sound = still_sound();
+                else sound = tree_sync_all(sound);
             }
-            tree_sync();
-            sound = still_sound();
+            sound = tree_sync_all(sound);
         }
         const uint64_t filled = min((uint64_t)fill + plan.n, (uint64_t)N);
         // (every CTA's warps have the cursor in hand once bar_vis is over)
@@ -823,7 +826,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
             // ---- the sample ----
             const float total32 = up[plan.up[0]];
             const double total = (double)total32;
-            const bool empty = sound && (filled == 0u || !(total32 > 0.0f));
+            const bool empty = filled == 0u || !(total32 > 0.0f);
             const bool holds = k < k_hi;
             uint32_t leaf = 0;
             float p = 1.0f;
@@ -867,7 +870,7 @@ prb_step_kernel(const __grid_constant__ StepPlan plan)
                 __syncwarp();
                 asm volatile("bar.arrive 2, %0;" ::"n"(kThreads) : "memory");      // the copying warps may go on
                 if (wflags) atomicOr(&plan.state->status, wflags);
-                if (empty) {
+                if (empty && sound) {
                     if (rank == 0u && tid == 0u) atomicOr(&plan.state->status, PEARL_ST_EMPTY);
                     return;
                 }

@@ -25,6 +25,6 @@ def test_no_wait_is_taken_for_granted():
     for at in waits:
         assert re.match(r" == kPrb(InTime|Never)", text[at:]), text[at - 80:at + 40]
     # level U's wait decides about the sums that CTA 0 stores, and with the visibility's about cursor, walk and indices
-    assert text.count("rank == 0u && sound, l, from, i)") == 4
+    assert text.count("rank == 0u && sound, l, from, i)") == 4 and text.count("sound = tree_sync_all(sound);") == 2
     assert "if (sound) move_cursor();" in text and "&& sound) move_cursor();" in text
     assert "if (walks && sound)" in text and "if (holds && sound) plan.out_idx[k]" in text
