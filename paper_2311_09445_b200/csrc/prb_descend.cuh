@@ -23,9 +23,12 @@ __device__ __forceinline__ uint32_t philox4x32_10_word0(uint32_t c0, uint32_t c1
     return c0;
 }
 
-// a / b rounded to nearest, from y = 1 / b rounded to nearest: one correction of a y by its exact remainder gives the correctly rounded
-// quotient (P. W. Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", IBM J. Res. Dev. 34 (1990),
-// theorem 8.3; no overflow or underflow here: a is a binary32 sum, b a batch size).  Three dependent operations where y is known ahead.
+// a / b rounded to nearest, from y = 1 / b rounded to nearest: one correction of a y by its exact remainder (P. W. Markstein, "Computation of
+// elementary functions on the IBM RISC System/6000 processor", IBM J. Res. Dev. 34 (1990), theorem 8.3).  The theorem wants a first
+// quotient within a unit in the last place; here it is the operands that make the result exact: a has 24 bits (a binary32 sum) and b 11 (strata of a
+// cluster), so a / b lies at least 2^-65 of itself from any midpoint of two binary64, and the corrected value is
+// within 2^-100 of it before its one rounding.  No overflow or underflow: a is a finite binary32.  Three dependent operations where y is known ahead.
+// (tests/test_step_plan.py compares it with the rounded quotient.)
 __device__ __forceinline__ double prb_quotient(double a, double b, double y)
 {
     const double q = __dmul_rn(a, y);
