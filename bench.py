@@ -575,7 +575,7 @@ def run_ours(args, wl, rank, world):
                              "peak": peak, "unit": "GB/s", "frac": step_bytes / (ms / args.steps * 1e-3) / 1e9 / peak}
     if n_ins:
         ins_bytes = n_ins * (2 * E + 4)
-        line["roofline_insert"] = {"kernel": "prb_insert_rows_kernel" if long_rows else "prb_tree_kernel", "bound": "hbm",
+        line["roofline_insert"] = {"kernel": "prb_insert_rows_kernel" if long_rows else "prb_step_kernel" if n_ins <= 256 else "prb_tree_kernel", "bound": "hbm",
                                    "bytes_per_launch": ins_bytes,
                                    "achieved": ins_bytes / (m["ms_insert"] * 1e-3) / 1e9, "peak": peak, "unit": "GB/s",
                                    "frac": ins_bytes / (m["ms_insert"] * 1e-3) / 1e9 / peak}

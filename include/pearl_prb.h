@@ -248,8 +248,10 @@ int pearl_prb_update_insert(pearl_prb_t* prb, uint32_t B, const int32_t* d_idx, 
  * eps, n, d_new_*...) -- followed by the sample of the next batch -- exactly pearl_prb_sample(prb, B,
  * beta, seed, d_idx, d_w, d_obs ...): same results, same state, same status bits as the two calls.
  * What the one call buys is one host call per iteration with all arguments checked before anything is
- * enqueued; the kernels are those of the two calls (for rows of 8 KB and more: the tree kernel beside the
- * copy of the new rows, then the sample).  d_upd_idx may be the d_idx of the previous step: it is read
+ * enqueued, and for short rows (the fields given come to at most 64 words) one launch: up to 1024 updates, 1024 insertions with
+ * priorities and 1536 strata, no frames, no min-tree, and no array that is read overlapping one that is written
+ * (d_upd_idx and d_idx excepted).  Otherwise the kernels are those of the two calls (for rows of 8 KB and
+ * more: the tree kernel beside the copy of the new rows, then the sample).  d_upd_idx may be the d_idx of the previous step: it is read
  * before d_idx is written.
  * n == 0 stands for an iteration without new transitions (update, then sample; the d_new_* are not read).
  * Arguments and errors as for the two calls; nothing is enqueued if any argument is refused. */

@@ -633,8 +633,8 @@ static int step_in_one(pearl_prb_t* h, uint32_t B_upd, const int32_t* d_upd_idx,
                        float* d_w, void* const out[PRB_NUM_FIELDS])
 {
     if (h->view.stack || h->view.min_off || (n && !d_new_prio)) return PEARL_STEP_IN_PARTS;
-    // (inputs over the link, which every CTA reads: 256 + 256 entries 37.9 -> 36.4 us, but a larger batch is better read by the four CTAs of the other
-    // route)
+    // (inputs over the link, which every CTA reads: from pinned arrays, fanout 16, 2^20 slots, two launches / one: 64 + 64 entries 31.9 / 31.3 us, 128 + 128 33.3 / 32.7, 256 + 256
+    // 37.7 / 36.4; fanout 2, 2^17 slots 33.4 / 31.0, 34.9 / 32.5, 39.6 / 36.1; a larger batch is better read by the four CTAs of the other route)
     if (h->linked_inputs && (B_upd > 256u || n > 256u)) return PEARL_STEP_IN_PARTS;
     struct Range { uintptr_t at, end; };
     Range reads[PRB_NUM_FIELDS + 3], writes[PRB_NUM_FIELDS + 2];

@@ -20,7 +20,7 @@
 // Two shapes, by batch size.  Up to kClusterStrata strata: one thread-block cluster of up to 16 CTAs; p_min goes
 // through distributed shared memory (each transfer signals the receiver's barrier), nothing through global
 // memory.  More: a grid; p_min by an atomic per CTA, and no CTA depends on another's being there: one that has copied its rows and does not
-// soon see that all have given theirs leaves its weights to the last that does.  (As a cooperative launch whose CTAs waited for the others it could be no
+// see within some 150 us that all have given theirs leaves its weights to the last that does.  (As a cooperative launch whose CTAs waited for the others it could be no
 // programmatic dependent: 4096 strata 24.6 -> 22.6 us a step with its tree kernel, 65536 55.4 -> 53.9.)
 #include "prb_walk.cuh"
 #include "prb_rows.cuh"
@@ -334,7 +334,7 @@ prb_sample_grid_kernel(const __grid_constant__ ShortPlan plan)
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     if (poisoned) {
-        // (a launch of co-resident CTAs gave up at its barrier once: see PrbState::wide_poisoned)
+        // (CTAs that wait for one another gave up once: see PrbState::wide_poisoned)
         if (tid == 0 && blockIdx.x == 0) atomicOr(&plan.state->status, PEARL_ST_INTERNAL);
         return;
     }

@@ -20,8 +20,8 @@
 //  * rows of the insertion are copied by warps of their own meanwhile, and a sampled slot that this very call inserts is
 //    read from the insertion's batch: nobody waits for the copy.
 // us a step, two kernels / this one: captured, fanout 16, 2^20 slots, 256 + 256 entries 10.0 / 8.3; fanout 2, 10^6 slots, 1000 + 777
-// 14.9 / 12.6; called eagerly, 32 entries of a 4096-slot binary tree 10.2 / 7.5, 64 + 64 of 2^20 slots 11.8 / 8.8; through host
-// buffers, 256 + 256 37.9 / 36.4.  Of the 8.3: 1.4 between the kernels, 1.4 until the groups are there, 1.2 up to level U, 0.7 to
+// 14.9 / 12.6; called eagerly, 32 entries of a 4096-slot binary tree 10.2 / 7.5, 64 + 64 of 2^20 slots 11.8 / 8.8; through pinned host
+// arrays, 256 + 256 entries, fanout 16, 2^20 slots 37.7 / 36.4, fanout 2, 2^17 slots 39.6 / 36.1.  Of the 8.3: 1.4 between the kernels, 1.4 until the groups are there, 1.2 up to level U, 0.7 to
 // the root, 2.1 down to the leaf, 1.2 for weights and rows.
 #include "prb_walk.cuh"
 #include "prb_groups.cuh"
@@ -38,7 +38,9 @@ template <uint32_t kEach> constexpr uint32_t kStepThreads = kTreeThreads + kCopy
 constexpr uint32_t kStepParts = 16;                         // CTAs of the cluster, at most
 constexpr uint32_t kMostEach = 4;                           // entries of the batch a thread looks at, at most
 constexpr uint32_t kMostEntries = kTreeThreads * kMostEach; // update entries, and inserted leaves
-constexpr uint32_t kMostUpper = 1024;                       // nodes of level U
+// Nodes of level U; half of it but for fanout 32, whose next cut would be 32 times coarser.  (Up to 1024 for all: fanout 16, 2^18 slots, steps of 256 + 256 7.02 -> 7.35 us,
+// fanout 4 9.20 -> 9.59, fanout 2, 2^14 slots 7.00 -> 7.34.)
+constexpr uint32_t kMostUpper = 1024;
 constexpr uint32_t kUpperLevels = 12;
 // Staged entries below level U, per CTA: of a batch of one entry a thread, and of larger ones.  All of them are fetched and every staged group is looked
 // at whatever the batch, so a small batch rather works one more level off as groups of its own: us a call in a graph, 14336 / 8192: fanout 8, 2^20 slots, updates
